@@ -61,12 +61,21 @@ int xg_ctx::pick_cfg(int kind, uint32_t nstreams) const
 {
     const int fixed = cfg[kind == xg::kNormalSum ? xg::kNormal : kind];
     if (fixed >= 0) return fixed;
-    // Without a tuned choice: many streams -> few lanes per stream (fewer
-    // shuffles and 128-bit stores); few streams -> more lanes per stream.
-    const uint64_t lanes_wanted = (uint64_t)sm_count * 32 * 24;  // ~24 resident warps per SM
-    if ((uint64_t)nstreams * 8 >= lanes_wanted / 2) return xg::cfg_index(8, 4);
-    if ((uint64_t)nstreams * 16 >= lanes_wanted / 2) return xg::cfg_index(16, 2);
-    return xg::cfg_index(32, 2);
+    // Without a tuned choice, from a sweep of 100 .. 131072 streams at 2^28
+    // outputs on GB300 (ps per output):
+    //  * words, normals and fused sums: one warp per stream at every count.
+    //    Words 0.598 (32,2) against 0.735 (8,4) at 10000 streams, 0.603 / 0.641
+    //    at 16384; normals 1.258 / 1.779 and 1.211 / 1.456 ((8,4) needs 98
+    //    registers: 20 warps per SM, so its last wave is mostly empty).
+    //  * uniforms, bound by the integer pipe when few lanes idle, gain from
+    //    fewer shuffles once every SM sub-partition has warps enough: (16,2)
+    //    from 9 and (8,4) from 18 streams per sub-partition (5472 and 10944
+    //    streams): 0.735 (32,2) / 0.785 (16,2) / 0.885 (8,4) at 5000 streams,
+    //    0.679 / 0.659 / 0.743 at 6000, 0.685 / 0.695 / 0.727 at 10000,
+    //    0.670 / 0.648 / 0.633 at 12000, 0.663 / 0.662 / 0.641 at 16384.
+    const uint64_t parts = (uint64_t)sm_count * 4;
+    if (kind != xg::kUniform || nstreams < 9 * parts) return xg::cfg_index(32, 2);
+    return nstreams < 18 * parts ? xg::cfg_index(16, 2) : xg::cfg_index(8, 4);
 }
 
 int xg_ctx::pick_block(int kind, int c) const
