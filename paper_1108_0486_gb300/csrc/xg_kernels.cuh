@@ -374,10 +374,55 @@ struct UnitSrc {
     bool write_state = true;
 };
 
+// Run one round, of which the call takes the first h words (0 < h < W), and
+// move the ring on by h words in registers, so that the next round starts
+// with the call's word h.  Afterwards lane j holds words W j + h ..  of each
+// row: one shuffle and one select per row and word moved.
+template <class E, class Emit>
+__device__ __forceinline__ void advance_words(E& eng, Emit& em, uint32_t h)
+{
+    constexpr int W = E::WPL_, TPG = E::TPG_, N = E::NROWS;
+    uint32_t row[N + 1][W];   // the ring, oldest first, then the new round
+#pragma unroll
+    for (int t = 0; t < N; ++t)
+#pragma unroll
+        for (int i = 0; i < W; ++i) row[t][i] = eng.ring[t][i];
+    eng.template round<0>();
+    em.template tail<0>(eng, 0);
+#pragma unroll
+    for (int i = 0; i < W; ++i) row[N][i] = eng.ring[0][i];
+#pragma unroll 1
+    for (uint32_t c = 0; c < h; ++c) {
+#pragma unroll
+        for (int t = 0; t <= N; ++t) {
+            // the last lane takes the next row's first word; past the new
+            // round it takes a word that the ring does not keep
+            const uint32_t send = (t < N && eng.lane == 0) ? row[t < N ? t + 1 : N][0] : row[t][0];
+            const uint32_t in = __shfl_sync(eng.mask, send, (eng.lane + 1) % TPG, TPG);
+#pragma unroll
+            for (int i = 0; i + 1 < W; ++i) row[t][i] = row[t][i + 1];
+            row[t][W - 1] = in;
+        }
+    }
+#pragma unroll
+    for (int t = 0; t < N; ++t)
+#pragma unroll
+        for (int i = 0; i < W; ++i) eng.ring[t][i] = row[t][i];
+}
+
 // One call (or piece) on one stream s: n outputs of kind OUT written to row
 // (this stream's first output).  Returns the lane's partial sum for
 // kNormalSum.
-template <class P, int TPG, int WPL, int OUT, bool VEC, bool UNROLL2 = true>
+//
+// kShifted: words and uniforms take vector stores at any row address.  The
+// first 0 .. 3 words, up to the first aligned address, are written one by one
+// and the ring moves on by as many words (advance_words).  kScalar writes 4
+// bytes every 8 (W = 2) or 16 (W = 4) per instruction, which costs the L2 two
+// to four times the sectors: 10000 rows of 100003 words take 0.779 ms with it
+// at (32, 2) and 2.549 ms at (8, 4) against 0.618 and 0.677 ms kShifted
+// (0.588 and 0.713 ms for aligned rows of 100000).  Normals pair words inside
+// a lane and are bound by the transform: kScalar costs them 0.5%.
+template <class P, int TPG, int WPL, int OUT, int ST, bool UNROLL2 = true>
 __device__ __forceinline__ float run_stream(const State& st, uint32_t s, uint64_t n, uint32_t* row,
                                             uint32_t omega, int lane, unsigned mask,
                                             const UnitSrc& src = UnitSrc())
@@ -386,7 +431,8 @@ __device__ __forceinline__ float run_stream(const State& st, uint32_t s, uint64_
     constexpr int RW = E::RW;
     constexpr bool kNormalOut = (OUT == kNormal || OUT == kNormalSum);
     const uint64_t nwords = kNormalOut ? n + (n & 1u) : n;
-    Emit<E, OUT, VEC> em;
+    using Em = Emit<E, OUT, ST != kScalar>;
+    Em em;
     em.acc = 0.0f;
     if (nwords == 0) return 0.0f;
     E eng;
@@ -407,21 +453,36 @@ __device__ __forceinline__ float run_stream(const State& st, uint32_t s, uint64_
     em.wl = wp + (uint32_t)(WPL * lane + 1) * omega;
     em.dst = (OUT == kNormalSum) ? nullptr : row + em.lane_off;
     uint32_t retired[WPL];
-    const uint64_t nr = (nwords + RW - 1) / RW;
-    const int rot = drive<E, Emit<E, OUT, VEC>, UNROLL2>(eng, nr, em, retired);
+    uint64_t head = 0;
+    if constexpr (ST == kShifted) {
+        static_assert(!kNormalOut, "normals pair words inside a lane");
+        constexpr uint32_t A = WPL % 4 == 0 ? 4 : 2;   // words per vector store
+        const uint32_t h = (0u - (uint32_t)(reinterpret_cast<uintptr_t>(row) >> 2)) & (A - 1);
+        // a call of at most one turn of the ring has scalar stores only (tail)
+        if (h != 0 && nwords > (uint64_t)kR) {
+            em.limit = h;
+            advance_words(eng, em, h);
+            head = h;
+            em.limit = n - h;
+            em.wl = wp + (uint32_t)(WPL * lane + 1 + h) * omega;
+            em.dst = row + h + em.lane_off;
+        }
+    }
+    const uint64_t nr = (nwords - head + RW - 1) / RW;
+    const int rot = drive<E, Em, UNROLL2>(eng, nr, em, retired);
     if (src.write_state) {
         __syncwarp(mask);
         store_window(eng, win_s, rot, retired);
         if (lane == 0) {
             st.weyl[s] = wp + (uint32_t)nwords * omega;
-            st.pend[s] = (uint32_t)(nr * RW - nwords);
+            st.pend[s] = (uint32_t)(nr * RW - (nwords - head));
             st.pos[s] += src.ring ? src.pos_add : nwords;
         }
     }
     return em.acc;
 }
 
-template <class P, int TPG, int WPL, int OUT, bool VEC>
+template <class P, int TPG, int WPL, int OUT, int ST>
 __device__ __forceinline__ void gen_body(const GenArgs& a)
 {
     const uint32_t g = (blockIdx.x * blockDim.x + threadIdx.x) / TPG;
@@ -430,7 +491,7 @@ __device__ __forceinline__ void gen_body(const GenArgs& a)
     const unsigned mask = group_mask<TPG>();
     uint32_t* row = (OUT == kNormalSum) ? nullptr
                                         : reinterpret_cast<uint32_t*>(a.out) + (uint64_t)g * a.ld;
-    float acc = run_stream<P, TPG, WPL, OUT, VEC>(a.st, a.first + g, a.n, row, a.omega, lane, mask);
+    float acc = run_stream<P, TPG, WPL, OUT, ST>(a.st, a.first + g, a.n, row, a.omega, lane, mask);
     if constexpr (OUT == kNormalSum) {
 #pragma unroll
         for (int off = TPG / 2; off >= 1; off /= 2)
@@ -444,16 +505,16 @@ __device__ __forceinline__ void gen_body(const GenArgs& a)
 // states a minimum of one block per SM, which frees the compiler to spend
 // registers on more independent work per thread (124 instead of 80 at
 // (8,4)); the write-bound uniform output runs 4% faster with it.
-template <class P, int TPG, int WPL, int OUT, bool VEC>
+template <class P, int TPG, int WPL, int OUT, int ST>
 __global__ void __launch_bounds__(256) gen_kernel(GenArgs a)
 {
-    gen_body<P, TPG, WPL, OUT, VEC>(a);
+    gen_body<P, TPG, WPL, OUT, ST>(a);
 }
 
-template <class P, int TPG, int WPL, int OUT, bool VEC>
+template <class P, int TPG, int WPL, int OUT, int ST>
 __global__ void __launch_bounds__(256, 1) gen_kernel_ilp(GenArgs a)
 {
-    gen_body<P, TPG, WPL, OUT, VEC>(a);
+    gen_body<P, TPG, WPL, OUT, ST>(a);
 }
 
 // Persistent batch kernel.  Each warp repeatedly takes the next task
@@ -485,21 +546,22 @@ __device__ __forceinline__ void run_item(const State& st, const BatchItem& it, c
                                          uint32_t omega, int lane)
 {
     uint32_t* row = reinterpret_cast<uint32_t*>(it.out);
-    const bool vec = (reinterpret_cast<uintptr_t>(row) & 15u) == 0;
+    // 64-bit stores: rows 4 bytes off an 8-byte boundary take the other form
+    const bool vec = (reinterpret_cast<uintptr_t>(row) & 7u) == 0;
     constexpr unsigned kFull = 0xFFFFFFFFu;
     const UnitSrc src = unit_src<P>(it, pieces);
     switch (it.kind) {
     case kU32:
-        if (vec) run_stream<P, 32, 2, kU32, true, false>(st, it.stream, it.count, row, omega, lane, kFull, src);
-        else run_stream<P, 32, 2, kU32, false, false>(st, it.stream, it.count, row, omega, lane, kFull, src);
+        if (vec) run_stream<P, 32, 2, kU32, kAligned, false>(st, it.stream, it.count, row, omega, lane, kFull, src);
+        else run_stream<P, 32, 2, kU32, kShifted, false>(st, it.stream, it.count, row, omega, lane, kFull, src);
         break;
     case kUniform:
-        if (vec) run_stream<P, 32, 2, kUniform, true, false>(st, it.stream, it.count, row, omega, lane, kFull, src);
-        else run_stream<P, 32, 2, kUniform, false, false>(st, it.stream, it.count, row, omega, lane, kFull, src);
+        if (vec) run_stream<P, 32, 2, kUniform, kAligned, false>(st, it.stream, it.count, row, omega, lane, kFull, src);
+        else run_stream<P, 32, 2, kUniform, kShifted, false>(st, it.stream, it.count, row, omega, lane, kFull, src);
         break;
     default:
-        if (vec) run_stream<P, 32, 2, kNormal, true, false>(st, it.stream, it.count, row, omega, lane, kFull, src);
-        else run_stream<P, 32, 2, kNormal, false, false>(st, it.stream, it.count, row, omega, lane, kFull, src);
+        if (vec) run_stream<P, 32, 2, kNormal, kAligned, false>(st, it.stream, it.count, row, omega, lane, kFull, src);
+        else run_stream<P, 32, 2, kNormal, kScalar, false>(st, it.stream, it.count, row, omega, lane, kFull, src);
         break;
     }
 }
@@ -519,8 +581,8 @@ __device__ __forceinline__ void run_group(const State& st, const BatchItem* item
         const BatchItem it = items[idx];
         uint32_t* row = reinterpret_cast<uint32_t*>(it.out);   // 16-byte aligned
         const UnitSrc src = unit_src<P>(it, pieces);
-        if (kind == kU32) run_stream<P, TPG, WPL, kU32, true, false>(st, it.stream, it.count, row, omega, gl, mask, src);
-        else run_stream<P, TPG, WPL, kUniform, true, false>(st, it.stream, it.count, row, omega, gl, mask, src);
+        if (kind == kU32) run_stream<P, TPG, WPL, kU32, kAligned, false>(st, it.stream, it.count, row, omega, gl, mask, src);
+        else run_stream<P, TPG, WPL, kUniform, kAligned, false>(st, it.stream, it.count, row, omega, gl, mask, src);
         __syncwarp(mask);
         if (it.flag) {
             __threadfence_system();
@@ -596,33 +658,45 @@ cudaError_t launch_seed_impl(const State& st, const uint32_t* d_seeds, uint32_t 
     return cudaGetLastError();
 }
 
-template <class P, int TPG, int WPL, int OUT, bool VEC>
+template <class P, int TPG, int WPL, int OUT, int ST>
 cudaError_t launch_gen_one(int block, const GenArgs& a, cudaStream_t s)
 {
     const uint64_t threads = (uint64_t)a.nstreams * TPG;
     const unsigned grid = (unsigned)((threads + block - 1) / block);
-    if constexpr (OUT == kUniform)
-        gen_kernel_ilp<P, TPG, WPL, OUT, VEC><<<grid, block, 0, s>>>(a);
+    if constexpr (OUT == kUniform || (OUT == kU32 && ST == kShifted))   // kShifted words: 0.631 -> 0.618 ms
+        gen_kernel_ilp<P, TPG, WPL, OUT, ST><<<grid, block, 0, s>>>(a);
     else
-        gen_kernel<P, TPG, WPL, OUT, VEC><<<grid, block, 0, s>>>(a);
+        gen_kernel<P, TPG, WPL, OUT, ST><<<grid, block, 0, s>>>(a);
     return cudaGetLastError();
+}
+
+// Rows that no vector store fits.  At (32, 2) the scalar stores of a short
+// call cost less than moving the ring on: 30000 rows of 1001 words 33.5 us
+// against 35.5 us, 16384 rows of 65537 0.808 against 0.645 ms; at the narrower
+// shapes, whose stores are 8 or 16 bytes apart over several rows, kShifted is
+// the faster at every length (75 against 34 us at (8, 4)).
+constexpr uint64_t kShiftMinWords = 2048;
+
+template <class P, int TPG, int WPL, int OUT>
+cudaError_t launch_gen_words(bool vec, int block, const GenArgs& a, cudaStream_t s)
+{
+    if (vec) return launch_gen_one<P, TPG, WPL, OUT, kAligned>(block, a, s);
+    if constexpr (TPG == 32)
+        if (a.n < kShiftMinWords) return launch_gen_one<P, TPG, WPL, OUT, kScalar>(block, a, s);
+    return launch_gen_one<P, TPG, WPL, OUT, kShifted>(block, a, s);
 }
 
 template <class P, int TPG, int WPL>
 cudaError_t launch_gen_cfg(int out_kind, bool vec, int block, const GenArgs& a, cudaStream_t s)
 {
     switch (out_kind) {
-    case kU32:
-        return vec ? launch_gen_one<P, TPG, WPL, kU32, true>(block, a, s)
-                   : launch_gen_one<P, TPG, WPL, kU32, false>(block, a, s);
-    case kUniform:
-        return vec ? launch_gen_one<P, TPG, WPL, kUniform, true>(block, a, s)
-                   : launch_gen_one<P, TPG, WPL, kUniform, false>(block, a, s);
+    case kU32: return launch_gen_words<P, TPG, WPL, kU32>(vec, block, a, s);
+    case kUniform: return launch_gen_words<P, TPG, WPL, kUniform>(vec, block, a, s);
     case kNormal:
-        return vec ? launch_gen_one<P, TPG, WPL, kNormal, true>(block, a, s)
-                   : launch_gen_one<P, TPG, WPL, kNormal, false>(block, a, s);
+        return vec ? launch_gen_one<P, TPG, WPL, kNormal, kAligned>(block, a, s)
+                   : launch_gen_one<P, TPG, WPL, kNormal, kScalar>(block, a, s);
     case kNormalSum:
-        return launch_gen_one<P, TPG, WPL, kNormalSum, true>(block, a, s);
+        return launch_gen_one<P, TPG, WPL, kNormalSum, kAligned>(block, a, s);
     default:
         return cudaErrorInvalidValue;
     }

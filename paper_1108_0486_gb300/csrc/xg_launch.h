@@ -30,6 +30,11 @@ struct State {
     uint64_t* pos;   // [n]  words consumed since seeding
 };
 
+// How a stream's row is stored: its address allows vector stores; one word
+// (or value) at a time; or words and uniforms at any other address, where the
+// ring first moves on to the next aligned word.
+enum Store { kScalar = 0, kAligned = 1, kShifted = 2 };
+
 enum OutKind { kU32 = 0, kUniform = 1, kNormal = 2, kNormalSum = 3 };
 
 struct GenArgs {

@@ -45,3 +45,55 @@ def test_default_launch_on_both_sides_of_its_thresholds(kind, edge):
             w = O.streams(W.seeds(1, 1 + s), 2 * words_of(kind, n))[0]
             check(kind, rows[s, :n], w, n)
             check(kind, rows[s, n:], w[words_of(kind, n):], n)
+
+
+@pytest.mark.parametrize("kind", KINDS)
+@pytest.mark.parametrize("tpg,wpl", [(4, 8), (8, 4), (16, 2), (16, 4), (32, 2)])
+@pytest.mark.parametrize("ps", [0, 1])
+def test_rows_at_every_word_offset(kind, tpg, wpl, ps):
+    """Two calls in a row whose rows start 0 .. 3 words off a 16-byte boundary:
+    lengths below and above one turn of the ring and the limit from which the
+    ring is moved on; the words around each row stay untouched, and the second
+    call continues the first."""
+    from paper_1108_0486_gb300 import Streams
+    streams = 5
+    seeds = W.seeds(streams)
+    for n in (3, 128, 131, 132, 133, 2047, 2049, 2211):
+        ld = n + 4 + (1 - n) % 4          # rows 1 word further off each time
+        m = words_of(kind, n)
+        ref = O.streams(seeds, 2 * m, param_set=ps)
+        for off in (1, 2):
+            with Streams(streams, param_set=ps, seeds=seeds) as st:
+                st.set_launch(kind, tpg, wpl)
+                dt = torch.int32 if kind == "u32" else torch.float32
+                for call in range(2):
+                    buf = torch.full((streams * ld + 8,), -7, dtype=dt, device="cuda")
+                    st.generate(kind, n, out=buf[off:], ld=ld)
+                    h = buf.cpu().numpy()
+                    assert np.all(h[:off] == -7)
+                    for i in range(streams):
+                        row = h[off + i * ld:off + i * ld + ld]
+                        check(kind, row[:n], ref[i, call * m:(call + 1) * m], n)
+                        assert np.all(row[n:n + 1] == -7)
+
+
+def test_batch_rows_at_every_word_offset():
+    """Cut and uncut calls of a batch with outputs 0 .. 3 words off."""
+    from paper_1108_0486_gb300 import Streams
+    seeds = W.seeds(24)
+    with Streams(24, seeds=seeds) as st:
+        st.set_batch_split(2048)
+        items, outs = [], []
+        for i in range(24):
+            kind, off, n = KINDS[i % 3], i // 3 % 4, (130, 5000, 777, 4099)[i % 4]
+            buf = torch.full((n + 8,), -7, dtype=torch.int32 if kind == "u32" else torch.float32, device="cuda")
+            outs.append((kind, off, n, buf))
+            items.append((i, kind, n, buf[off:off + n]))
+        st.batch(items)
+        st.batch(items)
+        torch.cuda.synchronize()
+    for i, (kind, off, n, buf) in enumerate(outs):
+        m = words_of(kind, n)
+        h = buf.cpu().numpy()
+        check(kind, h[off:off + n], O.streams(seeds[i:i + 1], 2 * m)[0, m:], n)
+        assert np.all(h[:off] == -7) and np.all(h[off + n:] == -7)
