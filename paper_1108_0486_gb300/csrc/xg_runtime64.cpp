@@ -54,14 +54,15 @@ bool is_device_pointer(const void* p)
     return attr.type == cudaMemoryTypeDevice || attr.type == cudaMemoryTypeManaged;
 }
 
-int pick_cfg(const xg_w64_ctx* c, int kind, uint32_t nstreams)
+// Without a tuned choice, one warp per stream: the fastest shape for both
+// outputs in a sweep of 100 .. 65536 streams (ps per output at 1000 / 8000 /
+// 16384 streams: u64 1.59 / 1.21 / 1.16 against 2.39 / 1.27 / 1.20 at (16,2)
+// and 4.19 / 1.95 / 2.04 at (8,4); uniforms 1.90 / 1.52 / 1.43 against
+// 2.66 / 1.54 / 1.47 and 4.62 / 1.85 / 1.56), and its stores are whole lines
+// at every row address (rows of an odd length at (8,4): 3.62).
+int pick_cfg(const xg_w64_ctx* c, int kind)
 {
-    if (c->cfg[kind] >= 0) return c->cfg[kind];
-    // many streams: few lanes per stream (fewer shuffles, 16-byte stores)
-    const uint64_t lanes_wanted = (uint64_t)c->sm_count * 32 * 24;
-    if ((uint64_t)nstreams * 8 >= lanes_wanted / 2) return xg64::cfg_index(8, 4);
-    if ((uint64_t)nstreams * 16 >= lanes_wanted / 2) return xg64::cfg_index(16, 2);
-    return xg64::cfg_index(32, 1);
+    return c->cfg[kind] >= 0 ? c->cfg[kind] : xg64::cfg_index(32, 1);
 }
 
 xg_status enqueue(xg_w64_ctx* c, int kind, uint32_t first, uint32_t nstreams, uint64_t n, void* d_out,
@@ -75,7 +76,7 @@ xg_status enqueue(xg_w64_ctx* c, int kind, uint32_t first, uint32_t nstreams, ui
     a.out = d_out;
     a.ld = ld;
     a.omega = c->weyl_on ? xg64::kOmega : 0;
-    const int cfg = force_cfg >= 0 ? force_cfg : pick_cfg(c, kind, nstreams);
+    const int cfg = force_cfg >= 0 ? force_cfg : pick_cfg(c, kind);
     int block = force_block;
     if (block <= 0) block = (c->cfg[kind] == cfg && c->blk[kind] > 0) ? c->blk[kind] : xg64::kCfgs[cfg].block;
     const bool vec = ((reinterpret_cast<uintptr_t>(d_out) & 15u) == 0) && (nstreams == 1 || ld % 2 == 0);

@@ -73,22 +73,27 @@ __device__ __noinline__ uint64_t to_uniform_bits_any(uint64_t o)
     return ((uint64_t)(1023 + p - 53) << 52) | frac;
 }
 
-// The same on 32-bit halves.  When m = mh:ml has its leading one in mh (all
-// but 2^-21 of the words), lz = clz(mh) is 11..31 and the normalising shift
-// k = lz - 11 is below 32, so m << k is two funnel shifts; the leading one
-// (bit 52) is then added into the exponent field, whose value before the
-// carry is 1033 - lz - 1.  Other words take the general path above.
-__device__ __forceinline__ uint64_t to_uniform_bits(uint64_t o)
+// The same on 32-bit halves for the words whose leading one is in the upper
+// 21 bits (all but 2^-21 of them: oh >= kNarrow).  m = mh:ml = o >> 11 has
+// clz(mh) = clz(oh) + 11, so the normalising shift is k = clz(oh) < 21 and
+// m << k is two shifts; the leading one (bit 52) is added into the exponent
+// field, whose value before the carry is 1021 - k.  A smaller oh gives a
+// wrong value and no fault.
+constexpr uint32_t kNarrow = 1u << 11;
+__device__ __forceinline__ uint64_t to_uniform_bits_wide(uint64_t o)
 {
     const uint32_t oh = (uint32_t)(o >> 32), ol = (uint32_t)o;
     const uint32_t mh = oh >> 11;
     const uint32_t ml = __funnelshift_r(ol, oh, 11);
-    if (mh == 0) return to_uniform_bits_any(o);
-    const int lz = __clz(mh);
-    const int k = lz - 11;
-    const uint32_t hi = __funnelshift_l(ml, mh, k) + ((uint32_t)(1032 - lz) << 20);
-    const uint32_t lo = ml << k;
+    const uint32_t k = (uint32_t)__clz(oh);
+    const uint32_t hi = __funnelshift_l(ml, mh, k) + (1021u << 20) - (k << 20);
+    const uint32_t lo = __funnelshift_l(0u, ml, k);
     return ((uint64_t)hi << 32) | lo;
+}
+
+__device__ __forceinline__ uint64_t to_uniform_bits(uint64_t o)
+{
+    return (uint32_t)(o >> 32) < kNarrow ? to_uniform_bits_any(o) : to_uniform_bits_wide(o);
 }
 
 template <int TPG, int WPL>
@@ -171,30 +176,47 @@ __device__ __forceinline__ void store_window(const E& eng, uint64_t* win_s, int 
 
 // nr rounds: full blocks of NROWS rounds through emit.full(), the last
 // 1..NROWS through emit.tail(); the last round saves the row it overwrites.
-// U blocks per loop iteration (FP64 uniforms, bound by integer issue: 4
-// blocks take 7.6% off the kernel; the raw u64 kernel is bound by HBM and
-// keeps 1).
+// U blocks per loop iteration: FP64 uniforms are bound by integer issue and
+// take 8 at one word per lane (16384 streams x 2^14: 1.434 ps per value; 4
+// blocks 1.450, 2 blocks 1.478) and 4 otherwise; the raw u64 kernel is bound
+// by HBM and keeps 1.
+//
+// Uniforms take the conversion that holds for all but 2^-21 of the words; an
+// iteration in which a lane met another word is run again from the ring kept
+// at its start (the group votes, so its lanes stay together for the
+// shuffles).  That is one vote per U * NROWS words instead of a branch per
+// word: 1.594 -> 1.434 ps per value there, with the larger register budget of
+// gen_kernel_ilp (1.503 ps without it), and 8.55 -> 6.1 at 300 streams.
 template <class E, class Emit, int U = 1>
 __device__ __forceinline__ int drive(E& eng, uint64_t nr, Emit& emit, uint64_t (&retired)[E::WPL_])
 {
     uint64_t r = 0;
-    if constexpr (U > 1) {
-        for (; r + U * E::NROWS < nr; r += U * E::NROWS) {
-            static_for<0, U * E::NROWS>([&](auto kc) {
-                constexpr int K = decltype(kc)::value % E::NROWS;
-                eng.template round<K>();
-                emit.template full<K>(eng);
-            });
-        }
-    }
-    while (r + E::NROWS < nr) {
-        static_for<0, E::NROWS>([&](auto kc) {
-            constexpr int K = decltype(kc)::value;
+    auto blocks = [&](auto uc, auto anyc) {
+        static_for<0, decltype(uc)::value * E::NROWS>([&](auto kc) {
+            constexpr int K = decltype(kc)::value % E::NROWS;
             eng.template round<K>();
-            emit.template full<K>(eng);
+            emit.template full<K, decltype(anyc)::value>(eng);
         });
-        r += E::NROWS;
-    }
+    };
+    auto iteration = [&](auto uc) {
+        if constexpr (Emit::kVoted) {
+            const E start = eng;
+            const Emit estart = emit;
+            emit.low = 0xFFFFFFFFu;
+            blocks(uc, std::false_type{});
+            if (__any_sync(eng.mask, emit.low < kNarrow)) {
+                eng = start;
+                emit = estart;
+                blocks(uc, std::true_type{});
+            }
+        } else {
+            blocks(uc, std::true_type{});
+        }
+        r += decltype(uc)::value * E::NROWS;
+    };
+    if constexpr (U > 1)
+        while (r + U * E::NROWS < nr) iteration(std::integral_constant<int, U>{});
+    while (r + E::NROWS < nr) iteration(std::integral_constant<int, 1>{});
     const int rem = (int)(nr - r);
     static_for<0, E::NROWS>([&](auto kc) {
         constexpr int K = decltype(kc)::value;
@@ -211,7 +233,8 @@ __device__ __forceinline__ int drive(E& eng, uint64_t nr, Emit& emit, uint64_t (
 }
 
 struct NoEmit {
-    template <int K, class E> __device__ __forceinline__ void full(const E&) {}
+    static constexpr bool kVoted = false;
+    template <int K, bool ANY, class E> __device__ __forceinline__ void full(const E&) {}
     template <int K, class E> __device__ __forceinline__ void tail(const E&, uint64_t) {}
 };
 
@@ -221,28 +244,39 @@ template <class E, int OUT, bool VEC>
 struct Emit {
     static constexpr int W = E::WPL_;
     static constexpr int RW = E::RW;
+    static constexpr bool kVoted = OUT == kUniformF64;
     uint64_t* dst;
     uint64_t limit;
     uint64_t lane_off;
     uint64_t wl;
     uint64_t omega;
+    uint32_t low;   // least upper half of this iteration's words
 
-    template <int K>
+    // ANY: the conversion for every word, else the one for upper halves of at
+    // least kNarrow (low tells whether that held).
+    template <int K, bool ANY>
     __device__ __forceinline__ void values(const E& eng, uint64_t (&v)[W])
     {
 #pragma unroll
         for (int i = 0; i < W; ++i) {
             const uint64_t o = combine(eng.ring[K][i], wl + (uint64_t)i * omega);
-            v[i] = (OUT == kU64) ? o : to_uniform_bits(o);
+            if constexpr (OUT == kU64) {
+                v[i] = o;
+            } else if constexpr (ANY) {
+                v[i] = to_uniform_bits(o);
+            } else {
+                low = min(low, (uint32_t)(o >> 32));
+                v[i] = to_uniform_bits_wide(o);
+            }
         }
         wl += (uint64_t)RW * omega;
     }
 
-    template <int K>
+    template <int K, bool ANY>
     __device__ __forceinline__ void full(const E& eng)
     {
         uint64_t v[W];
-        values<K>(eng, v);
+        values<K, ANY>(eng, v);
         if constexpr (VEC && W % 2 == 0) {
 #pragma unroll
             for (int q = 0; q < W / 2; ++q)
@@ -258,7 +292,7 @@ struct Emit {
     __device__ __forceinline__ void tail(const E& eng, uint64_t round)
     {
         uint64_t v[W];
-        values<K>(eng, v);
+        values<K, true>(eng, v);
         const uint64_t off = (uint64_t)RW * round + lane_off;
 #pragma unroll
         for (int i = 0; i < W; ++i)
@@ -313,7 +347,7 @@ __global__ void __launch_bounds__(256) seed_kernel(State st, const uint32_t* __r
 }
 
 template <int TPG, int WPL, int OUT, bool VEC>
-__global__ void __launch_bounds__(256) gen_kernel(GenArgs a)
+__device__ __forceinline__ void gen_body(const GenArgs& a)
 {
     using E = Engine<TPG, WPL>;
     constexpr int RW = E::RW;
@@ -336,7 +370,7 @@ __global__ void __launch_bounds__(256) gen_kernel(GenArgs a)
     em.dst = reinterpret_cast<uint64_t*>(a.out) + (uint64_t)g * a.ld + em.lane_off;
     uint64_t retired[WPL];
     const uint64_t nr = (a.n + RW - 1) / RW;
-    const int rot = drive<E, Emit<E, OUT, VEC>, OUT == kUniformF64 ? 4 : 1>(eng, nr, em, retired);
+    const int rot = drive<E, Emit<E, OUT, VEC>, OUT == kUniformF64 ? (WPL == 1 ? 8 : 4) : 1>(eng, nr, em, retired);
     __syncwarp(eng.mask);
     store_window(eng, win_s, rot, retired);
     if (lane == 0) {
@@ -346,22 +380,42 @@ __global__ void __launch_bounds__(256) gen_kernel(GenArgs a)
     }
 }
 
+// Two register budgets: one warp per stream runs uniforms with a stated
+// minimum of one block per SM, which lets the compiler keep more of an
+// iteration in flight.
+template <int TPG, int WPL, int OUT, bool VEC>
+__global__ void __launch_bounds__(256) gen_kernel(GenArgs a)
+{
+    gen_body<TPG, WPL, OUT, VEC>(a);
+}
+
+template <int TPG, int WPL, int OUT, bool VEC>
+__global__ void __launch_bounds__(256, 1) gen_kernel_ilp(GenArgs a)
+{
+    gen_body<TPG, WPL, OUT, VEC>(a);
+}
+
 template <int TPG, int WPL, int OUT, bool VEC>
 static cudaError_t launch_one(int block, const GenArgs& a, cudaStream_t s)
 {
     const uint64_t threads = (uint64_t)a.nstreams * TPG;
     const unsigned grid = (unsigned)((threads + block - 1) / block);
-    gen_kernel<TPG, WPL, OUT, VEC><<<grid, block, 0, s>>>(a);
+    if constexpr (OUT == kUniformF64 && WPL == 1)
+        gen_kernel_ilp<TPG, WPL, OUT, VEC><<<grid, block, 0, s>>>(a);
+    else
+        gen_kernel<TPG, WPL, OUT, VEC><<<grid, block, 0, s>>>(a);
     return cudaGetLastError();
 }
 
 template <int TPG, int WPL>
 static cudaError_t launch_cfg(int kind, bool vec, int block, const GenArgs& a, cudaStream_t s)
 {
+    if constexpr (WPL == 1) vec = false;   // one 8-byte store per word at any row address
+    constexpr bool kVec = WPL > 1;
     if (kind == kU64)
-        return vec ? launch_one<TPG, WPL, kU64, true>(block, a, s) : launch_one<TPG, WPL, kU64, false>(block, a, s);
+        return vec ? launch_one<TPG, WPL, kU64, kVec>(block, a, s) : launch_one<TPG, WPL, kU64, false>(block, a, s);
     if (kind == kUniformF64)
-        return vec ? launch_one<TPG, WPL, kUniformF64, true>(block, a, s)
+        return vec ? launch_one<TPG, WPL, kUniformF64, kVec>(block, a, s)
                    : launch_one<TPG, WPL, kUniformF64, false>(block, a, s);
     return cudaErrorInvalidValue;
 }

@@ -97,3 +97,28 @@ def test_batch_rows_at_every_word_offset():
         h = buf.cpu().numpy()
         check(kind, h[off:off + n], O.streams(seeds[i:i + 1], 2 * m)[0, m:], n)
         assert np.all(h[:off] == -7) and np.all(h[off + n:] == -7)
+
+
+@pytest.mark.parametrize("tpg,wpl", [(0, 0), (4, 8), (8, 4), (16, 2), (32, 1)])
+def test_fp64_uniforms_of_words_with_many_leading_zeros(tpg, wpl):
+    """A nearly empty ring without the Weyl word gives zeros and words of every
+    small size, which leave the conversion of the common words: values against
+    the closed form of the words themselves, at lengths around one and two
+    iterations of the kernel's loop and ends of rows."""
+    from paper_1108_0486_gb300 import Streams64
+    for n in (1, 33, 511, 512, 513, 577, 1025, 4000):
+        got = []
+        for kind in ("u64", "uniform"):
+            with Streams64(3, weyl=False, seeds=W.seeds(3)) as st:
+                for s in range(3):
+                    ring = np.zeros(64, dtype=np.uint64)
+                    ring[(7 * s + 1) % 64] = 1 << (20 * s)
+                    st.set_state(s, ring, 0)
+                if tpg:
+                    st.set_launch(kind, tpg, wpl)
+                got.append(np.concatenate([st.generate(kind, n).cpu().numpy(), st.generate(kind, n).cpu().numpy()], 1))
+        words = got[0].view(np.uint64)
+        assert np.array_equal(got[1], O.uniform64_of(words).reshape(words.shape))
+        if n > 1000:
+            small = words < (1 << 43)
+            assert small.any() and not small.all()
