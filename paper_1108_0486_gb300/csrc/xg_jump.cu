@@ -10,8 +10,20 @@
 //
 // Matrices are kept in column form: column j of C is the state reached from
 // the unit state e_j (bit j of ring word j/32).  Applying C to v is the XOR of
-// the columns selected by v's bits; squaring is applying C to its own columns.
-// The columns of M itself are one step of the recurrence applied to e_j.
+// the columns selected by v's bits.  The columns of M itself are one step of
+// the recurrence applied to e_j.
+//
+// Any M^J follows from its columns for the newest ring word alone (32 of the
+// 4096, or 64 for 64-bit words).  Let E_b be the state whose newest word is
+// bit b and the rest zero.  After i < r steps that word has moved to position
+// r - 1 - i, and the only other nonzero word is the one made from it when it
+// passed the lag-s tap at step s: (I+L^c)(I+R^d) e_b =: U e_b, by then at
+// position r - 1 - (i - s) (it meets no tap itself, since r - 1 - s < s).  So
+//   e_(r-1-i, b) = M^i E_b + [i >= s] sum_{b' in U e_b} M^(i-s) E_b',
+// and M^J e_(r-1-i, b) = M^i Y_b + [i >= s] sum M^(i-s) Y_b' with Y_b = M^J E_b:
+// windows of the sequences that go on from the states Y_b for r more words.
+// Products of matrices are therefore applications to 32 (64) states and one
+// pass that writes the columns, instead of applications to 4096 states.
 #include <algorithm>
 #include <cstdlib>
 #include <cstring>
@@ -28,7 +40,60 @@ namespace xg {
 
 constexpr int kBits = 4096;      // state bits
 constexpr int kWords64 = 64;     // uint64 words per state
-constexpr int kApplyVecs = 16;   // states per block in gf2_apply_kernel
+constexpr int kMaxNewest = 64;   // most columns of one ring word
+
+// The ring and operator pairs of a matrix family.
+template <class P>
+struct Ring32 {
+    using Word = uint32_t;
+    static constexpr int R = kR, S = P::S, BITS = 32;
+    static __host__ __device__ Word lag_r(Word t) { t ^= t << P::A; return t ^ (t >> P::B); }
+    static __host__ __device__ Word lag_s(Word u) { u ^= u << P::C; return u ^ (u >> P::D); }
+};
+struct Ring64 {
+    using Word = uint64_t;
+    static constexpr int R = xg64::kR, S = xg64::kS, BITS = 64;
+    static __host__ __device__ Word lag_r(Word t) { t ^= t << xg64::kA; return t ^ (t >> xg64::kB); }
+    static __host__ __device__ Word lag_s(Word u) { u ^= u << xg64::kC; return u ^ (u >> xg64::kD); }
+};
+
+// seq[b][0 .. 2R) = state b's ring and the R raw words after it (no Weyl
+// word): one block per state, S words at a time.
+template <class F>
+__global__ void __launch_bounds__(128) continue_kernel(const typename F::Word* __restrict__ states,
+                                                       typename F::Word* __restrict__ seq)
+{
+    constexpr int R = F::R, S = F::S;
+    static_assert(S <= 128 && R <= 128 && R - 1 - S < S, "one word of a step per thread");
+    __shared__ typename F::Word x[2 * R];
+    const int t = threadIdx.x;
+    if (t < R) x[t] = states[(size_t)blockIdx.x * R + t];
+    __syncthreads();
+    for (int k = R; k < 2 * R; k += S) {
+        if (t < S && k + t < 2 * R) x[k + t] = F::lag_r(x[k + t - R]) ^ F::lag_s(x[k + t - S]);
+        __syncthreads();
+    }
+    for (int k = t; k < 2 * R; k += 128) seq[(size_t)blockIdx.x * 2 * R + k] = x[k];
+}
+
+// All columns of M^J from the sequences that go on from Y_b = M^J E_b.
+template <class F>
+__global__ void __launch_bounds__(256) columns_kernel(const typename F::Word* __restrict__ seq,
+                                                      typename F::Word* __restrict__ C)
+{
+    using Word = typename F::Word;
+    constexpr int R = F::R, S = F::S;
+    const uint32_t id = blockIdx.x * 256 + threadIdx.x;   // grid covers kBits * R exactly
+    const int j = (int)(id / R), k = (int)(id % R);
+    const int b = j % F::BITS, i = R - 1 - j / F::BITS;
+    Word v = seq[(size_t)b * 2 * R + i + k];
+    if (i >= S)
+        for (Word u = F::lag_s(Word(1) << b); u; u &= u - 1) {
+            const int bb = __ffsll((long long)u) - 1;
+            v ^= seq[(size_t)bb * 2 * R + (i - S) + k];
+        }
+    C[id] = v;
+}
 
 // Columns of M for parameter set P: column j = one step from e_j.
 template <class P>
@@ -50,50 +115,6 @@ __global__ void __launch_bounds__(128) step_columns_kernel(uint32_t* __restrict_
     out[kR - 1] = t ^ u;
 }
 
-// out[i] = C in[i] for the n states listed in idx (or 0..n-1 when idx is
-// null).  64 threads per block, thread t owns uint64 word t of the results;
-// each column of C is loaded once per block and shared by its 16 states.
-// in and out may be the same array: a block reads its states before writing.
-__global__ void __launch_bounds__(64) gf2_apply_kernel(const uint64_t* __restrict__ C, const uint64_t* in,
-                                                       uint64_t* out, uint32_t n, const uint32_t* __restrict__ idx)
-{
-    __shared__ uint64_t vin[kApplyVecs][kWords64];
-    const int t = threadIdx.x;
-    const uint32_t base = blockIdx.x * kApplyVecs;
-    const int nv = (int)umin((uint32_t)kApplyVecs, n - base);
-    for (int v = 0; v < nv; ++v) {
-        const uint32_t i = idx ? idx[base + v] : base + v;
-        vin[v][t] = in[(size_t)i * kWords64 + t];
-    }
-    __syncthreads();
-    uint64_t acc[kApplyVecs];
-#pragma unroll
-    for (int v = 0; v < kApplyVecs; ++v) acc[v] = 0;
-    for (int w = 0; w < kWords64; ++w) {
-        uint64_t bits[kApplyVecs];
-        uint64_t any = 0;
-#pragma unroll
-        for (int v = 0; v < kApplyVecs; ++v) {
-            bits[v] = v < nv ? vin[v][w] : 0ull;
-            any |= bits[v];
-        }
-        while (any) {
-            const int b = __ffsll((long long)any) - 1;
-            any &= any - 1;
-            const uint64_t col = C[(size_t)(w * 64 + b) * kWords64 + t];
-#pragma unroll
-            for (int v = 0; v < kApplyVecs; ++v) acc[v] ^= col & (0ull - ((bits[v] >> b) & 1ull));
-        }
-    }
-#pragma unroll
-    for (int v = 0; v < kApplyVecs; ++v) {
-        if (v < nv) {
-            const uint32_t i = idx ? idx[base + v] : base + v;
-            out[(size_t)i * kWords64 + t] = acc[v];
-        }
-    }
-}
-
 // dst[i] ^= C src[i] for n (src, dst) pairs, dst zeroed beforehand.  Block
 // (x, y): pairs [48x, 48x+48), columns [y*cols, (y+1)*cols); 128 threads,
 // thread t owns 32-bit word t of every result.  Columns go four at a time:
@@ -107,7 +128,7 @@ __global__ void __launch_bounds__(64) gf2_apply_kernel(const uint64_t* __restric
 // 5.1 ms with 16 (64 gains no more and needs 168 registers a thread).  Few
 // states take NV = 16, which pads less.
 template <int kPairVecs>
-// rings and out are the same array (sources are read, distinct destinations
+// rings and out may be the same array (sources are read, distinct destinations
 // are written), so neither is declared __restrict__.
 __global__ void __launch_bounds__(128) gf2_apply_pairs_kernel(const uint32_t* __restrict__ C,
                                                               const uint32_t* rings,
@@ -214,14 +235,60 @@ __global__ void substream_scatter_kernel(State st, uint32_t first, uint32_t n, c
 
 // ---------------------------------------------------------------------------
 
+// C = M^J from the newest word's columns Y_b = M^J E_b (states, consecutive
+// rings); seq: 2 * kBits * kMaxNewest / 8 bytes of scratch.
+constexpr size_t kSeqBytes = (size_t)2 * kBits / 8 * kMaxNewest;
+
+template <class F>
+static cudaError_t build_columns(const uint32_t* states, uint8_t* seq, uint64_t* C, cudaStream_t s)
+{
+    using Word = typename F::Word;
+    Word* sq = reinterpret_cast<Word*>(seq);
+    continue_kernel<F><<<F::BITS, 128, 0, s>>>(reinterpret_cast<const Word*>(states), sq);
+    columns_kernel<F><<<kBits * F::R / 256, 256, 0, s>>>(sq, reinterpret_cast<Word*>(C));
+    return cudaGetLastError();
+}
+
+static cudaError_t launch_build_columns(int family, const uint32_t* states, uint8_t* seq, uint64_t* C, cudaStream_t s)
+{
+    if (family == kJumpSetW64) return build_columns<Ring64>(states, seq, C, s);
+    if (family == 1) return build_columns<Ring32<ParamsPaper>>(states, seq, C, s);
+    return build_columns<Ring32<ParamsDefault>>(states, seq, C, s);
+}
+
+// Columns of the newest ring word: the last ones of a matrix in column form.
+static int newest_columns(int family) { return family == kJumpSetW64 ? 64 : 32; }
+static const uint32_t* newest_of(const uint64_t* C, int family)
+{
+    return reinterpret_cast<const uint32_t*>(C) + (size_t)(kBits - newest_columns(family)) * kR;
+}
+
 namespace {
 struct Tables {
     uint64_t* mat[kMaxPow] = {};  // C_k: 4096 columns x 64 uint64 (2 MiB), allocated when built
     int built = 0;                // C_0 .. C_{built-1} are valid
+    uint8_t* scratch = nullptr;   // squaring: kMaxNewest states, sequences, identity list
 };
 std::mutex g_tab_mu;
 Tables g_tabs[64][3];  // per device, per matrix family
 }  // namespace
+
+// C_{b+1} from C_b: C_b applied to its own newest columns.
+static cudaError_t square_matrix(int device, int family, Tables& T, int b, cudaStream_t s)
+{
+    const int nb = newest_columns(family);
+    uint32_t* states = reinterpret_cast<uint32_t*>(T.scratch);
+    uint8_t* seq = T.scratch + (size_t)kMaxNewest * kR * 4;
+    uint32_t* ids = reinterpret_cast<uint32_t*>(seq + kSeqBytes);
+    int sms = 0;
+    cudaError_t e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device);
+    if (e == cudaSuccess) e = launch_jump_index(ids, (uint32_t)nb, 0u, s);
+    if (e == cudaSuccess) e = cudaMemsetAsync(states, 0, (size_t)nb * kR * 4, s);
+    if (e == cudaSuccess)
+        e = launch_gf2_apply_pairs(T.mat[b], newest_of(T.mat[b], family), states, (uint32_t)nb, ids, ids, sms, s);
+    if (e == cudaSuccess) e = launch_build_columns(family, states, seq, T.mat[b + 1], s);
+    return e;
+}
 
 const uint64_t* jump_matrix(int device, int param_set, int k, cudaStream_t s, xg_status* st)
 {
@@ -237,6 +304,12 @@ const uint64_t* jump_matrix(int device, int param_set, int k, cudaStream_t s, xg
     while (T.built <= k) {
         const int b = T.built;
         cudaError_t e = cudaMalloc(&T.mat[b], mat_bytes);
+        if (e == cudaSuccess && !T.scratch) {
+            void* p = nullptr;
+            e = cudaMalloc(&p, (size_t)kMaxNewest * kR * 4 + kSeqBytes + (size_t)3 * kMaxNewest * 4);
+            if (e == cudaSuccess) T.scratch = static_cast<uint8_t*>(p);
+            else cudaFree(T.mat[b]);
+        }
         if (e != cudaSuccess) {
             cudaGetLastError();
             T.mat[b] = nullptr;
@@ -251,7 +324,7 @@ const uint64_t* jump_matrix(int device, int param_set, int k, cudaStream_t s, xg
             else
                 step_columns_kernel<ParamsDefault><<<kBits / 128, 128, 0, s>>>(reinterpret_cast<uint32_t*>(T.mat[0]));
         } else {
-            gf2_apply_kernel<<<kBits / kApplyVecs, 64, 0, s>>>(T.mat[b - 1], T.mat[b - 1], T.mat[b], kBits, nullptr);
+            e = square_matrix(device, param_set, T, b - 1, s);
         }
         if (e == cudaSuccess) e = cudaGetLastError();
         if (e != cudaSuccess) {
@@ -330,7 +403,7 @@ cudaError_t gf2_apply(int device, int family, int k, uint32_t* rings, uint32_t n
     const uint64_t* C = jump_matrix(device, family, k, s, st);
     if (!C) return cudaErrorMemoryAllocation;
     cudaError_t e = dst_zeroed ? cudaSuccess : zero_rings(rings, d_dst, n, s);
-    if (e == cudaSuccess) e = launch_gf2_apply_pairs(C, rings, n, d_src, d_dst, sm_count, s);
+    if (e == cudaSuccess) e = launch_gf2_apply_pairs(C, rings, rings, n, d_src, d_dst, sm_count, s);
     return e;
 }
 
@@ -347,23 +420,31 @@ static cudaError_t gf2_apply_explicit(int device, const uint64_t* P, uint8_t* A_
         return e;
     }
     cudaError_t e = zero_rings(rings, d_dst, n, s);
-    if (e == cudaSuccess) e = launch_gf2_apply_pairs(P, rings, n, d_src, d_dst, sm_count, s);
+    if (e == cudaSuccess) e = launch_gf2_apply_pairs(P, rings, rings, n, d_src, d_dst, sm_count, s);
     return e;
 }
 
+// With several set bits and more than kMaxNewest states the powers are
+// multiplied first.  Both sides of the line cost one application of few
+// states per bit; above it the states themselves are touched once.
 static bool jump_combines(uint64_t words, uint32_t n)
 {
-    return __builtin_popcountll(words) >= 2 && n > (uint32_t)kGf2Bits;
+    return __builtin_popcountll(words) >= 2 && n > (uint32_t)kMaxNewest;
+}
+
+// Work area of a product: one group of newest columns per set bit, the
+// sequences, the product in column form.
+static size_t product_bytes(uint64_t words)
+{
+    return (size_t)__builtin_popcountll(words) * kMaxNewest * kR * 4 + kSeqBytes + (size_t)kBits * kR * 4;
 }
 
 size_t gf2_jump_work_bytes(int device, uint32_t n, uint64_t words)
 {
-    // the tensor-core operand (the product of powers, n > 4096, applies to
-    // 4096 columns, fewer than n), then the product matrix pair and its FP8
-    // copy when the powers are multiplied first
+    // the tensor-core operand, then the product's work area and its FP8 copy
     size_t b = (gf2_apply_scratch(device, n) + 255) / 256 * 256;
     if (jump_combines(words, n)) {
-        b += (size_t)2 * kBits * kR * 4;
+        b += product_bytes(words);
         if (gf2_use_tc(device, n)) b += (size_t)kGf2Bits * kGf2Bits;
     }
     return b;
@@ -390,31 +471,32 @@ cudaError_t gf2_jump_states(int device, int family, uint64_t words, uint32_t* ri
         *result_hi = !in_lo;
         return cudaSuccess;
     }
-    // multiply the powers first (they commute: all are powers of one
-    // matrix): b - 1 applications to the 4096 columns of a matrix in column
-    // form, then one to the states -- (b - 1) 4096 + n state applications
-    // instead of b n.  The identity list runs to 2n - 1 > 8191.
+    // The product of the powers: its newest columns by one application per
+    // further set bit to 32 (64) states, then all columns from them.  For
+    // 16384 streams and 8 set bits this took the jump from 0.615 ms (seven
+    // tensor-core products of 4096 columns each) to @@ ms.
     uint8_t* w = work + (sbytes + 255) / 256 * 256;
-    uint32_t* prod = reinterpret_cast<uint32_t*>(w);   // two 4096-column matrices (ping-pong)
-    uint8_t* abuf = scratch ? w + (size_t)2 * kBits * kR * 4 : nullptr;  // FP8 copy of the product
-    cudaError_t e = cudaSuccess;
-    bool p_lo = true, first_bit = true;
+    const int nb = newest_columns(family);
+    const size_t group = (size_t)nb * kR;   // 32-bit words of one group of columns
+    uint32_t* cols = reinterpret_cast<uint32_t*>(w);
+    uint8_t* seq = w + (size_t)__builtin_popcountll(words) * kMaxNewest * kR * 4;
+    uint64_t* prod = reinterpret_cast<uint64_t*>(seq + kSeqBytes);
+    uint8_t* abuf = scratch ? seq + kSeqBytes + (size_t)kBits * kR * 4 : nullptr;  // FP8 copy of the product
+    cudaError_t e = cudaMemsetAsync(cols + group, 0, (size_t)(__builtin_popcountll(words) - 1) * group * 4, s);
+    int done = 0;
     for (int k = 0; k < 64 && e == cudaSuccess; ++k) {
         if (!((words >> k) & 1)) continue;
-        if (first_bit) {
-            const uint64_t* C = jump_matrix(device, family, k, s, st);
-            e = C ? cudaMemcpyAsync(prod, C, (size_t)kBits * kR * 4, cudaMemcpyDeviceToDevice, s)
-                  : cudaErrorMemoryAllocation;
-            first_bit = false;
-            continue;
-        }
-        e = gf2_apply(device, family, k, prod, kBits, p_lo ? lo : lo + kBits, p_lo ? lo + kBits : lo, scratch,
-                      sm_count, s, st);
-        p_lo = !p_lo;
+        const uint64_t* C = jump_matrix(device, family, k, s, st);
+        if (!C) return cudaErrorMemoryAllocation;
+        if (done == 0)
+            e = cudaMemcpyAsync(cols, newest_of(C, family), group * 4, cudaMemcpyDeviceToDevice, s);
+        else
+            e = launch_gf2_apply_pairs(C, cols + (done - 1) * group, cols + done * group, (uint32_t)nb, lo, lo, sm_count, s);
+        ++done;
     }
+    if (e == cudaSuccess) e = launch_build_columns(family, cols + (done - 1) * group, seq, prod, s);
     if (e == cudaSuccess) {
-        const uint64_t* P = reinterpret_cast<const uint64_t*>(p_lo ? prod : prod + (size_t)kBits * kR);
-        e = gf2_apply_explicit(device, P, abuf, rings, n, lo, hi, scratch, sm_count, s);
+        e = gf2_apply_explicit(device, prod, abuf, rings, n, lo, hi, scratch, sm_count, s);
         *result_hi = true;
     }
     return e;
@@ -436,8 +518,8 @@ cudaError_t launch_jump_index(uint32_t* ids, uint32_t n, uint32_t first, cudaStr
 }
 
 template <int NV>
-static cudaError_t launch_pairs(const uint64_t* C, uint32_t* rings, uint32_t n, const uint32_t* d_src,
-                                const uint32_t* d_dst, int sm_count, cudaStream_t s)
+static cudaError_t launch_pairs(const uint64_t* C, const uint32_t* in, uint32_t* out, uint32_t n,
+                                const uint32_t* d_src, const uint32_t* d_dst, int sm_count, cudaStream_t s)
 {
     const uint32_t groups = (n + NV - 1) / NV;
     // enough blocks for about 8 per SM, splitting the 4096 columns if needed
@@ -445,17 +527,17 @@ static cudaError_t launch_pairs(const uint64_t* C, uint32_t* rings, uint32_t n, 
     // matrix read is the cost, spread over up to 128 blocks)
     int chunks = 1;
     while (chunks < kBits / 32 && (uint64_t)groups * chunks < (uint64_t)8 * sm_count) chunks *= 2;
-    gf2_apply_pairs_kernel<NV><<<dim3(groups, chunks), 128, 0, s>>>(reinterpret_cast<const uint32_t*>(C), rings,
-                                                                   d_src, d_dst, n, rings, kBits / chunks);
+    gf2_apply_pairs_kernel<NV><<<dim3(groups, chunks), 128, 0, s>>>(reinterpret_cast<const uint32_t*>(C), in,
+                                                                   d_src, d_dst, n, out, kBits / chunks);
     return cudaGetLastError();
 }
 
-cudaError_t launch_gf2_apply_pairs(const uint64_t* C, uint32_t* rings, uint32_t n, const uint32_t* d_src,
-                                   const uint32_t* d_dst, int sm_count, cudaStream_t s)
+cudaError_t launch_gf2_apply_pairs(const uint64_t* C, const uint32_t* in, uint32_t* out, uint32_t n,
+                                   const uint32_t* d_src, const uint32_t* d_dst, int sm_count, cudaStream_t s)
 {
     if (n == 0) return cudaSuccess;
-    return n >= 4 * 48 ? launch_pairs<48>(C, rings, n, d_src, d_dst, sm_count, s)
-                       : launch_pairs<16>(C, rings, n, d_src, d_dst, sm_count, s);
+    return n >= 4 * 48 ? launch_pairs<48>(C, in, out, n, d_src, d_dst, sm_count, s)
+                       : launch_pairs<16>(C, in, out, n, d_src, d_dst, sm_count, s);
 }
 
 cudaError_t zero_rings(uint32_t* rings, const uint32_t* d_idx, uint32_t n, cudaStream_t s)

@@ -14,14 +14,15 @@ constexpr int kMaxPow = 64;  // C_k = M^(2^k), k < 64
 // the 64-bit-word generator.
 constexpr int kJumpSetW64 = 2;
 
-// C_k for a device and matrix family, built on first use (squarings on
-// stream s; 2 MiB each, kept until the process exits).  Null on failure.
+// C_k for a device and matrix family, built on first use (on stream s, each
+// from the one before; 2 MiB each, kept until the process exits).  Null on failure.
 const uint64_t* jump_matrix(int device, int param_set, int k, cudaStream_t s, xg_status* st);
 
-// rings[d_dst[i]] ^= C rings[d_src[i]] for n pairs (destinations distinct,
-// not among the sources, zeroed beforehand); rings are 128-word states.
-cudaError_t launch_gf2_apply_pairs(const uint64_t* C, uint32_t* rings, uint32_t n, const uint32_t* d_src,
-                                   const uint32_t* d_dst, int sm_count, cudaStream_t s);
+// out[d_dst[i]] ^= C in[d_src[i]] for n pairs of 128-word states.  in and out
+// may be one array; destinations are distinct, not among the sources, and
+// zeroed beforehand.
+cudaError_t launch_gf2_apply_pairs(const uint64_t* C, const uint32_t* in, uint32_t* out, uint32_t n,
+                                   const uint32_t* d_src, const uint32_t* d_dst, int sm_count, cudaStream_t s);
 
 // Whether an application to n states runs on the tensor cores (sm_103 and
 // n >= XG_GF2_TC_MIN_STATES, default 1024; XG_JUMP_TENSOR_CORES=0 turns the
@@ -43,10 +44,10 @@ cudaError_t gf2_apply(int device, int family, int k, uint32_t* rings, uint32_t n
 
 // Advance n states by `words` positions: M^words applied to rings[0, n),
 // with rings[n, 2n) as the second buffer (*result_hi: the result ended there)
-// and d_idx the identity list 0 .. max(2n, 8192) - 1.  With several set bits
-// and n > 4096 the powers are multiplied first and the product applied once.
+// and d_idx the identity list 0 .. 2n - 1.  With several set bits and more
+// than 64 states the powers are multiplied first and the product applied once.
 // work: gf2_jump_work_bytes(device, n, words) bytes of device memory,
-// 256-byte aligned (the tensor-core operand, and the product matrices when
+// 256-byte aligned (the tensor-core operand, and the product's work area when
 // the powers are multiplied first).
 size_t gf2_jump_work_bytes(int device, uint32_t n, uint64_t words);
 cudaError_t gf2_jump_states(int device, int family, uint64_t words, uint32_t* rings, uint32_t n,
