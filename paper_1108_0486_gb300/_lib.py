@@ -7,6 +7,7 @@ built; nothing here computes random numbers itself.
 """
 from __future__ import annotations
 
+import array
 import ctypes
 import os
 import threading
@@ -27,6 +28,7 @@ class XGError(RuntimeError):
 
 _lock = threading.Lock()
 _lib = None
+_entry = {}   # name -> bound entry point, filled when the library is loaded
 
 u32, u64, vp, i32 = ctypes.c_uint32, ctypes.c_uint64, ctypes.c_void_p, ctypes.c_int
 P_u32, P_u64, P_vp, P_i32 = (ctypes.POINTER(ctypes.c_uint32), ctypes.POINTER(ctypes.c_uint64),
@@ -133,6 +135,7 @@ def lib() -> ctypes.CDLL:
                 fn = getattr(L, name)
                 fn.argtypes = args
                 fn.restype = _RESTYPES.get(name, ctypes.c_int)
+                _entry[name] = fn
             _lib = L
     return _lib
 
@@ -147,7 +150,14 @@ def check(status: int) -> None:
 
 
 def call(name: str, *args) -> None:
-    check(getattr(lib(), name)(*args))
+    """Call an entry point.  Pointer arguments may be plain integers or None:
+    the argument types bound at load convert them."""
+    fn = _entry.get(name)
+    if fn is None:
+        fn = getattr(lib(), name)
+    status = fn(*args)
+    if status:
+        check(status)
 
 
 # ---- functions with the C names (argument marshalling only) -------------
@@ -199,19 +209,19 @@ def xg_set_states(ctx, first, count, rings_ptr, weyl_ptr, pos_ptr=0) -> None:
 
 
 def xg_generate_u32(ctx, first, nstreams, n_per_stream, out_ptr, ld) -> None:
-    call("xg_generate_u32", ctypes.c_void_p(ctx), first, nstreams, n_per_stream, ctypes.c_void_p(out_ptr), ld)
+    call("xg_generate_u32", ctx, first, nstreams, n_per_stream, out_ptr, ld)
 
 
 def xg_generate_uniform(ctx, first, nstreams, n_per_stream, out_ptr, ld) -> None:
-    call("xg_generate_uniform", ctypes.c_void_p(ctx), first, nstreams, n_per_stream, ctypes.c_void_p(out_ptr), ld)
+    call("xg_generate_uniform", ctx, first, nstreams, n_per_stream, out_ptr, ld)
 
 
 def xg_generate_normal(ctx, first, nstreams, n_per_stream, out_ptr, ld) -> None:
-    call("xg_generate_normal", ctypes.c_void_p(ctx), first, nstreams, n_per_stream, ctypes.c_void_p(out_ptr), ld)
+    call("xg_generate_normal", ctx, first, nstreams, n_per_stream, out_ptr, ld)
 
 
 def xg_generate_normal_sum(ctx, first, nstreams, n_per_stream, sums_ptr) -> None:
-    call("xg_generate_normal_sum", ctypes.c_void_p(ctx), first, nstreams, n_per_stream, ctypes.c_void_p(sums_ptr))
+    call("xg_generate_normal_sum", ctx, first, nstreams, n_per_stream, sums_ptr)
 
 
 def xg_transform_uniform(ctx, words_ptr, n, out_ptr) -> None:
@@ -222,19 +232,50 @@ def xg_transform_normal(ctx, words_ptr, n, out_ptr) -> None:
     call("xg_transform_normal", ctypes.c_void_p(ctx), ctypes.c_void_p(words_ptr), n, ctypes.c_void_p(out_ptr))
 
 
+_ROW = [("stream", "<u4"), ("type", "<u4"), ("count", "<u8"), ("out", "<u8")]   # xg_item and xg_request
+
+
+def pack_columns(streams, types, counts, pointers):
+    """The columns of xg_item[] / xg_request[] as a record array.  Sequences of
+    integers go through machine-integer arrays, a quarter of the time that one
+    nested list of rows takes to convert."""
+    import numpy as np
+    rec = np.zeros(len(streams), dtype=_ROW)
+    for (name, _), c in zip(_ROW, (streams, types, counts, pointers)):
+        try:
+            c = array.array("Q", c)
+        except TypeError:                  # not integers as they stand
+            c = array.array("Q", [int(v) for v in c])
+        rec[name] = np.frombuffer(c, dtype=np.uint64)
+    return rec
+
+
+def pack_rows(rows):
+    """Rows (stream, type, count, pointer) as pack_columns gives them; a record
+    array that it made is returned as it is."""
+    import numpy as np
+    if isinstance(rows, np.ndarray):
+        if rows.dtype.names:
+            return rows
+        rows = rows.astype(np.uint64, copy=False).reshape(-1, 4)
+        return pack_columns(*(rows[:, k].tolist() for k in range(4)))
+    rows = rows if isinstance(rows, (list, tuple)) else list(rows)
+    try:
+        cols = list(zip(*rows, strict=True))
+    except (TypeError, ValueError):        # no equal rows
+        cols = []
+    if len(cols) != 4:                     # numpy sorts out or refuses the rest
+        return pack_rows(np.asarray(rows, dtype=np.uint64))
+    return pack_columns(*cols)
+
+
 def make_items(items):
     """A ctypes xg_item array from (stream, type, count, out_ptr) tuples (build
     it once to reuse it across calls)."""
     if isinstance(items, ctypes.Array):
         return items
-    import numpy as np
-    a = np.asarray(items, dtype=np.uint64).reshape(-1, 4)
-    rec = np.zeros(a.shape[0], dtype=[("stream", "<u4"), ("type", "<u4"), ("count", "<u8"),
-                                     ("out", "<u8")])
-    rec["stream"], rec["type"], rec["count"], rec["out"] = a[:, 0], a[:, 1], a[:, 2], a[:, 3]
-    arr = (XgItem * a.shape[0])()
-    ctypes.memmove(arr, rec.ctypes.data, rec.nbytes)
-    return arr
+    rec = pack_rows(items)
+    return (XgItem * rec.shape[0]).from_buffer(rec) if rec.shape[0] else (XgItem * 0)()
 
 
 def xg_generate_batch(ctx, items) -> None:
@@ -295,18 +336,14 @@ def xg_server_stop(ctx) -> None:
 def xg_submit(ctx, stream, out_type, count, d_out=0) -> int:
     req = XgRequest(stream, out_type, count, d_out)
     t = ctypes.c_uint64()
-    call("xg_submit", ctypes.c_void_p(ctx), ctypes.byref(req), ctypes.byref(t))
+    call("xg_submit", ctx, ctypes.byref(req), ctypes.byref(t))
     return t.value
 
 
 def make_requests(reqs):
     """A numpy record array laid out as xg_request[] from (stream, type,
     count, d_out) tuples (build it once, submit slices of it)."""
-    import numpy as np
-    a = np.asarray(reqs, dtype=np.uint64).reshape(-1, 4)
-    rec = np.zeros(a.shape[0], dtype=[("stream", "<u4"), ("type", "<u4"), ("count", "<u8"),
-                                     ("d_out", "<u8")])
-    rec["stream"], rec["type"], rec["count"], rec["d_out"] = a[:, 0], a[:, 1], a[:, 2], a[:, 3]
+    rec = pack_rows(reqs).view([(n if n != "out" else "d_out", t) for n, t in _ROW])
     assert rec.itemsize == ctypes.sizeof(XgRequest)
     return rec
 
@@ -325,18 +362,18 @@ def xg_submit_many(ctx, rec, first, n, tickets):
 
 def xg_poll(ctx, ticket):
     done, ptr = ctypes.c_int(), ctypes.c_void_p()
-    call("xg_poll", ctypes.c_void_p(ctx), ticket, ctypes.byref(done), ctypes.byref(ptr))
+    call("xg_poll", ctx, ticket, ctypes.byref(done), ctypes.byref(ptr))
     return bool(done.value), ptr.value
 
 
 def xg_wait(ctx, ticket, timeout_ms=10000):
     ptr = ctypes.c_void_p()
-    call("xg_wait", ctypes.c_void_p(ctx), ticket, timeout_ms, ctypes.byref(ptr))
+    call("xg_wait", ctx, ticket, timeout_ms, ctypes.byref(ptr))
     return ptr.value
 
 
 def xg_release(ctx, ticket) -> None:
-    call("xg_release", ctypes.c_void_p(ctx), ticket)
+    call("xg_release", ctx, ticket)
 
 
 def xg_cancel(ctx, ticket) -> None:
@@ -439,12 +476,11 @@ def xg_w64_set_state(ctx: int, stream: int, host_ring_ptr: int, weyl: int) -> No
 
 
 def xg_w64_generate_u64(ctx, first, nstreams, n_per_stream, out_ptr, ld) -> None:
-    call("xg_w64_generate_u64", ctypes.c_void_p(ctx), first, nstreams, n_per_stream, ctypes.c_void_p(out_ptr), ld)
+    call("xg_w64_generate_u64", ctx, first, nstreams, n_per_stream, out_ptr, ld)
 
 
 def xg_w64_generate_uniform_f64(ctx, first, nstreams, n_per_stream, out_ptr, ld) -> None:
-    call("xg_w64_generate_uniform_f64", ctypes.c_void_p(ctx), first, nstreams, n_per_stream,
-         ctypes.c_void_p(out_ptr), ld)
+    call("xg_w64_generate_uniform_f64", ctx, first, nstreams, n_per_stream, out_ptr, ld)
 
 
 def xg_w64_transform_uniform_f64(ctx, words_ptr, n, out_ptr) -> None:

@@ -22,6 +22,18 @@ def _stream_handle(stream) -> int:
     return int(stream.cuda_stream)
 
 
+def _rows(items):
+    """(stream, kind, count, out) tuples as L.pack_rows records: kinds by name
+    or number, out a device tensor or None."""
+    items = items if isinstance(items, (list, tuple)) else list(items)
+    if not items:
+        return L.pack_rows([])
+    s, k, c, o = zip(*items, strict=True)
+    kinds = [TYPES[x] if isinstance(x, str) else int(x) for x in k]
+    ptrs = [0 if x is None else x.data_ptr() for x in o]
+    return L.pack_columns(s, kinds, c, ptrs)
+
+
 class Streams:
     """A context of n independent xorgens streams resident on the GPU.
 
@@ -149,8 +161,7 @@ class Streams:
     def batch(self, items):
         """One persistent-kernel launch for items (stream, kind, count, out)
         with out a device tensor (or None for count 0)."""
-        L.xg_generate_batch(self.ctx, [(int(s), TYPES[k] if isinstance(k, str) else int(k), int(c),
-                                        0 if o is None else o.data_ptr()) for s, k, c, o in items])
+        L.xg_generate_batch(self.ctx, _rows(items))
 
     def set_batch_shape(self, kind, tpg: int, wpl: int):
         """Batch-kernel shape for single calls of one type: (32,2), (16,4) or (8,4)."""
@@ -162,8 +173,7 @@ class Streams:
     def autotune_batch(self, items) -> dict:
         """Pick the batch-kernel shape per type on this batch (streams do not
         advance; the outputs are written).  Returns {kind: (tpg, wpl, ms)}."""
-        res = L.xg_autotune_batch(self.ctx, [(int(s), TYPES[k] if isinstance(k, str) else int(k), int(c),
-                                              0 if o is None else o.data_ptr()) for s, k, c, o in items])
+        res = L.xg_autotune_batch(self.ctx, _rows(items))
         return {name: res[TYPES[name]] for name in TYPES}
 
     def set_batch_split(self, piece_words: int):
@@ -201,11 +211,7 @@ class Server:
     def submit_many(self, requests, tickets=None):
         """Submit (stream, kind, count[, out]) tuples in one call; returns the
         tickets of the admitted ones (all of them unless the cap refused one)."""
-        rows = []
-        for r in requests:
-            k = TYPES[r[1]] if isinstance(r[1], str) else int(r[1])
-            out = r[3] if len(r) > 3 else None
-            rows.append((int(r[0]), k, int(r[2]), 0 if out is None else out.data_ptr()))
+        rows = _rows([r if len(r) == 4 else (r[0], r[1], r[2], r[3] if len(r) > 3 else None) for r in requests])
         rec = L.make_requests(rows)
         t = np.zeros(len(rows), dtype=np.uint64)
         n = L.xg_submit_many(self.ctx, rec, 0, len(rows), t)
