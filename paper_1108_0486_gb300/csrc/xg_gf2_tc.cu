@@ -5,22 +5,31 @@
 // Over the integers, with 0/1 entries, (C x)_i counts the set bits of row i
 // of C that meet set bits of x; the GF(2) result is that count's parity.  The
 // counts are at most 4096, which an FP32 accumulator holds exactly, and 0/1
-// are exact in FP8 E4M3, so the product of the matrix and a batch of states
-// is a plain FP8 GEMM with an FP32 accumulator:
+// are exact in FP4 E2M1, so the product of the matrix and a batch of states
+// is a block-scaled FP4 GEMM whose scales are all 1 (mxf4: UE8M0 127):
 //   D[i][s] = sum_k A[i][k] B[s][k],  A[i][k] = C[i][k],  B[s][k] = bit k of x_s
 // (M = 4096 output bits, N = states, K = 4096 input bits, both operands
 // K-major), followed by a parity epilogue that packs bits back into 32-bit
-// ring words.
+// ring words.  FP4 halves the bytes per operand of the same kernel in FP8
+// (kind::f8f6f4): one application to 16384 states 149 -> 98.6 us.  Bound by
+// the bytes into shared memory, 47 KB per 128 x 240 x 256 block or about
+// 114 B/ns per SM (17 TB/s over the GPU); the tensor pipe is 61% active.
 //
-// Kernel: persistent, one CTA per SM, 128 x 256 output tiles.  Warp 0 (one
-// lane) streams 128-byte-wide K blocks of A and B into a 4-stage
-// shared-memory ring with TMA (128B swizzle, mbarrier transaction counts);
-// warp 1 (one lane) issues tcgen05.mma (kind::f8f6f4, E4M3 x E4M3 -> F32,
-// 128 x 256 x 32 each) into one of two TMEM accumulators and frees each
-// stage with tcgen05.commit; four epilogue warps read the other accumulator
-// with tcgen05.ld (32 TMEM lanes = 32 output bits each), take each count's
-// parity and pack the 32 lanes' bits with a warp ballot: one ballot is one
-// ring word of one state.
+// Order of K: both operands hold the 32 bits of an input word as 32 nibbles
+// in the order that three shifts and masks give (spread32); a dot product
+// does not depend on it.
+//
+// Kernel: persistent, one CTA per SM, 128 x 240 output tiles (two FP32
+// accumulators of 240 columns and 32 columns of scales fill the 512 TMEM
+// columns).  Warp 0 (one lane) streams 128-byte-wide K blocks (256 bits) of A
+// and B into a 4-stage shared-memory ring with TMA (128B swizzle, mbarrier
+// transaction counts); warp 1 (one lane) issues tcgen05.mma (kind::mxf4,
+// E2M1 x E2M1 -> F32, 128 x 240 x 64 each) into one of two TMEM accumulators
+// and frees each stage with tcgen05.commit; four epilogue warps read the
+// other accumulator with tcgen05.ld (32 TMEM lanes = 32 output bits each),
+// take each count's parity and pack the 32 lanes' bits with a warp ballot:
+// one ballot is one ring word of one state.  The scales are written once: every byte of their
+// columns is 127, so no layout of them matters.
 //
 // Every wait is bounded (2 s of %globaltimer); a wait that gives up records
 // a failure in a host-visible status word, the CTA waits (bounded) for its
@@ -42,9 +51,13 @@ namespace xg {
 namespace {
 
 constexpr int kBM = 128;                  // output bits per tile (TMEM lanes)
-constexpr int kBN = 256;                  // states per tile (TMEM columns)
-constexpr int kBK = 128;                  // K per stage: one 128-byte swizzle row
-constexpr int kKBlocks = kGf2Bits / kBK;  // 32
+constexpr int kBN = 240;                  // states per tile (TMEM columns)
+constexpr int kRowBytes = kGf2Bits / 2;   // 4096 nibbles
+constexpr int kBK = 128;                  // bytes of K per stage: one 128-byte swizzle row
+constexpr int kKBlocks = kRowBytes / kBK; // 16
+constexpr int kTmemCols = 512;
+constexpr int kScaleA = 2 * kBN, kScaleB = 2 * kBN + 16;   // TMEM columns of the scales
+static_assert(kScaleB + 16 <= kTmemCols, "TMEM columns");
 constexpr int kStages = 4;
 constexpr int kABytes = kBM * kBK;        // 16 KiB
 constexpr int kBBytes = kBN * kBK;        // 32 KiB
@@ -52,7 +65,6 @@ constexpr int kStageBytes = kABytes + kBBytes;
 constexpr int kSmemBytes = kStages * kStageBytes + 1024 /* barriers */ + 1024 /* alignment */;
 constexpr int kEpilogueWarps = 4;
 constexpr int kThreads = 32 * (2 + kEpilogueWarps);
-constexpr uint8_t kOneE4M3 = 0x38;        // 1.0 in FP8 E4M3
 constexpr uint64_t kWaitLimitNs = 2000000000ull;
 
 __device__ __forceinline__ uint32_t smem_addr(const void* p)
@@ -118,19 +130,21 @@ __device__ __forceinline__ uint64_t smem_desc(const void* p)
            | (2ull << 61);                   // layout: 128-byte swizzle
 }
 
-// Instruction descriptor, kind::f8f6f4: D F32, A and B E4M3, both K-major,
-// N = kBN, M = kBM.
-constexpr uint32_t kInstrDesc = (1u << 4)                    // D format F32
-                                | (0u << 7) | (0u << 10)     // A, B: E4M3
-                                | ((uint32_t)(kBN >> 3) << 17) | ((uint32_t)(kBM >> 4) << 24);
+// Instruction descriptor, kind::mxf4: A and B E2M1, both K-major, UE8M0
+// scales (data id 0), K = 64, N = kBN, M = kBM.
+constexpr uint32_t kInstrDesc = (1u << 7) | (1u << 10)       // A, B: E2M1
+                                | (1u << 23)                 // scale type UE8M0
+                                | ((uint32_t)(kBN >> 3) << 17) | ((uint32_t)(kBM >> 7) << 27);
 
-__device__ __forceinline__ void mma_f8(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t accumulate)
+__device__ __forceinline__ void mma_f4(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t sa_tmem,
+                                       uint32_t sb_tmem, uint32_t accumulate)
 {
     asm volatile(
         "{\n\t.reg .pred p;\n\t"
         "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f8f6f4 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
-        "l"(adesc), "l"(bdesc), "r"(kInstrDesc), "r"(accumulate)
+        "tcgen05.mma.cta_group::1.kind::mxf4.block_scale.scale_vec::2X [%0], %1, %2, %3, [%5], [%6], p;\n\t}" ::"r"(
+            d_tmem),
+        "l"(adesc), "l"(bdesc), "r"(kInstrDesc), "r"(accumulate), "r"(sa_tmem), "r"(sb_tmem)
         : "memory");
 }
 
@@ -143,19 +157,27 @@ __device__ __forceinline__ void mma_commit(uint64_t* bar)
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 
-// 32 consecutive columns of this warp's 32 TMEM lanes: v[j] = column col + j.
-__device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&v)[32])
+// 16 consecutive columns of this warp's 32 TMEM lanes: v[j] = column col + j.
+__device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t* v)
 {
     asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
-        "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
-        "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
+        "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
         : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
-          "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15]),
-          "=r"(v[16]), "=r"(v[17]), "=r"(v[18]), "=r"(v[19]), "=r"(v[20]), "=r"(v[21]), "=r"(v[22]), "=r"(v[23]),
-          "=r"(v[24]), "=r"(v[25]), "=r"(v[26]), "=r"(v[27]), "=r"(v[28]), "=r"(v[29]), "=r"(v[30]), "=r"(v[31])
+          "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
         : "r"(taddr));
-    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
+
+// The same word to 16 consecutive columns of this warp's 32 TMEM lanes.
+__device__ __forceinline__ void tmem_fill16(uint32_t taddr, uint32_t x)
+{
+    asm volatile(
+        "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], "
+        "{%1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1};" ::"r"(taddr),
+        "r"(x)
+        : "memory");
+    asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
 }
 
 __device__ __forceinline__ void mbar_arrive(uint64_t* bar)
@@ -206,7 +228,7 @@ __global__ void __launch_bounds__(kThreads, 1) gf2_tc_kernel(const __grid_consta
     }
     if (warp == 1) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_addr(tmem_slot)),
-                     "r"((uint32_t)(2 * kBN))
+                     "r"((uint32_t)kTmemCols)
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
@@ -214,6 +236,14 @@ __global__ void __launch_bounds__(kThreads, 1) gf2_tc_kernel(const __grid_consta
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
+    if (warp >= 2) {
+        const uint32_t lanes = tmem + ((uint32_t)(warp & 3) * 32 << 16);
+        tmem_fill16(lanes + kScaleA, 0x7F7F7F7Fu);
+        tmem_fill16(lanes + kScaleB, 0x7F7F7F7Fu);
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
 
     uint32_t issued = 0;  // producer: K blocks whose copies were started
     if (warp == 0) {
@@ -256,7 +286,7 @@ __global__ void __launch_bounds__(kThreads, 1) gf2_tc_kernel(const __grid_consta
                     const uint64_t bd = smem_desc(sb + s * kBBytes);
 #pragma unroll
                     for (int kk = 0; kk < kBK / 32; ++kk)  // K = 32 bytes per instruction: +2 in 16-byte units
-                        mma_f8(d, ad + 2 * kk, bd + 2 * kk, (kb | kk) != 0);
+                        mma_f4(d, ad + 2 * kk, bd + 2 * kk, tmem + kScaleA, tmem + kScaleB, (kb | kk) != 0);
                     mma_commit(&empty[s]);
                 }
                 mma_commit(&tfull[acc]);  // arrives once this tile's MMAs have completed
@@ -277,19 +307,24 @@ __global__ void __launch_bounds__(kThreads, 1) gf2_tc_kernel(const __grid_consta
             if (failed(&s_failed)) break;
             const uint32_t mt = t % kMTiles, nt = t / kMTiles;
             const uint32_t word = mt * (kBM / 32) + q;  // ring word of these 32 bits
+            static_assert(kBN % 16 == 0, "columns are read 16 at a time");
             for (int c = 0; c < kBN; c += 32) {
                 uint32_t vals[32];
-                tmem_ld32(tmem + ((q * 32) << 16) + acc * kBN + (uint32_t)c, vals);
+                const uint32_t col = tmem + ((q * 32) << 16) + acc * kBN + (uint32_t)c;
+                tmem_ld16(col, vals);
+                if (c + 16 < kBN) tmem_ld16(col + 16, vals + 16);
+                tmem_ld_wait();
                 uint32_t mine = 0;
 #pragma unroll
                 for (int j = 0; j < 32; ++j) {
+                    if (j >= 16 && c + 16 >= kBN) break;
                     // the count is an integer <= 4096: adding 2^23 puts its parity in the last bit
                     const uint32_t bit = __float_as_uint(__uint_as_float(vals[j]) + 8388608.0f) & 1u;
                     const uint32_t b = __ballot_sync(0xFFFFFFFFu, bit);
                     if (lane == j) mine = b;
                 }
                 const uint32_t st = nt * kBN + (uint32_t)c + (uint32_t)lane;
-                if (st < n) rings[(size_t)dst[st] * kGf2Words + word] = mine;
+                if (st < n && c + lane < kBN) rings[(size_t)dst[st] * kGf2Words + word] = mine;
             }
             tc_fence_before();
             __syncwarp();
@@ -312,51 +347,48 @@ __global__ void __launch_bounds__(kThreads, 1) gf2_tc_kernel(const __grid_consta
     }
     if (warp == 1) {
         tc_fence_after();
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"((uint32_t)(2 * kBN))
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"((uint32_t)kTmemCols)
                      : "memory");
     }
 }
 
-// A[i][k] = bit i of column k of C (column form: column k = 128 ring words).
-// Thread (k, w): one word of one column, 32 rows of A.
-__global__ void expand_matrix_kernel(const uint32_t* __restrict__ cols, uint8_t* __restrict__ A)
+// 32 bits to 32 nibbles of 0 or 1.0 (E2M1: 2): nibble n of word j is bit 4 n + j.
+__device__ __forceinline__ uint4 spread32(uint32_t x)
 {
-    const uint32_t k = blockIdx.x * blockDim.x + threadIdx.x;
-    const uint32_t w = blockIdx.y;
-    if (k >= (uint32_t)kGf2Bits) return;
-    const uint32_t word = cols[(size_t)k * kGf2Words + w];
-#pragma unroll 8
-    for (int b = 0; b < 32; ++b) A[(size_t)(32 * w + b) * kGf2Bits + k] = ((word >> b) & 1u) ? kOneE4M3 : 0;
+    return make_uint4((x << 1) & 0x22222222u, x & 0x22222222u, (x >> 1) & 0x22222222u, (x >> 2) & 0x22222222u);
 }
 
-// Four bits to four E4M3 bytes (byte b = 1.0 when bit b is set).
-__device__ __forceinline__ uint32_t spread4(uint32_t x)
+// A[i][k] = bit i of column k of C (column form: column k = 128 ring words).
+// A warp transposes 32 x 32 bits: lane l holds output word w of column
+// 32 kw + l, and the ballot of bit b is row 32 w + b over those columns.
+// Neighbouring warps of a block take neighbouring kw, so a row's 16-byte
+// pieces are written by one block.
+__global__ void __launch_bounds__(256) expand_matrix_kernel(const uint32_t* __restrict__ cols,
+                                                            uint8_t* __restrict__ A)
 {
-    return ((x & 1u) | ((x & 2u) << 7) | ((x & 4u) << 14) | ((x & 8u) << 21)) * (uint32_t)kOneE4M3;
+    const uint32_t lane = threadIdx.x & 31u, kw = blockIdx.x * 8 + (threadIdx.x >> 5), w = blockIdx.y;
+    const uint32_t word = cols[(size_t)(32 * kw + lane) * kGf2Words + w];
+    uint32_t row = 0;
+#pragma unroll
+    for (int b = 0; b < 32; ++b) {
+        const uint32_t v = __ballot_sync(0xFFFFFFFFu, (word >> b) & 1u);
+        if (lane == (uint32_t)b) row = v;
+    }
+    *reinterpret_cast<uint4*>(A + (size_t)(32 * w + lane) * kRowBytes + 16 * kw) = spread32(row);
 }
 
 // B[s][k] = bit k of state src[s] (s < n), 0 for n <= s < n_pad.  Thread =
-// one ring word = 32 bytes of B.
-__global__ void expand_states_kernel(const uint32_t* __restrict__ rings, const uint32_t* __restrict__ src,
-                                     uint32_t n, uint32_t n_pad, uint8_t* __restrict__ B)
+// one ring word = 16 bytes of B.
+__global__ void __launch_bounds__(256) expand_states_kernel(const uint32_t* __restrict__ rings,
+                                                            const uint32_t* __restrict__ src, uint32_t n,
+                                                            uint32_t n_pad, uint8_t* __restrict__ B)
 {
     const uint64_t t = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= (uint64_t)n_pad * kGf2Words) return;
     const uint32_t s = (uint32_t)(t / kGf2Words), w = (uint32_t)(t % kGf2Words);
     uint32_t x = 0;
     if (s < n) x = rings[(size_t)(src ? src[s] : s) * kGf2Words + w];
-    uint4 lo, hi;
-    lo.x = spread4(x);
-    lo.y = spread4(x >> 4);
-    lo.z = spread4(x >> 8);
-    lo.w = spread4(x >> 12);
-    hi.x = spread4(x >> 16);
-    hi.y = spread4(x >> 20);
-    hi.z = spread4(x >> 24);
-    hi.w = spread4(x >> 28);
-    uint4* out = reinterpret_cast<uint4*>(B + (size_t)s * kGf2Bits + 32 * w);
-    out[0] = lo;
-    out[1] = hi;
+    *reinterpret_cast<uint4*>(B + (size_t)s * kRowBytes + 16 * w) = spread32(x);
 }
 
 // ---- host side -------------------------------------------------------------
@@ -404,8 +436,8 @@ bool init_locked()
 
 bool make_map(CUtensorMap* m, const uint8_t* base, uint64_t rows, uint32_t box_rows)
 {
-    const cuuint64_t dims[2] = {(cuuint64_t)kGf2Bits, (cuuint64_t)rows};
-    const cuuint64_t strides[1] = {(cuuint64_t)kGf2Bits};
+    const cuuint64_t dims[2] = {(cuuint64_t)kRowBytes, (cuuint64_t)rows};
+    const cuuint64_t strides[1] = {(cuuint64_t)kRowBytes};
     const cuuint32_t box[2] = {(cuuint32_t)kBK, box_rows};
     const cuuint32_t estr[2] = {1, 1};
     return g_encode(m, CU_TENSOR_MAP_DATA_TYPE_UINT8, 2, const_cast<uint8_t*>(base), dims, strides, box, estr,
@@ -430,11 +462,11 @@ bool gf2_tc_available(int device)
 
 uint32_t gf2_tc_padded(uint32_t n) { return (n + kBN - 1) / kBN * kBN; }
 
-size_t gf2_tc_scratch_bytes(uint32_t n) { return (size_t)gf2_tc_padded(n) * kGf2Bits; }
+size_t gf2_tc_scratch_bytes(uint32_t n) { return (size_t)gf2_tc_padded(n) * kRowBytes; }
 
 cudaError_t gf2_tc_expand_matrix(const uint64_t* C, uint8_t* A, cudaStream_t s)
 {
-    expand_matrix_kernel<<<dim3(kGf2Bits / 128, kGf2Words), 128, 0, s>>>(reinterpret_cast<const uint32_t*>(C), A);
+    expand_matrix_kernel<<<dim3(kGf2Words / 8, kGf2Words), 256, 0, s>>>(reinterpret_cast<const uint32_t*>(C), A);
     return cudaGetLastError();
 }
 

@@ -15,13 +15,16 @@ constexpr int kGf2Words = kGf2Bits / 32;   // 32-bit ring words per state
 // True on sm_103 with the driver's tensor-map encoder available.
 bool gf2_tc_available(int device);
 
-// States are padded to whole tiles of 256; the B operand scratch holds
-// gf2_tc_padded(n) * 4096 bytes.
+// States are padded to whole tiles of 240; the B operand scratch holds
+// gf2_tc_padded(n) * 2048 bytes.
 uint32_t gf2_tc_padded(uint32_t n);
 size_t gf2_tc_scratch_bytes(uint32_t n);
 
-// A (4096 x 4096 bytes, 16 MiB) = C in FP8 E4M3, row i over input bits k,
-// from C in column form (column k = the 128 ring words of C e_k).
+// Bytes of a matrix as the A operand.
+constexpr size_t kGf2TcMatrixBytes = (size_t)kGf2Bits * kGf2Bits / 2;
+
+// A (4096 x 2048 bytes, 8 MiB) = C in FP4 E2M1, row i over input bits k, from
+// C in column form (column k = the 128 ring words of C e_k).
 cudaError_t gf2_tc_expand_matrix(const uint64_t* C, uint8_t* A, cudaStream_t s);
 
 // rings_out[dst[i]] = C rings_in[src[i]] (src null: i) for i < n, with A from

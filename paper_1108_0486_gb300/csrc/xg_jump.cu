@@ -343,7 +343,7 @@ const uint64_t* jump_matrix(int device, int param_set, int k, cudaStream_t s, xg
 }
 
 namespace {
-// FP8 copies of the powers for the tensor-core path: 16 MiB each, built on
+// FP4 copies of the powers for the tensor-core path: 8 MiB each, built on
 // first use and kept until exit.
 std::mutex g_tc_mu;
 uint8_t* g_tc_mats[64][3][kMaxPow] = {};
@@ -356,17 +356,17 @@ const uint8_t* jump_matrix_tc(int device, int family, int k, cudaStream_t s, xg_
     uint8_t*& A = g_tc_mats[device][family][k];
     if (A) return A;
     void* p = nullptr;
-    cudaError_t e = cudaMalloc(&p, (size_t)kGf2Bits * kGf2Bits);
+    cudaError_t e = cudaMalloc(&p, kGf2TcMatrixBytes);
     if (e != cudaSuccess) {
         cudaGetLastError();
-        *st = fail(XG_ENOMEM, "jump tables: cudaMalloc(16 MiB) failed for the FP8 power %d", k);
+        *st = fail(XG_ENOMEM, "jump tables: cudaMalloc(8 MiB) failed for the FP4 power %d", k);
         return nullptr;
     }
     e = gf2_tc_expand_matrix(C, static_cast<uint8_t*>(p), s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);  // other CUDA streams may use it next
     if (e != cudaSuccess) {
         cudaFree(p);
-        *st = cuda_fail(e, "jump tables: FP8 expansion");
+        *st = cuda_fail(e, "jump tables: FP4 expansion");
         return nullptr;
     }
     A = static_cast<uint8_t*>(p);
@@ -380,7 +380,10 @@ bool gf2_use_tc(int device, uint32_t n)
     const char* off = std::getenv("XG_JUMP_TENSOR_CORES");
     if (off && std::strcmp(off, "0") == 0) return false;
     const char* v = std::getenv("XG_GF2_TC_MIN_STATES");
-    const uint32_t min_states = v ? (uint32_t)std::strtoul(v, nullptr, 10) : 1024u;
+    // One application in a call, table kernel against tensor cores: 31 / 35 us
+    // for 64 states, 35 / 38 for 160, 39 / 36 for 192, 57 / 38 for 512,
+    // 68 / 42 for 1024 (the tensor cores take one tile's time up to 1140).
+    const uint32_t min_states = v ? (uint32_t)std::strtoul(v, nullptr, 10) : 192u;
     return n >= std::max(1u, min_states) && gf2_tc_available(device);
 }
 
@@ -408,7 +411,7 @@ cudaError_t gf2_apply(int device, int family, int k, uint32_t* rings, uint32_t n
 }
 
 // rings[dst[i]] = P rings[src[i]] for a matrix P in column form that is not
-// one of the cached powers; A_buf (16 MiB) receives its FP8 copy when the
+// one of the cached powers; A_buf (8 MiB) receives its FP4 copy when the
 // tensor cores are used.
 static cudaError_t gf2_apply_explicit(int device, const uint64_t* P, uint8_t* A_buf, uint32_t* rings, uint32_t n,
                                       const uint32_t* d_src, const uint32_t* d_dst, uint8_t* scratch, int sm_count,
@@ -441,11 +444,11 @@ static size_t product_bytes(uint64_t words)
 
 size_t gf2_jump_work_bytes(int device, uint32_t n, uint64_t words)
 {
-    // the tensor-core operand, then the product's work area and its FP8 copy
+    // the tensor-core operand, then the product's work area and its FP4 copy
     size_t b = (gf2_apply_scratch(device, n) + 255) / 256 * 256;
     if (jump_combines(words, n)) {
         b += product_bytes(words);
-        if (gf2_use_tc(device, n)) b += (size_t)kGf2Bits * kGf2Bits;
+        if (gf2_use_tc(device, n)) b += kGf2TcMatrixBytes;
     }
     return b;
 }
@@ -474,14 +477,14 @@ cudaError_t gf2_jump_states(int device, int family, uint64_t words, uint32_t* ri
     // The product of the powers: its newest columns by one application per
     // further set bit to 32 (64) states, then all columns from them.  For
     // 16384 streams and 8 set bits this took the jump from 0.615 ms (seven
-    // tensor-core products of 4096 columns each) to @@ ms.
+    // tensor-core products of 4096 columns each) to 0.311 ms.
     uint8_t* w = work + (sbytes + 255) / 256 * 256;
     const int nb = newest_columns(family);
     const size_t group = (size_t)nb * kR;   // 32-bit words of one group of columns
     uint32_t* cols = reinterpret_cast<uint32_t*>(w);
     uint8_t* seq = w + (size_t)__builtin_popcountll(words) * kMaxNewest * kR * 4;
     uint64_t* prod = reinterpret_cast<uint64_t*>(seq + kSeqBytes);
-    uint8_t* abuf = scratch ? seq + kSeqBytes + (size_t)kBits * kR * 4 : nullptr;  // FP8 copy of the product
+    uint8_t* abuf = scratch ? seq + kSeqBytes + (size_t)kBits * kR * 4 : nullptr;  // FP4 copy of the product
     cudaError_t e = cudaMemsetAsync(cols + group, 0, (size_t)(__builtin_popcountll(words) - 1) * group * 4, s);
     int done = 0;
     for (int k = 0; k < 64 && e == cudaSuccess; ++k) {

@@ -25,7 +25,7 @@ cudaError_t launch_gf2_apply_pairs(const uint64_t* C, const uint32_t* in, uint32
                                    const uint32_t* d_src, const uint32_t* d_dst, int sm_count, cudaStream_t s);
 
 // Whether an application to n states runs on the tensor cores (sm_103 and
-// n >= XG_GF2_TC_MIN_STATES, default 1024; XG_JUMP_TENSOR_CORES=0 turns the
+// n >= XG_GF2_TC_MIN_STATES, default 192; XG_JUMP_TENSOR_CORES=0 turns the
 // tensor-core path off), and the device scratch it then needs (0 otherwise).
 bool gf2_use_tc(int device, uint32_t n);
 size_t gf2_apply_scratch(int device, uint32_t n);

@@ -128,7 +128,7 @@ def test_fp64_uniforms_of_words_with_many_leading_zeros(tpg, wpl):
 @pytest.mark.parametrize("words", [3, (1 << 40) + (1 << 20) + 12345, 0x9E3779B97F4A7C15])
 def test_jump_on_both_sides_of_its_thresholds(family, words):
     """The same jump of 64 states (one power after another), 65 (product of the
-    powers, table kernel) and 1024 (product, tensor cores): equal streams end
+    powers, table kernel) and 192 or 1024 (product, tensor cores): equal streams end
     in equal states, and those of the single-stream jump; short jumps equal
     stepping by the oracle."""
     from paper_1108_0486_gb300 import Streams, Streams64
@@ -141,13 +141,28 @@ def test_jump_on_both_sides_of_its_thresholds(family, words):
         return (st.u64(70) if family == 64 else st.u32(140)).cpu().numpy()
 
     rows = {}
-    for n in (1, 64, 65, 1024):
+    for n in (1, 64, 65, 192, 1024):
         with make(n) as st:
             st.jump(words)
             rows[n] = draw(st)
     assert np.array_equal(rows[64], rows[65][:64]) and np.array_equal(rows[65], rows[1024][:65])
+    assert np.array_equal(rows[192], rows[1024][:192])
     assert np.array_equal(rows[1][0], rows[64][0])
     if words == 3:
         seeds = W.seeds(4)
         ref = O.streams64(seeds, 73) if family == 64 else O.streams(seeds, 143, param_set=family)
         assert np.array_equal(rows[65][:4].view(ref.dtype), ref[:, 3:])
+
+
+@pytest.mark.parametrize("n", [191, 192, 239, 240, 241, 480, 1141])
+def test_tensor_core_jump_at_tile_edges(n, monkeypatch):
+    """One power applied to n states on the tensor cores (tiles of 240 states,
+    used from 192) equals the table kernel's result."""
+    from paper_1108_0486_gb300 import Streams
+    rows = []
+    for tc in ("1", "0"):
+        monkeypatch.setenv("XG_JUMP_TENSOR_CORES", tc)
+        with Streams(n, seeds=W.seeds(n)) as st:
+            st.jump(1 << 37)
+            rows.append(st.u32(128).cpu().numpy())
+    assert np.array_equal(rows[0], rows[1])
