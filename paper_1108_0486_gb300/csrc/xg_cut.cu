@@ -1,0 +1,242 @@
+// Cut calls (see xg_cut.h): choice of the piece length, the jump-ahead
+// prologue and its launch.
+//
+// One stream is a serial chain of rounds that one warp runs (Sec. 2), so a
+// call on few streams leaves most of the GPU idle.  Piece m of a stream starts
+// from its ring advanced by m 2^q words.  The prologue computes those rings in
+// a few steps: a step takes the pieces m < B of every stream to the pieces
+// m + j B, j = 1 .. J, with the matrices M^(j B 2^q).  All of it is regular,
+// so the index lists are built on the device and nothing is uploaded.
+//
+// One stream of 2^20 words: 73 us with a planned batch (two uploads, a gather,
+// five doubling steps, pieces of 2^15 words), @@ us this way.
+#include "xg_cut.h"
+
+#include <algorithm>
+
+#include "xg_gf2_tc.h"
+#include "xg_jump.h"
+#include "xg_launch.h"
+#include "xg_runtime.h"
+
+namespace xg {
+namespace {
+
+constexpr int kMaxSteps = 32;
+constexpr uint64_t kMaxPieces = uint64_t(1) << 22;   // 2 GiB of rings
+
+// One prologue step: sources are the pieces m < have of every stream,
+// destinations m + j have for j = 1 .. mats (kNoState past the last piece).
+struct Step {
+    uint32_t have;
+    uint32_t mats;
+    uint64_t at;    // its sources in the list, then mats destination lists
+};
+struct Steps {
+    Step step[kMaxSteps];
+    int n;
+    uint64_t entries;
+};
+
+// Up to 7 matrices per step while the states are few (a step then costs a
+// launch and the matrix read, not the lookups): up to 16 sources 3.5 us with
+// one matrix and @@ with 7; single doubling steps from 49 on, whose 192 or more
+// states run on the tensor cores.
+Steps plan_steps(uint32_t nstreams, uint32_t pieces)
+{
+    Steps p{};
+    for (uint64_t have = 1; have < pieces && p.n < kMaxSteps; ++p.n) {
+        const uint64_t sources = have * nstreams;
+        const uint64_t most = sources <= 16 ? 7 : sources <= 48 ? 3 : 1;
+        const uint64_t mats = std::min<uint64_t>(most, (pieces + have - 1) / have - 1);
+        p.step[p.n] = Step{(uint32_t)have, (uint32_t)mats, p.entries};
+        p.entries += sources * (1 + mats);
+        have *= 1 + mats;
+    }
+    return p;
+}
+
+// Piece 0 of a stream takes its ring, the other pieces zero rings (the table
+// kernel XORs into them); weyl0[i] = stream i's Weyl word; then the lists of
+// all steps.  A warp per piece, 8 to a block; blocks past the pieces write
+// the lists.
+__global__ void __launch_bounds__(256) cut_setup_kernel(State st, uint32_t first, uint32_t nstreams, uint32_t pieces,
+                                                        uint32_t piece_blocks, uint32_t* __restrict__ rings,
+                                                        uint32_t* __restrict__ weyl0, Steps steps,
+                                                        uint32_t* __restrict__ lists)
+{
+    cudaTriggerProgrammaticLaunchCompletion();
+    if (blockIdx.x < piece_blocks) {
+        const uint32_t p = blockIdx.x * 8 + threadIdx.x / 32, lane = threadIdx.x % 32;
+        if (p >= nstreams * pieces) return;
+        uint4 v = make_uint4(0, 0, 0, 0);
+        if (p % pieces == 0) {
+            const uint32_t s = first + p / pieces;
+            const uint32_t* src = st.win + (size_t)s * kWin + (kRingBase - st.pend[s]) + 4 * lane;
+            v = make_uint4(src[0], src[1], src[2], src[3]);
+            if (lane == 0) weyl0[p / pieces] = st.weyl[s];
+        }
+        reinterpret_cast<uint4*>(rings + (size_t)p * 128)[lane] = v;
+        return;
+    }
+    const uint64_t e = (uint64_t)(blockIdx.x - piece_blocks) * 256 + threadIdx.x;
+    if (e >= steps.entries) return;
+    int k = 0;
+    while (k + 1 < steps.n && e >= steps.step[k + 1].at) ++k;
+    const uint32_t have = steps.step[k].have, sources = have * nstreams;
+    const uint64_t r = e - steps.step[k].at;
+    const uint32_t j = (uint32_t)(r / sources), x = (uint32_t)(r % sources);   // j = 0: the sources
+    const uint32_t i = x / have, m = x % have + j * have;
+    lists[e] = m < pieces ? i * pieces + m : kNoState;
+}
+
+// Time of one word on a sub-partition of an SM that runs w warps, in ns,
+// fitted to a sweep of 100 .. 4000 whole streams: one warp alone is bound by
+// its own chain, several by the pipes.
+double word_ns(int kind, double w)
+{
+    switch (kind) {
+    case kU32: return std::max(0.585, 0.365 * w);
+    case kUniform: return std::max(0.62, 0.42 * w);
+    default: return std::max(1.34, 0.55 + 0.68 * w);
+    }
+}
+
+// Prologue time in us: the set-up launch, then per step a table-kernel launch
+// or, from 192 states, one tensor-core application (a wave of output tiles is
+// 240 states on 32 of the SMs).
+double prologue_us(uint32_t nstreams, uint64_t pieces, int sm_count)
+{
+    const Steps p = plan_steps(nstreams, (uint32_t)pieces);
+    double t = 6.0;
+    for (int k = 0; k < p.n; ++k) {
+        const uint64_t n = (uint64_t)p.step[k].have * nstreams;
+        if (n < 192) {
+            t += 5.5 + 0.025 * (double)n * p.step[k].mats;
+        } else {
+            const uint64_t tiles = (n + 239) / 240 * 32;
+            t += 6.0 + 6.6 * (double)((tiles + sm_count - 1) / sm_count);
+        }
+    }
+    return t;
+}
+
+}  // namespace
+
+int cut_choose(int kind, uint32_t nstreams, uint64_t n, int sm_count, uint64_t forced)
+{
+    const uint64_t words = kind == kNormal ? n + (n & 1u) : n;
+    if (forced) {
+        int q = 6;
+        while ((uint64_t(1) << q) < forced) ++q;
+        if (words < (uint64_t)2 << q || ((words + (uint64_t(1) << q) - 1) >> q) * nstreams > kMaxPieces) return 0;
+        return q;
+    }
+    const double parts = 4.0 * sm_count;
+    if (nstreams > 6 * parts) return 0;   // the pipes are busy as it is
+    auto warps = [&](double units) { return std::max(1.0, (double)(uint64_t)((units + parts - 1) / parts)); };
+    // the whole call, less 10% so that a cut has to be clearly the faster
+    double best = 0.9e-3 * (double)words * word_ns(kind, warps(nstreams));
+    int best_q = 0;
+    for (int q = 12; q <= 32; ++q) {
+        const uint64_t len = uint64_t(1) << q;
+        if (words < 2 * len) break;
+        const uint64_t pieces = (words + len - 1) / len;
+        if (pieces * nstreams > kMaxPieces) continue;
+        const double t = prologue_us(nstreams, pieces, sm_count) +
+                         1e-3 * (double)len * word_ns(kind, warps((double)nstreams * (double)pieces));
+        if (t < best) {
+            best = t;
+            best_q = q;
+        }
+    }
+    return best_q;
+}
+
+xg_status cut_generate(xg_ctx* c, int kind, uint32_t first, uint32_t nstreams, uint64_t n, void* out, uint64_t ld,
+                       int q, bool* ran)
+{
+    *ran = false;
+    const uint64_t words = kind == kNormal ? n + (n & 1u) : n;
+    const uint32_t pieces = (uint32_t)((words + (uint64_t(1) << q) - 1) >> q);
+    const uint32_t total = pieces * nstreams;
+    const Steps steps = plan_steps(nstreams, pieces);
+    cudaStream_t s = c->stream;
+    uint32_t most_tc = 0;   // states of the largest tensor-core step
+    for (int k = 0; k < steps.n; ++k) {
+        const uint32_t m = steps.step[k].have * nstreams;
+        if (steps.step[k].mats == 1 && gf2_use_tc(c->device, m)) most_tc = std::max(most_tc, m);
+    }
+    const size_t weyl_off = (size_t)total * 512;
+    const size_t list_off = (weyl_off + (size_t)nstreams * 4 + 255) / 256 * 256;
+    const size_t tc_off = (list_off + (size_t)steps.entries * 4 + 255) / 256 * 256;
+    const size_t bytes = tc_off + (most_tc ? gf2_tc_scratch_bytes(most_tc) : 0);
+    if (c->ensure_cut_ws(bytes) != XG_OK) return XG_OK;
+    char* ws = static_cast<char*>(c->cut_ws);
+    uint32_t* rings = reinterpret_cast<uint32_t*>(ws);
+    uint32_t* weyl0 = reinterpret_cast<uint32_t*>(ws + weyl_off);
+    uint32_t* lists = reinterpret_cast<uint32_t*>(ws + list_off);
+    uint8_t* tc = most_tc ? reinterpret_cast<uint8_t*>(ws + tc_off) : nullptr;
+    // the matrices first: building one on its first use synchronises
+    const uint64_t* mats[kMaxSteps][kMaxMats] = {};
+    xg_status st = XG_OK;
+    for (int k = 0; k < steps.n; ++k)
+        for (uint32_t j = 1; j <= steps.step[k].mats; ++j) {
+            uint64_t f = (uint64_t)j * steps.step[k].have;   // the exponent is f 2^q
+            int e = q;
+            while (f % 2 == 0) {
+                f /= 2;
+                ++e;
+            }
+            mats[k][j - 1] = jump_matrix_multiple(c->device, (int)c->param_set, (int)f, e, s, &st);
+            if (!mats[k][j - 1]) return st == XG_ENOMEM ? XG_OK : st;   // no memory: the whole call needs none
+        }
+    *ran = true;
+    if (xg_status w = c->cut_ws_acquire()) return w;
+    const uint32_t piece_blocks = (total + 7) / 8;
+    const uint32_t list_blocks = (uint32_t)((steps.entries + 255) / 256);
+    cut_setup_kernel<<<piece_blocks + list_blocks, 256, 0, s>>>(c->st, first, nstreams, pieces, piece_blocks, rings,
+                                                                weyl0, steps, lists);
+    cudaError_t e = cudaGetLastError();
+    bool dependent = true;   // the launch before is the set-up or a table kernel
+    for (int k = 0; k < steps.n && e == cudaSuccess; ++k) {
+        const uint32_t m = steps.step[k].have * nstreams;
+        const uint32_t* src = lists + steps.step[k].at;
+        const uint32_t* dst = src + m;
+        if (steps.step[k].mats == 1 && tc && gf2_use_tc(c->device, m)) {
+            int e2 = q;
+            uint64_t f = steps.step[k].have;
+            while (f % 2 == 0) {
+                f /= 2;
+                ++e2;
+            }
+            e = gf2_apply_matrix_tc(c->device, (int)c->param_set, (int)f, e2, rings, m, src, dst, tc, s, &st);
+            dependent = false;
+        } else {
+            e = launch_gf2_apply_multi(mats[k], (int)steps.step[k].mats, rings, rings, m, src, dst, c->sm_count, s,
+                                       dependent);
+            dependent = true;
+        }
+    }
+    if (e == cudaSuccess) {
+        CutArgs a{};
+        a.st = c->st;
+        a.first = first;
+        a.nstreams = nstreams;
+        a.pieces = pieces;
+        a.log2_len = (uint32_t)q;
+        a.n = n;
+        a.out = out;
+        a.ld = ld;
+        a.rings = rings;
+        a.weyl0 = weyl0;
+        a.omega = c->weyl_on ? 0x9E3779B9u : 0u;
+        a.dependent = dependent;
+        const bool vec = ((reinterpret_cast<uintptr_t>(out) & 15u) == 0) && (ld % 4 == 0 || nstreams == 1);
+        e = launch_cut((int)c->param_set, kind, vec, a, s);
+    }
+    if (e != cudaSuccess) return st != XG_OK ? st : cuda_fail(e, "cut generation");
+    return c->cut_ws_release(most_tc != 0);
+}
+
+}  // namespace xg

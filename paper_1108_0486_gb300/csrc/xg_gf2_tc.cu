@@ -324,7 +324,10 @@ __global__ void __launch_bounds__(kThreads, 1) gf2_tc_kernel(const __grid_consta
                     if (lane == j) mine = b;
                 }
                 const uint32_t st = nt * kBN + (uint32_t)c + (uint32_t)lane;
-                if (st < n && c + lane < kBN) rings[(size_t)dst[st] * kGf2Words + word] = mine;
+                if (st < n && c + lane < kBN) {
+                    const uint32_t d = dst[st];
+                    if (d != kNoState) rings[(size_t)d * kGf2Words + word] = mine;
+                }
             }
             tc_fence_before();
             __syncwarp();

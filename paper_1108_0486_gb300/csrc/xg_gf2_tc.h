@@ -12,6 +12,9 @@ namespace xg {
 constexpr int kGf2Bits = 4096;             // state bits = matrix order
 constexpr int kGf2Words = kGf2Bits / 32;   // 32-bit ring words per state
 
+// A destination index that takes no result.
+constexpr uint32_t kNoState = 0xFFFFFFFFu;
+
 // True on sm_103 with the driver's tensor-map encoder available.
 bool gf2_tc_available(int device);
 

@@ -15,6 +15,11 @@ cudaError_t launch_gen_default(int cfg, int out_kind, bool vec, int block, const
     return launch_gen_impl<ParamsDefault>(cfg, out_kind, vec, block, a, s);
 }
 
+cudaError_t launch_cut_default(int out_kind, bool vec, const CutArgs& a, cudaStream_t s)
+{
+    return launch_cut_impl<ParamsDefault>(out_kind, vec, a, s);
+}
+
 const void* batch_kernel_ptr_default(bool groups) { return batch_kernel_ptr<ParamsDefault>(groups); }
 
 }  // namespace xg

@@ -15,6 +15,11 @@ cudaError_t launch_gen_paper(int cfg, int out_kind, bool vec, int block, const G
     return launch_gen_impl<ParamsPaper>(cfg, out_kind, vec, block, a, s);
 }
 
+cudaError_t launch_cut_paper(int out_kind, bool vec, const CutArgs& a, cudaStream_t s)
+{
+    return launch_cut_impl<ParamsPaper>(out_kind, vec, a, s);
+}
+
 const void* batch_kernel_ptr_paper(bool groups) { return batch_kernel_ptr<ParamsPaper>(groups); }
 
 }  // namespace xg

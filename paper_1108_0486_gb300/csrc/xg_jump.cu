@@ -116,61 +116,85 @@ __global__ void __launch_bounds__(128) step_columns_kernel(uint32_t* __restrict_
 }
 
 // dst[i] ^= C src[i] for n (src, dst) pairs, dst zeroed beforehand.  Block
-// (x, y): pairs [48x, 48x+48), columns [y*cols, (y+1)*cols); 128 threads,
-// thread t owns 32-bit word t of every result.  Columns go four at a time:
-// each thread tabulates the 16 XOR combinations of its word of the four
-// columns (in shared memory, its own column of the table, so no barrier is
-// needed), and a state then costs one lookup and one XOR per four columns.
+// (x, y, z): matrix z, pairs [NV x, NV x + NV), columns [y*cols, (y+1)*cols);
+// 128 threads, thread t owns 32-bit word t of every result.  Columns go four
+// at a time: each thread tabulates the 16 XOR combinations of its word of the
+// four columns (in shared memory, its own column of the table, so no barrier
+// is needed), and a state then costs one lookup and one XOR per four columns.
 // Partial results are folded into dst with one atomic XOR per pair.  The
 // shared-memory traffic of the lookups and of building the tables bounds the
 // kernel, so many states per block (NV = 48) spread each table over more
 // lookups: on GB300, 16384 states x 8 applications take 3.3 ms against
 // 5.1 ms with 16 (64 gains no more and needs 168 registers a thread).  Few
-// states take NV = 16, which pads less.
+// states take NV = 16, which pads less, and up to 4 states NV = 4 without
+// tables: there the latency of the loads is the cost, so a block asks for its
+// first 32 columns, which no earlier kernel writes, before it waits for the
+// kernel before it (programmatic dependent launch).
+struct MatSet {
+    const uint32_t* C[kMaxMats];
+};
 template <int kPairVecs>
 // rings and out may be the same array (sources are read, distinct destinations
 // are written), so neither is declared __restrict__.
-__global__ void __launch_bounds__(128) gf2_apply_pairs_kernel(const uint32_t* __restrict__ C,
-                                                              const uint32_t* rings,
+__global__ void __launch_bounds__(128) gf2_apply_pairs_kernel(MatSet mats, const uint32_t* rings,
                                                               const uint32_t* __restrict__ src,
                                                               const uint32_t* __restrict__ dst, uint32_t n,
                                                               uint32_t* out, int cols)
 {
     __shared__ uint32_t vbits[kPairVecs][kR];
-    __shared__ uint32_t tbl[16][kR];
+    __shared__ uint32_t tbl[kPairVecs > 4 ? 16 : 1][kR];
+    const uint32_t* __restrict__ C = mats.C[blockIdx.z];
+    dst += (size_t)blockIdx.z * n;
     const int t = threadIdx.x;
     const uint32_t base = blockIdx.x * kPairVecs;
     const int nv = (int)umin((uint32_t)kPairVecs, n - base);
+    const int w0 = blockIdx.y * (cols / 32), w1 = w0 + cols / 32;
+    uint32_t col[32];   // 32 columns of one input word
+    auto load_columns = [&](int w) {
+        const uint32_t* colw = C + (size_t)w * 32 * kR + t;
+#pragma unroll
+        for (int b = 0; b < 32; ++b) col[b] = __ldg(colw + (size_t)b * kR);
+    };
+    cudaTriggerProgrammaticLaunchCompletion();
+    load_columns(w0);
+    cudaGridDependencySynchronize();
     for (int v = 0; v < kPairVecs; ++v)
         vbits[v][t] = v < nv ? rings[(size_t)src[base + v] * kR + t] : 0u;
     __syncthreads();
     uint32_t acc[kPairVecs];
 #pragma unroll
     for (int v = 0; v < kPairVecs; ++v) acc[v] = 0;
-    const int w0 = blockIdx.y * (cols / 32), w1 = w0 + cols / 32;
-    for (int w = w0; w < w1; ++w) {  // 32 columns per input word
-        const uint32_t* colw = C + (size_t)w * 32 * kR + t;
-        uint32_t col[32];
-#pragma unroll
-        for (int b = 0; b < 32; ++b) col[b] = __ldg(colw + (size_t)b * kR);
+    for (int w = w0;;) {
         uint32_t bw[kPairVecs];
 #pragma unroll
         for (int v = 0; v < kPairVecs; ++v) bw[v] = vbits[v][w];
+        if constexpr (kPairVecs <= 4) {
 #pragma unroll
-        for (int g = 0; g < 8; ++g) {
-            const uint32_t c0 = col[4 * g], c1 = col[4 * g + 1], c2 = col[4 * g + 2], c3 = col[4 * g + 3];
-            const uint32_t c01 = c0 ^ c1, c23 = c2 ^ c3;
-            tbl[0][t] = 0u;        tbl[1][t] = c0;         tbl[2][t] = c1;         tbl[3][t] = c01;
-            tbl[4][t] = c2;        tbl[5][t] = c2 ^ c0;    tbl[6][t] = c2 ^ c1;    tbl[7][t] = c2 ^ c01;
-            tbl[8][t] = c3;        tbl[9][t] = c3 ^ c0;    tbl[10][t] = c3 ^ c1;   tbl[11][t] = c3 ^ c01;
-            tbl[12][t] = c23;      tbl[13][t] = c23 ^ c0;  tbl[14][t] = c23 ^ c1;  tbl[15][t] = c23 ^ c01;
+            for (int b = 0; b < 32; ++b)
 #pragma unroll
-            for (int v = 0; v < kPairVecs; ++v) acc[v] ^= tbl[(bw[v] >> (4 * g)) & 15u][t];
+                for (int v = 0; v < kPairVecs; ++v) acc[v] ^= col[b] & (0u - ((bw[v] >> b) & 1u));
+        } else {
+#pragma unroll
+            for (int g = 0; g < 8; ++g) {
+                const uint32_t c0 = col[4 * g], c1 = col[4 * g + 1], c2 = col[4 * g + 2], c3 = col[4 * g + 3];
+                const uint32_t c01 = c0 ^ c1, c23 = c2 ^ c3;
+                tbl[0][t] = 0u;        tbl[1][t] = c0;         tbl[2][t] = c1;         tbl[3][t] = c01;
+                tbl[4][t] = c2;        tbl[5][t] = c2 ^ c0;    tbl[6][t] = c2 ^ c1;    tbl[7][t] = c2 ^ c01;
+                tbl[8][t] = c3;        tbl[9][t] = c3 ^ c0;    tbl[10][t] = c3 ^ c1;   tbl[11][t] = c3 ^ c01;
+                tbl[12][t] = c23;      tbl[13][t] = c23 ^ c0;  tbl[14][t] = c23 ^ c1;  tbl[15][t] = c23 ^ c01;
+#pragma unroll
+                for (int v = 0; v < kPairVecs; ++v) acc[v] ^= tbl[(bw[v] >> (4 * g)) & 15u][t];
+            }
         }
+        if (++w == w1) break;
+        load_columns(w);
     }
 #pragma unroll
     for (int v = 0; v < kPairVecs; ++v)
-        if (v < nv && acc[v]) atomicXor(&out[(size_t)dst[base + v] * kR + t], acc[v]);
+        if (v < nv && acc[v]) {
+            const uint32_t d = dst[base + v];
+            if (d != kNoState) atomicXor(&out[(size_t)d * kR + t], acc[v]);
+        }
 }
 
 __global__ void zero_listed_kernel(uint32_t* __restrict__ rings, const uint32_t* __restrict__ idx, uint32_t n)
@@ -267,14 +291,16 @@ namespace {
 struct Tables {
     uint64_t* mat[kMaxPow] = {};  // C_k: 4096 columns x 64 uint64 (2 MiB), allocated when built
     int built = 0;                // C_0 .. C_{built-1} are valid
+    uint64_t* odd[3][kMaxPow] = {};  // M^(j 2^k) for j = 3, 5, 7
     uint8_t* scratch = nullptr;   // squaring: kMaxNewest states, sequences, identity list
 };
 std::mutex g_tab_mu;
 Tables g_tabs[64][3];  // per device, per matrix family
 }  // namespace
 
-// C_{b+1} from C_b: C_b applied to its own newest columns.
-static cudaError_t square_matrix(int device, int family, Tables& T, int b, cudaStream_t s)
+// out = A B (powers of one matrix): A applied to B's newest columns.
+static cudaError_t multiply_matrices(int device, int family, Tables& T, const uint64_t* A, const uint64_t* B,
+                                     uint64_t* out, cudaStream_t s)
 {
     const int nb = newest_columns(family);
     uint32_t* states = reinterpret_cast<uint32_t*>(T.scratch);
@@ -285,8 +311,8 @@ static cudaError_t square_matrix(int device, int family, Tables& T, int b, cudaS
     if (e == cudaSuccess) e = launch_jump_index(ids, (uint32_t)nb, 0u, s);
     if (e == cudaSuccess) e = cudaMemsetAsync(states, 0, (size_t)nb * kR * 4, s);
     if (e == cudaSuccess)
-        e = launch_gf2_apply_pairs(T.mat[b], newest_of(T.mat[b], family), states, (uint32_t)nb, ids, ids, sms, s);
-    if (e == cudaSuccess) e = launch_build_columns(family, states, seq, T.mat[b + 1], s);
+        e = launch_gf2_apply_pairs(A, newest_of(B, family), states, (uint32_t)nb, ids, ids, sms, s);
+    if (e == cudaSuccess) e = launch_build_columns(family, states, seq, out, s);
     return e;
 }
 
@@ -324,7 +350,7 @@ const uint64_t* jump_matrix(int device, int param_set, int k, cudaStream_t s, xg
             else
                 step_columns_kernel<ParamsDefault><<<kBits / 128, 128, 0, s>>>(reinterpret_cast<uint32_t*>(T.mat[0]));
         } else {
-            e = square_matrix(device, param_set, T, b - 1, s);
+            e = multiply_matrices(device, param_set, T, T.mat[b - 1], T.mat[b - 1], T.mat[b], s);
         }
         if (e == cudaSuccess) e = cudaGetLastError();
         if (e != cudaSuccess) {
@@ -342,18 +368,55 @@ const uint64_t* jump_matrix(int device, int param_set, int k, cudaStream_t s, xg
     return T.mat[k];
 }
 
+const uint64_t* jump_matrix_multiple(int device, int param_set, int j, int k, cudaStream_t s, xg_status* st)
+{
+    while (j > 1 && j % 2 == 0) {
+        j /= 2;
+        ++k;
+    }
+    if (j == 1) return jump_matrix(device, param_set, k, s, st);
+    // j = 3, 5, 7: M^(2^k) times M^((j - 1) 2^k), itself an even multiple
+    const uint64_t* a = jump_matrix(device, param_set, k, s, st);
+    const uint64_t* b = a ? jump_matrix_multiple(device, param_set, j - 1, k, s, st) : nullptr;
+    if (!b) return nullptr;
+    std::lock_guard<std::mutex> lk(g_tab_mu);
+    Tables& T = g_tabs[device][param_set];
+    uint64_t*& C = T.odd[(j - 3) / 2][k];
+    if (C) return C;
+    void* p = nullptr;
+    cudaError_t e = cudaMalloc(&p, (size_t)kBits * kWords64 * 8);
+    if (e != cudaSuccess) {
+        cudaGetLastError();
+        *st = fail(XG_ENOMEM, "jump tables: cudaMalloc(2 MiB) failed for %d times power %d", j, k);
+        return nullptr;
+    }
+    e = multiply_matrices(device, param_set, T, a, b, static_cast<uint64_t*>(p), s);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s);  // other CUDA streams may use it next
+    if (e != cudaSuccess) {
+        cudaFree(p);
+        *st = cuda_fail(e, "jump table build");
+        return nullptr;
+    }
+    return C = static_cast<uint64_t*>(p);
+}
+
 namespace {
 // FP4 copies of the powers for the tensor-core path: 8 MiB each, built on
 // first use and kept until exit.
 std::mutex g_tc_mu;
-uint8_t* g_tc_mats[64][3][kMaxPow] = {};
+uint8_t* g_tc_mats[64][3][4][kMaxPow] = {};   // [.. j = 1, 3, 5, 7][k]
 
-const uint8_t* jump_matrix_tc(int device, int family, int k, cudaStream_t s, xg_status* st)
+// M^(j 2^k) as the A operand.
+const uint8_t* jump_matrix_tc(int device, int family, int j, int k, cudaStream_t s, xg_status* st)
 {
-    const uint64_t* C = jump_matrix(device, family, k, s, st);
+    while (j > 1 && j % 2 == 0) {
+        j /= 2;
+        ++k;
+    }
+    const uint64_t* C = jump_matrix_multiple(device, family, j, k, s, st);
     if (!C) return nullptr;
     std::lock_guard<std::mutex> lk(g_tc_mu);
-    uint8_t*& A = g_tc_mats[device][family][k];
+    uint8_t*& A = g_tc_mats[device][family][j / 2][k];
     if (A) return A;
     void* p = nullptr;
     cudaError_t e = cudaMalloc(&p, kGf2TcMatrixBytes);
@@ -399,7 +462,7 @@ cudaError_t gf2_apply(int device, int family, int k, uint32_t* rings, uint32_t n
     *st = XG_OK;
     if (n == 0) return cudaSuccess;
     if (scratch && gf2_use_tc(device, n)) {
-        const uint8_t* A = jump_matrix_tc(device, family, k, s, st);
+        const uint8_t* A = jump_matrix_tc(device, family, 1, k, s, st);
         if (!A) return cudaErrorMemoryAllocation;
         return gf2_tc_apply(device, A, rings, d_src, n, rings, d_dst, scratch, s);
     }
@@ -408,6 +471,15 @@ cudaError_t gf2_apply(int device, int family, int k, uint32_t* rings, uint32_t n
     cudaError_t e = dst_zeroed ? cudaSuccess : zero_rings(rings, d_dst, n, s);
     if (e == cudaSuccess) e = launch_gf2_apply_pairs(C, rings, rings, n, d_src, d_dst, sm_count, s);
     return e;
+}
+
+cudaError_t gf2_apply_matrix_tc(int device, int family, int j, int k, uint32_t* rings, uint32_t n,
+                                const uint32_t* d_src, const uint32_t* d_dst, uint8_t* scratch, cudaStream_t s,
+                                xg_status* st)
+{
+    const uint8_t* A = jump_matrix_tc(device, family, j, k, s, st);
+    if (!A) return cudaErrorMemoryAllocation;
+    return gf2_tc_apply(device, A, rings, d_src, n, rings, d_dst, scratch, s);
 }
 
 // rings[dst[i]] = P rings[src[i]] for a matrix P in column form that is not
@@ -494,7 +566,8 @@ cudaError_t gf2_jump_states(int device, int family, uint64_t words, uint32_t* ri
         if (done == 0)
             e = cudaMemcpyAsync(cols, newest_of(C, family), group * 4, cudaMemcpyDeviceToDevice, s);
         else
-            e = launch_gf2_apply_pairs(C, cols + (done - 1) * group, cols + done * group, (uint32_t)nb, lo, lo, sm_count, s);
+            e = launch_gf2_apply_pairs(C, cols + (done - 1) * group, cols + done * group, (uint32_t)nb, lo, lo, sm_count, s,
+                                       done > 1);
         ++done;
     }
     if (e == cudaSuccess) e = launch_build_columns(family, cols + (done - 1) * group, seq, prod, s);
@@ -521,26 +594,38 @@ cudaError_t launch_jump_index(uint32_t* ids, uint32_t n, uint32_t first, cudaStr
 }
 
 template <int NV>
-static cudaError_t launch_pairs(const uint64_t* C, const uint32_t* in, uint32_t* out, uint32_t n,
-                                const uint32_t* d_src, const uint32_t* d_dst, int sm_count, cudaStream_t s)
+static cudaError_t launch_pairs(const MatSet& mats, int n_mats, const uint32_t* in, uint32_t* out, uint32_t n,
+                                const uint32_t* d_src, const uint32_t* d_dst, int sm_count, cudaStream_t s,
+                                bool dependent)
 {
     const uint32_t groups = (n + NV - 1) / NV;
     // enough blocks for about 8 per SM, splitting the 4096 columns if needed
     // (down to one 32-column input word per block: with few states the
     // matrix read is the cost, spread over up to 128 blocks)
     int chunks = 1;
-    while (chunks < kBits / 32 && (uint64_t)groups * chunks < (uint64_t)8 * sm_count) chunks *= 2;
-    gf2_apply_pairs_kernel<NV><<<dim3(groups, chunks), 128, 0, s>>>(reinterpret_cast<const uint32_t*>(C), in,
-                                                                   d_src, d_dst, n, out, kBits / chunks);
-    return cudaGetLastError();
+    while (chunks < kBits / 32 && (uint64_t)groups * chunks * n_mats < (uint64_t)8 * sm_count) chunks *= 2;
+    return launch_dependent(dependent, dim3(groups, chunks, n_mats), dim3(128), s, gf2_apply_pairs_kernel<NV>, mats,
+                            in, d_src, d_dst, n, out, kBits / chunks);
+}
+
+cudaError_t launch_gf2_apply_multi(const uint64_t* const* C, int n_mats, const uint32_t* in, uint32_t* out, uint32_t n,
+                                   const uint32_t* d_src, const uint32_t* d_dst, int sm_count, cudaStream_t s,
+                                   bool dependent)
+{
+    if (n == 0 || n_mats == 0) return cudaSuccess;
+    if (n_mats > kMaxMats) return cudaErrorInvalidValue;
+    MatSet mats{};
+    for (int j = 0; j < n_mats; ++j) mats.C[j] = reinterpret_cast<const uint32_t*>(C[j]);
+    if (n >= 4 * 48) return launch_pairs<48>(mats, n_mats, in, out, n, d_src, d_dst, sm_count, s, dependent);
+    if (n > 4) return launch_pairs<16>(mats, n_mats, in, out, n, d_src, d_dst, sm_count, s, dependent);
+    return launch_pairs<4>(mats, n_mats, in, out, n, d_src, d_dst, sm_count, s, dependent);
 }
 
 cudaError_t launch_gf2_apply_pairs(const uint64_t* C, const uint32_t* in, uint32_t* out, uint32_t n,
-                                   const uint32_t* d_src, const uint32_t* d_dst, int sm_count, cudaStream_t s)
+                                   const uint32_t* d_src, const uint32_t* d_dst, int sm_count, cudaStream_t s,
+                                   bool dependent)
 {
-    if (n == 0) return cudaSuccess;
-    return n >= 4 * 48 ? launch_pairs<48>(C, in, out, n, d_src, d_dst, sm_count, s)
-                       : launch_pairs<16>(C, in, out, n, d_src, d_dst, sm_count, s);
+    return launch_gf2_apply_multi(&C, 1, in, out, n, d_src, d_dst, sm_count, s, dependent);
 }
 
 cudaError_t zero_rings(uint32_t* rings, const uint32_t* d_idx, uint32_t n, cudaStream_t s)

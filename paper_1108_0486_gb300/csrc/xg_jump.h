@@ -14,15 +14,31 @@ constexpr int kMaxPow = 64;  // C_k = M^(2^k), k < 64
 // the 64-bit-word generator.
 constexpr int kJumpSetW64 = 2;
 
+// Most matrices applied by one launch of the table kernel.
+constexpr int kMaxMats = 7;
+
 // C_k for a device and matrix family, built on first use (on stream s, each
 // from the one before; 2 MiB each, kept until the process exits).  Null on failure.
 const uint64_t* jump_matrix(int device, int param_set, int k, cudaStream_t s, xg_status* st);
 
 // out[d_dst[i]] ^= C in[d_src[i]] for n pairs of 128-word states.  in and out
 // may be one array; destinations are distinct, not among the sources, and
-// zeroed beforehand.
+// zeroed beforehand.  dependent: the kernel before it on the stream is one of
+// this file's or of the cut calls' set-up, so the launch may overlap its end
+// (both wait for each other where it matters).
 cudaError_t launch_gf2_apply_pairs(const uint64_t* C, const uint32_t* in, uint32_t* out, uint32_t n,
-                                   const uint32_t* d_src, const uint32_t* d_dst, int sm_count, cudaStream_t s);
+                                   const uint32_t* d_src, const uint32_t* d_dst, int sm_count, cudaStream_t s,
+                                   bool dependent = false);
+
+// The same for several matrices in one launch: out[d_dst[j n + i]] ^=
+// C[j] in[d_src[i]] for j < n_mats (<= kMaxMats); kNoState destinations are
+// skipped.
+cudaError_t launch_gf2_apply_multi(const uint64_t* const* C, int n_mats, const uint32_t* in, uint32_t* out, uint32_t n,
+                                   const uint32_t* d_src, const uint32_t* d_dst, int sm_count, cudaStream_t s,
+                                   bool dependent = false);
+
+// M^(j 2^k) for 1 <= j <= 7, built on first use like jump_matrix.
+const uint64_t* jump_matrix_multiple(int device, int param_set, int j, int k, cudaStream_t s, xg_status* st);
 
 // Whether an application to n states runs on the tensor cores (sm_103 and
 // n >= XG_GF2_TC_MIN_STATES, default 192; XG_JUMP_TENSOR_CORES=0 turns the
@@ -41,6 +57,12 @@ size_t gf2_apply_scratch(int device, uint32_t n);
 cudaError_t gf2_apply(int device, int family, int k, uint32_t* rings, uint32_t n, const uint32_t* d_src,
                       const uint32_t* d_dst, uint8_t* scratch, int sm_count, cudaStream_t s, xg_status* st,
                       bool dst_zeroed = false);
+
+// rings[d_dst[i]] = M^(j 2^k) rings[d_src[i]] on the tensor cores (1 <= j <= 7;
+// kNoState destinations are skipped); scratch as gf2_tc_apply's.
+cudaError_t gf2_apply_matrix_tc(int device, int family, int j, int k, uint32_t* rings, uint32_t n,
+                                const uint32_t* d_src, const uint32_t* d_dst, uint8_t* scratch, cudaStream_t s,
+                                xg_status* st);
 
 // Advance n states by `words` positions: M^words applied to rings[0, n),
 // with rings[n, 2n) as the second buffer (*result_hi: the result ended there)

@@ -369,7 +369,7 @@ __global__ void __launch_bounds__(256) seed_kernel(State st, const uint32_t* __r
 // piece writes the state back (adding the whole call's words to pos).
 struct UnitSrc {
     const uint32_t* ring = nullptr;   // null: the stream's window
-    const uint32_t* weyl0 = nullptr;  // with ring: Weyl word before the first word
+    uint32_t weyl0 = 0;               // with ring: Weyl word before the first word
     uint64_t pos_add = 0;             // with ring: words the whole call advances
     bool write_state = true;
 };
@@ -442,7 +442,7 @@ __device__ __forceinline__ float run_stream(const State& st, uint32_t s, uint64_
     uint32_t wp;
     if (src.ring) {
         load_ring(eng, src.ring - kRingBase, 0u);
-        wp = *src.weyl0;
+        wp = src.weyl0;
     } else {
         load_ring(eng, win_s, st.pend[s]);
         wp = st.weyl[s];
@@ -517,6 +517,40 @@ __global__ void __launch_bounds__(256, 1) gen_kernel_ilp(GenArgs a)
     gen_body<P, TPG, WPL, OUT, ST>(a);
 }
 
+// A cut call: warp p generates piece m = p % K of the call on stream
+// first + p / K, from the ring and the Weyl word that the jump-ahead prologue
+// prepared; the last piece writes the stream's state.  Register budgets as
+// for the whole calls.
+template <class P, int OUT, int ST>
+__device__ __forceinline__ void cut_body(const CutArgs& a)
+{
+    const uint32_t p = (blockIdx.x * blockDim.x + threadIdx.x) / 32;
+    const uint32_t i = p / a.pieces, m = p % a.pieces;
+    if (i >= a.nstreams) return;
+    cudaGridDependencySynchronize();   // the last prologue step
+    const uint64_t skip = (uint64_t)m << a.log2_len, len = uint64_t(1) << a.log2_len;
+    UnitSrc src;
+    src.ring = a.rings + (size_t)p * kR;
+    src.weyl0 = a.weyl0[i] + (uint32_t)skip * a.omega;
+    src.write_state = m + 1 == a.pieces;
+    src.pos_add = OUT == kNormal ? a.n + (a.n & 1u) : a.n;
+    uint32_t* row = reinterpret_cast<uint32_t*>(a.out) + (uint64_t)i * a.ld + skip;
+    run_stream<P, 32, 2, OUT, ST>(a.st, a.first + i, src.write_state ? a.n - skip : len, row, a.omega,
+                                  (int)(threadIdx.x & 31u), 0xFFFFFFFFu, src);
+}
+
+template <class P, int OUT, int ST>
+__global__ void __launch_bounds__(256) cut_kernel(CutArgs a)
+{
+    cut_body<P, OUT, ST>(a);
+}
+
+template <class P, int OUT, int ST>
+__global__ void __launch_bounds__(256, 1) cut_kernel_ilp(CutArgs a)
+{
+    cut_body<P, OUT, ST>(a);
+}
+
 // Persistent batch kernel.  Each warp repeatedly takes the next task
 // (atomic counter; tasks are ordered costliest first by the host).  A chain
 // task runs every item of one chain -- the calls on one stream, in order --
@@ -534,7 +568,7 @@ __device__ __forceinline__ UnitSrc unit_src(const BatchItem& it, const BatchPiec
     if (it.piece) {
         const BatchPiece& pc = pieces[it.piece - 1];
         src.ring = pc.ring;
-        src.weyl0 = pc.weyl0;
+        src.weyl0 = *pc.weyl0;
         src.pos_add = pc.item_words;
         src.write_state = pc.last != 0;
     }
@@ -699,6 +733,30 @@ cudaError_t launch_gen_cfg(int out_kind, bool vec, int block, const GenArgs& a, 
         return launch_gen_one<P, TPG, WPL, kNormalSum, kAligned>(block, a, s);
     default:
         return cudaErrorInvalidValue;
+    }
+}
+
+template <class P, int OUT, int ST>
+cudaError_t launch_cut_one(const CutArgs& a, cudaStream_t s)
+{
+    constexpr int block = 64;
+    const uint64_t threads = (uint64_t)a.nstreams * a.pieces * 32;
+    const unsigned grid = (unsigned)((threads + block - 1) / block);
+    if constexpr (OUT == kUniform || ST == kShifted)
+        return launch_dependent(a.dependent, dim3(grid), dim3(block), s, cut_kernel_ilp<P, OUT, ST>, a);
+    else
+        return launch_dependent(a.dependent, dim3(grid), dim3(block), s, cut_kernel<P, OUT, ST>, a);
+}
+
+template <class P>
+cudaError_t launch_cut_impl(int out_kind, bool vec, const CutArgs& a, cudaStream_t s)
+{
+    switch (out_kind) {
+    case kU32: return vec ? launch_cut_one<P, kU32, kAligned>(a, s) : launch_cut_one<P, kU32, kShifted>(a, s);
+    case kUniform:
+        return vec ? launch_cut_one<P, kUniform, kAligned>(a, s) : launch_cut_one<P, kUniform, kShifted>(a, s);
+    case kNormal: return vec ? launch_cut_one<P, kNormal, kAligned>(a, s) : launch_cut_one<P, kNormal, kScalar>(a, s);
+    default: return cudaErrorInvalidValue;
     }
 }
 

@@ -14,6 +14,28 @@
 
 namespace xg {
 
+// Launch f as an ordinary kernel, or (dependent) as one that may start while
+// the kernel before it on the stream still runs (programmatic dependent
+// launch): f then calls cudaGridDependencySynchronize() before it touches what
+// that kernel, or any before it, reads or writes.
+#if defined(__CUDACC__)
+template <class... KArgs, class... Args>
+inline cudaError_t launch_dependent(bool dependent, dim3 grid, dim3 block, cudaStream_t s, void (*f)(KArgs...),
+                                    Args... args)
+{
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.stream = s;
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = dependent ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, f, KArgs(args)...);
+}
+#endif
+
 // Per-stream window of recent words kept in device memory.  The ring that
 // the next call starts from is window[kRingBase - pend, kRingBase - pend + 128),
 // where pend (< 64, less than one round) counts words already computed past the
@@ -46,6 +68,24 @@ struct GenArgs {
     uint64_t ld;        // elements between consecutive streams' outputs
     float* sums;        // fused normal sum: one per stream
     uint32_t omega;     // Weyl increment, 0 when the Weyl generator is off
+};
+
+// A call cut into pieces of 2^log2_len outputs per stream, each its own warp
+// (32 lanes, two words per lane): piece m of stream first + i starts from
+// rings[i * pieces + m] and the Weyl word weyl0[i] + m 2^log2_len omega.
+struct CutArgs {
+    State st;
+    uint32_t first;
+    uint32_t nstreams;
+    uint32_t pieces;        // per stream, the last one shorter or equal
+    uint32_t log2_len;
+    uint64_t n;             // outputs per stream
+    void* out;
+    uint64_t ld;
+    const uint32_t* rings;
+    const uint32_t* weyl0;  // [nstreams]
+    uint32_t omega;
+    bool dependent;         // the last prologue step was a table-kernel launch
 };
 
 // ---- batches: work items of the persistent batch kernel -----------------
@@ -149,6 +189,7 @@ cudaError_t launch_export_states(const State& st, uint32_t first, uint32_t n, ui
                                  uint64_t* pos, cudaStream_t s);
 cudaError_t launch_import_states(const State& st, uint32_t first, uint32_t n, const uint32_t* rings,
                                  const uint32_t* weyl, const uint64_t* pos, uint32_t weyl_on, cudaStream_t s);
+cudaError_t launch_cut(int param_set, int out_kind, bool vec, const CutArgs& a, cudaStream_t s);
 // The persistent batch kernel of a parameter set; groups: the variant with
 // the group-task paths.
 const void* batch_kernel_ptr(int param_set, bool groups);
@@ -158,6 +199,8 @@ cudaError_t launch_seed_default(const State&, const uint32_t*, uint32_t, uint32_
 cudaError_t launch_seed_paper(const State&, const uint32_t*, uint32_t, uint32_t, cudaStream_t);
 cudaError_t launch_gen_default(int cfg, int out_kind, bool vec, int block, const GenArgs&, cudaStream_t);
 cudaError_t launch_gen_paper(int cfg, int out_kind, bool vec, int block, const GenArgs&, cudaStream_t);
+cudaError_t launch_cut_default(int out_kind, bool vec, const CutArgs&, cudaStream_t);
+cudaError_t launch_cut_paper(int out_kind, bool vec, const CutArgs&, cudaStream_t);
 const void* batch_kernel_ptr_default(bool groups);
 const void* batch_kernel_ptr_paper(bool groups);
 

@@ -145,6 +145,11 @@ cudaError_t launch_gen(int param_set, int cfg, int out_kind, bool vec, int block
                           : launch_gen_default(cfg, out_kind, vec, block, a, s);
 }
 
+cudaError_t launch_cut(int param_set, int out_kind, bool vec, const CutArgs& a, cudaStream_t s)
+{
+    return param_set == 1 ? launch_cut_paper(out_kind, vec, a, s) : launch_cut_default(out_kind, vec, a, s);
+}
+
 const void* batch_kernel_ptr(int param_set, bool groups)
 {
     return param_set == 1 ? batch_kernel_ptr_paper(groups) : batch_kernel_ptr_default(groups);

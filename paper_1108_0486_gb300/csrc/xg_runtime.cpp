@@ -13,6 +13,8 @@
 #include <vector>
 
 #include "xg_batch.h"
+#include "xg_cut.h"
+#include "xg_gf2_tc.h"
 #include "xg_launch.h"
 #include "xg_runtime.h"
 
@@ -101,6 +103,53 @@ xg_status xg_ctx::ensure_jump_ws(size_t bytes)
     return XG_OK;
 }
 
+xg_status xg_ctx::ensure_cut_ws(size_t bytes)
+{
+    if (cut_ws_bytes >= bytes) return XG_OK;
+    if (cut_ws) {
+        if (cut_used) cudaEventSynchronize(cut_event);
+        cudaFree(cut_ws);
+    }
+    cut_ws = nullptr;
+    cut_ws_bytes = 0;
+    if (!cut_event && cudaEventCreateWithFlags(&cut_event, cudaEventDisableTiming) != cudaSuccess) {
+        cudaGetLastError();
+        cut_event = nullptr;
+        return xg::fail(XG_ENOMEM, "cudaEventCreate(cut workspace) failed");
+    }
+    if (cudaMalloc(&cut_ws, bytes) != cudaSuccess) {
+        cudaGetLastError();
+        cut_ws = nullptr;
+        return xg::fail(XG_ENOMEM, "cudaMalloc(cut workspace, %zu bytes) failed", bytes);
+    }
+    cut_ws_bytes = bytes;
+    return XG_OK;
+}
+
+xg_status xg_ctx::cut_ws_acquire()
+{
+    if (!cut_used) return XG_OK;
+    // a tensor-core prologue that gave up waiting made its call's outputs
+    // invalid: reported by the first cut call after it has finished
+    if (cut_tc_pending && cudaEventQuery(cut_event) == cudaSuccess) {
+        cut_tc_pending = false;
+        if (xg::gf2_tc_take_failure())
+            return xg::fail(XG_EDEVICE, "an earlier cut call's tensor-core kernel gave up waiting; its streams are not valid");
+    }
+    if (cut_stream != stream && cudaStreamWaitEvent(stream, cut_event, 0) != cudaSuccess)
+        return xg::cuda_fail(cudaGetLastError(), "cut workspace");
+    return XG_OK;
+}
+
+xg_status xg_ctx::cut_ws_release(bool tensor_cores)
+{
+    cut_stream = stream;
+    cut_tc_pending = cut_tc_pending || tensor_cores;
+    if (cudaEventRecord(cut_event, stream) != cudaSuccess) return xg::cuda_fail(cudaGetLastError(), "cut workspace");
+    cut_used = true;
+    return XG_OK;
+}
+
 xg_status xg_ctx::ensure_staging(size_t bytes)
 {
     if (staging_bytes >= bytes) return XG_OK;
@@ -144,26 +193,25 @@ static xg_status enqueue_gen(Ctx* c, int kind, uint32_t first, uint32_t nstreams
     return XG_OK;
 }
 
-constexpr uint32_t kCutMaxStreams = 64;
-constexpr uint64_t kCutMinWords = uint64_t(1) << 18;
-
-static xg_status generate_cut(Ctx* c, int kind, uint32_t first, uint32_t nstreams, uint64_t n, void* out,
-                              uint64_t ld)
+// log2 of the piece length that a device call is cut into, 0 for a whole
+// call.  A piece length set by the caller applies to at most 64 streams of at
+// least 2^18 outputs; by itself the library cuts where its prediction says
+// so, unless a launch shape was set or tuned for more streams or shorter
+// calls than those.  Not while the stream is being captured: a first use builds matrices
+// and the workspace.
+static int cut_length(Ctx* c, int kind, uint32_t nstreams, uint64_t n)
 {
-    std::vector<xg::HostItem> items(nstreams);
-    for (uint32_t i = 0; i < nstreams; ++i)
-        items[i] = xg::HostItem{first + i, (uint32_t)kind, n, static_cast<char*>(out) + (uint64_t)i * ld * 4,
-                                nullptr};
-    xg::BatchLauncher*& L = c->batch[c->batch_next];
-    c->batch_next ^= 1;
-    if (!L) L = new (std::nothrow) xg::BatchLauncher();
-    if (!L) return fail(XG_ENOMEM, "host allocation failed");
-    xg_status st = L->launch(c, items.data(), nstreams, c->stream);
-    if (st != XG_OK) {
-        cudaError_t e = cudaGetLastError();
-        return fail(st, "cut generation failed (%s)", cudaGetErrorString(e));
+    if (c->split_words == 1 || n < (uint64_t(1) << 13)) return 0;
+    const bool always = nstreams <= 64 && n >= (uint64_t(1) << 18);   // whatever the launch shape set
+    if (!always && (c->split_words > 1 || c->cfg[kind] >= 0)) return 0;
+    const int q = xg::cut_choose(kind, nstreams, n, c->sm_count, c->split_words);
+    if (!q) return 0;
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(c->stream, &cap) != cudaSuccess) {
+        cudaGetLastError();
+        return 0;
     }
-    return XG_OK;
+    return cap == cudaStreamCaptureStatusNone ? q : 0;
 }
 
 static bool is_device_pointer(const void* p)
@@ -245,8 +293,11 @@ static xg_status generate_common(xg_ctx* ctx, int kind, uint32_t first, uint32_t
         // few streams, long calls: a single stream is one serial chain (one
         // warp, ~1.5e9 words/s), so cut each call into pieces that run on
         // many warps at once (jump-ahead; the output is the same)
-        if (nstreams <= kCutMaxStreams && n >= kCutMinWords && c->split_words != 1)
-            return generate_cut(c, kind, first, nstreams, n, out, ld);
+        if (const int q = cut_length(c, kind, nstreams, n)) {
+            bool ran = false;
+            const xg_status st = xg::cut_generate(c, kind, first, nstreams, n, out, ld, q, &ran);
+            if (ran || st != XG_OK) return st;
+        }
         return enqueue_gen(c, kind, first, nstreams, n, out, ld, nullptr, c->stream);
     }
     return generate_to_host(c, kind, first, nstreams, n, out, ld);
@@ -335,6 +386,11 @@ xg_status xg_destroy(xg_ctx* ctx)
         if (c->staging[b]) cudaFree(c->staging[b]);
     }
     if (c->jump_ws) cudaFree(c->jump_ws);
+    if (c->cut_event) {
+        if (c->cut_used) cudaEventSynchronize(c->cut_event);
+        cudaEventDestroy(c->cut_event);
+    }
+    if (c->cut_ws) cudaFree(c->cut_ws);
     if (c->state_mem) cudaFree(c->state_mem);
     delete c;
     return XG_OK;

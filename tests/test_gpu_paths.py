@@ -166,3 +166,73 @@ def test_tensor_core_jump_at_tile_edges(n, monkeypatch):
             st.jump(1 << 37)
             rows.append(st.u32(128).cpu().numpy())
     assert np.array_equal(rows[0], rows[1])
+
+
+@pytest.mark.parametrize("kind", KINDS)
+@pytest.mark.parametrize("streams,n,piece", [(1, 16385, 0), (1, (1 << 18) + 3, 0), (1, 1 << 18, 4096), (3, 262145, 64),
+                                              (7, 300001, 0), (64, 1 << 18, 65536), (100, 70001, 0), (600, 140002, 0)])
+def test_cut_calls_equal_whole_calls(kind, streams, n, piece):
+    """Calls cut into pieces (chosen by the library, or of a set length; one
+    and several prologue steps, on the tensor cores and not; the last piece
+    full, short and odd) against whole calls on the same streams, twice in a
+    row, at aligned and unaligned rows; two streams against the oracle."""
+    from paper_1108_0486_gb300 import Streams
+    ps = streams % 2
+    rows = []
+    for split in (piece, 1):
+        with Streams(streams, param_set=ps, seeds=W.seeds(streams)) as st:
+            st.set_batch_split(split)
+            a = st.generate(kind, n)
+            b = st.generate(kind, n, ld=n + 5)[:, :n]
+            c = st.generate(kind, 77)
+            rows.append([a, b, c])
+            pos = st.checkpoint()["pos"]
+            assert np.all(pos == 2 * words_of(kind, n) + words_of(kind, 77))
+    for x, y in zip(*rows):
+        assert torch.equal(x, y)
+    if streams <= 7:
+        m = words_of(kind, n)
+        for s in {0, streams - 1}:
+            w = O.streams(W.seeds(1, 1 + s), 2 * m, param_set=ps)[0]
+            check(kind, rows[0][1][s].cpu().numpy(), w[m:], n)
+
+
+def test_cut_calls_on_two_cuda_streams():
+    """Cut calls of one context on alternating CUDA streams, each ordered after
+    the other: the workspace they share follows."""
+    from paper_1108_0486_gb300 import Streams, _lib as L
+    n = 1 << 18
+    s1, s2 = torch.cuda.Stream(), torch.cuda.Stream()
+    with Streams(5, seeds=W.seeds(5)) as st:
+        outs = []
+        for k in range(6):
+            cs, other = (s1, s2) if k % 2 else (s2, s1)
+            # calls on disjoint streams need no order between the CUDA streams
+            L.xg_set_stream(st.ctx, cs.cuda_stream)
+            with torch.cuda.stream(cs):
+                outs.append(st.u32(n, first=k % 2, count=1))
+        torch.cuda.synchronize()
+        L.xg_set_stream(st.ctx, torch.cuda.current_stream().cuda_stream)
+        got = [o.cpu().numpy().view(np.uint32)[0] for o in outs]
+    for s in (0, 1):
+        w = O.streams(W.seeds(1, 1 + s), 3 * n)[0]
+        assert np.array_equal(np.concatenate(got[s::2]), w)
+
+
+def test_call_in_a_captured_graph_is_not_cut():
+    """A call that would be cut runs whole while its CUDA stream is captured;
+    replays continue the streams."""
+    from paper_1108_0486_gb300 import Streams
+    n, streams = 50000, 200
+    cs = torch.cuda.Stream()
+    with Streams(streams, seeds=W.seeds(streams), stream=cs) as st:
+        out = torch.empty((streams, n), dtype=torch.int32, device="cuda")
+        torch.cuda.synchronize()
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g, stream=cs):
+            st.u32(n, out=out)
+        for k in range(2):
+            g.replay()
+            torch.cuda.synchronize()
+            w = O.streams(W.seeds(1, streams), (k + 1) * n)[0, k * n:]
+            assert np.array_equal(out[streams - 1].cpu().numpy().view(np.uint32), w)
