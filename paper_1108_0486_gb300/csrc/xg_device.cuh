@@ -220,11 +220,16 @@ __device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b)
 }
 __device__ __forceinline__ f32x2 dup2(float v) { return pk2(v, v); }
 
+// TAIL = false leaves the FP64 tail out: the caller looks at the first words
+// (kNormalTail) and discards the results where one of them is in it.
+constexpr uint32_t kNormalTail = 62u << 8;   // o1 below this <=> m1 <= 62
+
+template <bool TAIL = true>
 __device__ __forceinline__ void normal_pair2(uint32_t o1a, uint32_t o2a, uint32_t o1b, uint32_t o2b, float& z1a,
                                              float& z2a, float& z1b, float& z2b)
 {
     const uint32_t m1a = (o1a >> 8) + 1u, m1b = (o1b >> 8) + 1u;
-    if (m1a <= 62u || m1b <= 62u) {
+    if (TAIL && (m1a <= 62u || m1b <= 62u)) {
         normal_pair(o1a, o2a, z1a, z2a);
         normal_pair(o1b, o2b, z1b, z2b);
         return;

@@ -121,12 +121,49 @@ __device__ __forceinline__ void store_window(const E& eng, uint32_t* win_s, int 
 // retired row).  Returns the final rotation.
 // UNROLL2 = false keeps one block per iteration (the batch kernel, whose
 // register count the longer body would raise).
-template <class E, class Emit, bool UNROLL2 = true>
+//
+// VOTED > 0 (normals): VOTED blocks per iteration with the FP64 tail's branch
+// taken out of each pair.  The branch keeps the compiler from moving a pair's
+// work across it, so a warp waits out the transform's latency pair by pair;
+// without it the transforms of an iteration overlap each other and the next
+// rounds.  The warp votes once per iteration, and the few iterations (0.1%)
+// in which a pair belongs to the tail are run again, with the branch, from
+// the ring kept at their start: same values, stored over the first ones.
+// Times in ms per call of 65536 normals (sums) per stream, before -> now:
+// 1 stream 0.090 -> 0.073 (0.088 -> 0.068), 608 0.096 -> 0.081 (0.094 ->
+// 0.076), 1216 0.131 -> 0.117 (0.121 -> 0.106), 3040 0.264 -> 0.252 (0.258 ->
+// 0.235), 8000 0.672 -> 0.664 (0.659 -> 0.622).  2 blocks gain the same on few
+// streams and less on many; 8 gain no more.
+template <class E, class Emit, bool UNROLL2 = true, int VOTED = 0>
 __device__ __forceinline__ int drive(E& eng, uint64_t nr, Emit& emit,
                                      uint32_t (&retired)[E::WPL_])
 {
     constexpr int W = E::WPL_;
     uint64_t r = 0;
+    if constexpr (VOTED > 0) {
+        static_assert(Emit::kPairRounds, "normals, two-row ring");
+        while (r + VOTED * E::NROWS < nr) {
+            const E start = eng;
+            const Emit estart = emit;
+            emit.low = 0xFFFFFFFFu;
+            static_for<0, VOTED>([&](auto) {
+                eng.template round<0>();
+                eng.template round<1>();
+                emit.template full_rounds01<false>(eng);
+            });
+            if (__any_sync(eng.mask, emit.low < kNormalTail)) {
+                eng = start;
+                emit = estart;
+#pragma unroll 1
+                for (int b = 0; b < VOTED; ++b) {
+                    eng.template round<0>();
+                    eng.template round<1>();
+                    emit.full_rounds01(eng);
+                }
+            }
+            r += VOTED * E::NROWS;
+        }
+    }
     if constexpr (UNROLL2) {
         for (; r + 2 * E::NROWS < nr; r += 2 * E::NROWS) {
             if constexpr (Emit::kPairRounds) {
@@ -200,6 +237,7 @@ struct Emit {
     uint32_t wl;       // Weyl word of this lane's element 0 in the current round
     uint32_t omega;    // omega, or 0 with the Weyl generator off
     float acc;         // fused sum
+    uint32_t low;      // smallest first word of the pairs since the last vote
 
     template <int K>
     __device__ __forceinline__ void words(const E& eng, uint32_t (&o)[W])
@@ -237,13 +275,15 @@ struct Emit {
 
     // Rounds 0 and 1 of a two-row ring (kPairRounds): the outputs of
     // full<0>() then full<1>(), both normal pairs through normal_pair2.
+    template <bool TAIL = true>
     __device__ __forceinline__ void full_rounds01(const E& eng)
     {
         uint32_t oa[W], ob[W];
         words<0>(eng, oa);
         words<1>(eng, ob);
+        if constexpr (!TAIL) low = umin(low, umin(oa[0], ob[0]));
         float z1a, z2a, z1b, z2b;
-        normal_pair2(oa[0], oa[1], ob[0], ob[1], z1a, z2a, z1b, z2b);
+        normal_pair2<TAIL>(oa[0], oa[1], ob[0], ob[1], z1a, z2a, z1b, z2b);
         if constexpr (OUT != kNormalSum) {
             if constexpr (VEC) {
                 *reinterpret_cast<uint2*>(dst) = make_uint2(__float_as_uint(z1a), __float_as_uint(z2a));
@@ -422,7 +462,7 @@ __device__ __forceinline__ void advance_words(E& eng, Emit& em, uint32_t h)
 // at (32, 2) and 2.549 ms at (8, 4) against 0.618 and 0.677 ms kShifted
 // (0.588 and 0.713 ms for aligned rows of 100000).  Normals pair words inside
 // a lane and are bound by the transform: kScalar costs them 0.5%.
-template <class P, int TPG, int WPL, int OUT, int ST, bool UNROLL2 = true>
+template <class P, int TPG, int WPL, int OUT, int ST, bool UNROLL2 = true, int VOTED = 0>
 __device__ __forceinline__ float run_stream(const State& st, uint32_t s, uint64_t n, uint32_t* row,
                                             uint32_t omega, int lane, unsigned mask,
                                             const UnitSrc& src = UnitSrc())
@@ -469,7 +509,7 @@ __device__ __forceinline__ float run_stream(const State& st, uint32_t s, uint64_
         }
     }
     const uint64_t nr = (nwords - head + RW - 1) / RW;
-    const int rot = drive<E, Em, UNROLL2>(eng, nr, em, retired);
+    const int rot = drive<E, Em, UNROLL2, VOTED>(eng, nr, em, retired);
     if (src.write_state) {
         __syncwarp(mask);
         store_window(eng, win_s, rot, retired);
@@ -482,7 +522,7 @@ __device__ __forceinline__ float run_stream(const State& st, uint32_t s, uint64_
     return em.acc;
 }
 
-template <class P, int TPG, int WPL, int OUT, int ST>
+template <class P, int TPG, int WPL, int OUT, int ST, int VOTED = 0>
 __device__ __forceinline__ void gen_body(const GenArgs& a)
 {
     const uint32_t g = (blockIdx.x * blockDim.x + threadIdx.x) / TPG;
@@ -491,7 +531,7 @@ __device__ __forceinline__ void gen_body(const GenArgs& a)
     const unsigned mask = group_mask<TPG>();
     uint32_t* row = (OUT == kNormalSum) ? nullptr
                                         : reinterpret_cast<uint32_t*>(a.out) + (uint64_t)g * a.ld;
-    float acc = run_stream<P, TPG, WPL, OUT, ST>(a.st, a.first + g, a.n, row, a.omega, lane, mask);
+    float acc = run_stream<P, TPG, WPL, OUT, ST, true, VOTED>(a.st, a.first + g, a.n, row, a.omega, lane, mask);
     if constexpr (OUT == kNormalSum) {
 #pragma unroll
         for (int off = TPG / 2; off >= 1; off /= 2)
@@ -517,10 +557,25 @@ __global__ void __launch_bounds__(256, 1) gen_kernel_ilp(GenArgs a)
     gen_body<P, TPG, WPL, OUT, ST>(a);
 }
 
+// Long calls of normals and fused sums at (32, 2): the voted loop (see drive),
+// with the larger budget (93 and 87 registers).  From kVotedMinNormals and
+// kVotedMinSums outputs per stream on; below, the warps that the registers
+// cost weigh more: 40000 streams of 1600 / 3200 / 6400, us: normals 86 / 161 /
+// 309 plain and 89 / 162 / 311 voted, sums 84 / 157 / 303 and 84 / 154 / 295.
+constexpr int kVotedBlocks = 4;
+constexpr uint64_t kVotedMinNormals = 8192;
+constexpr uint64_t kVotedMinSums = 3072;
+
+template <class P, int OUT, int ST>
+__global__ void __launch_bounds__(256, 1) gen_kernel_voted(GenArgs a)
+{
+    gen_body<P, 32, 2, OUT, ST, kVotedBlocks>(a);
+}
+
 // A cut call: warp p generates piece m = p % K of the call on stream
 // first + p / K, from the ring and the Weyl word that the jump-ahead prologue
-// prepared; the last piece writes the stream's state.  Register budgets as
-// for the whole calls.
+// prepared; the last piece writes the stream's state.  Register budgets and
+// the voted loop as for long whole calls.
 template <class P, int OUT, int ST>
 __device__ __forceinline__ void cut_body(const CutArgs& a)
 {
@@ -535,8 +590,8 @@ __device__ __forceinline__ void cut_body(const CutArgs& a)
     src.write_state = m + 1 == a.pieces;
     src.pos_add = OUT == kNormal ? a.n + (a.n & 1u) : a.n;
     uint32_t* row = reinterpret_cast<uint32_t*>(a.out) + (uint64_t)i * a.ld + skip;
-    run_stream<P, 32, 2, OUT, ST>(a.st, a.first + i, src.write_state ? a.n - skip : len, row, a.omega,
-                                  (int)(threadIdx.x & 31u), 0xFFFFFFFFu, src);
+    run_stream<P, 32, 2, OUT, ST, true, OUT == kNormal ? kVotedBlocks : 0>(
+        a.st, a.first + i, src.write_state ? a.n - skip : len, row, a.omega, (int)(threadIdx.x & 31u), 0xFFFFFFFFu, src);
 }
 
 template <class P, int OUT, int ST>
@@ -697,6 +752,11 @@ cudaError_t launch_gen_one(int block, const GenArgs& a, cudaStream_t s)
 {
     const uint64_t threads = (uint64_t)a.nstreams * TPG;
     const unsigned grid = (unsigned)((threads + block - 1) / block);
+    if constexpr (TPG == 32 && WPL == 2 && (OUT == kNormal || OUT == kNormalSum))
+        if (a.n >= (OUT == kNormal ? kVotedMinNormals : kVotedMinSums)) {
+            gen_kernel_voted<P, OUT, ST><<<grid, block, 0, s>>>(a);
+            return cudaGetLastError();
+        }
     if constexpr (OUT == kUniform || (OUT == kU32 && ST == kShifted))   // kShifted words: 0.631 -> 0.618 ms
         gen_kernel_ilp<P, TPG, WPL, OUT, ST><<<grid, block, 0, s>>>(a);
     else
@@ -742,7 +802,7 @@ cudaError_t launch_cut_one(const CutArgs& a, cudaStream_t s)
     constexpr int block = 64;
     const uint64_t threads = (uint64_t)a.nstreams * a.pieces * 32;
     const unsigned grid = (unsigned)((threads + block - 1) / block);
-    if constexpr (OUT == kUniform || ST == kShifted)
+    if constexpr (OUT != kU32 || ST == kShifted)
         return launch_dependent(a.dependent, dim3(grid), dim3(block), s, cut_kernel_ilp<P, OUT, ST>, a);
     else
         return launch_dependent(a.dependent, dim3(grid), dim3(block), s, cut_kernel<P, OUT, ST>, a);

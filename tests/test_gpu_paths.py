@@ -236,3 +236,34 @@ def test_call_in_a_captured_graph_is_not_cut():
             torch.cuda.synchronize()
             w = O.streams(W.seeds(1, streams), (k + 1) * n)[0, k * n:]
             assert np.array_equal(out[streams - 1].cpu().numpy().view(np.uint32), w)
+
+
+@pytest.mark.parametrize("n", [3071, 3072, 3327, 3329, 8191, 8192, 8193, 8447, 8448, 8449, 8703, 8705])
+@pytest.mark.parametrize("ps", [0, 1])
+def test_long_normals_and_sums_with_tail_pairs(n, ps):
+    """Lengths around the limits of the voted loop and around its iterations,
+    rows that vector stores fit and others; nearly empty rings without the Weyl
+    word, whose small words put many pairs into the FP64 tail, beside seeded
+    streams: the bits of another launch shape, and sums within the rounding of
+    each lane's additions."""
+    from paper_1108_0486_gb300 import Streams
+    streams = 40
+
+    def make():
+        st = Streams(streams, param_set=ps, weyl=False, seeds=W.seeds(streams))
+        for s in range(3):
+            ring = np.zeros(128, dtype=np.uint32)
+            ring[(41 * s + 1) % 128] = 1 << (9 * s)
+            st.set_state(s, ring, 0)
+        return st
+
+    with make() as a, make() as b, make() as c:
+        b.set_launch("normal", 16, 2)
+        for ld in (n, n + (-n) % 4):
+            x, y = a.normal(n, ld=ld)[:, :n], b.normal(n, ld=ld)[:, :n]
+            assert torch.equal(x, y)
+            assert torch.equal(torch.from_numpy(a.checkpoint()["rings"]), torch.from_numpy(b.checkpoint()["rings"]))
+            got = c.normal_sum(n).double()
+            z = x.double()
+            bound = (n / 32 + 6) * 2.0 ** -24 * z.abs().sum(1)
+            assert bool(((got - z.sum(1)).abs() <= bound).all())
