@@ -9,10 +9,10 @@ cudaError_t launch_seed_default(const State& st, const uint32_t* d_seeds, uint32
     return launch_seed_impl<ParamsDefault, 32, 2>(st, d_seeds, first, count, s);
 }
 
-cudaError_t launch_gen_default(int cfg, int out_kind, bool vec, int block, const GenArgs& a,
+cudaError_t launch_gen_default(int cfg, int out_kind, Store store, int block, const GenArgs& a,
                                cudaStream_t s)
 {
-    return launch_gen_impl<ParamsDefault>(cfg, out_kind, vec, block, a, s);
+    return launch_gen_impl<ParamsDefault>(cfg, out_kind, store, block, a, s);
 }
 
 cudaError_t launch_cut_default(int out_kind, bool vec, const CutArgs& a, cudaStream_t s)

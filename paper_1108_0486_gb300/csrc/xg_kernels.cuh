@@ -764,30 +764,23 @@ cudaError_t launch_gen_one(int block, const GenArgs& a, cudaStream_t s)
     return cudaGetLastError();
 }
 
-// Rows that no vector store fits.  At (32, 2) the scalar stores of a short
-// call cost less than moving the ring on: 30000 rows of 1001 words 33.5 us
-// against 35.5 us, 16384 rows of 65537 0.808 against 0.645 ms; at the narrower
-// shapes, whose stores are 8 or 16 bytes apart over several rows, kShifted is
-// the faster at every length (75 against 34 us at (8, 4)).
-constexpr uint64_t kShiftMinWords = 2048;
-
 template <class P, int TPG, int WPL, int OUT>
-cudaError_t launch_gen_words(bool vec, int block, const GenArgs& a, cudaStream_t s)
+cudaError_t launch_gen_words(Store store, int block, const GenArgs& a, cudaStream_t s)
 {
-    if (vec) return launch_gen_one<P, TPG, WPL, OUT, kAligned>(block, a, s);
-    if constexpr (TPG == 32)
-        if (a.n < kShiftMinWords) return launch_gen_one<P, TPG, WPL, OUT, kScalar>(block, a, s);
+    if (store == kAligned) return launch_gen_one<P, TPG, WPL, OUT, kAligned>(block, a, s);
+    if constexpr (TPG == 32)   // the narrower shapes have no scalar form (see pick_store)
+        if (store == kScalar) return launch_gen_one<P, TPG, WPL, OUT, kScalar>(block, a, s);
     return launch_gen_one<P, TPG, WPL, OUT, kShifted>(block, a, s);
 }
 
 template <class P, int TPG, int WPL>
-cudaError_t launch_gen_cfg(int out_kind, bool vec, int block, const GenArgs& a, cudaStream_t s)
+cudaError_t launch_gen_cfg(int out_kind, Store store, int block, const GenArgs& a, cudaStream_t s)
 {
     switch (out_kind) {
-    case kU32: return launch_gen_words<P, TPG, WPL, kU32>(vec, block, a, s);
-    case kUniform: return launch_gen_words<P, TPG, WPL, kUniform>(vec, block, a, s);
+    case kU32: return launch_gen_words<P, TPG, WPL, kU32>(store, block, a, s);
+    case kUniform: return launch_gen_words<P, TPG, WPL, kUniform>(store, block, a, s);
     case kNormal:
-        return vec ? launch_gen_one<P, TPG, WPL, kNormal, kAligned>(block, a, s)
+        return store == kAligned ? launch_gen_one<P, TPG, WPL, kNormal, kAligned>(block, a, s)
                    : launch_gen_one<P, TPG, WPL, kNormal, kScalar>(block, a, s);
     case kNormalSum:
         return launch_gen_one<P, TPG, WPL, kNormalSum, kAligned>(block, a, s);
@@ -828,16 +821,16 @@ const void* batch_kernel_ptr(bool groups)
 }
 
 template <class P>
-cudaError_t launch_gen_impl(int cfg, int out_kind, bool vec, int block, const GenArgs& a,
+cudaError_t launch_gen_impl(int cfg, int out_kind, Store store, int block, const GenArgs& a,
                             cudaStream_t s)
 {
     if (a.nstreams == 0) return cudaSuccess;
     switch (cfg) {
-    case 0: return launch_gen_cfg<P, 4, 8>(out_kind, vec, block, a, s);
-    case 1: return launch_gen_cfg<P, 8, 4>(out_kind, vec, block, a, s);
-    case 2: return launch_gen_cfg<P, 16, 2>(out_kind, vec, block, a, s);
-    case 3: return launch_gen_cfg<P, 16, 4>(out_kind, vec, block, a, s);
-    case 4: return launch_gen_cfg<P, 32, 2>(out_kind, vec, block, a, s);
+    case 0: return launch_gen_cfg<P, 4, 8>(out_kind, store, block, a, s);
+    case 1: return launch_gen_cfg<P, 8, 4>(out_kind, store, block, a, s);
+    case 2: return launch_gen_cfg<P, 16, 2>(out_kind, store, block, a, s);
+    case 3: return launch_gen_cfg<P, 16, 4>(out_kind, store, block, a, s);
+    case 4: return launch_gen_cfg<P, 32, 2>(out_kind, store, block, a, s);
     default: return cudaErrorInvalidValue;
     }
 }

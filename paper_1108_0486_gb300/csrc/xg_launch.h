@@ -179,7 +179,7 @@ int cfg_index(int tpg, int wpl);          // -1 if unsupported
 // Launchers (return the launch error, if any).
 cudaError_t launch_seed(int param_set, const State& st, const uint32_t* d_seeds,
                         uint32_t first, uint32_t count, cudaStream_t s);
-cudaError_t launch_gen(int param_set, int cfg, int out_kind, bool vec, int block,
+cudaError_t launch_gen(int param_set, int cfg, int out_kind, Store store, int block,
                        const GenArgs& a, cudaStream_t s);
 cudaError_t launch_transform(int out_kind, const uint32_t* in, uint64_t n, float* out,
                              cudaStream_t s);
@@ -197,8 +197,8 @@ const void* batch_kernel_ptr(int param_set, bool groups);
 // Per parameter set (defined in xg_inst_default.cu / xg_inst_paper.cu).
 cudaError_t launch_seed_default(const State&, const uint32_t*, uint32_t, uint32_t, cudaStream_t);
 cudaError_t launch_seed_paper(const State&, const uint32_t*, uint32_t, uint32_t, cudaStream_t);
-cudaError_t launch_gen_default(int cfg, int out_kind, bool vec, int block, const GenArgs&, cudaStream_t);
-cudaError_t launch_gen_paper(int cfg, int out_kind, bool vec, int block, const GenArgs&, cudaStream_t);
+cudaError_t launch_gen_default(int cfg, int out_kind, Store store, int block, const GenArgs&, cudaStream_t);
+cudaError_t launch_gen_paper(int cfg, int out_kind, Store store, int block, const GenArgs&, cudaStream_t);
 cudaError_t launch_cut_default(int out_kind, bool vec, const CutArgs&, cudaStream_t);
 cudaError_t launch_cut_paper(int out_kind, bool vec, const CutArgs&, cudaStream_t);
 const void* batch_kernel_ptr_default(bool groups);

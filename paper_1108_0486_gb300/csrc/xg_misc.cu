@@ -138,11 +138,11 @@ cudaError_t launch_seed(int param_set, const State& st, const uint32_t* d_seeds,
                           : launch_seed_default(st, d_seeds, first, count, s);
 }
 
-cudaError_t launch_gen(int param_set, int cfg, int out_kind, bool vec, int block, const GenArgs& a,
+cudaError_t launch_gen(int param_set, int cfg, int out_kind, Store store, int block, const GenArgs& a,
                        cudaStream_t s)
 {
-    return param_set == 1 ? launch_gen_paper(cfg, out_kind, vec, block, a, s)
-                          : launch_gen_default(cfg, out_kind, vec, block, a, s);
+    return param_set == 1 ? launch_gen_paper(cfg, out_kind, store, block, a, s)
+                          : launch_gen_default(cfg, out_kind, store, block, a, s);
 }
 
 cudaError_t launch_cut(int param_set, int out_kind, bool vec, const CutArgs& a, cudaStream_t s)

@@ -59,12 +59,12 @@ size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 
 }  // namespace
 
-int xg_ctx::pick_cfg(int kind, uint32_t nstreams) const
+int xg_ctx::pick_cfg(int kind, uint32_t nstreams, uint64_t n) const
 {
     const int fixed = cfg[kind == xg::kNormalSum ? xg::kNormal : kind];
     if (fixed >= 0) return fixed;
-    // Without a tuned choice, from a sweep of 100 .. 131072 streams at 2^28
-    // outputs on GB300 (ps per output):
+    // Without a tuned choice, from sweeps of 100 .. 131072 streams at 2^28
+    // outputs (ps per output) and of short calls (us per call) on GB300:
     //  * words, normals and fused sums: one warp per stream at every count.
     //    Words 0.598 (32,2) against 0.735 (8,4) at 10000 streams, 0.603 / 0.641
     //    at 16384; normals 1.258 / 1.779 and 1.211 / 1.456 ((8,4) needs 98
@@ -75,9 +75,38 @@ int xg_ctx::pick_cfg(int kind, uint32_t nstreams) const
     //    streams): 0.735 (32,2) / 0.785 (16,2) / 0.885 (8,4) at 5000 streams,
     //    0.679 / 0.659 / 0.743 at 6000, 0.685 / 0.695 / 0.727 at 10000,
     //    0.670 / 0.648 / 0.633 at 12000, 0.663 / 0.662 / 0.641 at 16384.
+    //  * short calls on many streams are waves of warps that load a ring, run
+    //    a few rounds and store it: two streams per warp.  40000 streams of
+    //    100 / 401 / 1600 words: 14.5 / 23.1 / 51.2 us (32,2), 12.5 / 20.6 /
+    //    49.9 (16,2), 14.5 / 22.4 / 50.5 (8,4); 3200: 87.6 / 88.1 / 88.8
+    //    (16000 uniform streams of 1600: 23.1 (8,4), 23.9 (16,2)).
+    //    Normals gain only below half a thousand: 64 / 100 / 400: 15.3 / 17.8 /
+    //    33.4 (32,2), 13.9 / 15.7 / 33.0 (16,4); 8000 streams of 200: 9.1 / 9.6.
     const uint64_t parts = (uint64_t)sm_count * 4;
-    if (kind != xg::kUniform || nstreams < 9 * parts) return xg::cfg_index(32, 2);
-    return nstreams < 18 * parts ? xg::cfg_index(16, 2) : xg::cfg_index(8, 4);
+    if (kind == xg::kU32 || kind == xg::kUniform) {
+        if (nstreams < 9 * parts) return xg::cfg_index(32, 2);
+        if (n < (kind == xg::kU32 ? 2048 : 1536)) return xg::cfg_index(16, 2);
+        if (kind == xg::kU32) return xg::cfg_index(32, 2);
+        return nstreams < 18 * parts ? xg::cfg_index(16, 2) : xg::cfg_index(8, 4);
+    }
+    return n < 512 && nstreams >= 18 * parts ? xg::cfg_index(16, 4) : xg::cfg_index(32, 2);
+}
+
+// How rows are stored.  Where no vector store fits, words and uniforms move
+// the ring on to the next aligned word first (kShifted), which is the faster
+// form at every shape but (32, 2): there the scalar stores are 8 bytes apart
+// and cost less than the move in a short call (30000 rows of 1001 words: 33.5
+// against 35.5 us) or where a warp's own chain is the limit: 600 / 1500 /
+// 2432 / 4000 rows of 25601 words 18.7 / 33.0 / 43.0 / 82.4 us scalar, 20.7 /
+// 34.9 / 43.2 / 70.9 us shifted (uniforms 20.8 / 39.0 / 49.6 / 86.6 and 22.7 /
+// 39.1 / 51.3 / 80.4), so shifted from 5 streams per SM sub-partition.
+xg::Store xg_ctx::pick_store(int kind, int c, uint32_t nstreams, uint64_t n, const void* out, uint64_t ld) const
+{
+    if (kind == xg::kNormalSum) return xg::kAligned;
+    if ((reinterpret_cast<uintptr_t>(out) & 15u) == 0 && (ld % 4 == 0 || nstreams == 1)) return xg::kAligned;
+    if (kind == xg::kNormal) return xg::kScalar;
+    const bool scalar = xg::kCfgs[c].tpg == 32 && (n < 2048 || nstreams < 5u * 4u * (uint32_t)sm_count);
+    return scalar ? xg::kScalar : xg::kShifted;
 }
 
 int xg_ctx::pick_block(int kind, int c) const
@@ -184,11 +213,10 @@ static xg_status enqueue_gen(Ctx* c, int kind, uint32_t first, uint32_t nstreams
     a.ld = ld;
     a.sums = d_sums;
     a.omega = c->weyl_on ? kOmegaHost : 0u;
-    const int cfg = force_cfg >= 0 ? force_cfg : c->pick_cfg(kind, nstreams);
-    const bool vec = kind == xg::kNormalSum ||
-                     (((reinterpret_cast<uintptr_t>(d_out) & 15u) == 0) && (ld % 4 == 0));
+    const int cfg = force_cfg >= 0 ? force_cfg : c->pick_cfg(kind, nstreams, n);
+    const xg::Store store = c->pick_store(kind, cfg, nstreams, n, d_out, ld);
     const int block = force_block > 0 ? force_block : c->pick_block(kind, cfg);
-    cudaError_t e = xg::launch_gen(c->param_set, cfg, kind, vec, block, a, s);
+    cudaError_t e = xg::launch_gen(c->param_set, cfg, kind, store, block, a, s);
     if (e != cudaSuccess) return cuda_fail(e, "generate kernel launch");
     return XG_OK;
 }

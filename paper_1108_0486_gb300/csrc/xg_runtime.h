@@ -63,7 +63,8 @@ struct xg_ctx {
     bool cut_used = false;      // cut_event has been recorded
     bool cut_tc_pending = false;  // a tensor-core prologue's status is unread
 
-    int pick_cfg(int kind, uint32_t nstreams) const;
+    int pick_cfg(int kind, uint32_t nstreams, uint64_t n) const;
+    xg::Store pick_store(int kind, int cfg, uint32_t nstreams, uint64_t n, const void* out, uint64_t ld) const;
     int pick_block(int kind, int cfg) const;
     xg_status ensure_staging(size_t bytes);
     xg_status ensure_jump_ws(size_t bytes);

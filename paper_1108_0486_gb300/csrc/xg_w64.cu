@@ -375,7 +375,7 @@ __global__ void __launch_bounds__(256) seed_kernel(State st, const uint32_t* __r
     }
 }
 
-template <int TPG, int WPL, int OUT, bool VEC>
+template <int TPG, int WPL, int OUT, bool VEC, int U>
 __device__ __forceinline__ void gen_body(const GenArgs& a)
 {
     constexpr bool kShared = WPL == 1 && OUT == kU64;
@@ -404,7 +404,7 @@ __device__ __forceinline__ void gen_body(const GenArgs& a)
     em.dst = reinterpret_cast<uint64_t*>(a.out) + (uint64_t)g * a.ld + em.lane_off;
     uint64_t retired[WPL];
     const uint64_t nr = (a.n + RW - 1) / RW;
-    const int rot = drive<E, Emit<E, OUT, VEC>, OUT == kUniformF64 ? (WPL == 1 ? 8 : 4) : 1>(eng, nr, em, retired);
+    const int rot = drive<E, Emit<E, OUT, VEC>, U>(eng, nr, em, retired);
     __syncwarp(eng.mask);
     store_window(eng, win_s, rot, retired);
     if (lane == 0) {
@@ -416,17 +416,24 @@ __device__ __forceinline__ void gen_body(const GenArgs& a)
 
 // Two register budgets: one warp per stream runs uniforms with a stated
 // minimum of one block per SM, which lets the compiler keep more of an
-// iteration in flight.
-template <int TPG, int WPL, int OUT, bool VEC>
+// iteration in flight.  Not in short calls on many streams, which are waves of
+// warps that load a ring, run a few rounds and store it: 40000 streams of
+// 100 / 401 / 800 / 1601 values take 26.8 / 53.4 / 69.1 / 106.6 us that way
+// and 16.6 / 38.0 / 57.5 / 106.7 us with the default budget and two blocks
+// per iteration; 1500 streams of 800 6.4 us either way, 300 4.4 and 6.2.
+constexpr uint64_t kShortWords = 1024;
+constexpr uint32_t kShortMinStreams = 2048;
+
+template <int TPG, int WPL, int OUT, bool VEC, int U>
 __global__ void __launch_bounds__(256) gen_kernel(GenArgs a)
 {
-    gen_body<TPG, WPL, OUT, VEC>(a);
+    gen_body<TPG, WPL, OUT, VEC, U>(a);
 }
 
-template <int TPG, int WPL, int OUT, bool VEC>
+template <int TPG, int WPL, int OUT, bool VEC, int U>
 __global__ void __launch_bounds__(256, 1) gen_kernel_ilp(GenArgs a)
 {
-    gen_body<TPG, WPL, OUT, VEC>(a);
+    gen_body<TPG, WPL, OUT, VEC, U>(a);
 }
 
 template <int TPG, int WPL, int OUT, bool VEC>
@@ -434,10 +441,13 @@ static cudaError_t launch_one(int block, const GenArgs& a, cudaStream_t s)
 {
     const uint64_t threads = (uint64_t)a.nstreams * TPG;
     const unsigned grid = (unsigned)((threads + block - 1) / block);
-    if constexpr (OUT == kUniformF64 && WPL == 1)
-        gen_kernel_ilp<TPG, WPL, OUT, VEC><<<grid, block, 0, s>>>(a);
-    else
-        gen_kernel<TPG, WPL, OUT, VEC>
+    if constexpr (OUT == kUniformF64 && WPL == 1) {
+        if (a.n < kShortWords && a.nstreams >= kShortMinStreams)
+            gen_kernel<TPG, WPL, OUT, VEC, 2><<<grid, block, 0, s>>>(a);
+        else
+            gen_kernel_ilp<TPG, WPL, OUT, VEC, 8><<<grid, block, 0, s>>>(a);
+    } else
+        gen_kernel<TPG, WPL, OUT, VEC, OUT == kUniformF64 ? 4 : 1>
             <<<grid, block, WPL == 1 && OUT == kU64 ? block / 32 * 4 * kRW * sizeof(uint64_t) : 0, s>>>(a);
     return cudaGetLastError();
 }

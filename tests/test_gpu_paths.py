@@ -267,3 +267,33 @@ def test_long_normals_and_sums_with_tail_pairs(n, ps):
             z = x.double()
             bound = (n / 32 + 6) * 2.0 ** -24 * z.abs().sum(1)
             assert bool(((got - z.sum(1)).abs() <= bound).all())
+
+
+@pytest.mark.parametrize("kind", KINDS)
+def test_short_calls_on_many_streams(kind):
+    """Lengths on both sides of the limits under which many streams take
+    another shape, and of the storing of rows that no vector store fits on both
+    sides of its stream count: two calls each, first and last streams."""
+    from paper_1108_0486_gb300 import Streams
+    parts = 4 * torch.cuda.get_device_properties(0).multi_processor_count
+    for streams, lengths in ((18 * parts, (3, 129, 511, 512, 1535, 1536, 2047, 2048)), (5 * parts - 1, (2047, 2049)),
+                             (5 * parts, (2047, 2049)), (1, (2049,))):
+        for n in lengths:
+            with Streams(streams, seeds=W.seeds(streams)) as st:
+                rows = torch.cat([st.generate(kind, n), st.generate(kind, n)], 1)
+                for s in (0, streams - 1):
+                    got = rows[s].cpu().numpy()
+                    w = O.streams(W.seeds(1, 1 + s), 2 * words_of(kind, n))[0]
+                    check(kind, got[:n], w, n)
+                    check(kind, got[n:], w[words_of(kind, n):], n)
+
+
+@pytest.mark.parametrize("streams", [2047, 2048])
+def test_short_fp64_uniforms_on_many_streams(streams):
+    from paper_1108_0486_gb300 import Streams64
+    for n in (1, 65, 255, 257, 1023, 1024):
+        with Streams64(streams, seeds=W.seeds(streams)) as st:
+            rows = torch.cat([st.uniform(n), st.uniform(n)], 1)
+            for s in (0, streams - 1):
+                ref = O.uniform64_of(O.streams64(W.seeds(1, 1 + s), 2 * n))
+                assert np.array_equal(rows[s].cpu().numpy(), np.asarray(ref).reshape(-1))
