@@ -151,7 +151,9 @@ xg_status xg_generate_normal(xg_ctx* ctx, uint32_t first, uint32_t nstreams,
  * their FP32 sum per stream to d_sums[i - first] (device memory).  The sum
  * order is fixed by the launch configuration (xg_get_launch): each lane adds
  * its own values in sequence order, then the lanes of a stream are combined
- * by a butterfly over lane offsets TPG/2, ..., 1. */
+ * by a butterfly over lane offsets TPG/2, ..., 1.  A long call on few streams
+ * without a set or tuned launch shape may be summed in pieces that way (see
+ * xg_set_batch_split), the pieces' sums added in FP64 and rounded once. */
 xg_status xg_generate_normal_sum(xg_ctx* ctx, uint32_t first, uint32_t nstreams,
                                  uint64_t n_per_stream, float* d_sums);
 

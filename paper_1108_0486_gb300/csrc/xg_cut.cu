@@ -90,6 +90,21 @@ __global__ void __launch_bounds__(256) cut_setup_kernel(State st, uint32_t first
     lists[e] = m < pieces ? i * pieces + m : kNoState;
 }
 
+// sums[i] = the sum of stream i's pieces' sums, in FP64 and rounded once.  A
+// warp per stream.
+__global__ void __launch_bounds__(64) cut_sum_kernel(const float* __restrict__ piece_sums, uint32_t pieces,
+                                                     uint32_t nstreams, float* __restrict__ sums)
+{
+    const uint32_t i = blockIdx.x * 2 + threadIdx.x / 32, lane = threadIdx.x % 32;
+    cudaGridDependencySynchronize();
+    if (i >= nstreams) return;
+    double acc = 0.0;
+    for (uint32_t m = lane; m < pieces; m += 32) acc += (double)piece_sums[(size_t)i * pieces + m];
+#pragma unroll
+    for (int off = 16; off >= 1; off /= 2) acc += __shfl_xor_sync(0xFFFFFFFFu, acc, off);
+    if (lane == 0) sums[i] = (float)acc;
+}
+
 // Time of one word on a sub-partition of an SM that runs w warps, in ns,
 // fitted to a sweep of 100 .. 4000 whole streams: one warp alone is bound by
 // its own chain, several by the pipes.
@@ -98,7 +113,8 @@ double word_ns(int kind, double w)
     switch (kind) {
     case kU32: return std::max(0.585, 0.365 * w);
     case kUniform: return std::max(0.62, 0.42 * w);
-    default: return std::max(1.34, 0.55 + 0.68 * w);
+    case kNormal: return std::max(1.18, 0.35 + 0.705 * w);
+    default: return std::max(1.08, 0.27 + 0.67 * w);   // fused sums
     }
 }
 
@@ -125,7 +141,7 @@ double prologue_us(uint32_t nstreams, uint64_t pieces, int sm_count)
 
 int cut_choose(int kind, uint32_t nstreams, uint64_t n, int sm_count, uint64_t forced)
 {
-    const uint64_t words = kind == kNormal ? n + (n & 1u) : n;
+    const uint64_t words = kind == kNormal || kind == kNormalSum ? n + (n & 1u) : n;
     if (forced) {
         int q = 6;
         while ((uint64_t(1) << q) < forced) ++q;
@@ -143,7 +159,7 @@ int cut_choose(int kind, uint32_t nstreams, uint64_t n, int sm_count, uint64_t f
         if (words < 2 * len) break;
         const uint64_t pieces = (words + len - 1) / len;
         if (pieces * nstreams > kMaxPieces) continue;
-        const double t = prologue_us(nstreams, pieces, sm_count) +
+        const double t = prologue_us(nstreams, pieces, sm_count) + (kind == kNormalSum ? 2.0 : 0.0) +
                          1e-3 * (double)len * word_ns(kind, warps((double)nstreams * (double)pieces));
         if (t < best) {
             best = t;
@@ -157,7 +173,8 @@ xg_status cut_generate(xg_ctx* c, int kind, uint32_t first, uint32_t nstreams, u
                        int q, bool* ran)
 {
     *ran = false;
-    const uint64_t words = kind == kNormal ? n + (n & 1u) : n;
+    const bool sum = kind == kNormalSum;
+    const uint64_t words = kind == kNormal || sum ? n + (n & 1u) : n;
     const uint32_t pieces = (uint32_t)((words + (uint64_t(1) << q) - 1) >> q);
     const uint32_t total = pieces * nstreams;
     const Steps steps = plan_steps(nstreams, pieces);
@@ -170,7 +187,8 @@ xg_status cut_generate(xg_ctx* c, int kind, uint32_t first, uint32_t nstreams, u
     const size_t weyl_off = (size_t)total * 512;
     const size_t list_off = (weyl_off + (size_t)nstreams * 4 + 255) / 256 * 256;
     const size_t tc_off = (list_off + (size_t)steps.entries * 4 + 255) / 256 * 256;
-    const size_t bytes = tc_off + (most_tc ? gf2_tc_scratch_bytes(most_tc) : 0);
+    const size_t sums_off = (tc_off + (most_tc ? gf2_tc_scratch_bytes(most_tc) : 0) + 255) / 256 * 256;
+    const size_t bytes = sums_off + (sum ? (size_t)total * 4 : 0);
     if (c->ensure_cut_ws(bytes) != XG_OK) return XG_OK;
     char* ws = static_cast<char*>(c->cut_ws);
     uint32_t* rings = reinterpret_cast<uint32_t*>(ws);
@@ -226,14 +244,18 @@ xg_status cut_generate(xg_ctx* c, int kind, uint32_t first, uint32_t nstreams, u
         a.pieces = pieces;
         a.log2_len = (uint32_t)q;
         a.n = n;
-        a.out = out;
+        a.out = sum ? ws + sums_off : out;
         a.ld = ld;
         a.rings = rings;
         a.weyl0 = weyl0;
         a.omega = c->weyl_on ? 0x9E3779B9u : 0u;
         a.dependent = dependent;
-        const bool vec = ((reinterpret_cast<uintptr_t>(out) & 15u) == 0) && (ld % 4 == 0 || nstreams == 1);
+        const bool vec = sum || ((reinterpret_cast<uintptr_t>(out) & 15u) == 0 && (ld % 4 == 0 || nstreams == 1));
         e = launch_cut((int)c->param_set, kind, vec, a, s);
+        if (sum && e == cudaSuccess)
+            e = launch_dependent(true, dim3((nstreams + 1) / 2), dim3(64), s, cut_sum_kernel,
+                                 reinterpret_cast<const float*>(ws + sums_off), pieces, nstreams,
+                                 static_cast<float*>(out));
     }
     if (e != cudaSuccess) return st != XG_OK ? st : cuda_fail(e, "cut generation");
     return c->cut_ws_release(most_tc != 0);

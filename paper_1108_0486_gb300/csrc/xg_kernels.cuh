@@ -574,7 +574,8 @@ __global__ void __launch_bounds__(256, 1) gen_kernel_voted(GenArgs a)
 
 // A cut call: warp p generates piece m = p % K of the call on stream
 // first + p / K, from the ring and the Weyl word that the jump-ahead prologue
-// prepared; the last piece writes the stream's state.  Register budgets and
+// prepared; the last piece writes the stream's state.  Fused sums: out[p] is
+// the piece's sum.  Register budgets and
 // the voted loop as for long whole calls.
 template <class P, int OUT, int ST>
 __device__ __forceinline__ void cut_body(const CutArgs& a)
@@ -588,10 +589,17 @@ __device__ __forceinline__ void cut_body(const CutArgs& a)
     src.ring = a.rings + (size_t)p * kR;
     src.weyl0 = a.weyl0[i] + (uint32_t)skip * a.omega;
     src.write_state = m + 1 == a.pieces;
-    src.pos_add = OUT == kNormal ? a.n + (a.n & 1u) : a.n;
-    uint32_t* row = reinterpret_cast<uint32_t*>(a.out) + (uint64_t)i * a.ld + skip;
-    run_stream<P, 32, 2, OUT, ST, true, OUT == kNormal ? kVotedBlocks : 0>(
-        a.st, a.first + i, src.write_state ? a.n - skip : len, row, a.omega, (int)(threadIdx.x & 31u), 0xFFFFFFFFu, src);
+    constexpr bool kSum = OUT == kNormalSum, kNormalOut = OUT == kNormal || kSum;
+    src.pos_add = kNormalOut ? a.n + (a.n & 1u) : a.n;
+    uint32_t* row = kSum ? nullptr : reinterpret_cast<uint32_t*>(a.out) + (uint64_t)i * a.ld + skip;
+    const int lane = (int)(threadIdx.x & 31u);
+    float acc = run_stream<P, 32, 2, OUT, ST, true, kNormalOut ? kVotedBlocks : 0>(
+        a.st, a.first + i, src.write_state ? a.n - skip : len, row, a.omega, lane, 0xFFFFFFFFu, src);
+    if constexpr (kSum) {
+#pragma unroll
+        for (int off = 16; off >= 1; off /= 2) acc = __fadd_rn(acc, __shfl_xor_sync(0xFFFFFFFFu, acc, off));
+        if (lane == 0) reinterpret_cast<float*>(a.out)[p] = acc;
+    }
 }
 
 template <class P, int OUT, int ST>
@@ -809,6 +817,7 @@ cudaError_t launch_cut_impl(int out_kind, bool vec, const CutArgs& a, cudaStream
     case kUniform:
         return vec ? launch_cut_one<P, kUniform, kAligned>(a, s) : launch_cut_one<P, kUniform, kShifted>(a, s);
     case kNormal: return vec ? launch_cut_one<P, kNormal, kAligned>(a, s) : launch_cut_one<P, kNormal, kScalar>(a, s);
+    case kNormalSum: return launch_cut_one<P, kNormalSum, kAligned>(a, s);
     default: return cudaErrorInvalidValue;
     }
 }

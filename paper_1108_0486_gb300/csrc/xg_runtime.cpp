@@ -230,8 +230,11 @@ static xg_status enqueue_gen(Ctx* c, int kind, uint32_t first, uint32_t nstreams
 static int cut_length(Ctx* c, int kind, uint32_t nstreams, uint64_t n)
 {
     if (c->split_words == 1 || n < (uint64_t(1) << 13)) return 0;
+    // fused sums: a launch shape that was set fixes the order of the additions
+    const bool shaped = c->cfg[kind == xg::kNormalSum ? xg::kNormal : kind] >= 0;
+    if (kind == xg::kNormalSum && shaped) return 0;
     const bool always = nstreams <= 64 && n >= (uint64_t(1) << 18);   // whatever the launch shape set
-    if (!always && (c->split_words > 1 || c->cfg[kind] >= 0)) return 0;
+    if (!always && (c->split_words > 1 || shaped)) return 0;
     const int q = xg::cut_choose(kind, nstreams, n, c->sm_count, c->split_words);
     if (!q) return 0;
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
@@ -574,6 +577,11 @@ xg_status xg_generate_normal_sum(xg_ctx* ctx, uint32_t first, uint32_t nstreams,
     if (!is_device_pointer(d_sums)) return fail(XG_EINVAL, "sums must be device memory");
     if (c->server) return fail(XG_EINVAL, "the request server owns this context; use xg_submit");
     std::lock_guard<std::mutex> lk(c->mu);
+    if (const int q = cut_length(c, xg::kNormalSum, nstreams, n)) {
+        bool ran = false;
+        const xg_status st = xg::cut_generate(c, xg::kNormalSum, first, nstreams, n, d_sums, 0, q, &ran);
+        if (ran || st != XG_OK) return st;
+    }
     return enqueue_gen(c, xg::kNormalSum, first, nstreams, n, nullptr, 0, d_sums, c->stream);
 }
 

@@ -297,3 +297,28 @@ def test_short_fp64_uniforms_on_many_streams(streams):
             for s in (0, streams - 1):
                 ref = O.uniform64_of(O.streams64(W.seeds(1, 1 + s), 2 * n))
                 assert np.array_equal(rows[s].cpu().numpy(), np.asarray(ref).reshape(-1))
+
+
+@pytest.mark.parametrize("streams,n,piece", [(1, 16385, 0), (1, (1 << 18) + 3, 4096), (3, 262145, 64), (7, 300001, 0),
+                                              (64, 1 << 18, 65536), (100, 70001, 0), (600, 140002, 0)])
+def test_cut_sums(streams, n, piece):
+    """Sums of calls cut into pieces (chosen by the library, or of a set
+    length): within the rounding of each lane's additions of the FP64 sum of
+    the same normals, twice in a row; the streams end where whole calls end,
+    and a set launch shape keeps its order of additions."""
+    from paper_1108_0486_gb300 import Streams
+    ps = streams % 2
+    make = lambda: Streams(streams, param_set=ps, seeds=W.seeds(streams))
+    with make() as a, make() as b, make() as c, make() as d:
+        a.set_batch_split(piece)
+        b.set_batch_split(1)
+        c.set_launch("normal", 32, 2)
+        d.set_batch_split(1)
+        d.set_launch("normal", 32, 2)
+        for _ in range(2):
+            z = b.normal(n).double()
+            bound = (n / 32 + 6) * 2.0 ** -24 * z.abs().sum(1)
+            assert bool(((a.normal_sum(n).double() - z.sum(1)).abs() <= bound).all())
+            assert torch.equal(c.normal_sum(n), d.normal_sum(n))
+        assert torch.equal(a.u32(77), b.u32(77))
+        assert np.array_equal(a.checkpoint()["pos"], b.checkpoint()["pos"])
