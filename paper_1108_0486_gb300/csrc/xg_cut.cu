@@ -9,7 +9,8 @@
 // so the index lists are built on the device and nothing is uploaded.
 //
 // One stream of 2^20 words: 73 us with a planned batch (two uploads, a gather,
-// five doubling steps, pieces of 2^15 words), @@ us this way.
+// five doubling steps, pieces of 2^15 words), 28 us this way; 500 streams of
+// 500000 normals 537 us whole, 379 us cut; 200 streams of 2^18 words 153 and 70.
 #include "xg_cut.h"
 
 #include <algorithm>
@@ -30,6 +31,7 @@ constexpr uint64_t kMaxPieces = uint64_t(1) << 22;   // 2 GiB of rings
 struct Step {
     uint32_t have;
     uint32_t mats;
+    uint32_t tc;    // by the tensor cores, where they are to be had
     uint64_t at;    // its sources in the list, then mats destination lists
 };
 struct Steps {
@@ -38,20 +40,21 @@ struct Steps {
     uint64_t entries;
 };
 
-// Up to 7 matrices per step while the states are few (a step then costs a
-// launch and the matrix read, not the lookups): up to 16 sources 3.5 us with
-// one matrix and @@ with 7; single doubling steps from 49 on, whose 192 or more
-// states run on the tensor cores.
+// Up to 7 matrices per step, which makes the pieces eight times as many.  By
+// the table kernel as long as the states are few, where a step costs a launch
+// and the matrix read rather than the lookups (0.07 us per state and matrix);
+// by the tensor cores from about 200 results on, where it costs the launches
+// and one tile's time and hardly more for seven matrices than for one.
 Steps plan_steps(uint32_t nstreams, uint32_t pieces)
 {
     Steps p{};
     for (uint64_t have = 1; have < pieces && p.n < kMaxSteps; ++p.n) {
         const uint64_t sources = have * nstreams;
-        const uint64_t most = sources <= 16 ? 7 : sources <= 48 ? 3 : 1;
-        const uint64_t mats = std::min<uint64_t>(most, (pieces + have - 1) / have - 1);
-        p.step[p.n] = Step{(uint32_t)have, (uint32_t)mats, p.entries};
-        p.entries += sources * (1 + mats);
-        have *= 1 + mats;
+        const uint64_t left = std::min<uint64_t>(7, (pieces + have - 1) / have - 1);
+        const bool table = sources <= 16 || (sources <= 48 && left <= 3) || (sources < 192 && left == 1);
+        p.step[p.n] = Step{(uint32_t)have, (uint32_t)left, table ? 0u : 1u, p.entries};
+        p.entries += sources * (1 + left);
+        have *= 1 + left;
     }
     return p;
 }
@@ -119,19 +122,19 @@ double word_ns(int kind, double w)
 }
 
 // Prologue time in us: the set-up launch, then per step a table-kernel launch
-// or, from 192 states, one tensor-core application (a wave of output tiles is
-// 240 states on 32 of the SMs).
+// or an application on the tensor cores (a wave of output tiles is 240 states
+// by one matrix on 32 of the SMs).
 double prologue_us(uint32_t nstreams, uint64_t pieces, int sm_count)
 {
     const Steps p = plan_steps(nstreams, (uint32_t)pieces);
-    double t = 6.0;
+    double t = 5.0;
     for (int k = 0; k < p.n; ++k) {
         const uint64_t n = (uint64_t)p.step[k].have * nstreams;
-        if (n < 192) {
-            t += 5.5 + 0.025 * (double)n * p.step[k].mats;
+        if (!p.step[k].tc) {
+            t += 5.5 + 0.05 * (double)(n * p.step[k].mats);
         } else {
-            const uint64_t tiles = (n + 239) / 240 * 32;
-            t += 6.0 + 6.6 * (double)((tiles + sm_count - 1) / sm_count);
+            const uint64_t tiles = (n + 239) / 240 * 32 * p.step[k].mats;
+            t += 18.0 + 4.5 * (double)((tiles + sm_count - 1) / sm_count - 1);
         }
     }
     return t;
@@ -150,17 +153,21 @@ int cut_choose(int kind, uint32_t nstreams, uint64_t n, int sm_count, uint64_t f
     }
     const double parts = 4.0 * sm_count;
     if (nstreams > 6 * parts) return 0;   // the pipes are busy as it is
-    auto warps = [&](double units) { return std::max(1.0, (double)(uint64_t)((units + parts - 1) / parts)); };
-    // the whole call, less 10% so that a cut has to be clearly the faster
-    double best = 0.9e-3 * (double)words * word_ns(kind, warps(nstreams));
+    // warps on the fullest sub-partition: blocks of two warps over the SMs
+    auto warps = [&](uint64_t blocks) { return (double)(((blocks + sm_count - 1) / sm_count + 1) / 2); };
+    // A launch's own start and end are 3.5 us; a piece's ring comes from
+    // memory that was just written.  5% in favour of the whole call, so that a
+    // cut has to be clearly the faster.
+    double best = 0.95 * (3.5 + 1e-3 * (double)words * word_ns(kind, warps((nstreams + 1) / 2)));
     int best_q = 0;
     for (int q = 12; q <= 32; ++q) {
         const uint64_t len = uint64_t(1) << q;
         if (words < 2 * len) break;
         const uint64_t pieces = (words + len - 1) / len;
         if (pieces * nstreams > kMaxPieces) continue;
-        const double t = prologue_us(nstreams, pieces, sm_count) + (kind == kNormalSum ? 2.0 : 0.0) +
-                         1e-3 * (double)len * word_ns(kind, warps((double)nstreams * (double)pieces));
+        const double run = 6.0 + 1e-3 * (double)len * word_ns(kind, warps(nstreams * ((pieces + 1) / 2)));
+        if (run >= best) continue;
+        const double t = prologue_us(nstreams, pieces, sm_count) + run + (kind == kNormalSum ? 2.0 : 0.0);
         if (t < best) {
             best = t;
             best_q = q;
@@ -180,9 +187,11 @@ xg_status cut_generate(xg_ctx* c, int kind, uint32_t first, uint32_t nstreams, u
     const Steps steps = plan_steps(nstreams, pieces);
     cudaStream_t s = c->stream;
     uint32_t most_tc = 0;   // states of the largest tensor-core step
+    bool use_tc[kMaxSteps] = {};
     for (int k = 0; k < steps.n; ++k) {
         const uint32_t m = steps.step[k].have * nstreams;
-        if (steps.step[k].mats == 1 && gf2_use_tc(c->device, m)) most_tc = std::max(most_tc, m);
+        use_tc[k] = steps.step[k].tc && gf2_use_tc(c->device, m * steps.step[k].mats);
+        if (use_tc[k]) most_tc = std::max(most_tc, m);
     }
     const size_t weyl_off = (size_t)total * 512;
     const size_t list_off = (weyl_off + (size_t)nstreams * 4 + 255) / 256 * 256;
@@ -197,6 +206,8 @@ xg_status cut_generate(xg_ctx* c, int kind, uint32_t first, uint32_t nstreams, u
     uint8_t* tc = most_tc ? reinterpret_cast<uint8_t*>(ws + tc_off) : nullptr;
     // the matrices first: building one on its first use synchronises
     const uint64_t* mats[kMaxSteps][kMaxMats] = {};
+    const uint8_t* tc_mats[kMaxSteps][kGf2TcMaxMats] = {};
+    static_assert(kMaxMats >= 7 && kGf2TcMaxMats >= 7, "matrices per step");
     xg_status st = XG_OK;
     for (int k = 0; k < steps.n; ++k)
         for (uint32_t j = 1; j <= steps.step[k].mats; ++j) {
@@ -206,8 +217,10 @@ xg_status cut_generate(xg_ctx* c, int kind, uint32_t first, uint32_t nstreams, u
                 f /= 2;
                 ++e;
             }
-            mats[k][j - 1] = jump_matrix_multiple(c->device, (int)c->param_set, (int)f, e, s, &st);
-            if (!mats[k][j - 1]) return st == XG_ENOMEM ? XG_OK : st;   // no memory: the whole call needs none
+            if (use_tc[k]) tc_mats[k][j - 1] = jump_matrix_tc(c->device, (int)c->param_set, (int)f, e, s, &st);
+            else mats[k][j - 1] = jump_matrix_multiple(c->device, (int)c->param_set, (int)f, e, s, &st);
+            if (!(use_tc[k] ? (const void*)tc_mats[k][j - 1] : (const void*)mats[k][j - 1]))
+                return st == XG_ENOMEM ? XG_OK : st;   // no memory: the whole call needs none
         }
     *ran = true;
     if (xg_status w = c->cut_ws_acquire()) return w;
@@ -216,25 +229,15 @@ xg_status cut_generate(xg_ctx* c, int kind, uint32_t first, uint32_t nstreams, u
     cut_setup_kernel<<<piece_blocks + list_blocks, 256, 0, s>>>(c->st, first, nstreams, pieces, piece_blocks, rings,
                                                                 weyl0, steps, lists);
     cudaError_t e = cudaGetLastError();
-    bool dependent = true;   // the launch before is the set-up or a table kernel
     for (int k = 0; k < steps.n && e == cudaSuccess; ++k) {
         const uint32_t m = steps.step[k].have * nstreams;
+        const int n_mats = (int)steps.step[k].mats;
         const uint32_t* src = lists + steps.step[k].at;
         const uint32_t* dst = src + m;
-        if (steps.step[k].mats == 1 && tc && gf2_use_tc(c->device, m)) {
-            int e2 = q;
-            uint64_t f = steps.step[k].have;
-            while (f % 2 == 0) {
-                f /= 2;
-                ++e2;
-            }
-            e = gf2_apply_matrix_tc(c->device, (int)c->param_set, (int)f, e2, rings, m, src, dst, tc, s, &st);
-            dependent = false;
-        } else {
-            e = launch_gf2_apply_multi(mats[k], (int)steps.step[k].mats, rings, rings, m, src, dst, c->sm_count, s,
-                                       dependent);
-            dependent = true;
-        }
+        if (use_tc[k])
+            e = gf2_tc_apply(c->device, tc_mats[k], n_mats, rings, src, m, rings, dst, tc, s, true);
+        else
+            e = launch_gf2_apply_multi(mats[k], n_mats, rings, rings, m, src, dst, c->sm_count, s, true, k + 1 < steps.n);
     }
     if (e == cudaSuccess) {
         CutArgs a{};
@@ -249,7 +252,6 @@ xg_status cut_generate(xg_ctx* c, int kind, uint32_t first, uint32_t nstreams, u
         a.rings = rings;
         a.weyl0 = weyl0;
         a.omega = c->weyl_on ? 0x9E3779B9u : 0u;
-        a.dependent = dependent;
         const bool vec = sum || ((reinterpret_cast<uintptr_t>(out) & 15u) == 0 && (ld % 4 == 0 || nstreams == 1));
         e = launch_cut((int)c->param_set, kind, vec, a, s);
         if (sum && e == cudaSuccess)

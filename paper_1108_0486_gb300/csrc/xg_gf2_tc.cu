@@ -29,7 +29,9 @@
 // other accumulator with tcgen05.ld (32 TMEM lanes = 32 output bits each),
 // take each count's parity and pack the 32 lanes' bits with a warp ballot:
 // one ballot is one ring word of one state.  The scales are written once: every byte of their
-// columns is 127, so no layout of them matters.
+// columns is 127, so no layout of them matters.  The set-up runs beside the end
+// of the kernel before it; the launch after it starts when it ends: kernels that
+// were resident earlier would crowd onto the SMs that have no tile.
 //
 // Every wait is bounded (2 s of %globaltimer); a wait that gives up records
 // a failure in a host-visible status word, the CTA waits (bounded) for its
@@ -187,17 +189,25 @@ __device__ __forceinline__ void mbar_arrive(uint64_t* bar)
 
 __device__ __forceinline__ bool failed(const volatile int* flag) { return *flag != 0; }
 
-// out[dst[s]] = C x_s for the n states of the B operand (rows >= n of B are
-// zero padding).  Persistent: CTA b takes tiles b, b + gridDim.x, ... of the
-// (4096 / kBM) x (n_pad / kBN) tiles, M fastest (consecutive tiles share a B
-// tile in L2).  192 threads: warp 0 = TMA producer, warp 1 = TMEM owner and
+struct TcMaps {
+    CUtensorMap a[kGf2TcMaxMats];
+    CUtensorMap b;
+};
+
+// out[dst[j n + s]] = C_j x_s for the n states of the B operand (rows >= n of
+// B are zero padding) and j < n_mats.  Persistent: CTA b takes tiles b, b +
+// gridDim.x, ... of the n_mats x (4096 / kBM) x (n_pad / kBN) tiles, M fastest
+// (consecutive tiles share a B tile in L2).  A few hundred states fill a part
+// of the SMs with one matrix, and a launch costs as much as its first tile
+// (14 us, each further wave 4), so several matrices share one: 500 states by 7
+// matrices 35 us, in three doubling launches 75 us.  192 threads: warp 0 = TMA producer, warp 1 = TMEM owner and
 // MMA issuer, warps 2-5 = epilogue (warp w reads TMEM lanes 32 (w mod 4) ..).
 // Two accumulators of kBN columns alternate, so that the epilogue of one
 // tile overlaps the MMAs of the next.
-__global__ void __launch_bounds__(kThreads, 1) gf2_tc_kernel(const __grid_constant__ CUtensorMap tmA,
-                                                              const __grid_constant__ CUtensorMap tmB, uint32_t n,
-                                                              uint32_t n_tiles, const uint32_t* __restrict__ dst,
-                                                              uint32_t* rings, uint32_t* status, uint32_t stall)
+__global__ void __launch_bounds__(kThreads, 1) gf2_tc_kernel(const __grid_constant__ TcMaps maps, uint32_t n_mats,
+                                                              uint32_t n, uint32_t n_tiles,
+                                                              const uint32_t* __restrict__ dst, uint32_t* rings,
+                                                              uint32_t* status, uint32_t stall)
 {
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -212,7 +222,7 @@ __global__ void __launch_bounds__(kThreads, 1) gf2_tc_kernel(const __grid_consta
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     constexpr uint32_t kMTiles = kGf2Bits / kBM;
-    const uint32_t total = kMTiles * n_tiles;
+    const uint32_t total = kMTiles * n_tiles * n_mats;
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < kStages; ++s) {
@@ -244,12 +254,14 @@ __global__ void __launch_bounds__(kThreads, 1) gf2_tc_kernel(const __grid_consta
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
+    cudaGridDependencySynchronize();   // B, and the rings that an earlier kernel still reads
 
     uint32_t issued = 0;  // producer: K blocks whose copies were started
     if (warp == 0) {
         if (lane == 0) {
             for (uint32_t t = blockIdx.x; t < total && !failed(&s_failed); t += gridDim.x) {
-                const int mt = (int)(t % kMTiles), nt = (int)(t / kMTiles);
+                const int mt = (int)(t % kMTiles), nt = (int)(t / kMTiles % n_tiles);
+                const CUtensorMap* ma = &maps.a[t / kMTiles / n_tiles];
                 for (int kb = 0; kb < kKBlocks; ++kb, ++issued) {
                     const uint32_t s = issued % kStages, u = issued / kStages;
                     if (issued >= (uint32_t)kStages && !mbar_wait(&empty[s], (u & 1) ^ 1, global_ns() + kWaitLimitNs)) {
@@ -258,8 +270,8 @@ __global__ void __launch_bounds__(kThreads, 1) gf2_tc_kernel(const __grid_consta
                     }
                     mbar_expect_tx(&full[s], kStageBytes);
                     if (stall && blockIdx.x == 0 && issued == 0) continue;   // the failure-path test
-                    tma_load_2d(sa + s * kABytes, &tmA, &full[s], kb * kBK, mt * kBM);
-                    tma_load_2d(sb + s * kBBytes, &tmB, &full[s], kb * kBK, nt * kBN);
+                    tma_load_2d(sa + s * kABytes, ma, &full[s], kb * kBK, mt * kBM);
+                    tma_load_2d(sb + s * kBBytes, &maps.b, &full[s], kb * kBK, nt * kBN);
                 }
             }
         }
@@ -305,7 +317,8 @@ __global__ void __launch_bounds__(kThreads, 1) gf2_tc_kernel(const __grid_consta
             }
             tc_fence_after();
             if (failed(&s_failed)) break;
-            const uint32_t mt = t % kMTiles, nt = t / kMTiles;
+            const uint32_t mt = t % kMTiles, nt = t / kMTiles % n_tiles;
+            const uint32_t* to = dst + (size_t)(t / kMTiles / n_tiles) * n;
             const uint32_t word = mt * (kBM / 32) + q;  // ring word of these 32 bits
             static_assert(kBN % 16 == 0, "columns are read 16 at a time");
             for (int c = 0; c < kBN; c += 32) {
@@ -325,7 +338,7 @@ __global__ void __launch_bounds__(kThreads, 1) gf2_tc_kernel(const __grid_consta
                 }
                 const uint32_t st = nt * kBN + (uint32_t)c + (uint32_t)lane;
                 if (st < n && c + lane < kBN) {
-                    const uint32_t d = dst[st];
+                    const uint32_t d = to[st];
                     if (d != kNoState) rings[(size_t)d * kGf2Words + word] = mine;
                 }
             }
@@ -387,6 +400,8 @@ __global__ void __launch_bounds__(256) expand_states_kernel(const uint32_t* __re
                                                             uint32_t n_pad, uint8_t* __restrict__ B)
 {
     const uint64_t t = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    cudaTriggerProgrammaticLaunchCompletion();
+    cudaGridDependencySynchronize();
     if (t >= (uint64_t)n_pad * kGf2Words) return;
     const uint32_t s = (uint32_t)(t / kGf2Words), w = (uint32_t)(t % kGf2Words);
     uint32_t x = 0;
@@ -473,16 +488,20 @@ cudaError_t gf2_tc_expand_matrix(const uint64_t* C, uint8_t* A, cudaStream_t s)
     return cudaGetLastError();
 }
 
-cudaError_t gf2_tc_apply(int device, const uint8_t* A, const uint32_t* rings_in, const uint32_t* src, uint32_t n,
-                         uint32_t* rings_out, const uint32_t* dst, uint8_t* scratch, cudaStream_t s)
+cudaError_t gf2_tc_apply(int device, const uint8_t* const* A, int n_mats, const uint32_t* rings_in,
+                         const uint32_t* src, uint32_t n, uint32_t* rings_out, const uint32_t* dst, uint8_t* scratch,
+                         cudaStream_t s, bool dependent)
 {
-    if (n == 0) return cudaSuccess;
+    if (n == 0 || n_mats == 0) return cudaSuccess;
+    if (n_mats < 0 || n_mats > kGf2TcMaxMats) return cudaErrorInvalidValue;
     const uint32_t n_pad = gf2_tc_padded(n);
-    CUtensorMap ma, mb;
+    TcMaps maps{};
     {
         std::lock_guard<std::mutex> lk(g_mu);
         if (!init_locked()) return cudaErrorNotSupported;
-        if (!make_map(&ma, A, kGf2Bits, kBM) || !make_map(&mb, scratch, n_pad, kBN)) return cudaErrorInvalidValue;
+        for (int j = 0; j < n_mats; ++j)
+            if (!make_map(&maps.a[j], A[j], kGf2Bits, kBM)) return cudaErrorInvalidValue;
+        if (!make_map(&maps.b, scratch, n_pad, kBN)) return cudaErrorInvalidValue;
         if (device >= 0 && device < 64 && !g_attr_set[device]) {
             cudaError_t e = cudaFuncSetAttribute(gf2_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
             if (e != cudaSuccess) return e;
@@ -490,18 +509,27 @@ cudaError_t gf2_tc_apply(int device, const uint8_t* A, const uint32_t* rings_in,
         }
     }
     const uint64_t words = (uint64_t)n_pad * kGf2Words;
-    expand_states_kernel<<<(unsigned)((words + 255) / 256), 256, 0, s>>>(rings_in, src, n, n_pad, scratch);
-    cudaError_t e = cudaGetLastError();
+    cudaError_t e = launch_dependent(dependent, dim3((unsigned)((words + 255) / 256)), dim3(256), s,
+                                     expand_states_kernel, rings_in, src, n, n_pad, scratch);
     if (e != cudaSuccess) return e;
     const uint32_t n_tiles = n_pad / kBN;
-    const uint32_t tiles = (kGf2Bits / kBM) * n_tiles;
+    const uint64_t tiles = (uint64_t)(kGf2Bits / kBM) * n_tiles * n_mats;
     int sms = 0;
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess || sms <= 0) sms = 1;
-    const unsigned grid = (unsigned)std::min<uint32_t>(tiles, (uint32_t)sms);
+    const unsigned grid = (unsigned)std::min<uint64_t>(tiles, (uint64_t)sms);
     const char* stall = std::getenv("XG_TC_TEST_STALL");
-    gf2_tc_kernel<<<grid, kThreads, kSmemBytes, s>>>(ma, mb, n, n_tiles, dst, rings_out, g_status_dev,
-                                                     (stall && stall[0] == '1') ? 1u : 0u);
-    return cudaGetLastError();
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(kThreads);
+    cfg.dynamicSmemBytes = kSmemBytes;
+    cfg.stream = s;
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, gf2_tc_kernel, maps, (uint32_t)n_mats, n, n_tiles, dst, rings_out, g_status_dev,
+                              (stall && stall[0] == '1') ? 1u : 0u);
 }
 
 bool gf2_tc_take_failure()

@@ -30,13 +30,19 @@ constexpr size_t kGf2TcMatrixBytes = (size_t)kGf2Bits * kGf2Bits / 2;
 // C in column form (column k = the 128 ring words of C e_k).
 cudaError_t gf2_tc_expand_matrix(const uint64_t* C, uint8_t* A, cudaStream_t s);
 
-// rings_out[dst[i]] = C rings_in[src[i]] (src null: i) for i < n, with A from
-// gf2_tc_expand_matrix; the destination rings are overwritten, and may be in
-// the same array as the sources if no destination is a source.  scratch:
-// gf2_tc_scratch_bytes(n) bytes, 16-byte aligned, reused once the launch has
-// finished.  Asynchronous on s.
-cudaError_t gf2_tc_apply(int device, const uint8_t* A, const uint32_t* rings_in, const uint32_t* src, uint32_t n,
-                         uint32_t* rings_out, const uint32_t* dst, uint8_t* scratch, cudaStream_t s);
+// Most matrices applied by one launch.
+constexpr int kGf2TcMaxMats = 7;
+
+// rings_out[dst[j n + i]] = C_j rings_in[src[i]] (src null: i) for i < n and
+// j < n_mats (<= kGf2TcMaxMats), with A[j] from gf2_tc_expand_matrix; the
+// destination rings are overwritten, and may be in the same array as the
+// sources if no destination is a source; kNoState destinations are skipped.
+// scratch: gf2_tc_scratch_bytes(n) bytes, 16-byte aligned, reused once the
+// launch has finished.  Asynchronous on s.  dependent: as in
+// launch_gf2_apply_pairs.
+cudaError_t gf2_tc_apply(int device, const uint8_t* const* A, int n_mats, const uint32_t* rings_in,
+                         const uint32_t* src, uint32_t n, uint32_t* rings_out, const uint32_t* dst, uint8_t* scratch,
+                         cudaStream_t s, bool dependent = false);
 
 // True (and cleared) if a tensor-core launch gave up a wait since the last
 // call: its results are not valid.  Read after synchronising.

@@ -139,7 +139,7 @@ template <int kPairVecs>
 __global__ void __launch_bounds__(128) gf2_apply_pairs_kernel(MatSet mats, const uint32_t* rings,
                                                               const uint32_t* __restrict__ src,
                                                               const uint32_t* __restrict__ dst, uint32_t n,
-                                                              uint32_t* out, int cols)
+                                                              uint32_t* out, int cols, bool early)
 {
     __shared__ uint32_t vbits[kPairVecs][kR];
     __shared__ uint32_t tbl[kPairVecs > 4 ? 16 : 1][kR];
@@ -155,7 +155,7 @@ __global__ void __launch_bounds__(128) gf2_apply_pairs_kernel(MatSet mats, const
 #pragma unroll
         for (int b = 0; b < 32; ++b) col[b] = __ldg(colw + (size_t)b * kR);
     };
-    cudaTriggerProgrammaticLaunchCompletion();
+    if (early) cudaTriggerProgrammaticLaunchCompletion();
     load_columns(w0);
     cudaGridDependencySynchronize();
     for (int v = 0; v < kPairVecs; ++v)
@@ -405,8 +405,8 @@ namespace {
 // first use and kept until exit.
 std::mutex g_tc_mu;
 uint8_t* g_tc_mats[64][3][4][kMaxPow] = {};   // [.. j = 1, 3, 5, 7][k]
+}  // namespace
 
-// M^(j 2^k) as the A operand.
 const uint8_t* jump_matrix_tc(int device, int family, int j, int k, cudaStream_t s, xg_status* st)
 {
     while (j > 1 && j % 2 == 0) {
@@ -435,7 +435,6 @@ const uint8_t* jump_matrix_tc(int device, int family, int j, int k, cudaStream_t
     A = static_cast<uint8_t*>(p);
     return A;
 }
-}  // namespace
 
 bool gf2_use_tc(int device, uint32_t n)
 {
@@ -464,22 +463,13 @@ cudaError_t gf2_apply(int device, int family, int k, uint32_t* rings, uint32_t n
     if (scratch && gf2_use_tc(device, n)) {
         const uint8_t* A = jump_matrix_tc(device, family, 1, k, s, st);
         if (!A) return cudaErrorMemoryAllocation;
-        return gf2_tc_apply(device, A, rings, d_src, n, rings, d_dst, scratch, s);
+        return gf2_tc_apply(device, &A, 1, rings, d_src, n, rings, d_dst, scratch, s);
     }
     const uint64_t* C = jump_matrix(device, family, k, s, st);
     if (!C) return cudaErrorMemoryAllocation;
     cudaError_t e = dst_zeroed ? cudaSuccess : zero_rings(rings, d_dst, n, s);
     if (e == cudaSuccess) e = launch_gf2_apply_pairs(C, rings, rings, n, d_src, d_dst, sm_count, s);
     return e;
-}
-
-cudaError_t gf2_apply_matrix_tc(int device, int family, int j, int k, uint32_t* rings, uint32_t n,
-                                const uint32_t* d_src, const uint32_t* d_dst, uint8_t* scratch, cudaStream_t s,
-                                xg_status* st)
-{
-    const uint8_t* A = jump_matrix_tc(device, family, j, k, s, st);
-    if (!A) return cudaErrorMemoryAllocation;
-    return gf2_tc_apply(device, A, rings, d_src, n, rings, d_dst, scratch, s);
 }
 
 // rings[dst[i]] = P rings[src[i]] for a matrix P in column form that is not
@@ -491,7 +481,8 @@ static cudaError_t gf2_apply_explicit(int device, const uint64_t* P, uint8_t* A_
 {
     if (scratch && A_buf && gf2_use_tc(device, n)) {
         cudaError_t e = gf2_tc_expand_matrix(P, A_buf, s);
-        if (e == cudaSuccess) e = gf2_tc_apply(device, A_buf, rings, d_src, n, rings, d_dst, scratch, s);
+        const uint8_t* A = A_buf;
+        if (e == cudaSuccess) e = gf2_tc_apply(device, &A, 1, rings, d_src, n, rings, d_dst, scratch, s);
         return e;
     }
     cudaError_t e = zero_rings(rings, d_dst, n, s);
@@ -596,7 +587,7 @@ cudaError_t launch_jump_index(uint32_t* ids, uint32_t n, uint32_t first, cudaStr
 template <int NV>
 static cudaError_t launch_pairs(const MatSet& mats, int n_mats, const uint32_t* in, uint32_t* out, uint32_t n,
                                 const uint32_t* d_src, const uint32_t* d_dst, int sm_count, cudaStream_t s,
-                                bool dependent)
+                                bool dependent, bool early)
 {
     const uint32_t groups = (n + NV - 1) / NV;
     // enough blocks for about 8 per SM, splitting the 4096 columns if needed
@@ -605,20 +596,20 @@ static cudaError_t launch_pairs(const MatSet& mats, int n_mats, const uint32_t* 
     int chunks = 1;
     while (chunks < kBits / 32 && (uint64_t)groups * chunks * n_mats < (uint64_t)8 * sm_count) chunks *= 2;
     return launch_dependent(dependent, dim3(groups, chunks, n_mats), dim3(128), s, gf2_apply_pairs_kernel<NV>, mats,
-                            in, d_src, d_dst, n, out, kBits / chunks);
+                            in, d_src, d_dst, n, out, kBits / chunks, early);
 }
 
 cudaError_t launch_gf2_apply_multi(const uint64_t* const* C, int n_mats, const uint32_t* in, uint32_t* out, uint32_t n,
                                    const uint32_t* d_src, const uint32_t* d_dst, int sm_count, cudaStream_t s,
-                                   bool dependent)
+                                   bool dependent, bool early)
 {
     if (n == 0 || n_mats == 0) return cudaSuccess;
     if (n_mats > kMaxMats) return cudaErrorInvalidValue;
     MatSet mats{};
     for (int j = 0; j < n_mats; ++j) mats.C[j] = reinterpret_cast<const uint32_t*>(C[j]);
-    if (n >= 4 * 48) return launch_pairs<48>(mats, n_mats, in, out, n, d_src, d_dst, sm_count, s, dependent);
-    if (n > 4) return launch_pairs<16>(mats, n_mats, in, out, n, d_src, d_dst, sm_count, s, dependent);
-    return launch_pairs<4>(mats, n_mats, in, out, n, d_src, d_dst, sm_count, s, dependent);
+    if (n >= 4 * 48) return launch_pairs<48>(mats, n_mats, in, out, n, d_src, d_dst, sm_count, s, dependent, early);
+    if (n > 4) return launch_pairs<16>(mats, n_mats, in, out, n, d_src, d_dst, sm_count, s, dependent, early);
+    return launch_pairs<4>(mats, n_mats, in, out, n, d_src, d_dst, sm_count, s, dependent, early);
 }
 
 cudaError_t launch_gf2_apply_pairs(const uint64_t* C, const uint32_t* in, uint32_t* out, uint32_t n,

@@ -32,13 +32,19 @@ cudaError_t launch_gf2_apply_pairs(const uint64_t* C, const uint32_t* in, uint32
 
 // The same for several matrices in one launch: out[d_dst[j n + i]] ^=
 // C[j] in[d_src[i]] for j < n_mats (<= kMaxMats); kNoState destinations are
-// skipped.
+// skipped.  early: a dependent launch after it may become resident while it
+// runs.  Wrong for long kernels of many blocks, which would be spread over the
+// SMs by what this one has left free: 16 streams of 2^18 words in 128 pieces
+// 45 us early, 33 us not.
 cudaError_t launch_gf2_apply_multi(const uint64_t* const* C, int n_mats, const uint32_t* in, uint32_t* out, uint32_t n,
                                    const uint32_t* d_src, const uint32_t* d_dst, int sm_count, cudaStream_t s,
-                                   bool dependent = false);
+                                   bool dependent = false, bool early = true);
 
 // M^(j 2^k) for 1 <= j <= 7, built on first use like jump_matrix.
 const uint64_t* jump_matrix_multiple(int device, int param_set, int j, int k, cudaStream_t s, xg_status* st);
+
+// The same as the A operand of gf2_tc_apply.
+const uint8_t* jump_matrix_tc(int device, int family, int j, int k, cudaStream_t s, xg_status* st);
 
 // Whether an application to n states runs on the tensor cores (sm_103 and
 // n >= XG_GF2_TC_MIN_STATES, default 192; XG_JUMP_TENSOR_CORES=0 turns the
@@ -57,12 +63,6 @@ size_t gf2_apply_scratch(int device, uint32_t n);
 cudaError_t gf2_apply(int device, int family, int k, uint32_t* rings, uint32_t n, const uint32_t* d_src,
                       const uint32_t* d_dst, uint8_t* scratch, int sm_count, cudaStream_t s, xg_status* st,
                       bool dst_zeroed = false);
-
-// rings[d_dst[i]] = M^(j 2^k) rings[d_src[i]] on the tensor cores (1 <= j <= 7;
-// kNoState destinations are skipped); scratch as gf2_tc_apply's.
-cudaError_t gf2_apply_matrix_tc(int device, int family, int j, int k, uint32_t* rings, uint32_t n,
-                                const uint32_t* d_src, const uint32_t* d_dst, uint8_t* scratch, cudaStream_t s,
-                                xg_status* st);
 
 // Advance n states by `words` positions: M^words applied to rings[0, n),
 // with rings[n, 2n) as the second buffer (*result_hi: the result ended there)

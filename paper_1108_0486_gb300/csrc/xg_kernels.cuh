@@ -572,46 +572,44 @@ __global__ void __launch_bounds__(256, 1) gen_kernel_voted(GenArgs a)
     gen_body<P, 32, 2, OUT, ST, kVotedBlocks>(a);
 }
 
-// A cut call: warp p generates piece m = p % K of the call on stream
-// first + p / K, from the ring and the Weyl word that the jump-ahead prologue
-// prepared; the last piece writes the stream's state.  Fused sums: out[p] is
-// the piece's sum.  Register budgets and
-// the voted loop as for long whole calls.
+// A cut call: a warp generates piece m of the call on stream first + i (grid:
+// pieces, streams), from the ring and the Weyl word that the jump-ahead
+// prologue prepared; the last piece writes the stream's state.  Fused sums:
+// out[i pieces + m] is the piece's sum.
+//
+// The recurrence's chain is what a warp waits for, as in a whole call on as
+// many streams, but the loop is compiled worse once its length is not the
+// grid's: with the length as it is, 800 pieces of 65536 words (uniforms) take
+// 63.4 (69.4) us against 52.8 (62.8) us for whole calls on 800 streams.  Read
+// from one lane by a shuffle, it makes the compiler keep that loop: 57.1
+// (65.6) us with the larger register budget; normals are as fast without
+// (114 us, whole 110).
 template <class P, int OUT, int ST>
-__device__ __forceinline__ void cut_body(const CutArgs& a)
+__global__ void __launch_bounds__(256, 1) cut_kernel(CutArgs a)
 {
-    const uint32_t p = (blockIdx.x * blockDim.x + threadIdx.x) / 32;
-    const uint32_t i = p / a.pieces, m = p % a.pieces;
-    if (i >= a.nstreams) return;
+    const uint32_t m = (blockIdx.x * blockDim.x + threadIdx.x) / 32, i = blockIdx.y;
+    if (m >= a.pieces) return;
     cudaGridDependencySynchronize();   // the last prologue step
-    const uint64_t skip = (uint64_t)m << a.log2_len, len = uint64_t(1) << a.log2_len;
+    constexpr bool kSum = OUT == kNormalSum, kNormalOut = OUT == kNormal || kSum;
+    const size_t p = (size_t)i * a.pieces + m;
+    const uint64_t skip = (uint64_t)m << a.log2_len;
     UnitSrc src;
-    src.ring = a.rings + (size_t)p * kR;
+    src.ring = a.rings + p * kR;
     src.weyl0 = a.weyl0[i] + (uint32_t)skip * a.omega;
     src.write_state = m + 1 == a.pieces;
-    constexpr bool kSum = OUT == kNormalSum, kNormalOut = OUT == kNormal || kSum;
     src.pos_add = kNormalOut ? a.n + (a.n & 1u) : a.n;
+    uint64_t n = src.write_state ? a.n - skip : uint64_t(1) << a.log2_len;
+    if constexpr (!kNormalOut)
+        n = ((uint64_t)__shfl_sync(0xFFFFFFFFu, (uint32_t)(n >> 32), 0) << 32) | __shfl_sync(0xFFFFFFFFu, (uint32_t)n, 0);
     uint32_t* row = kSum ? nullptr : reinterpret_cast<uint32_t*>(a.out) + (uint64_t)i * a.ld + skip;
     const int lane = (int)(threadIdx.x & 31u);
-    float acc = run_stream<P, 32, 2, OUT, ST, true, kNormalOut ? kVotedBlocks : 0>(
-        a.st, a.first + i, src.write_state ? a.n - skip : len, row, a.omega, lane, 0xFFFFFFFFu, src);
+    float acc = run_stream<P, 32, 2, OUT, ST, true, kNormalOut ? kVotedBlocks : 0>(a.st, a.first + i, n, row, a.omega,
+                                                                                  lane, 0xFFFFFFFFu, src);
     if constexpr (kSum) {
 #pragma unroll
         for (int off = 16; off >= 1; off /= 2) acc = __fadd_rn(acc, __shfl_xor_sync(0xFFFFFFFFu, acc, off));
         if (lane == 0) reinterpret_cast<float*>(a.out)[p] = acc;
     }
-}
-
-template <class P, int OUT, int ST>
-__global__ void __launch_bounds__(256) cut_kernel(CutArgs a)
-{
-    cut_body<P, OUT, ST>(a);
-}
-
-template <class P, int OUT, int ST>
-__global__ void __launch_bounds__(256, 1) cut_kernel_ilp(CutArgs a)
-{
-    cut_body<P, OUT, ST>(a);
 }
 
 // Persistent batch kernel.  Each warp repeatedly takes the next task
@@ -800,13 +798,9 @@ cudaError_t launch_gen_cfg(int out_kind, Store store, int block, const GenArgs& 
 template <class P, int OUT, int ST>
 cudaError_t launch_cut_one(const CutArgs& a, cudaStream_t s)
 {
-    constexpr int block = 64;
-    const uint64_t threads = (uint64_t)a.nstreams * a.pieces * 32;
-    const unsigned grid = (unsigned)((threads + block - 1) / block);
-    if constexpr (OUT != kU32 || ST == kShifted)
-        return launch_dependent(a.dependent, dim3(grid), dim3(block), s, cut_kernel_ilp<P, OUT, ST>, a);
-    else
-        return launch_dependent(a.dependent, dim3(grid), dim3(block), s, cut_kernel<P, OUT, ST>, a);
+    constexpr unsigned block = 64;
+    const dim3 grid((a.pieces + block / 32 - 1) / (block / 32), a.nstreams);   // at most 6 streams per SM sub-partition
+    return launch_dependent(true, grid, dim3(block), s, cut_kernel<P, OUT, ST>, a);
 }
 
 template <class P>

@@ -85,7 +85,6 @@ struct CutArgs {
     const uint32_t* rings;
     const uint32_t* weyl0;  // [nstreams]
     uint32_t omega;
-    bool dependent;         // the last prologue step was a table-kernel launch
 };
 
 // ---- batches: work items of the persistent batch kernel -----------------

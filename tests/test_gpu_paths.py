@@ -322,3 +322,22 @@ def test_cut_sums(streams, n, piece):
             assert torch.equal(c.normal_sum(n), d.normal_sum(n))
         assert torch.equal(a.u32(77), b.u32(77))
         assert np.array_equal(a.checkpoint()["pos"], b.checkpoint()["pos"])
+
+
+@pytest.mark.parametrize("streams,piece,pieces", [(33, 65536, 5), (40, 32768, 9), (60, 8192, 33), (64, 4096, 65),
+                                                  (17, 16384, 17), (49, 131072, 2), (49, 131072, 3), (64, 32768, 8)])
+@pytest.mark.parametrize("tensor_cores", ["1", "0"])
+def test_cut_prologue_steps(streams, piece, pieces, tensor_cores, monkeypatch):
+    """Piece counts that make the steps of the prologue take one to seven
+    matrices, the last one only in part, on the tensor cores and by the table
+    kernel: outputs and streams of whole calls."""
+    from paper_1108_0486_gb300 import Streams
+    monkeypatch.setenv("XG_JUMP_TENSOR_CORES", tensor_cores)
+    n = max(1 << 18, piece * (pieces - 1) + 321)
+    rows = []
+    for split in (piece, 1):
+        with Streams(streams, param_set=streams % 2, seeds=W.seeds(streams)) as st:
+            st.set_batch_split(split)
+            rows.append((st.u32(n), st.u32(n), st.u32(99)))
+    for x, y in zip(*rows):
+        assert torch.equal(x, y)
