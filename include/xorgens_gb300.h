@@ -135,10 +135,12 @@ xg_status xg_set_states(xg_ctx* ctx, uint32_t first, uint32_t count, const uint3
  * memory (the library generates into its own device buffer in chunks and
  * copies them to the host, overlapping both; returns when the data is there).
  * The fast path needs out and ld*4 bytes 16-byte aligned; other alignments
- * are accepted and use scalar stores.  Calls on at most 64 streams with at
- * least 2^18 outputs each go through the batch path, which cuts them into
- * pieces generated at once (see xg_set_batch_split; 1 turns this off); the
- * outputs are the same. */
+ * are accepted: words and uniforms take vector stores there too after a few
+ * scalar ones, normals scalar stores.  Long calls on few streams are cut into
+ * pieces generated at once where that is predicted to be the faster (see
+ * xg_set_batch_split; 1 turns this off; a set or tuned launch shape keeps it
+ * to at most 64 streams of at least 2^18 outputs), but not while the CUDA
+ * stream is being captured; the outputs are the same. */
 xg_status xg_generate_u32(xg_ctx* ctx, uint32_t first, uint32_t nstreams,
                           uint64_t n_per_stream, uint32_t* out, uint64_t ld);
 xg_status xg_generate_uniform(xg_ctx* ctx, uint32_t first, uint32_t nstreams,

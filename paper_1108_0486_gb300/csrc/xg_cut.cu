@@ -63,10 +63,10 @@ Steps plan_steps(uint32_t nstreams, uint32_t pieces)
 // kernel XORs into them); weyl0[i] = stream i's Weyl word; then the lists of
 // all steps.  A warp per piece, 8 to a block; blocks past the pieces write
 // the lists.
-__global__ void __launch_bounds__(256) cut_setup_kernel(State st, uint32_t first, uint32_t nstreams, uint32_t pieces,
-                                                        uint32_t piece_blocks, uint32_t* __restrict__ rings,
-                                                        uint32_t* __restrict__ weyl0, Steps steps,
-                                                        uint32_t* __restrict__ lists)
+__global__ void __launch_bounds__(256) cut_setup_kernel(CutStreams st, uint32_t first, uint32_t nstreams,
+                                                        uint32_t pieces, uint32_t piece_blocks,
+                                                        uint32_t* __restrict__ rings, uint32_t* __restrict__ weyl0,
+                                                        Steps steps, uint32_t* __restrict__ lists)
 {
     cudaTriggerProgrammaticLaunchCompletion();
     if (blockIdx.x < piece_blocks) {
@@ -75,9 +75,9 @@ __global__ void __launch_bounds__(256) cut_setup_kernel(State st, uint32_t first
         uint4 v = make_uint4(0, 0, 0, 0);
         if (p % pieces == 0) {
             const uint32_t s = first + p / pieces;
-            const uint32_t* src = st.win + (size_t)s * kWin + (kRingBase - st.pend[s]) + 4 * lane;
+            const uint32_t* src = st.win + (size_t)s * kWin + (kRingBase - st.pend[s] * st.word) + 4 * lane;
             v = make_uint4(src[0], src[1], src[2], src[3]);
-            if (lane == 0) weyl0[p / pieces] = st.weyl[s];
+            if (lane < st.word) weyl0[p / pieces * st.word + lane] = st.weyl[(size_t)s * st.word + lane];
         }
         reinterpret_cast<uint4*>(rings + (size_t)p * 128)[lane] = v;
         return;
@@ -117,7 +117,9 @@ double word_ns(int kind, double w)
     case kU32: return std::max(0.585, 0.365 * w);
     case kUniform: return std::max(0.62, 0.42 * w);
     case kNormal: return std::max(1.18, 0.35 + 0.705 * w);
-    default: return std::max(1.08, 0.27 + 0.67 * w);   // fused sums
+    case kNormalSum: return std::max(1.08, 0.27 + 0.67 * w);
+    case kCutU64: return std::max(1.19, 0.735 * w);
+    default: return std::max(1.26, 0.25 + 0.86 * w);   // kCutUniform64
     }
 }
 
@@ -176,34 +178,87 @@ int cut_choose(int kind, uint32_t nstreams, uint64_t n, int sm_count, uint64_t f
     return best_q;
 }
 
-xg_status cut_generate(xg_ctx* c, int kind, uint32_t first, uint32_t nstreams, uint64_t n, void* out, uint64_t ld,
-                       int q, bool* ran)
+xg_status CutWorkspace::ensure(size_t want)
+{
+    if (bytes >= want) return XG_OK;
+    if (mem) {
+        if (used) cudaEventSynchronize(event);
+        cudaFree(mem);
+    }
+    mem = nullptr;
+    bytes = 0;
+    if (!event && cudaEventCreateWithFlags(&event, cudaEventDisableTiming) != cudaSuccess) {
+        cudaGetLastError();
+        event = nullptr;
+        return fail(XG_ENOMEM, "cudaEventCreate(cut workspace) failed");
+    }
+    if (cudaMalloc(&mem, want) != cudaSuccess) {
+        cudaGetLastError();
+        mem = nullptr;
+        return fail(XG_ENOMEM, "cudaMalloc(cut workspace, %zu bytes) failed", want);
+    }
+    bytes = want;
+    return XG_OK;
+}
+
+xg_status CutWorkspace::acquire(cudaStream_t s)
+{
+    if (!used) return XG_OK;
+    // a tensor-core prologue that gave up waiting made its call's outputs
+    // invalid: reported by the first cut call after it has finished
+    if (tc_pending && cudaEventQuery(event) == cudaSuccess) {
+        tc_pending = false;
+        if (gf2_tc_take_failure())
+            return fail(XG_EDEVICE, "an earlier cut call's tensor-core kernel gave up waiting; its streams are not valid");
+    }
+    if (stream != s && cudaStreamWaitEvent(s, event, 0) != cudaSuccess)
+        return cuda_fail(cudaGetLastError(), "cut workspace");
+    return XG_OK;
+}
+
+xg_status CutWorkspace::release(cudaStream_t s, bool tensor_cores)
+{
+    stream = s;
+    tc_pending = tc_pending || tensor_cores;
+    if (cudaEventRecord(event, s) != cudaSuccess) return cuda_fail(cudaGetLastError(), "cut workspace");
+    used = true;
+    return XG_OK;
+}
+
+void CutWorkspace::destroy()
+{
+    if (event) {
+        if (used) cudaEventSynchronize(event);
+        cudaEventDestroy(event);
+    }
+    if (mem) cudaFree(mem);
+    *this = CutWorkspace{};
+}
+
+xg_status cut_prologue(CutWorkspace& ws, const CutStreams& streams, uint32_t first, uint32_t nstreams, uint32_t pieces,
+                       int q, size_t extra_bytes, cudaStream_t s, CutRings* out, bool* ran)
 {
     *ran = false;
-    const bool sum = kind == kNormalSum;
-    const uint64_t words = kind == kNormal || sum ? n + (n & 1u) : n;
-    const uint32_t pieces = (uint32_t)((words + (uint64_t(1) << q) - 1) >> q);
     const uint32_t total = pieces * nstreams;
     const Steps steps = plan_steps(nstreams, pieces);
-    cudaStream_t s = c->stream;
     uint32_t most_tc = 0;   // states of the largest tensor-core step
     bool use_tc[kMaxSteps] = {};
     for (int k = 0; k < steps.n; ++k) {
         const uint32_t m = steps.step[k].have * nstreams;
-        use_tc[k] = steps.step[k].tc && gf2_use_tc(c->device, m * steps.step[k].mats);
+        use_tc[k] = steps.step[k].tc && gf2_use_tc(streams.device, m * steps.step[k].mats);
         if (use_tc[k]) most_tc = std::max(most_tc, m);
     }
+    auto up = [](size_t v) { return (v + 255) / 256 * 256; };
     const size_t weyl_off = (size_t)total * 512;
-    const size_t list_off = (weyl_off + (size_t)nstreams * 4 + 255) / 256 * 256;
-    const size_t tc_off = (list_off + (size_t)steps.entries * 4 + 255) / 256 * 256;
-    const size_t sums_off = (tc_off + (most_tc ? gf2_tc_scratch_bytes(most_tc) : 0) + 255) / 256 * 256;
-    const size_t bytes = sums_off + (sum ? (size_t)total * 4 : 0);
-    if (c->ensure_cut_ws(bytes) != XG_OK) return XG_OK;
-    char* ws = static_cast<char*>(c->cut_ws);
-    uint32_t* rings = reinterpret_cast<uint32_t*>(ws);
-    uint32_t* weyl0 = reinterpret_cast<uint32_t*>(ws + weyl_off);
-    uint32_t* lists = reinterpret_cast<uint32_t*>(ws + list_off);
-    uint8_t* tc = most_tc ? reinterpret_cast<uint8_t*>(ws + tc_off) : nullptr;
+    const size_t list_off = up(weyl_off + (size_t)nstreams * streams.word * 4);
+    const size_t tc_off = up(list_off + (size_t)steps.entries * 4);
+    const size_t extra_off = up(tc_off + (most_tc ? gf2_tc_scratch_bytes(most_tc) : 0));
+    if (ws.ensure(extra_off + extra_bytes) != XG_OK) return XG_OK;
+    char* base = static_cast<char*>(ws.mem);
+    uint32_t* rings = reinterpret_cast<uint32_t*>(base);
+    uint32_t* weyl0 = reinterpret_cast<uint32_t*>(base + weyl_off);
+    uint32_t* lists = reinterpret_cast<uint32_t*>(base + list_off);
+    uint8_t* tc = reinterpret_cast<uint8_t*>(base + tc_off);
     // the matrices first: building one on its first use synchronises
     const uint64_t* mats[kMaxSteps][kMaxMats] = {};
     const uint8_t* tc_mats[kMaxSteps][kGf2TcMaxMats] = {};
@@ -217,16 +272,16 @@ xg_status cut_generate(xg_ctx* c, int kind, uint32_t first, uint32_t nstreams, u
                 f /= 2;
                 ++e;
             }
-            if (use_tc[k]) tc_mats[k][j - 1] = jump_matrix_tc(c->device, (int)c->param_set, (int)f, e, s, &st);
-            else mats[k][j - 1] = jump_matrix_multiple(c->device, (int)c->param_set, (int)f, e, s, &st);
-            if (!(use_tc[k] ? (const void*)tc_mats[k][j - 1] : (const void*)mats[k][j - 1]))
-                return st == XG_ENOMEM ? XG_OK : st;   // no memory: the whole call needs none
+            const void* m;
+            if (use_tc[k]) m = tc_mats[k][j - 1] = jump_matrix_tc(streams.device, streams.family, (int)f, e, s, &st);
+            else m = mats[k][j - 1] = jump_matrix_multiple(streams.device, streams.family, (int)f, e, s, &st);
+            if (!m) return st == XG_ENOMEM ? XG_OK : st;   // no memory: the whole call needs none
         }
     *ran = true;
-    if (xg_status w = c->cut_ws_acquire()) return w;
+    if (xg_status w = ws.acquire(s)) return w;
     const uint32_t piece_blocks = (total + 7) / 8;
     const uint32_t list_blocks = (uint32_t)((steps.entries + 255) / 256);
-    cut_setup_kernel<<<piece_blocks + list_blocks, 256, 0, s>>>(c->st, first, nstreams, pieces, piece_blocks, rings,
+    cut_setup_kernel<<<piece_blocks + list_blocks, 256, 0, s>>>(streams, first, nstreams, pieces, piece_blocks, rings,
                                                                 weyl0, steps, lists);
     cudaError_t e = cudaGetLastError();
     for (int k = 0; k < steps.n && e == cudaSuccess; ++k) {
@@ -235,32 +290,46 @@ xg_status cut_generate(xg_ctx* c, int kind, uint32_t first, uint32_t nstreams, u
         const uint32_t* src = lists + steps.step[k].at;
         const uint32_t* dst = src + m;
         if (use_tc[k])
-            e = gf2_tc_apply(c->device, tc_mats[k], n_mats, rings, src, m, rings, dst, tc, s, true);
+            e = gf2_tc_apply(streams.device, tc_mats[k], n_mats, rings, src, m, rings, dst, tc, s, true);
         else
-            e = launch_gf2_apply_multi(mats[k], n_mats, rings, rings, m, src, dst, c->sm_count, s, true, k + 1 < steps.n);
+            e = launch_gf2_apply_multi(mats[k], n_mats, rings, rings, m, src, dst, streams.sm_count, s, true,
+                                       k + 1 < steps.n);
     }
-    if (e == cudaSuccess) {
-        CutArgs a{};
-        a.st = c->st;
-        a.first = first;
-        a.nstreams = nstreams;
-        a.pieces = pieces;
-        a.log2_len = (uint32_t)q;
-        a.n = n;
-        a.out = sum ? ws + sums_off : out;
-        a.ld = ld;
-        a.rings = rings;
-        a.weyl0 = weyl0;
-        a.omega = c->weyl_on ? 0x9E3779B9u : 0u;
-        const bool vec = sum || ((reinterpret_cast<uintptr_t>(out) & 15u) == 0 && (ld % 4 == 0 || nstreams == 1));
-        e = launch_cut((int)c->param_set, kind, vec, a, s);
-        if (sum && e == cudaSuccess)
-            e = launch_dependent(true, dim3((nstreams + 1) / 2), dim3(64), s, cut_sum_kernel,
-                                 reinterpret_cast<const float*>(ws + sums_off), pieces, nstreams,
-                                 static_cast<float*>(out));
-    }
-    if (e != cudaSuccess) return st != XG_OK ? st : cuda_fail(e, "cut generation");
-    return c->cut_ws_release(most_tc != 0);
+    if (e != cudaSuccess) return cuda_fail(e, "cut prologue");
+    *out = CutRings{rings, weyl0, base + extra_off, most_tc != 0};
+    return XG_OK;
+}
+
+xg_status cut_generate(xg_ctx* c, int kind, uint32_t first, uint32_t nstreams, uint64_t n, void* out, uint64_t ld,
+                       int q, bool* ran)
+{
+    const bool sum = kind == kNormalSum;
+    const uint64_t words = kind == kNormal || sum ? n + (n & 1u) : n;
+    const uint32_t pieces = (uint32_t)((words + (uint64_t(1) << q) - 1) >> q);
+    const CutStreams streams{c->device, c->sm_count, (int)c->param_set, c->st.win, c->st.pend, c->st.weyl, 1};
+    CutRings r{};
+    xg_status st = cut_prologue(c->cut, streams, first, nstreams, pieces, q, sum ? (size_t)pieces * nstreams * 4 : 0,
+                                c->stream, &r, ran);
+    if (st != XG_OK || !*ran) return st;
+    CutArgs a{};
+    a.st = c->st;
+    a.first = first;
+    a.nstreams = nstreams;
+    a.pieces = pieces;
+    a.log2_len = (uint32_t)q;
+    a.n = n;
+    a.out = sum ? r.extra : out;
+    a.ld = ld;
+    a.rings = r.rings;
+    a.weyl0 = r.weyl0;
+    a.omega = c->weyl_on ? 0x9E3779B9u : 0u;
+    const bool vec = sum || ((reinterpret_cast<uintptr_t>(out) & 15u) == 0 && (ld % 4 == 0 || nstreams == 1));
+    cudaError_t e = launch_cut((int)c->param_set, kind, vec, a, c->stream);
+    if (sum && e == cudaSuccess)
+        e = launch_dependent(true, dim3((nstreams + 1) / 2), dim3(64), c->stream, cut_sum_kernel,
+                             reinterpret_cast<const float*>(r.extra), pieces, nstreams, static_cast<float*>(out));
+    if (e != cudaSuccess) return cuda_fail(e, "cut generation");
+    return c->cut.release(c->stream, r.tensor_cores);
 }
 
 }  // namespace xg

@@ -132,53 +132,6 @@ xg_status xg_ctx::ensure_jump_ws(size_t bytes)
     return XG_OK;
 }
 
-xg_status xg_ctx::ensure_cut_ws(size_t bytes)
-{
-    if (cut_ws_bytes >= bytes) return XG_OK;
-    if (cut_ws) {
-        if (cut_used) cudaEventSynchronize(cut_event);
-        cudaFree(cut_ws);
-    }
-    cut_ws = nullptr;
-    cut_ws_bytes = 0;
-    if (!cut_event && cudaEventCreateWithFlags(&cut_event, cudaEventDisableTiming) != cudaSuccess) {
-        cudaGetLastError();
-        cut_event = nullptr;
-        return xg::fail(XG_ENOMEM, "cudaEventCreate(cut workspace) failed");
-    }
-    if (cudaMalloc(&cut_ws, bytes) != cudaSuccess) {
-        cudaGetLastError();
-        cut_ws = nullptr;
-        return xg::fail(XG_ENOMEM, "cudaMalloc(cut workspace, %zu bytes) failed", bytes);
-    }
-    cut_ws_bytes = bytes;
-    return XG_OK;
-}
-
-xg_status xg_ctx::cut_ws_acquire()
-{
-    if (!cut_used) return XG_OK;
-    // a tensor-core prologue that gave up waiting made its call's outputs
-    // invalid: reported by the first cut call after it has finished
-    if (cut_tc_pending && cudaEventQuery(cut_event) == cudaSuccess) {
-        cut_tc_pending = false;
-        if (xg::gf2_tc_take_failure())
-            return xg::fail(XG_EDEVICE, "an earlier cut call's tensor-core kernel gave up waiting; its streams are not valid");
-    }
-    if (cut_stream != stream && cudaStreamWaitEvent(stream, cut_event, 0) != cudaSuccess)
-        return xg::cuda_fail(cudaGetLastError(), "cut workspace");
-    return XG_OK;
-}
-
-xg_status xg_ctx::cut_ws_release(bool tensor_cores)
-{
-    cut_stream = stream;
-    cut_tc_pending = cut_tc_pending || tensor_cores;
-    if (cudaEventRecord(cut_event, stream) != cudaSuccess) return xg::cuda_fail(cudaGetLastError(), "cut workspace");
-    cut_used = true;
-    return XG_OK;
-}
-
 xg_status xg_ctx::ensure_staging(size_t bytes)
 {
     if (staging_bytes >= bytes) return XG_OK;
@@ -417,11 +370,7 @@ xg_status xg_destroy(xg_ctx* ctx)
         if (c->staging[b]) cudaFree(c->staging[b]);
     }
     if (c->jump_ws) cudaFree(c->jump_ws);
-    if (c->cut_event) {
-        if (c->cut_used) cudaEventSynchronize(c->cut_event);
-        cudaEventDestroy(c->cut_event);
-    }
-    if (c->cut_ws) cudaFree(c->cut_ws);
+    c->cut.destroy();
     if (c->state_mem) cudaFree(c->state_mem);
     delete c;
     return XG_OK;

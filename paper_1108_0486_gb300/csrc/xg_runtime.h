@@ -6,6 +6,7 @@
 #include <cstdint>
 #include <mutex>
 
+#include "xg_cut.h"
 #include "xg_launch.h"
 #include "xorgens_gb300.h"
 
@@ -53,24 +54,13 @@ struct xg_ctx {
     void* jump_ws = nullptr;
     size_t jump_ws_bytes = 0;
 
-    // cut calls' workspace (grow-only, freed by xg_destroy).  Used on the
-    // context's stream of the moment: cut_event follows the last use, and a
-    // use on another stream waits for it.
-    void* cut_ws = nullptr;
-    size_t cut_ws_bytes = 0;
-    cudaEvent_t cut_event = nullptr;
-    cudaStream_t cut_stream = nullptr;
-    bool cut_used = false;      // cut_event has been recorded
-    bool cut_tc_pending = false;  // a tensor-core prologue's status is unread
+    xg::CutWorkspace cut;
 
     int pick_cfg(int kind, uint32_t nstreams, uint64_t n) const;
     xg::Store pick_store(int kind, int cfg, uint32_t nstreams, uint64_t n, const void* out, uint64_t ld) const;
     int pick_block(int kind, int cfg) const;
     xg_status ensure_staging(size_t bytes);
     xg_status ensure_jump_ws(size_t bytes);
-    xg_status ensure_cut_ws(size_t bytes);
-    xg_status cut_ws_acquire();                // before the first launch that uses it
-    xg_status cut_ws_release(bool tensor_cores);  // after the last
     void shutdown_server();
 };
 

@@ -7,8 +7,8 @@
 #include <cstring>
 #include <mutex>
 #include <new>
-#include <vector>
 
+#include "xg_cut.h"
 #include "xg_gf2_tc.h"
 #include "xg_jump.h"
 #include "xg_runtime.h"
@@ -31,6 +31,7 @@ struct xg_w64_ctx {
     void* staging = nullptr;
     size_t staging_bytes = 0;
     uint64_t split_words = 0;   // cut calls: 0 automatic, 1 never, else the piece length
+    xg::CutWorkspace cut;
     std::mutex mu;
 };
 
@@ -84,104 +85,62 @@ xg_status enqueue(xg_w64_ctx* c, int kind, uint32_t first, uint32_t nstreams, ui
     return e == cudaSuccess ? XG_OK : cuda_fail(e, "64-bit generate kernel launch");
 }
 
-// Few streams, long calls: one stream is one serial chain (one warp), so the
-// call is cut into K pieces of L = 2^q words per stream whose start states
-// come from the jump-ahead matrices (piece m = the stream advanced m L
-// words), generated as K streams of a scratch state, and the stream then
-// takes the state of its last piece.  The output is exactly the uncut call's.
-constexpr uint32_t kCutMaxStreams = 16;
-constexpr uint64_t kCutMinWords = uint64_t(1) << 18;
-
-xg_status generate_cut(xg_w64_ctx* c, int kind, uint32_t first, uint32_t nstreams, uint64_t n, void* d_out,
-                       uint64_t ld)
+// log2 of the piece length that a device call is cut into (one stream is one
+// serial chain of one warp), 0 for a whole call.  A piece length set by the
+// caller applies to at most 16 streams of at least 2^18 outputs; by itself the
+// library cuts where its prediction says so, unless a launch shape was set or
+// tuned for other calls than those.  Not while the stream is being captured: a
+// first use builds matrices and the workspace.
+//
+// 16 streams of 400000 words: 476 us whole, 1648 us in pieces of 2^16 words
+// with one launch per stream and a doubling step per factor of two (the
+// earlier form of the cut), 52 us this way; one stream 131 and 28 us; 200
+// streams of 400000 FP64 uniforms 505 us whole, 211 us.
+int cut_length(const xg_w64_ctx* c, int kind, uint32_t nstreams, uint64_t n)
 {
-    // piece length: about four pieces per SM sub-partition in all, at least 2^16
-    int q = 16;
-    if (c->split_words > 1) {
-        while ((uint64_t(1) << q) < c->split_words) ++q;
-    } else {
-        const uint64_t target = std::max<uint64_t>(1, (uint64_t)c->sm_count * 4 / nstreams);
-        while (q < 40 && (uint64_t(1) << q) * target < n) ++q;
+    if (c->split_words == 1 || n < (uint64_t(1) << 13)) return 0;
+    const bool always = nstreams <= 16 && n >= (uint64_t(1) << 18);   // whatever the launch shape set
+    if (!always && (c->split_words > 1 || c->cfg[kind] >= 0)) return 0;
+    const int q = xg::cut_choose(kind == xg64::kU64 ? xg::kCutU64 : xg::kCutUniform64, nstreams, n, c->sm_count,
+                                 c->split_words);
+    if (!q) return 0;
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(c->stream, &cap) != cudaSuccess) {
+        cudaGetLastError();
+        return 0;
     }
-    const uint64_t L = uint64_t(1) << q;
-    const uint64_t K64 = (n + L - 1) / L;
-    if (K64 < 2 || K64 * nstreams > (uint64_t(1) << 20)) return enqueue(c, kind, first, nstreams, n, d_out, ld);
-    const uint32_t K = (uint32_t)K64;
-    const uint32_t P = nstreams * K;
-    cudaStream_t s = c->stream;
-    int steps = 0;   // doubling steps: bits of K - 1
-    while (((uint64_t)(K - 1) >> steps)) ++steps;
-    xg_status st = XG_OK;
-    for (int b = 0; b < steps; ++b)
-        if (!xg::jump_matrix(c->device, xg::kJumpSetW64, q + b, s, &st)) return st;
-    // pair lists per step b: sources i K + m - 2^b, destinations i K + m
-    std::vector<uint32_t> h;
-    std::vector<size_t> src_off(steps), dst_off(steps);
-    std::vector<uint32_t> cnt(steps);
-    for (int b = 0; b < steps; ++b) {
-        const uint32_t lo = 1u << b, hi = (uint32_t)std::min<uint64_t>((uint64_t)lo << 1, K);
-        cnt[b] = (hi - lo) * nstreams;
-        src_off[b] = h.size();
-        for (uint32_t i = 0; i < nstreams; ++i)
-            for (uint32_t m = lo; m < hi; ++m) h.push_back(i * K + m - lo);
-        dst_off[b] = h.size();
-        for (uint32_t i = 0; i < nstreams; ++i)
-            for (uint32_t m = lo; m < hi; ++m) h.push_back(i * K + m);
-    }
-    // scratch: rings[P][64] | piece state (window, Weyl, pend, pos) | lists
-    const size_t off_win = (size_t)P * xg64::kR * 8;
-    const size_t off_weyl = off_win + (size_t)P * xg64::kWin * 8;
-    const size_t off_pos = off_weyl + (size_t)P * 8;
-    const size_t off_pend = off_pos + (size_t)P * 8;
-    const size_t off_lists = align_up(off_pend + (size_t)P * 4, 16);
-    const uint32_t most = steps ? *std::max_element(cnt.begin(), cnt.end()) : 0u;
-    const size_t tc_bytes = xg::gf2_apply_scratch(c->device, most);  // tensor-core operand, when used
-    const size_t off_tc = align_up(off_lists + h.size() * 4 + 4, 256);
-    const size_t total = off_tc + tc_bytes;
-    char* scratch = nullptr;
-    XG_CUDA(cudaMallocAsync(reinterpret_cast<void**>(&scratch), total, s), "cut scratch");
-    uint64_t* rings = reinterpret_cast<uint64_t*>(scratch);
-    uint32_t* rings32 = reinterpret_cast<uint32_t*>(scratch);
-    uint32_t* lists = reinterpret_cast<uint32_t*>(scratch + off_lists);
-    xg64::State pieces{reinterpret_cast<uint64_t*>(scratch + off_win), reinterpret_cast<uint64_t*>(scratch + off_weyl),
-                       reinterpret_cast<uint32_t*>(scratch + off_pend), reinterpret_cast<uint64_t*>(scratch + off_pos)};
-    cudaError_t e = cudaSuccess;
-    if (!h.empty()) e = cudaMemcpyAsync(lists, h.data(), h.size() * 4, cudaMemcpyHostToDevice, s);
-    // every ring zeroed once (the doubling steps XOR into the pieces m > 0),
-    // then piece 0 of each stream: the stream's own ring (one stream at a time)
-    if (e == cudaSuccess) e = cudaMemsetAsync(rings, 0, off_win, s);
-    for (uint32_t i = 0; i < nstreams && e == cudaSuccess; ++i)
-        e = xg64::launch_gather_rings(c->st, first + i, 1, rings + (size_t)i * K * xg64::kR, s);
-    uint8_t* tc_scratch = tc_bytes ? reinterpret_cast<uint8_t*>(scratch + off_tc) : nullptr;
-    for (int b = 0; b < steps && e == cudaSuccess; ++b)
-        e = xg::gf2_apply(c->device, xg::kJumpSetW64, q + b, rings32, cnt[b], lists + src_off[b], lists + dst_off[b],
-                          tc_scratch, c->sm_count, s, &st, true);
-    const uint64_t omega = c->weyl_on ? xg64::kOmega : 0;
-    if (e == cudaSuccess) e = xg64::launch_init_pieces(c->st, first, nstreams, K, L, rings, pieces, omega, s);
-    xg_status gst = XG_OK;
-    if (e == cudaSuccess) {
-        // the full pieces of each stream as K - 1 streams with ld = L, then its last piece
-        xg_w64_ctx view = {};
-        view.sm_count = c->sm_count;
-        view.stream = s;
-        view.st = pieces;
-        view.weyl_on = c->weyl_on;
-        view.cfg[0] = c->cfg[0];
-        view.cfg[1] = c->cfg[1];
-        view.blk[0] = c->blk[0];
-        view.blk[1] = c->blk[1];
-        const uint64_t last = n - (uint64_t)(K - 1) * L;
-        for (uint32_t i = 0; i < nstreams && gst == XG_OK; ++i) {
-            char* row = static_cast<char*>(d_out) + (uint64_t)i * ld * 8;
-            gst = enqueue(&view, kind, i * K, K - 1, L, row, L);
-            if (gst == XG_OK) gst = enqueue(&view, kind, i * K + K - 1, 1, last, row + (uint64_t)(K - 1) * L * 8, last);
-        }
-        if (gst == XG_OK) e = xg64::launch_adopt_last_piece(c->st, first, nstreams, K, pieces, n, s);
-    }
-    cudaFreeAsync(scratch, s);
-    if (gst != XG_OK) return gst;
+    return cap == cudaStreamCaptureStatusNone ? q : 0;
+}
+
+// The call in pieces of 2^q outputs; *ran = false when the whole call is to be
+// taken (no memory for the workspace).  The output is exactly the whole call's.
+xg_status generate_cut(xg_w64_ctx* c, int kind, uint32_t first, uint32_t nstreams, uint64_t n, void* d_out, uint64_t ld,
+                       int q, bool* ran)
+{
+    // the prologue reads windows and rings as 32-bit words, two per word
+    static_assert(xg64::kWin * 2 == xg::kWin && xg64::kRingBase * 2 == xg::kRingBase && xg64::kR * 2 == 128,
+                  "window layout in 32-bit words");
+    const uint32_t pieces = (uint32_t)((n + (uint64_t(1) << q) - 1) >> q);
+    const xg::CutStreams streams{c->device, c->sm_count, xg::kJumpSetW64, reinterpret_cast<const uint32_t*>(c->st.win),
+                                 c->st.pend, reinterpret_cast<const uint32_t*>(c->st.weyl), 2};
+    xg::CutRings r{};
+    xg_status st = xg::cut_prologue(c->cut, streams, first, nstreams, pieces, q, 0, c->stream, &r, ran);
+    if (st != XG_OK || !*ran) return st;
+    xg64::CutArgs a{};
+    a.st = c->st;
+    a.first = first;
+    a.nstreams = nstreams;
+    a.pieces = pieces;
+    a.log2_len = (uint32_t)q;
+    a.n = n;
+    a.out = d_out;
+    a.ld = ld;
+    a.rings = reinterpret_cast<const uint64_t*>(r.rings);
+    a.weyl0 = reinterpret_cast<const uint64_t*>(r.weyl0);
+    a.omega = c->weyl_on ? xg64::kOmega : 0;
+    const cudaError_t e = xg64::launch_cut(kind, a, c->stream);
     if (e != cudaSuccess) return cuda_fail(e, "64-bit cut generation");
-    return XG_OK;
+    return c->cut.release(c->stream, r.tensor_cores);
 }
 
 // Host output: generate into one device buffer piece by piece and copy each
@@ -233,8 +192,11 @@ xg_status generate(xg_w64_ctx* c, int kind, uint32_t first, uint32_t nstreams, u
     if (reinterpret_cast<uintptr_t>(out) & 7u) return fail(XG_EINVAL, "output must be 8-byte aligned");
     std::lock_guard<std::mutex> lk(c->mu);
     if (is_device_pointer(out)) {
-        if (nstreams <= kCutMaxStreams && n >= kCutMinWords && c->split_words != 1)
-            return generate_cut(c, kind, first, nstreams, n, out, ld);
+        if (const int q = cut_length(c, kind, nstreams, n)) {
+            bool ran = false;
+            const xg_status st = generate_cut(c, kind, first, nstreams, n, out, ld, q, &ran);
+            if (ran || st != XG_OK) return st;
+        }
         return enqueue(c, kind, first, nstreams, n, out, ld);
     }
     return to_host(c, kind, first, nstreams, n, out, ld);
@@ -299,6 +261,7 @@ xg_status xg_w64_destroy(xg_w64_ctx* c)
     if (!c) return XG_OK;
     if (c->state_mem) cudaStreamSynchronize(c->stream);
     if (c->staging) cudaFree(c->staging);
+    c->cut.destroy();
     if (c->state_mem) cudaFree(c->state_mem);
     delete c;
     return XG_OK;

@@ -10,6 +10,7 @@
 // same lane.
 #include <type_traits>
 
+#include "xg_launch.h"
 #include "xg_w64.h"
 
 namespace xg64 {
@@ -375,43 +376,68 @@ __global__ void __launch_bounds__(256) seed_kernel(State st, const uint32_t* __r
     }
 }
 
+// Where a call's words start from and what it leaves behind: a whole call
+// reads the stream's window and writes the stream state back, a piece of a cut
+// call starts from the ring and the Weyl word that the jump-ahead prologue
+// prepared, and the last one writes the state (pos advances by the whole
+// call's words).
+struct UnitSrc {
+    const uint64_t* ring = nullptr;   // null: the stream's window
+    uint64_t weyl0 = 0;
+    uint64_t pos_add = 0;
+    bool write_state = true;
+};
+
+// n outputs of stream s to row; rows: 4 * kRW words of shared memory (one word
+// per lane, raw words).
 template <int TPG, int WPL, int OUT, bool VEC, int U>
-__device__ __forceinline__ void gen_body(const GenArgs& a)
+__device__ __forceinline__ void run_stream(const State& st, uint32_t s, uint64_t n, uint64_t* row, uint64_t omega,
+                                           uint64_t* rows, const UnitSrc& src = UnitSrc())
 {
     constexpr bool kShared = WPL == 1 && OUT == kU64;
     using E = Engine<TPG, WPL, kShared>;
     constexpr int RW = E::RW;
-    const uint32_t g = (blockIdx.x * blockDim.x + threadIdx.x) / TPG;
-    if (g >= a.nstreams || a.n == 0) return;
     const int lane = threadIdx.x % TPG;
-    const uint32_t s = a.first + g;
     E eng;
     eng.lane = lane;
     eng.mask = group_mask<TPG>();
-    const State& st = a.st;
     uint64_t* win_s = st.win + (uint64_t)s * kWin;
-    load_ring(eng, win_s, st.pend[s]);
-    if constexpr (kShared) {
-        extern __shared__ uint64_t rows[];   // 4 * RW words per warp
-        eng.share(rows + threadIdx.x / 32 * (4 * RW));
+    uint64_t wp;
+    if (src.ring) {
+        load_ring(eng, src.ring - kRingBase, 0u);
+        wp = src.weyl0;
+    } else {
+        load_ring(eng, win_s, st.pend[s]);
+        wp = st.weyl[s];
     }
-    const uint64_t wp = st.weyl[s];
+    if constexpr (kShared) eng.share(rows);
     Emit<E, OUT, VEC> em;
-    em.omega = a.omega;
-    em.limit = a.n;
+    em.omega = omega;
+    em.limit = n;
     em.lane_off = (uint64_t)WPL * lane;
-    em.wl = wp + (uint64_t)(WPL * lane + 1) * a.omega;
-    em.dst = reinterpret_cast<uint64_t*>(a.out) + (uint64_t)g * a.ld + em.lane_off;
+    em.wl = wp + (uint64_t)(WPL * lane + 1) * omega;
+    em.dst = row + em.lane_off;
     uint64_t retired[WPL];
-    const uint64_t nr = (a.n + RW - 1) / RW;
+    const uint64_t nr = (n + RW - 1) / RW;
     const int rot = drive<E, Emit<E, OUT, VEC>, U>(eng, nr, em, retired);
+    if (!src.write_state) return;
     __syncwarp(eng.mask);
     store_window(eng, win_s, rot, retired);
     if (lane == 0) {
-        st.weyl[s] = wp + a.n * a.omega;
-        st.pend[s] = (uint32_t)(nr * RW - a.n);
-        st.pos[s] += a.n;
+        st.weyl[s] = wp + n * omega;
+        st.pend[s] = (uint32_t)(nr * RW - n);
+        st.pos[s] += src.ring ? src.pos_add : n;
     }
+}
+
+template <int TPG, int WPL, int OUT, bool VEC, int U>
+__device__ __forceinline__ void gen_body(const GenArgs& a)
+{
+    const uint32_t g = (blockIdx.x * blockDim.x + threadIdx.x) / TPG;
+    if (g >= a.nstreams || a.n == 0) return;
+    extern __shared__ uint64_t rows[];   // 4 * kRW words per warp, for raw words with one word per lane
+    run_stream<TPG, WPL, OUT, VEC, U>(a.st, a.first + g, a.n, reinterpret_cast<uint64_t*>(a.out) + (uint64_t)g * a.ld,
+                                      a.omega, rows + threadIdx.x / 32 * (4 * kRW));
 }
 
 // Two register budgets: one warp per stream runs uniforms with a stated
@@ -434,6 +460,30 @@ template <int TPG, int WPL, int OUT, bool VEC, int U>
 __global__ void __launch_bounds__(256, 1) gen_kernel_ilp(GenArgs a)
 {
     gen_body<TPG, WPL, OUT, VEC, U>(a);
+}
+
+// A cut call: a warp generates piece m of the call on stream first + i (grid:
+// pieces, streams).  The length is read by a shuffle, which makes the compiler
+// keep the whole call's loop (see the 32-bit cut kernel).
+template <int OUT>
+__global__ void __launch_bounds__(64, 1) cut_kernel(CutArgs a)
+{
+    const uint32_t m = (blockIdx.x * blockDim.x + threadIdx.x) / 32, i = blockIdx.y;
+    if (m >= a.pieces) return;
+    __shared__ uint64_t rows[OUT == kU64 ? 2 * 4 * kRW : 1];
+    cudaGridDependencySynchronize();   // the last prologue step
+    const uint64_t skip = (uint64_t)m << a.log2_len;
+    UnitSrc src;
+    src.ring = a.rings + ((size_t)i * a.pieces + m) * kR;
+    src.weyl0 = a.weyl0[i] + skip * a.omega;
+    src.write_state = m + 1 == a.pieces;
+    src.pos_add = a.n;
+    uint64_t n = src.write_state ? a.n - skip : uint64_t(1) << a.log2_len;
+    n = __shfl_sync(0xFFFFFFFFu, n, 0);
+    uint64_t* row = reinterpret_cast<uint64_t*>(a.out) + (uint64_t)i * a.ld + skip;
+    run_stream<32, 1, OUT, false, OUT == kUniformF64 ? 8 : 1>(a.st, a.first + i, n, row, a.omega,
+                                                              OUT == kU64 ? rows + threadIdx.x / 32 * (4 * kRW) : rows,
+                                                              src);
 }
 
 template <int TPG, int WPL, int OUT, bool VEC>
@@ -475,6 +525,14 @@ cudaError_t launch_gen(int cfg, int kind, bool vec, int block, const GenArgs& a,
     case 3: return launch_cfg<32, 1>(kind, vec, block, a, s);
     default: return cudaErrorInvalidValue;
     }
+}
+
+cudaError_t launch_cut(int kind, const CutArgs& a, cudaStream_t s)
+{
+    constexpr unsigned block = 64;
+    const dim3 grid((a.pieces + 1) / 2, a.nstreams);
+    return kind == kU64 ? xg::launch_dependent(true, grid, dim3(block), s, cut_kernel<kU64>, a)
+                        : xg::launch_dependent(true, grid, dim3(block), s, cut_kernel<kUniformF64>, a);
 }
 
 // FP64 uniform conversion of n given words (grid-stride).
@@ -570,48 +628,6 @@ cudaError_t launch_substream_scatter(const State& st, uint32_t first, uint32_t n
 {
     if (n == 0) return cudaSuccess;
     substream_scatter_kernel<<<n, kR, 0, s>>>(st, first, n, rings, w0, q, omega);
-    return cudaGetLastError();
-}
-
-__global__ void __launch_bounds__(64) init_pieces_kernel(State real, uint32_t first, uint32_t K, uint64_t L,
-                                                         const uint64_t* __restrict__ rings, State pieces,
-                                                         uint64_t omega)
-{
-    const uint32_t p = blockIdx.x;   // piece p = i K + m
-    const uint32_t i = p / K, m = p % K;
-    pieces.win[(size_t)p * kWin + kRingBase + threadIdx.x] = rings[(size_t)p * kR + threadIdx.x];
-    if (threadIdx.x == 0) {
-        pieces.weyl[p] = real.weyl[first + i] + (uint64_t)m * L * omega;
-        pieces.pend[p] = 0;
-        pieces.pos[p] = 0;
-    }
-}
-
-__global__ void __launch_bounds__(96) adopt_last_piece_kernel(State real, uint32_t first, uint32_t K, State pieces,
-                                                              uint64_t n)
-{
-    const uint32_t i = blockIdx.x;
-    const uint32_t p = i * K + (K - 1);
-    const uint32_t s = first + i;
-    real.win[(size_t)s * kWin + threadIdx.x] = pieces.win[(size_t)p * kWin + threadIdx.x];
-    if (threadIdx.x == 0) {
-        real.weyl[s] = pieces.weyl[p];
-        real.pend[s] = pieces.pend[p];
-        real.pos[s] += n;
-    }
-}
-
-cudaError_t launch_init_pieces(const State& real, uint32_t first, uint32_t nstreams, uint32_t K, uint64_t L,
-                               const uint64_t* rings, const State& pieces, uint64_t omega, cudaStream_t s)
-{
-    init_pieces_kernel<<<nstreams * K, kR, 0, s>>>(real, first, K, L, rings, pieces, omega);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_adopt_last_piece(const State& real, uint32_t first, uint32_t nstreams, uint32_t K,
-                                    const State& pieces, uint64_t n, cudaStream_t s)
-{
-    adopt_last_piece_kernel<<<nstreams, kWin, 0, s>>>(real, first, K, pieces, n);
     return cudaGetLastError();
 }
 

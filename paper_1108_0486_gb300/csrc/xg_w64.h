@@ -44,6 +44,23 @@ struct GenArgs {
     uint64_t omega;   // kOmega, or 0 with the Weyl generator off
 };
 
+// A call cut into pieces of 2^log2_len outputs per stream, each its own warp
+// (one word per lane): piece m of stream first + i starts from
+// rings[i * pieces + m] and the Weyl word weyl0[i] + m 2^log2_len omega.
+struct CutArgs {
+    State st;
+    uint32_t first;
+    uint32_t nstreams;
+    uint32_t pieces;
+    uint32_t log2_len;
+    uint64_t n;
+    void* out;
+    uint64_t ld;
+    const uint64_t* rings;
+    const uint64_t* weyl0;
+    uint64_t omega;
+};
+
 // Launch configurations: lanes per stream x words per lane = 32.
 struct LaunchCfg {
     int tpg, wpl, block;
@@ -55,6 +72,8 @@ int cfg_index(int tpg, int wpl);
 cudaError_t launch_seed(const State& st, const uint32_t* d_seeds, uint32_t first, uint32_t count,
                         cudaStream_t s);
 cudaError_t launch_gen(int cfg, int kind, bool vec, int block, const GenArgs& a, cudaStream_t s);
+// Launched as a dependent of the prologue's last kernel.
+cudaError_t launch_cut(int kind, const CutArgs& a, cudaStream_t s);
 cudaError_t launch_transform_uniform(const uint64_t* in, uint64_t n, uint64_t* out, int sms, cudaStream_t s);
 
 // Jump-ahead.  The 64-word ring is a 4096-bit state like the 32-bit sets'
@@ -73,16 +92,5 @@ cudaError_t launch_scatter_rings(const State& st, uint32_t first, uint32_t n, co
 // *w0 advanced by m 2^q omega, and position m 2^q.
 cudaError_t launch_substream_scatter(const State& st, uint32_t first, uint32_t n, const uint64_t* rings,
                                      const uint64_t* w0, int q, uint64_t omega, cudaStream_t s);
-
-// Cut calls: a long call on stream first + i is generated as K pieces of L
-// words, piece m by stream i K + m of a scratch state `pieces` whose ring is
-// rings[i K + m] (the real ring advanced m L words) and whose Weyl word is
-// the real one advanced by m L omega.
-cudaError_t launch_init_pieces(const State& real, uint32_t first, uint32_t nstreams, uint32_t K, uint64_t L,
-                               const uint64_t* rings, const State& pieces, uint64_t omega, cudaStream_t s);
-// After the pieces ran: stream first + i takes the state of its last piece
-// (window, Weyl word, pending words) and its position advances by n.
-cudaError_t launch_adopt_last_piece(const State& real, uint32_t first, uint32_t nstreams, uint32_t K,
-                                    const State& pieces, uint64_t n, cudaStream_t s);
 
 }  // namespace xg64

@@ -341,3 +341,41 @@ def test_cut_prologue_steps(streams, piece, pieces, tensor_cores, monkeypatch):
             rows.append((st.u32(n), st.u32(n), st.u32(99)))
     for x, y in zip(*rows):
         assert torch.equal(x, y)
+
+
+@pytest.mark.parametrize("kind", ["u64", "uniform"])
+@pytest.mark.parametrize("streams,n,piece", [(1, 32769, 0), (1, (1 << 18) + 3, 4096), (3, 262145, 64), (16, 1 << 18, 32768),
+                                              (17, 70001, 0), (100, 131072, 0), (400, 262147, 0)])
+def test_cut_64bit_calls_equal_whole_calls(kind, streams, n, piece):
+    """64-bit calls cut into pieces (chosen by the library, or of a set length)
+    against whole calls on the same streams, twice in a row, with rows of odd
+    strides; a stream against the oracle."""
+    from paper_1108_0486_gb300 import Streams64
+    rows = []
+    for split in (piece, 1):
+        with Streams64(streams, seeds=W.seeds(streams)) as st:
+            st.set_split(split)
+            rows.append([st.generate(kind, n), st.generate(kind, n, ld=n + 5)[:, :n], st.generate(kind, 77)])
+            rows[-1].append(torch.from_numpy(np.concatenate([st.get_state(streams - 1)[0]]).view(np.int64)))
+    for x, y in zip(*rows):
+        assert torch.equal(x, y)
+    w = O.streams64(W.seeds(1, streams), 2 * n)[0, n:]
+    got = rows[0][1][streams - 1].cpu().numpy()
+    assert np.array_equal(got.view(np.uint64), w) if kind == "u64" else np.array_equal(got, O.uniform64_of(w))
+
+
+def test_64bit_call_in_a_captured_graph_is_not_cut():
+    from paper_1108_0486_gb300 import Streams64
+    n, streams = 1 << 18, 3
+    cs = torch.cuda.Stream()
+    with Streams64(streams, seeds=W.seeds(streams), stream=cs) as st:
+        out = torch.empty((streams, n), dtype=torch.int64, device="cuda")
+        torch.cuda.synchronize()
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g, stream=cs):
+            st.u64(n, out=out)
+        for k in range(2):
+            g.replay()
+            torch.cuda.synchronize()
+            w = O.streams64(W.seeds(1, streams), (k + 1) * n)[0, k * n:]
+            assert np.array_equal(out[streams - 1].cpu().numpy().view(np.uint64), w)
