@@ -290,7 +290,8 @@ xg_status cut_prologue(CutWorkspace& ws, const CutStreams& streams, uint32_t fir
         const uint32_t* src = lists + steps.step[k].at;
         const uint32_t* dst = src + m;
         if (use_tc[k])
-            e = gf2_tc_apply(streams.device, tc_mats[k], n_mats, rings, src, m, rings, dst, tc, s, true);
+            e = gf2_tc_apply(streams.device, tc_mats[k], n_mats, TcStates{rings, kGf2Words, src, nullptr, 0}, m, rings, kGf2Words,
+                             dst, tc, s, true);
         else
             e = launch_gf2_apply_multi(mats[k], n_mats, rings, rings, m, src, dst, streams.sm_count, s, true,
                                        k + 1 < steps.n);

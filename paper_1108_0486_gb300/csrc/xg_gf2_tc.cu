@@ -206,8 +206,8 @@ struct TcMaps {
 // tile overlaps the MMAs of the next.
 __global__ void __launch_bounds__(kThreads, 1) gf2_tc_kernel(const __grid_constant__ TcMaps maps, uint32_t n_mats,
                                                               uint32_t n, uint32_t n_tiles,
-                                                              const uint32_t* __restrict__ dst, uint32_t* rings,
-                                                              uint32_t* status, uint32_t stall)
+                                                              const uint32_t* __restrict__ dst, uint32_t* out,
+                                                              uint32_t out_stride, uint32_t* status, uint32_t stall)
 {
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -318,7 +318,7 @@ __global__ void __launch_bounds__(kThreads, 1) gf2_tc_kernel(const __grid_consta
             tc_fence_after();
             if (failed(&s_failed)) break;
             const uint32_t mt = t % kMTiles, nt = t / kMTiles % n_tiles;
-            const uint32_t* to = dst + (size_t)(t / kMTiles / n_tiles) * n;
+            const uint32_t* to = dst ? dst + (size_t)(t / kMTiles / n_tiles) * n : nullptr;
             const uint32_t word = mt * (kBM / 32) + q;  // ring word of these 32 bits
             static_assert(kBN % 16 == 0, "columns are read 16 at a time");
             for (int c = 0; c < kBN; c += 32) {
@@ -338,8 +338,8 @@ __global__ void __launch_bounds__(kThreads, 1) gf2_tc_kernel(const __grid_consta
                 }
                 const uint32_t st = nt * kBN + (uint32_t)c + (uint32_t)lane;
                 if (st < n && c + lane < kBN) {
-                    const uint32_t d = to[st];
-                    if (d != kNoState) rings[(size_t)d * kGf2Words + word] = mine;
+                    const uint32_t d = to ? to[st] : st;
+                    if (d != kNoState) out[(size_t)d * out_stride + word] = mine;
                 }
             }
             tc_fence_before();
@@ -393,11 +393,10 @@ __global__ void __launch_bounds__(256) expand_matrix_kernel(const uint32_t* __re
     *reinterpret_cast<uint4*>(A + (size_t)(32 * w + lane) * kRowBytes + 16 * kw) = spread32(row);
 }
 
-// B[s][k] = bit k of state src[s] (s < n), 0 for n <= s < n_pad.  Thread =
+// B[s][k] = bit k of state s of `in` (s < n), 0 for n <= s < n_pad.  Thread =
 // one ring word = 16 bytes of B.
-__global__ void __launch_bounds__(256) expand_states_kernel(const uint32_t* __restrict__ rings,
-                                                            const uint32_t* __restrict__ src, uint32_t n,
-                                                            uint32_t n_pad, uint8_t* __restrict__ B)
+__global__ void __launch_bounds__(256) expand_states_kernel(TcStates in, uint32_t n, uint32_t n_pad,
+                                                            uint8_t* __restrict__ B)
 {
     const uint64_t t = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
     cudaTriggerProgrammaticLaunchCompletion();
@@ -405,7 +404,11 @@ __global__ void __launch_bounds__(256) expand_states_kernel(const uint32_t* __re
     if (t >= (uint64_t)n_pad * kGf2Words) return;
     const uint32_t s = (uint32_t)(t / kGf2Words), w = (uint32_t)(t % kGf2Words);
     uint32_t x = 0;
-    if (s < n) x = rings[(size_t)(src ? src[s] : s) * kGf2Words + w];
+    if (s < n) {
+        const uint32_t* ring = in.base + (size_t)(in.list ? in.list[s] : s) * in.stride;
+        if (in.pend) ring -= in.pend[s] * in.word;
+        x = ring[w];
+    }
     *reinterpret_cast<uint4*>(B + (size_t)s * kRowBytes + 16 * w) = spread32(x);
 }
 
@@ -488,9 +491,8 @@ cudaError_t gf2_tc_expand_matrix(const uint64_t* C, uint8_t* A, cudaStream_t s)
     return cudaGetLastError();
 }
 
-cudaError_t gf2_tc_apply(int device, const uint8_t* const* A, int n_mats, const uint32_t* rings_in,
-                         const uint32_t* src, uint32_t n, uint32_t* rings_out, const uint32_t* dst, uint8_t* scratch,
-                         cudaStream_t s, bool dependent)
+cudaError_t gf2_tc_apply(int device, const uint8_t* const* A, int n_mats, const TcStates& in, uint32_t n, uint32_t* out,
+                         uint32_t out_stride, const uint32_t* dst, uint8_t* scratch, cudaStream_t s, bool dependent)
 {
     if (n == 0 || n_mats == 0) return cudaSuccess;
     if (n_mats < 0 || n_mats > kGf2TcMaxMats) return cudaErrorInvalidValue;
@@ -510,7 +512,7 @@ cudaError_t gf2_tc_apply(int device, const uint8_t* const* A, int n_mats, const 
     }
     const uint64_t words = (uint64_t)n_pad * kGf2Words;
     cudaError_t e = launch_dependent(dependent, dim3((unsigned)((words + 255) / 256)), dim3(256), s,
-                                     expand_states_kernel, rings_in, src, n, n_pad, scratch);
+                                     expand_states_kernel, in, n, n_pad, scratch);
     if (e != cudaSuccess) return e;
     const uint32_t n_tiles = n_pad / kBN;
     const uint64_t tiles = (uint64_t)(kGf2Bits / kBM) * n_tiles * n_mats;
@@ -528,7 +530,7 @@ cudaError_t gf2_tc_apply(int device, const uint8_t* const* A, int n_mats, const 
     attr.val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = &attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, gf2_tc_kernel, maps, (uint32_t)n_mats, n, n_tiles, dst, rings_out, g_status_dev,
+    return cudaLaunchKernelEx(&cfg, gf2_tc_kernel, maps, (uint32_t)n_mats, n, n_tiles, dst, out, out_stride, g_status_dev,
                               (stall && stall[0] == '1') ? 1u : 0u);
 }
 

@@ -33,16 +33,27 @@ cudaError_t gf2_tc_expand_matrix(const uint64_t* C, uint8_t* A, cudaStream_t s);
 // Most matrices applied by one launch.
 constexpr int kGf2TcMaxMats = 7;
 
-// rings_out[dst[j n + i]] = C_j rings_in[src[i]] (src null: i) for i < n and
-// j < n_mats (<= kGf2TcMaxMats), with A[j] from gf2_tc_expand_matrix; the
-// destination rings are overwritten, and may be in the same array as the
-// sources if no destination is a source; kNoState destinations are skipped.
-// scratch: gf2_tc_scratch_bytes(n) bytes, 16-byte aligned, reused once the
-// launch has finished.  Asynchronous on s.  dependent: as in
+// The states that are read: state i is the 128 words at base + list[i] stride
+// (list null: i), or, with pend, at base + i stride - pend[i] word (the ring in
+// a stream's window, base its position without pending words).
+struct TcStates {
+    const uint32_t* base;
+    uint32_t stride;
+    const uint32_t* list;
+    const uint32_t* pend;
+    uint32_t word;
+};
+
+// out[dst[j n + i] out_stride ..] = C_j (state i) for i < n and j < n_mats (<=
+// kGf2TcMaxMats; dst null: one matrix, i), with A[j] from gf2_tc_expand_matrix.
+// All states are read before the first is written: out may overlap the states
+// with one matrix, else if no destination is a source.  kNoState destinations
+// are skipped.  scratch: gf2_tc_scratch_bytes(n) bytes, 16-byte aligned, reused
+// once the launch has finished.  Asynchronous on s.  dependent: as in
 // launch_gf2_apply_pairs.
-cudaError_t gf2_tc_apply(int device, const uint8_t* const* A, int n_mats, const uint32_t* rings_in,
-                         const uint32_t* src, uint32_t n, uint32_t* rings_out, const uint32_t* dst, uint8_t* scratch,
-                         cudaStream_t s, bool dependent = false);
+cudaError_t gf2_tc_apply(int device, const uint8_t* const* A, int n_mats, const TcStates& in, uint32_t n, uint32_t* out,
+                         uint32_t out_stride, const uint32_t* dst, uint8_t* scratch, cudaStream_t s,
+                         bool dependent = false);
 
 // True (and cleared) if a tensor-core launch gave up a wait since the last
 // call: its results are not valid.  Read after synchronising.

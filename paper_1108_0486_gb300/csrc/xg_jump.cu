@@ -144,7 +144,7 @@ __global__ void __launch_bounds__(128) gf2_apply_pairs_kernel(MatSet mats, const
     __shared__ uint32_t vbits[kPairVecs][kR];
     __shared__ uint32_t tbl[kPairVecs > 4 ? 16 : 1][kR];
     const uint32_t* __restrict__ C = mats.C[blockIdx.z];
-    dst += (size_t)blockIdx.z * n;
+    if (dst) dst += (size_t)blockIdx.z * n;
     const int t = threadIdx.x;
     const uint32_t base = blockIdx.x * kPairVecs;
     const int nv = (int)umin((uint32_t)kPairVecs, n - base);
@@ -159,7 +159,7 @@ __global__ void __launch_bounds__(128) gf2_apply_pairs_kernel(MatSet mats, const
     load_columns(w0);
     cudaGridDependencySynchronize();
     for (int v = 0; v < kPairVecs; ++v)
-        vbits[v][t] = v < nv ? rings[(size_t)src[base + v] * kR + t] : 0u;
+        vbits[v][t] = v < nv ? rings[(size_t)(src ? src[base + v] : base + v) * kR + t] : 0u;
     __syncthreads();
     uint32_t acc[kPairVecs];
 #pragma unroll
@@ -192,7 +192,7 @@ __global__ void __launch_bounds__(128) gf2_apply_pairs_kernel(MatSet mats, const
 #pragma unroll
     for (int v = 0; v < kPairVecs; ++v)
         if (v < nv && acc[v]) {
-            const uint32_t d = dst[base + v];
+            const uint32_t d = dst ? dst[base + v] : blockIdx.z * n + base + v;
             if (d != kNoState) atomicXor(&out[(size_t)d * kR + t], acc[v]);
         }
 }
@@ -237,6 +237,17 @@ __global__ void scatter_rings_kernel(State st, uint32_t first, uint32_t n, const
         st.pend[s] = 0;
         st.pos[s] += jump;
     }
+}
+
+// The same where the windows hold the jumped rings already.
+__global__ void finish_jump_kernel(State st, uint32_t first, uint32_t n, uint64_t jump, uint32_t omega)
+{
+    const uint32_t k = blockIdx.x * blockDim.x + threadIdx.x;
+    if (k >= n) return;
+    const uint32_t s = first + k;
+    st.weyl[s] += (uint32_t)jump * omega;
+    st.pend[s] = 0;
+    st.pos[s] += jump;
 }
 
 // Substreams: stream first + m takes rings[m] (its ring after m * 2^q words
@@ -463,30 +474,13 @@ cudaError_t gf2_apply(int device, int family, int k, uint32_t* rings, uint32_t n
     if (scratch && gf2_use_tc(device, n)) {
         const uint8_t* A = jump_matrix_tc(device, family, 1, k, s, st);
         if (!A) return cudaErrorMemoryAllocation;
-        return gf2_tc_apply(device, &A, 1, rings, d_src, n, rings, d_dst, scratch, s);
+        return gf2_tc_apply(device, &A, 1, TcStates{rings, kGf2Words, d_src, nullptr, 0}, n, rings, kGf2Words, d_dst, scratch,
+                            s);
     }
     const uint64_t* C = jump_matrix(device, family, k, s, st);
     if (!C) return cudaErrorMemoryAllocation;
     cudaError_t e = dst_zeroed ? cudaSuccess : zero_rings(rings, d_dst, n, s);
     if (e == cudaSuccess) e = launch_gf2_apply_pairs(C, rings, rings, n, d_src, d_dst, sm_count, s);
-    return e;
-}
-
-// rings[dst[i]] = P rings[src[i]] for a matrix P in column form that is not
-// one of the cached powers; A_buf (8 MiB) receives its FP4 copy when the
-// tensor cores are used.
-static cudaError_t gf2_apply_explicit(int device, const uint64_t* P, uint8_t* A_buf, uint32_t* rings, uint32_t n,
-                                      const uint32_t* d_src, const uint32_t* d_dst, uint8_t* scratch, int sm_count,
-                                      cudaStream_t s)
-{
-    if (scratch && A_buf && gf2_use_tc(device, n)) {
-        cudaError_t e = gf2_tc_expand_matrix(P, A_buf, s);
-        const uint8_t* A = A_buf;
-        if (e == cudaSuccess) e = gf2_tc_apply(device, &A, 1, rings, d_src, n, rings, d_dst, scratch, s);
-        return e;
-    }
-    cudaError_t e = zero_rings(rings, d_dst, n, s);
-    if (e == cudaSuccess) e = launch_gf2_apply_pairs(P, rings, rings, n, d_src, d_dst, sm_count, s);
     return e;
 }
 
@@ -516,6 +510,68 @@ size_t gf2_jump_work_bytes(int device, uint32_t n, uint64_t words)
     return b;
 }
 
+// The product of the powers in `words` in column form (in w, product_bytes):
+// its newest columns by one application per further set bit to 32 (64) states,
+// then all columns from them.  For 16384 streams and 8 set bits this took the
+// jump from 0.615 ms (seven tensor-core products of 4096 columns each) to
+// 0.311 ms.  The applications are one dependent chain, 5.6 us each: the launch
+// that waits for the one before it, the states, 8 rounds of tables.
+static cudaError_t power_product(int device, int family, uint64_t words, uint8_t* w, int sm_count, cudaStream_t s,
+                                 const uint64_t** product, xg_status* st)
+{
+    const int nb = newest_columns(family);
+    const size_t group = (size_t)nb * kR;   // 32-bit words of one group of columns
+    const int bits = __builtin_popcountll(words);
+    uint32_t* cols = reinterpret_cast<uint32_t*>(w);
+    uint8_t* seq = w + (size_t)bits * kMaxNewest * kR * 4;
+    uint64_t* prod = reinterpret_cast<uint64_t*>(seq + kSeqBytes);
+    cudaError_t e = cudaMemsetAsync(cols, 0, (size_t)(bits - 1) * group * 4, s);
+    const uint32_t* have = nullptr;   // the newest columns of the product so far
+    int done = 0;
+    for (int k = 0; k < 64 && e == cudaSuccess; ++k) {
+        if (!((words >> k) & 1)) continue;
+        const uint64_t* C = jump_matrix(device, family, k, s, st);
+        if (!C) return cudaErrorMemoryAllocation;
+        if (!have) {
+            have = newest_of(C, family);
+            continue;
+        }
+        uint32_t* to = cols + done * group;
+        e = launch_gf2_apply_pairs(C, have, to, (uint32_t)nb, nullptr, nullptr, sm_count, s, done > 0);
+        have = to;
+        ++done;
+    }
+    if (e == cudaSuccess) e = launch_build_columns(family, have, seq, prod, s);
+    *product = prod;
+    return e;
+}
+
+bool gf2_jump_in_place(int device, uint32_t n, uint64_t words)
+{
+    return gf2_use_tc(device, n) && (__builtin_popcountll(words) == 1 || jump_combines(words, n));
+}
+
+cudaError_t gf2_jump_windows(int device, int family, uint64_t words, const JumpWindows& win, uint32_t n, uint8_t* work,
+                             int sm_count, cudaStream_t s, xg_status* st)
+{
+    *st = XG_OK;
+    const uint8_t* A = nullptr;
+    if (__builtin_popcountll(words) == 1) {
+        A = jump_matrix_tc(device, family, 1, __builtin_ctzll(words), s, st);
+        if (!A) return cudaErrorMemoryAllocation;
+    } else {
+        uint8_t* w = work + (gf2_apply_scratch(device, n) + 255) / 256 * 256;
+        uint8_t* abuf = w + product_bytes(words);
+        const uint64_t* P = nullptr;
+        cudaError_t e = power_product(device, family, words, w, sm_count, s, &P, st);
+        if (e == cudaSuccess) e = gf2_tc_expand_matrix(P, abuf, s);
+        if (e != cudaSuccess) return e;
+        A = abuf;
+    }
+    uint32_t* ring = win.win + kRingBase;
+    return gf2_tc_apply(device, &A, 1, TcStates{ring, kWin, nullptr, win.pend, win.word}, n, ring, kWin, nullptr, work, s);
+}
+
 cudaError_t gf2_jump_states(int device, int family, uint64_t words, uint32_t* rings, uint32_t n,
                             const uint32_t* d_idx, uint8_t* work, int sm_count, cudaStream_t s, xg_status* st,
                             bool* result_hi)
@@ -525,8 +581,8 @@ cudaError_t gf2_jump_states(int device, int family, uint64_t words, uint32_t* ri
     const uint32_t* lo = d_idx;       // 0 .. n-1
     const uint32_t* hi = d_idx + n;   // n .. 2n-1
     const size_t sbytes = gf2_apply_scratch(device, n);
-    uint8_t* scratch = sbytes ? work : nullptr;
     if (!jump_combines(words, n)) {
+        uint8_t* scratch = sbytes ? work : nullptr;
         bool in_lo = true;
         for (int k = 0; k < 64; ++k) {
             if (!((words >> k) & 1)) continue;
@@ -537,35 +593,11 @@ cudaError_t gf2_jump_states(int device, int family, uint64_t words, uint32_t* ri
         *result_hi = !in_lo;
         return cudaSuccess;
     }
-    // The product of the powers: its newest columns by one application per
-    // further set bit to 32 (64) states, then all columns from them.  For
-    // 16384 streams and 8 set bits this took the jump from 0.615 ms (seven
-    // tensor-core products of 4096 columns each) to 0.311 ms.
-    uint8_t* w = work + (sbytes + 255) / 256 * 256;
-    const int nb = newest_columns(family);
-    const size_t group = (size_t)nb * kR;   // 32-bit words of one group of columns
-    uint32_t* cols = reinterpret_cast<uint32_t*>(w);
-    uint8_t* seq = w + (size_t)__builtin_popcountll(words) * kMaxNewest * kR * 4;
-    uint64_t* prod = reinterpret_cast<uint64_t*>(seq + kSeqBytes);
-    uint8_t* abuf = scratch ? seq + kSeqBytes + (size_t)kBits * kR * 4 : nullptr;  // FP4 copy of the product
-    cudaError_t e = cudaMemsetAsync(cols + group, 0, (size_t)(__builtin_popcountll(words) - 1) * group * 4, s);
-    int done = 0;
-    for (int k = 0; k < 64 && e == cudaSuccess; ++k) {
-        if (!((words >> k) & 1)) continue;
-        const uint64_t* C = jump_matrix(device, family, k, s, st);
-        if (!C) return cudaErrorMemoryAllocation;
-        if (done == 0)
-            e = cudaMemcpyAsync(cols, newest_of(C, family), group * 4, cudaMemcpyDeviceToDevice, s);
-        else
-            e = launch_gf2_apply_pairs(C, cols + (done - 1) * group, cols + done * group, (uint32_t)nb, lo, lo, sm_count, s,
-                                       done > 1);
-        ++done;
-    }
-    if (e == cudaSuccess) e = launch_build_columns(family, cols + (done - 1) * group, seq, prod, s);
-    if (e == cudaSuccess) {
-        e = gf2_apply_explicit(device, prod, abuf, rings, n, lo, hi, scratch, sm_count, s);
-        *result_hi = true;
-    }
+    const uint64_t* P = nullptr;
+    cudaError_t e = power_product(device, family, words, work + (sbytes + 255) / 256 * 256, sm_count, s, &P, st);
+    if (e == cudaSuccess) e = zero_rings(rings, hi, n, s);
+    if (e == cudaSuccess) e = launch_gf2_apply_pairs(P, rings, rings, n, lo, hi, sm_count, s);
+    *result_hi = true;
     return e;
 }
 
@@ -651,30 +683,41 @@ extern "C" xg_status xg_jump(xg_ctx* ctx, uint32_t first, uint32_t nstreams, uin
     xg_status st = XG_OK;
     for (int k = 0; k <= top; ++k)
         if (((words >> k) & 1) && !jump_matrix(ctx->device, (int)ctx->param_set, k, s, &st)) return st;
-    // workspace kept in the context (grow-only): rings[0, n) hold the
-    // states, rings[n, 2n) receive the results; index lists (stream ids for
-    // the gather, then 0 .. 2n-1); the jump's own work area
-    const size_t rings_bytes = (size_t)2 * nstreams * kR * 4;
-    const size_t ids_off = rings_bytes;
-    const size_t work_off = (ids_off + (size_t)3 * nstreams * 4 + 255) / 256 * 256;
+    const uint32_t omega = ctx->weyl_on ? 0x9E3779B9u : 0u;
     const size_t wbytes = gf2_jump_work_bytes(ctx->device, nstreams, words);
-    if (xg_status g = ctx->ensure_jump_ws(work_off + wbytes)) return g;
-    char* ws = static_cast<char*>(ctx->jump_ws);
-    uint32_t* rings = reinterpret_cast<uint32_t*>(ws);
-    uint32_t* ids = reinterpret_cast<uint32_t*>(ws + ids_off);
-    const uint32_t* lo_idx = ids + nstreams;  // 0 .. 2n-1
-    cudaError_t e = launch_jump_index(ids, nstreams, first, s);
-    if (e == cudaSuccess) e = launch_gather_rings(ctx->st, ids, nstreams, rings, nullptr, nullptr, 0, 0, s);
-    bool hi = false;
-    if (e == cudaSuccess)
-        e = gf2_jump_states(ctx->device, (int)ctx->param_set, words, rings, nstreams, lo_idx,
-                            reinterpret_cast<uint8_t*>(ws + work_off), ctx->sm_count, s, &st, &hi);
-    const bool in_lo = !hi;
-    if (e == cudaSuccess) {
-        const uint32_t* res = in_lo ? rings : rings + (size_t)nstreams * kR;
-        scatter_rings_kernel<<<nstreams, 128, 0, s>>>(ctx->st, first, nstreams, res, words,
-                                                      ctx->weyl_on ? 0x9E3779B9u : 0u);
-        e = cudaGetLastError();
+    cudaError_t e;
+    if (gf2_jump_in_place(ctx->device, nstreams, words)) {
+        if (xg_status g = ctx->ensure_jump_ws(wbytes)) return g;
+        e = gf2_jump_windows(ctx->device, (int)ctx->param_set, words,
+                             JumpWindows{ctx->st.win + (size_t)first * kWin, ctx->st.pend + first, 1}, nstreams,
+                             static_cast<uint8_t*>(ctx->jump_ws), ctx->sm_count, s, &st);
+        if (e == cudaSuccess) {
+            finish_jump_kernel<<<(nstreams + 255) / 256, 256, 0, s>>>(ctx->st, first, nstreams, words, omega);
+            e = cudaGetLastError();
+        }
+    } else {
+        // workspace kept in the context (grow-only): rings[0, n) hold the
+        // states, rings[n, 2n) receive the results; index lists (stream ids for
+        // the gather, then 0 .. 2n-1); the jump's own work area
+        const size_t rings_bytes = (size_t)2 * nstreams * kR * 4;
+        const size_t ids_off = rings_bytes;
+        const size_t work_off = (ids_off + (size_t)3 * nstreams * 4 + 255) / 256 * 256;
+        if (xg_status g = ctx->ensure_jump_ws(work_off + wbytes)) return g;
+        char* ws = static_cast<char*>(ctx->jump_ws);
+        uint32_t* rings = reinterpret_cast<uint32_t*>(ws);
+        uint32_t* ids = reinterpret_cast<uint32_t*>(ws + ids_off);
+        const uint32_t* lo_idx = ids + nstreams;  // 0 .. 2n-1
+        e = launch_jump_index(ids, nstreams, first, s);
+        if (e == cudaSuccess) e = launch_gather_rings(ctx->st, ids, nstreams, rings, nullptr, nullptr, 0, 0, s);
+        bool hi = false;
+        if (e == cudaSuccess)
+            e = gf2_jump_states(ctx->device, (int)ctx->param_set, words, rings, nstreams, lo_idx,
+                                reinterpret_cast<uint8_t*>(ws + work_off), ctx->sm_count, s, &st, &hi);
+        if (e == cudaSuccess) {
+            const uint32_t* res = hi ? rings + (size_t)nstreams * kR : rings;
+            scatter_rings_kernel<<<nstreams, 128, 0, s>>>(ctx->st, first, nstreams, res, words, omega);
+            e = cudaGetLastError();
+        }
     }
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     const size_t sbytes = gf2_apply_scratch(ctx->device, nstreams);

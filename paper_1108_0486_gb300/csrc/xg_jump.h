@@ -70,11 +70,26 @@ cudaError_t gf2_apply(int device, int family, int k, uint32_t* rings, uint32_t n
 // than 64 states the powers are multiplied first and the product applied once.
 // work: gf2_jump_work_bytes(device, n, words) bytes of device memory,
 // 256-byte aligned (the tensor-core operand, and the product's work area when
-// the powers are multiplied first).
+// the powers are multiplied first).  Not for jumps that gf2_jump_in_place takes.
 size_t gf2_jump_work_bytes(int device, uint32_t n, uint64_t words);
 cudaError_t gf2_jump_states(int device, int family, uint64_t words, uint32_t* rings, uint32_t n,
                             const uint32_t* d_idx, uint8_t* work, int sm_count, cudaStream_t s, xg_status* st,
                             bool* result_hi);
+
+// Whether a jump applies one matrix (a power, or the product of several) on
+// the tensor cores; then gf2_jump_windows reads the rings of n consecutive
+// streams in their windows and writes them back there, without pending words:
+// for 16384 streams it saves the copies of all rings out of the windows and
+// back (25 of 229 us).  The caller resets pend and advances the Weyl words.
+// work as for gf2_jump_states.
+struct JumpWindows {
+    uint32_t* win;    // the first stream's window, kWin 32-bit words each
+    uint32_t* pend;   // of the first stream
+    uint32_t word;    // 32-bit words per generator word
+};
+bool gf2_jump_in_place(int device, uint32_t n, uint64_t words);
+cudaError_t gf2_jump_windows(int device, int family, uint64_t words, const JumpWindows& win, uint32_t n, uint8_t* work,
+                             int sm_count, cudaStream_t s, xg_status* st);
 
 // ids[i] = first + i for i < n, then ids[n + j] = j for j < 2n (3n entries).
 cudaError_t launch_jump_index(uint32_t* ids, uint32_t n, uint32_t first, cudaStream_t s);

@@ -606,6 +606,24 @@ __global__ void __launch_bounds__(64) scatter_rings_kernel(State st, uint32_t fi
     }
 }
 
+// The same where the windows hold the jumped rings already.
+__global__ void finish_jump_kernel(State st, uint32_t first, uint32_t n, uint64_t jump, uint64_t omega)
+{
+    const uint32_t k = blockIdx.x * blockDim.x + threadIdx.x;
+    if (k >= n) return;
+    const uint32_t s = first + k;
+    st.weyl[s] += jump * omega;
+    st.pend[s] = 0;
+    st.pos[s] += jump;
+}
+
+cudaError_t launch_finish_jump(const State& st, uint32_t first, uint32_t n, uint64_t jump, uint64_t omega, cudaStream_t s)
+{
+    if (n == 0) return cudaSuccess;
+    finish_jump_kernel<<<(n + 255) / 256, 256, 0, s>>>(st, first, n, jump, omega);
+    return cudaGetLastError();
+}
+
 __global__ void __launch_bounds__(64) substream_scatter_kernel(State st, uint32_t first, uint32_t n,
                                                                const uint64_t* __restrict__ rings,
                                                                const uint64_t* __restrict__ w0, int q,

@@ -379,3 +379,30 @@ def test_64bit_call_in_a_captured_graph_is_not_cut():
             torch.cuda.synchronize()
             w = O.streams64(W.seeds(1, streams), (k + 1) * n)[0, k * n:]
             assert np.array_equal(out[streams - 1].cpu().numpy().view(np.uint64), w)
+
+
+@pytest.mark.parametrize("family", [0, 1, 64])
+@pytest.mark.parametrize("words", [1 << 21, (1 << 33) + (1 << 9) + 5, 0x9E3779B97F4A7C15])
+def test_jump_in_the_windows(family, words, monkeypatch):
+    """Jumps of 192 and more consecutive streams in the middle of a context, in
+    place on the tensor cores, after draws that leave pending words: the
+    states, positions and next words of the table kernel's jump, and the other
+    streams untouched."""
+    from paper_1108_0486_gb300 import Streams, Streams64
+    n = 500
+    for first, count in ((0, 500), (7, 192), (3, 241)):
+        got = []
+        for tc in ("1", "0"):
+            monkeypatch.setenv("XG_JUMP_TENSOR_CORES", tc)
+            seeds = W.seeds(n)
+            with (Streams64(n, seeds=seeds) if family == 64 else Streams(n, param_set=family, seeds=seeds)) as st:
+                draw = st.u64 if family == 64 else st.u32
+                draw(77)
+                st.jump(words, first=first, count=count)
+                rows = [draw(45), draw(200)]
+                if family != 64:
+                    c = st.checkpoint()
+                    rows += [torch.from_numpy(c[k].view(np.int64 if k == "pos" else np.int32)) for k in ("rings", "weyl", "pos")]
+                got.append([r.cpu() for r in rows])
+        for x, y in zip(*got):
+            assert torch.equal(x, y)
