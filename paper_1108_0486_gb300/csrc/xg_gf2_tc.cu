@@ -383,6 +383,8 @@ __global__ void __launch_bounds__(256) expand_matrix_kernel(const uint32_t* __re
                                                             uint8_t* __restrict__ A)
 {
     const uint32_t lane = threadIdx.x & 31u, kw = blockIdx.x * 8 + (threadIdx.x >> 5), w = blockIdx.y;
+    cudaTriggerProgrammaticLaunchCompletion();
+    cudaGridDependencySynchronize();
     const uint32_t word = cols[(size_t)(32 * kw + lane) * kGf2Words + w];
     uint32_t row = 0;
 #pragma unroll
@@ -400,16 +402,19 @@ __global__ void __launch_bounds__(256) expand_states_kernel(TcStates in, uint32_
 {
     const uint64_t t = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
     cudaTriggerProgrammaticLaunchCompletion();
-    cudaGridDependencySynchronize();
-    if (t >= (uint64_t)n_pad * kGf2Words) return;
-    const uint32_t s = (uint32_t)(t / kGf2Words), w = (uint32_t)(t % kGf2Words);
-    uint32_t x = 0;
-    if (s < n) {
-        const uint32_t* ring = in.base + (size_t)(in.list ? in.list[s] : s) * in.stride;
-        if (in.pend) ring -= in.pend[s] * in.word;
-        x = ring[w];
+    if (!in.settled) cudaGridDependencySynchronize();
+    if (t < (uint64_t)n_pad * kGf2Words) {
+        const uint32_t s = (uint32_t)(t / kGf2Words), w = (uint32_t)(t % kGf2Words);
+        uint32_t x = 0;
+        if (s < n) {
+            const uint32_t* ring = in.base + (size_t)(in.list ? in.list[s] : s) * in.stride;
+            if (in.pend) ring -= in.pend[s] * in.word;
+            x = ring[w];
+        }
+        *reinterpret_cast<uint4*>(B + (size_t)s * kRowBytes + 16 * w) = spread32(x);
     }
-    *reinterpret_cast<uint4*>(B + (size_t)s * kRowBytes + 16 * w) = spread32(x);
+    // the product waits for this kernel only: it ends after the one before it
+    if (in.settled) cudaGridDependencySynchronize();
 }
 
 // ---- host side -------------------------------------------------------------
@@ -485,10 +490,10 @@ uint32_t gf2_tc_padded(uint32_t n) { return (n + kBN - 1) / kBN * kBN; }
 
 size_t gf2_tc_scratch_bytes(uint32_t n) { return (size_t)gf2_tc_padded(n) * kRowBytes; }
 
-cudaError_t gf2_tc_expand_matrix(const uint64_t* C, uint8_t* A, cudaStream_t s)
+cudaError_t gf2_tc_expand_matrix(const uint64_t* C, uint8_t* A, cudaStream_t s, bool dependent)
 {
-    expand_matrix_kernel<<<dim3(kGf2Words / 8, kGf2Words), 256, 0, s>>>(reinterpret_cast<const uint32_t*>(C), A);
-    return cudaGetLastError();
+    return launch_dependent(dependent, dim3(kGf2Words / 8, kGf2Words), dim3(256), s, expand_matrix_kernel,
+                            reinterpret_cast<const uint32_t*>(C), A);
 }
 
 cudaError_t gf2_tc_apply(int device, const uint8_t* const* A, int n_mats, const TcStates& in, uint32_t n, uint32_t* out,

@@ -28,20 +28,24 @@ constexpr size_t kGf2TcMatrixBytes = (size_t)kGf2Bits * kGf2Bits / 2;
 
 // A (4096 x 2048 bytes, 8 MiB) = C in FP4 E2M1, row i over input bits k, from
 // C in column form (column k = the 128 ring words of C e_k).
-cudaError_t gf2_tc_expand_matrix(const uint64_t* C, uint8_t* A, cudaStream_t s);
+// dependent: as in launch_gf2_apply_pairs.
+cudaError_t gf2_tc_expand_matrix(const uint64_t* C, uint8_t* A, cudaStream_t s, bool dependent = false);
 
 // Most matrices applied by one launch.
 constexpr int kGf2TcMaxMats = 7;
 
 // The states that are read: state i is the 128 words at base + list[i] stride
 // (list null: i), or, with pend, at base + i stride - pend[i] word (the ring in
-// a stream's window, base its position without pending words).
+// a stream's window, base its position without pending words).  settled: no
+// kernel since the last ordinary launch writes them, so that a dependent launch
+// may read them beside the kernels before it.
 struct TcStates {
     const uint32_t* base;
     uint32_t stride;
     const uint32_t* list;
     const uint32_t* pend;
     uint32_t word;
+    bool settled = false;
 };
 
 // out[dst[j n + i] out_stride ..] = C_j (state i) for i < n and j < n_mats (<=

@@ -67,6 +67,8 @@ __global__ void __launch_bounds__(128) continue_kernel(const typename F::Word* _
     static_assert(S <= 128 && R <= 128 && R - 1 - S < S, "one word of a step per thread");
     __shared__ typename F::Word x[2 * R];
     const int t = threadIdx.x;
+    cudaTriggerProgrammaticLaunchCompletion();
+    cudaGridDependencySynchronize();
     if (t < R) x[t] = states[(size_t)blockIdx.x * R + t];
     __syncthreads();
     for (int k = R; k < 2 * R; k += S) {
@@ -86,6 +88,8 @@ __global__ void __launch_bounds__(256) columns_kernel(const typename F::Word* __
     const uint32_t id = blockIdx.x * 256 + threadIdx.x;   // grid covers kBits * R exactly
     const int j = (int)(id / R), k = (int)(id % R);
     const int b = j % F::BITS, i = R - 1 - j / F::BITS;
+    cudaTriggerProgrammaticLaunchCompletion();
+    cudaGridDependencySynchronize();
     Word v = seq[(size_t)b * 2 * R + i + k];
     if (i >= S)
         for (Word u = F::lag_s(Word(1) << b); u; u &= u - 1) {
@@ -132,23 +136,24 @@ __global__ void __launch_bounds__(128) step_columns_kernel(uint32_t* __restrict_
 // kernel before it (programmatic dependent launch).
 struct MatSet {
     const uint32_t* C[kMaxMats];
+    const uint32_t* in[kMaxMats];   // the states that each one is applied to
 };
 template <int kPairVecs>
-// rings and out may be the same array (sources are read, distinct destinations
-// are written), so neither is declared __restrict__.
-__global__ void __launch_bounds__(128) gf2_apply_pairs_kernel(MatSet mats, const uint32_t* rings,
-                                                              const uint32_t* __restrict__ src,
+// The states and out may be the same array (sources are read, distinct
+// destinations are written), so neither is declared __restrict__.
+__global__ void __launch_bounds__(128) gf2_apply_pairs_kernel(MatSet mats, const uint32_t* __restrict__ src,
                                                               const uint32_t* __restrict__ dst, uint32_t n,
                                                               uint32_t* out, int cols, bool early)
 {
-    __shared__ uint32_t vbits[kPairVecs][kR];
+    __shared__ uint32_t vbits[kPairVecs * kR];   // this block's words of its states
     __shared__ uint32_t tbl[kPairVecs > 4 ? 16 : 1][kR];
     const uint32_t* __restrict__ C = mats.C[blockIdx.z];
+    const uint32_t* rings = mats.in[blockIdx.z];
     if (dst) dst += (size_t)blockIdx.z * n;
     const int t = threadIdx.x;
     const uint32_t base = blockIdx.x * kPairVecs;
     const int nv = (int)umin((uint32_t)kPairVecs, n - base);
-    const int w0 = blockIdx.y * (cols / 32), w1 = w0 + cols / 32;
+    const int nw = cols / 32, w0 = blockIdx.y * nw;
     uint32_t col[32];   // 32 columns of one input word
     auto load_columns = [&](int w) {
         const uint32_t* colw = C + (size_t)w * 32 * kR + t;
@@ -158,16 +163,18 @@ __global__ void __launch_bounds__(128) gf2_apply_pairs_kernel(MatSet mats, const
     if (early) cudaTriggerProgrammaticLaunchCompletion();
     load_columns(w0);
     cudaGridDependencySynchronize();
-    for (int v = 0; v < kPairVecs; ++v)
-        vbits[v][t] = v < nv ? rings[(size_t)(src ? src[base + v] : base + v) * kR + t] : 0u;
+    for (int k = t; k < kPairVecs * nw; k += 128) {
+        const int v = k / nw;
+        vbits[k] = v < nv ? rings[(size_t)(src ? src[base + v] : base + v) * kR + w0 + k % nw] : 0u;
+    }
     __syncthreads();
     uint32_t acc[kPairVecs];
 #pragma unroll
     for (int v = 0; v < kPairVecs; ++v) acc[v] = 0;
-    for (int w = w0;;) {
+    for (int w = 0;;) {
         uint32_t bw[kPairVecs];
 #pragma unroll
-        for (int v = 0; v < kPairVecs; ++v) bw[v] = vbits[v][w];
+        for (int v = 0; v < kPairVecs; ++v) bw[v] = vbits[v * nw + w];
         if constexpr (kPairVecs <= 4) {
 #pragma unroll
             for (int b = 0; b < 32; ++b)
@@ -186,8 +193,8 @@ __global__ void __launch_bounds__(128) gf2_apply_pairs_kernel(MatSet mats, const
                 for (int v = 0; v < kPairVecs; ++v) acc[v] ^= tbl[(bw[v] >> (4 * g)) & 15u][t];
             }
         }
-        if (++w == w1) break;
-        load_columns(w);
+        if (++w == nw) break;
+        load_columns(w0 + w);
     }
 #pragma unroll
     for (int v = 0; v < kPairVecs; ++v)
@@ -270,25 +277,70 @@ __global__ void substream_scatter_kernel(State st, uint32_t first, uint32_t n, c
 
 // ---------------------------------------------------------------------------
 
+template <int NV>
+static cudaError_t launch_pairs(const MatSet& mats, int n_mats, uint32_t* out, uint32_t n, const uint32_t* d_src,
+                                const uint32_t* d_dst, int sm_count, cudaStream_t s, bool dependent, bool early)
+{
+    const uint32_t groups = (n + NV - 1) / NV;
+    // enough blocks for about 8 per SM, splitting the 4096 columns if needed
+    // (down to one 32-column input word per block: with few states the
+    // matrix read is the cost, spread over up to 128 blocks)
+    int chunks = 1;
+    while (chunks < kBits / 32 && (uint64_t)groups * chunks * n_mats < (uint64_t)8 * sm_count) chunks *= 2;
+    return launch_dependent(dependent, dim3(groups, chunks, n_mats), dim3(128), s, gf2_apply_pairs_kernel<NV>, mats,
+                            d_src, d_dst, n, out, kBits / chunks, early);
+}
+
+// Matrix j applied to the states in[j] (null lists: state i to state j n + i).
+static cudaError_t apply_sets(const uint64_t* const* C, int n_mats, const uint32_t* const* in, uint32_t* out, uint32_t n,
+                              const uint32_t* d_src, const uint32_t* d_dst, int sm_count, cudaStream_t s, bool dependent,
+                              bool early)
+{
+    if (n == 0 || n_mats == 0) return cudaSuccess;
+    if (n_mats > kMaxMats) return cudaErrorInvalidValue;
+    MatSet mats{};
+    for (int j = 0; j < n_mats; ++j) {
+        mats.C[j] = reinterpret_cast<const uint32_t*>(C[j]);
+        mats.in[j] = in[j];
+    }
+    if (n >= 4 * 48) return launch_pairs<48>(mats, n_mats, out, n, d_src, d_dst, sm_count, s, dependent, early);
+    if (n > 4) return launch_pairs<16>(mats, n_mats, out, n, d_src, d_dst, sm_count, s, dependent, early);
+    return launch_pairs<4>(mats, n_mats, out, n, d_src, d_dst, sm_count, s, dependent, early);
+}
+
+cudaError_t launch_gf2_apply_multi(const uint64_t* const* C, int n_mats, const uint32_t* in, uint32_t* out, uint32_t n,
+                                   const uint32_t* d_src, const uint32_t* d_dst, int sm_count, cudaStream_t s,
+                                   bool dependent, bool early)
+{
+    const uint32_t* all[kMaxMats];
+    for (const uint32_t*& p : all) p = in;
+    return apply_sets(C, n_mats, all, out, n, d_src, d_dst, sm_count, s, dependent, early);
+}
+
 // C = M^J from the newest word's columns Y_b = M^J E_b (states, consecutive
 // rings); seq: 2 * kBits * kMaxNewest / 8 bytes of scratch.
 constexpr size_t kSeqBytes = (size_t)2 * kBits / 8 * kMaxNewest;
 
 template <class F>
-static cudaError_t build_columns(const uint32_t* states, uint8_t* seq, uint64_t* C, cudaStream_t s)
+static cudaError_t build_columns(const uint32_t* states, uint8_t* seq, uint64_t* C, cudaStream_t s, bool dependent)
 {
     using Word = typename F::Word;
     Word* sq = reinterpret_cast<Word*>(seq);
-    continue_kernel<F><<<F::BITS, 128, 0, s>>>(reinterpret_cast<const Word*>(states), sq);
-    columns_kernel<F><<<kBits * F::R / 256, 256, 0, s>>>(sq, reinterpret_cast<Word*>(C));
-    return cudaGetLastError();
+    cudaError_t e = launch_dependent(dependent, dim3(F::BITS), dim3(128), s, continue_kernel<F>,
+                                     reinterpret_cast<const Word*>(states), sq);
+    if (e == cudaSuccess)
+        e = launch_dependent(true, dim3(kBits * F::R / 256), dim3(256), s, columns_kernel<F>,
+                             static_cast<const Word*>(sq), reinterpret_cast<Word*>(C));
+    return e;
 }
 
-static cudaError_t launch_build_columns(int family, const uint32_t* states, uint8_t* seq, uint64_t* C, cudaStream_t s)
+// dependent: as in launch_gf2_apply_pairs.
+static cudaError_t launch_build_columns(int family, const uint32_t* states, uint8_t* seq, uint64_t* C, cudaStream_t s,
+                                        bool dependent = false)
 {
-    if (family == kJumpSetW64) return build_columns<Ring64>(states, seq, C, s);
-    if (family == 1) return build_columns<Ring32<ParamsPaper>>(states, seq, C, s);
-    return build_columns<Ring32<ParamsDefault>>(states, seq, C, s);
+    if (family == kJumpSetW64) return build_columns<Ring64>(states, seq, C, s, dependent);
+    if (family == 1) return build_columns<Ring32<ParamsPaper>>(states, seq, C, s, dependent);
+    return build_columns<Ring32<ParamsDefault>>(states, seq, C, s, dependent);
 }
 
 // Columns of the newest ring word: the last ones of a matrix in column form.
@@ -484,19 +536,23 @@ cudaError_t gf2_apply(int device, int family, int k, uint32_t* rings, uint32_t n
     return e;
 }
 
-// With several set bits and more than kMaxNewest states the powers are
-// multiplied first.  Both sides of the line cost one application of few
-// states per bit; above it the states themselves are touched once.
+// With several set bits the powers are multiplied first: one chain of
+// applications to 32 (64) states, or two at half the length, instead of one to
+// all states.  From 2 bits on for more than kMaxNewest states; fewer states
+// cost hardly more than the columns do, so there the product has to save
+// launches: us per jump power by power / by the product, 16 streams 4 bits 60 /
+// 54, 8 bits 101 / 67, 1 stream 4 bits 44 / 50, 8 bits 68 / 60.
 static bool jump_combines(uint64_t words, uint32_t n)
 {
-    return __builtin_popcountll(words) >= 2 && n > (uint32_t)kMaxNewest;
+    const int bits = __builtin_popcountll(words);
+    return bits >= (n > (uint32_t)kMaxNewest ? 2 : n > 4 ? 4 : 7);
 }
 
 // Work area of a product: one group of newest columns per set bit, the
-// sequences, the product in column form.
+// sequences, the product and one factor in column form.
 static size_t product_bytes(uint64_t words)
 {
-    return (size_t)__builtin_popcountll(words) * kMaxNewest * kR * 4 + kSeqBytes + (size_t)kBits * kR * 4;
+    return (size_t)__builtin_popcountll(words) * kMaxNewest * kR * 4 + kSeqBytes + (size_t)2 * kBits * kR * 4;
 }
 
 size_t gf2_jump_work_bytes(int device, uint32_t n, uint64_t words)
@@ -514,34 +570,56 @@ size_t gf2_jump_work_bytes(int device, uint32_t n, uint64_t words)
 // its newest columns by one application per further set bit to 32 (64) states,
 // then all columns from them.  For 16384 streams and 8 set bits this took the
 // jump from 0.615 ms (seven tensor-core products of 4096 columns each) to
-// 0.311 ms.  The applications are one dependent chain, 5.6 us each: the launch
-// that waits for the one before it, the states, 8 rounds of tables.
+// 0.311 ms.  The applications are one dependent chain, 3 us each (the launch
+// that waits for the one before it, the states, 8 rounds of tables), so from
+// kTwoChains bits on the powers form two chains that share their launches; one
+// of them then gets all its columns (5 us) and is applied to the other.  300
+// streams, 8 / 16 / 30 bits: 78 / 113 / 180 -> 66 / 91 / 144 us.
+// Last launch: a dependent one may follow.
+constexpr int kTwoChains = 6;
+
 static cudaError_t power_product(int device, int family, uint64_t words, uint8_t* w, int sm_count, cudaStream_t s,
                                  const uint64_t** product, xg_status* st)
 {
-    const int nb = newest_columns(family);
+    const uint32_t nb = (uint32_t)newest_columns(family);
     const size_t group = (size_t)nb * kR;   // 32-bit words of one group of columns
-    const int bits = __builtin_popcountll(words);
     uint32_t* cols = reinterpret_cast<uint32_t*>(w);
+    const int bits = __builtin_popcountll(words);
     uint8_t* seq = w + (size_t)bits * kMaxNewest * kR * 4;
     uint64_t* prod = reinterpret_cast<uint64_t*>(seq + kSeqBytes);
-    cudaError_t e = cudaMemsetAsync(cols, 0, (size_t)(bits - 1) * group * 4, s);
-    const uint32_t* have = nullptr;   // the newest columns of the product so far
-    int done = 0;
-    for (int k = 0; k < 64 && e == cudaSuccess; ++k) {
+    uint64_t* factor = prod + (size_t)kBits * kWords64;
+    const uint64_t* C[64];
+    int n = 0;
+    for (int k = 0; k < 64; ++k) {
         if (!((words >> k) & 1)) continue;
-        const uint64_t* C = jump_matrix(device, family, k, s, st);
-        if (!C) return cudaErrorMemoryAllocation;
-        if (!have) {
-            have = newest_of(C, family);
-            continue;
-        }
-        uint32_t* to = cols + done * group;
-        e = launch_gf2_apply_pairs(C, have, to, (uint32_t)nb, nullptr, nullptr, sm_count, s, done > 0);
-        have = to;
-        ++done;
+        C[n] = jump_matrix(device, family, k, s, st);
+        if (!C[n++]) return cudaErrorMemoryAllocation;
     }
-    if (e == cudaSuccess) e = launch_build_columns(family, have, seq, prod, s);
+    cudaError_t e = cudaMemsetAsync(cols, 0, (size_t)(bits - 1) * group * 4, s);
+    // chain c starts with the newest columns of its first power
+    const int chains = bits >= kTwoChains ? 2 : 1;
+    const int len[2] = {(bits + chains - 1) / chains, chains == 2 ? bits / 2 : 0};
+    const uint64_t* const* power[2] = {C, C + len[0]};
+    const uint32_t* have[2] = {newest_of(C[0], family), chains == 2 ? newest_of(C[len[0]], family) : nullptr};
+    uint32_t* to = cols;
+    bool dependent = false;   // the launch before is one of this chain's
+    for (int i = 1; i < len[0] && e == cudaSuccess; ++i) {
+        const int now = i < len[1] ? 2 : 1;
+        const uint64_t* m[2] = {power[0][i], now == 2 ? power[1][i] : nullptr};
+        e = apply_sets(m, now, have, to, nb, nullptr, nullptr, sm_count, s, dependent, true);
+        dependent = true;
+        for (int c = 0; c < now; ++c, to += group) have[c] = to;
+    }
+    if (chains == 2) {
+        if (e == cudaSuccess) e = launch_build_columns(family, have[1], seq, factor, s, dependent);
+        // an ordinary launch: a dependent one would read the factor's first
+        // columns before the kernel that writes them has ended
+        const uint64_t* f = factor;
+        if (e == cudaSuccess) e = apply_sets(&f, 1, have, to, nb, nullptr, nullptr, sm_count, s, false, true);
+        dependent = true;
+        have[0] = to;
+    }
+    if (e == cudaSuccess) e = launch_build_columns(family, have[0], seq, prod, s, dependent);
     *product = prod;
     return e;
 }
@@ -564,12 +642,14 @@ cudaError_t gf2_jump_windows(int device, int family, uint64_t words, const JumpW
         uint8_t* abuf = w + product_bytes(words);
         const uint64_t* P = nullptr;
         cudaError_t e = power_product(device, family, words, w, sm_count, s, &P, st);
-        if (e == cudaSuccess) e = gf2_tc_expand_matrix(P, abuf, s);
+        if (e == cudaSuccess) e = gf2_tc_expand_matrix(P, abuf, s, true);
         if (e != cudaSuccess) return e;
         A = abuf;
     }
+    // the windows were last written before the product's first launch
     uint32_t* ring = win.win + kRingBase;
-    return gf2_tc_apply(device, &A, 1, TcStates{ring, kWin, nullptr, win.pend, win.word}, n, ring, kWin, nullptr, work, s);
+    return gf2_tc_apply(device, &A, 1, TcStates{ring, kWin, nullptr, win.pend, win.word, true}, n, ring, kWin, nullptr,
+                        work, s, __builtin_popcountll(words) > 1);
 }
 
 cudaError_t gf2_jump_states(int device, int family, uint64_t words, uint32_t* rings, uint32_t n,
@@ -614,34 +694,6 @@ cudaError_t launch_jump_index(uint32_t* ids, uint32_t n, uint32_t first, cudaStr
     const uint64_t total = (uint64_t)3 * n;
     jump_index_kernel<<<(unsigned)((total + 255) / 256), 256, 0, s>>>(ids, n, first);
     return cudaGetLastError();
-}
-
-template <int NV>
-static cudaError_t launch_pairs(const MatSet& mats, int n_mats, const uint32_t* in, uint32_t* out, uint32_t n,
-                                const uint32_t* d_src, const uint32_t* d_dst, int sm_count, cudaStream_t s,
-                                bool dependent, bool early)
-{
-    const uint32_t groups = (n + NV - 1) / NV;
-    // enough blocks for about 8 per SM, splitting the 4096 columns if needed
-    // (down to one 32-column input word per block: with few states the
-    // matrix read is the cost, spread over up to 128 blocks)
-    int chunks = 1;
-    while (chunks < kBits / 32 && (uint64_t)groups * chunks * n_mats < (uint64_t)8 * sm_count) chunks *= 2;
-    return launch_dependent(dependent, dim3(groups, chunks, n_mats), dim3(128), s, gf2_apply_pairs_kernel<NV>, mats,
-                            in, d_src, d_dst, n, out, kBits / chunks, early);
-}
-
-cudaError_t launch_gf2_apply_multi(const uint64_t* const* C, int n_mats, const uint32_t* in, uint32_t* out, uint32_t n,
-                                   const uint32_t* d_src, const uint32_t* d_dst, int sm_count, cudaStream_t s,
-                                   bool dependent, bool early)
-{
-    if (n == 0 || n_mats == 0) return cudaSuccess;
-    if (n_mats > kMaxMats) return cudaErrorInvalidValue;
-    MatSet mats{};
-    for (int j = 0; j < n_mats; ++j) mats.C[j] = reinterpret_cast<const uint32_t*>(C[j]);
-    if (n >= 4 * 48) return launch_pairs<48>(mats, n_mats, in, out, n, d_src, d_dst, sm_count, s, dependent, early);
-    if (n > 4) return launch_pairs<16>(mats, n_mats, in, out, n, d_src, d_dst, sm_count, s, dependent, early);
-    return launch_pairs<4>(mats, n_mats, in, out, n, d_src, d_dst, sm_count, s, dependent, early);
 }
 
 cudaError_t launch_gf2_apply_pairs(const uint64_t* C, const uint32_t* in, uint32_t* out, uint32_t n,

@@ -406,3 +406,31 @@ def test_jump_in_the_windows(family, words, monkeypatch):
                 got.append([r.cpu() for r in rows])
         for x, y in zip(*got):
             assert torch.equal(x, y)
+
+
+@pytest.mark.parametrize("family", [0, 1, 64])
+@pytest.mark.parametrize("bits", [2, 5, 6, 7, 9, 10, 11, 33])
+def test_jump_by_the_number_of_set_bits(family, bits):
+    """Jumps whose powers form one or two chains, few streams on both sides of
+    the number of bits from which their powers are multiplied first, and many:
+    the same power after power."""
+    from paper_1108_0486_gb300 import Streams, Streams64
+    rng = np.random.default_rng(bits)
+    at = sorted(rng.choice(45, bits, replace=False).tolist())
+    words = sum(1 << k for k in at)
+
+    def make(n):
+        seeds = W.seeds(n)
+        return Streams64(n, seeds=seeds) if family == 64 else Streams(n, param_set=family, seeds=seeds)
+
+    def draw(st):
+        return (st.u64(70) if family == 64 else st.u32(140)).cpu()
+
+    with make(3) as st:
+        for k in at:
+            st.jump(1 << k)
+        ref = draw(st)
+    for n in (3, 70, 200):
+        with make(n) as st:
+            st.jump(words)
+            assert torch.equal(draw(st)[:3], ref)
