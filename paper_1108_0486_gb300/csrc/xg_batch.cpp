@@ -319,38 +319,60 @@ xg_status BatchLauncher::reserve_jump(uint32_t pieces, uint32_t pairs)
 }
 
 // Start rings of the pieces.  Piece 0 of a call gets the stream's ring
-// (gather).  Then, doubling: step b gives every piece m in [2^b, 2^(b+1)) the
-// ring of piece m - 2^b advanced by 2^b pieces, i.e. C_{q+b} applied to it
-// (q = log2 of the piece length).  Each piece costs one application and a
-// call cut into K pieces needs ceil(log2 K) steps.
+// (gather).  Then in steps: step k gives every piece m + j 8^k, m < 8^k and
+// j = 1 .. 7, the ring of piece m advanced by j 8^k pieces, with the matrices
+// M^(j 8^k 2^q) (q = log2 of the piece length).  One launch per step applies
+// all seven: the sources are listed by how many results they have, most
+// first, so that matrix j applies to a prefix of them.  256 requests of a
+// server burst took 6 doubling launches of 15 to 25 us each, a batch of 4096
+// calls five of 25 to 37 us.
 xg_status BatchLauncher::prologue(xg_ctx* c, cudaStream_t s)
 {
     const uint32_t P = (uint32_t)plan_.pieces.size();
     if (P == 0) return XG_OK;
-    // per step b: (src, dst) piece pairs; pieces of one call are consecutive.
-    // Count them per step first, then write the lists straight into staging.
-    uint32_t per_step[32] = {0};
+    constexpr int kSteps = 11;   // 8^11 > 2^32 pieces
+    constexpr uint32_t kMats = 7;
+    static_assert(kMats <= (uint32_t)kMaxMats && kMats <= (uint32_t)kGf2TcMaxMats, "matrices per launch");
+    uint32_t with[kSteps][kMats + 1] = {};   // sources with exactly d results
     int nsteps = 0;
-    for (uint32_t k = 0; k < P; ++k) {
-        const uint32_t m = plan_.piece_index[k];
-        if (m == 0) continue;
-        const int b = 31 - __builtin_clz(m);
-        ++per_step[b];
-        nsteps = std::max(nsteps, b + 1);
+    // f(step, piece, results, 8^step) for every source
+    auto for_sources = [&](auto&& f) {
+        for (uint32_t k0 = 0, k1; k0 < P; k0 = k1) {
+            k1 = k0 + 1;
+            while (k1 < P && plan_.piece_index[k1] != 0) ++k1;
+            const uint64_t K = k1 - k0;
+            int step = 0;
+            for (uint64_t have = 1; have < K; have *= 8, ++step)
+                for (uint64_t m = 0; m < have && m + have < K; ++m)
+                    f(step, k0 + (uint32_t)m, (uint32_t)std::min<uint64_t>(kMats, (K - 1 - m) / have), (uint32_t)have);
+            nsteps = std::max(nsteps, step);
+        }
+    };
+    size_t entries = 0;
+    for_sources([&](int step, uint32_t, uint32_t d, uint32_t) {
+        ++with[step][d];
+        entries += 1 + d;
+    });
+    uint32_t counts[kSteps][kMats] = {};   // sources with more than j results
+    bool use_tc[kSteps] = {};
+    uint32_t most = 0;                     // states of the largest step on the tensor cores
+    for (int k = 0; k < nsteps; ++k) {
+        uint32_t results = 0;
+        for (uint32_t j = kMats; j-- > 0;) {
+            counts[k][j] = with[k][j + 1] + (j + 1 < kMats ? counts[k][j + 1] : 0u);
+            results += counts[k][j];
+        }
+        use_tc[k] = gf2_use_tc(c->device, results);
+        if (use_tc[k]) most = std::max(most, counts[k][0]);
     }
-    size_t npairs = 0;
-    for (int b = 0; b < nsteps; ++b) npairs += per_step[b];
-    // device buffer: rings | weyls | gather streams | gather skips | pair lists
+    // device buffer: rings | weyls | gather streams | gather skips | lists
     const size_t off_rings = 0;
     const size_t off_weyl = off_rings + (size_t)P * 512;
     const size_t off_streams = (off_weyl + (size_t)P * 4 + 15) / 16 * 16;
     const size_t off_skip = (off_streams + (size_t)P * 4 + 15) / 16 * 16;
     const size_t off_lists = off_skip + (size_t)P * 8;
-    uint32_t most = 0;
-    for (int b = 0; b < nsteps; ++b) most = std::max(most, per_step[b]);
-    const size_t tc_bytes = gf2_apply_scratch(c->device, most);  // tensor-core operand, when used
-    const size_t off_tc = (off_lists + 2 * npairs * 4 + 16 + 255) / 256 * 256;
-    const size_t total = off_tc + tc_bytes;
+    const size_t off_tc = (off_lists + entries * 4 + 16 + 255) / 256 * 256;
+    const size_t total = off_tc + (most ? gf2_tc_scratch_bytes(most) : 0);
     if (total > jbytes_) {
         if (xg_status st = grow_jump(total + total / 2)) return st;
     }
@@ -360,39 +382,42 @@ xg_status BatchLauncher::prologue(xg_ctx* c, cudaStream_t s)
     // from the gather (m = 0) or a doubling step
     std::memcpy(hb + off_streams, plan_.piece_stream.data(), (size_t)P * 4);
     std::memcpy(hb + off_skip, plan_.piece_skip.data(), (size_t)P * 8);
-    size_t src_off[32], dst_off[32];
-    uint32_t* src_w[32];
-    uint32_t* dst_w[32];
-    size_t o = off_lists;
-    for (int b = 0; b < nsteps; ++b) {
-        src_off[b] = o;
-        src_w[b] = reinterpret_cast<uint32_t*>(hb + o);
-        o += (size_t)per_step[b] * 4;
-        dst_off[b] = o;
-        dst_w[b] = reinterpret_cast<uint32_t*>(hb + o);
-        o += (size_t)per_step[b] * 4;
+    // per step: its sources, then each matrix's destinations
+    uint32_t* const lists = reinterpret_cast<uint32_t*>(hb + off_lists);
+    size_t src_at[kSteps], dst_at[kSteps][kMats];
+    uint32_t next[kSteps][kMats + 1];   // the next source with d results
+    size_t o = 0;
+    for (int k = 0; k < nsteps; ++k) {
+        src_at[k] = o;
+        o += counts[k][0];
+        for (uint32_t j = 0; j < kMats; ++j) {
+            dst_at[k][j] = o;
+            o += counts[k][j];
+            next[k][j + 1] = j + 1 < kMats ? counts[k][j + 1] : 0u;
+        }
     }
-    for (uint32_t k = 0; k < P; ++k) {
-        const uint32_t m = plan_.piece_index[k];
-        if (m == 0) continue;
-        const int b = 31 - __builtin_clz(m);
-        *src_w[b]++ = k - (1u << b);
-        *dst_w[b]++ = k;
-    }
+    for_sources([&](int step, uint32_t piece, uint32_t d, uint32_t have) {
+        const uint32_t at = next[step][d]++;
+        lists[src_at[step] + at] = piece;
+        for (uint32_t j = 0; j < d; ++j) lists[dst_at[step][j] + at] = piece + (j + 1) * have;
+    });
     for (uint32_t k = 0; k < P; ++k) {
         plan_.pieces[k].ring = reinterpret_cast<const uint32_t*>(db + off_rings + (size_t)k * 512);
         plan_.pieces[k].weyl0 = reinterpret_cast<const uint32_t*>(db + off_weyl + (size_t)k * 4);
     }
     // matrices first (the first use builds them and synchronises)
-    const uint64_t* mats[32] = {nullptr};
-    for (int b = 0; b < nsteps; ++b) {
-        if (per_step[b] == 0) continue;
-        xg_status st = XG_OK;
-        mats[b] = jump_matrix(c->device, (int)c->param_set, plan_.split_log2 + (int)b, s, &st);
-        if (!mats[b]) return st;
-    }
-    if (cudaMemcpyAsync(db + off_streams, hb + off_streams, o - off_streams, cudaMemcpyHostToDevice, s) !=
-        cudaSuccess)
+    const uint64_t* mats[kSteps][kMats] = {};
+    const uint8_t* tc_mats[kSteps][kMats] = {};
+    for (int k = 0; k < nsteps; ++k)
+        for (uint32_t j = 0; j < kMats && counts[k][j]; ++j) {
+            xg_status st = XG_OK;
+            const int e = plan_.split_log2 + 3 * k;
+            if (use_tc[k]) tc_mats[k][j] = jump_matrix_tc(c->device, (int)c->param_set, (int)j + 1, e, s, &st);
+            else mats[k][j] = jump_matrix_multiple(c->device, (int)c->param_set, (int)j + 1, e, s, &st);
+            if (!tc_mats[k][j] && !mats[k][j]) return st;
+        }
+    if (cudaMemcpyAsync(db + off_streams, hb + off_streams, off_lists + o * 4 - off_streams, cudaMemcpyHostToDevice,
+                        s) != cudaSuccess)
         return XG_ECUDA;
     // piece 0 of each call gets its stream's ring, the others (nonzero skip)
     // a zero ring, into which their doubling step XORs
@@ -402,15 +427,20 @@ xg_status BatchLauncher::prologue(xg_ctx* c, cudaStream_t s)
                             reinterpret_cast<uint32_t*>(db + off_weyl), 1u, c->weyl_on ? 0x9E3779B9u : 0u,
                             s) != cudaSuccess)
         return XG_ECUDA;
-    uint8_t* tc_scratch = tc_bytes ? reinterpret_cast<uint8_t*>(db + off_tc) : nullptr;
-    for (int b = 0; b < nsteps; ++b) {
-        if (per_step[b] == 0) continue;
-        xg_status st = XG_OK;
-        if (gf2_apply(c->device, (int)c->param_set, plan_.split_log2 + b, reinterpret_cast<uint32_t*>(db + off_rings),
-                      per_step[b], reinterpret_cast<const uint32_t*>(db + src_off[b]),
-                      reinterpret_cast<const uint32_t*>(db + dst_off[b]), tc_scratch, c->sm_count, s,
-                      &st, true) != cudaSuccess)
-            return st != XG_OK ? st : XG_ECUDA;
+    uint32_t* rings = reinterpret_cast<uint32_t*>(db + off_rings);
+    const uint32_t* d_lists = reinterpret_cast<const uint32_t*>(db + off_lists);
+    for (int k = 0; k < nsteps; ++k) {
+        int n_mats = 0;
+        while (n_mats < (int)kMats && counts[k][n_mats]) ++n_mats;
+        const uint32_t *src = d_lists + src_at[k], *dst = d_lists + dst_at[k][0];
+        cudaError_t e;
+        if (use_tc[k])
+            e = gf2_tc_apply(c->device, tc_mats[k], n_mats, TcStates{rings, kGf2Words, src, nullptr, 0}, counts[k][0],
+                             rings, kGf2Words, dst, reinterpret_cast<uint8_t*>(db + off_tc), s, k > 0, counts[k]);
+        else
+            e = launch_gf2_apply_multi(mats[k], n_mats, rings, rings, counts[k][0], src, dst, c->sm_count, s, k > 0,
+                                       k + 1 < nsteps, counts[k]);
+        if (e != cudaSuccess) return XG_ECUDA;
     }
     return XG_OK;
 }

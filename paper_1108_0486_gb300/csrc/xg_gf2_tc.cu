@@ -192,11 +192,14 @@ __device__ __forceinline__ bool failed(const volatile int* flag) { return *flag 
 struct TcMaps {
     CUtensorMap a[kGf2TcMaxMats];
     CUtensorMap b;
+    uint32_t n[kGf2TcMaxMats];    // matrix j applies to the first n[j] states
+    uint32_t at[kGf2TcMaxMats];   // its destinations in the list
+    uint32_t end[kGf2TcMaxMats];  // tiles of the matrices up to j
 };
 
-// out[dst[j n + s]] = C_j x_s for the n states of the B operand (rows >= n of
-// B are zero padding) and j < n_mats.  Persistent: CTA b takes tiles b, b +
-// gridDim.x, ... of the n_mats x (4096 / kBM) x (n_pad / kBN) tiles, M fastest
+// out[dst[at_j + s]] = C_j x_s for the first n_j states of the B operand (rows
+// past them count for nothing).  Persistent: CTA b takes tiles b, b +
+// gridDim.x, ... of the matrices' (4096 / kBM) x (n_j / kBN) tiles, M fastest
 // (consecutive tiles share a B tile in L2).  A few hundred states fill a part
 // of the SMs with one matrix, and a launch costs as much as its first tile
 // (14 us, each further wave 4), so several matrices share one: 500 states by 7
@@ -204,8 +207,18 @@ struct TcMaps {
 // MMA issuer, warps 2-5 = epilogue (warp w reads TMEM lanes 32 (w mod 4) ..).
 // Two accumulators of kBN columns alternate, so that the epilogue of one
 // tile overlaps the MMAs of the next.
-__global__ void __launch_bounds__(kThreads, 1) gf2_tc_kernel(const __grid_constant__ TcMaps maps, uint32_t n_mats,
-                                                              uint32_t n, uint32_t n_tiles,
+// Matrix and state tile of tile t.
+struct TcTile {
+    uint32_t j, nt;
+};
+__device__ __forceinline__ TcTile tc_tile(const TcMaps& maps, uint32_t t)
+{
+    uint32_t j = 0, from = 0;
+    while (t >= maps.end[j]) from = maps.end[j++];
+    return TcTile{j, (t - from) / (uint32_t)(kGf2Bits / kBM)};
+}
+
+__global__ void __launch_bounds__(kThreads, 1) gf2_tc_kernel(const __grid_constant__ TcMaps maps, uint32_t total,
                                                               const uint32_t* __restrict__ dst, uint32_t* out,
                                                               uint32_t out_stride, uint32_t* status, uint32_t stall)
 {
@@ -222,7 +235,6 @@ __global__ void __launch_bounds__(kThreads, 1) gf2_tc_kernel(const __grid_consta
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     constexpr uint32_t kMTiles = kGf2Bits / kBM;
-    const uint32_t total = kMTiles * n_tiles * n_mats;
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < kStages; ++s) {
@@ -260,8 +272,9 @@ __global__ void __launch_bounds__(kThreads, 1) gf2_tc_kernel(const __grid_consta
     if (warp == 0) {
         if (lane == 0) {
             for (uint32_t t = blockIdx.x; t < total && !failed(&s_failed); t += gridDim.x) {
-                const int mt = (int)(t % kMTiles), nt = (int)(t / kMTiles % n_tiles);
-                const CUtensorMap* ma = &maps.a[t / kMTiles / n_tiles];
+                const TcTile tile = tc_tile(maps, t);
+                const int mt = (int)(t % kMTiles), nt = (int)tile.nt;
+                const CUtensorMap* ma = &maps.a[tile.j];
                 for (int kb = 0; kb < kKBlocks; ++kb, ++issued) {
                     const uint32_t s = issued % kStages, u = issued / kStages;
                     if (issued >= (uint32_t)kStages && !mbar_wait(&empty[s], (u & 1) ^ 1, global_ns() + kWaitLimitNs)) {
@@ -317,8 +330,9 @@ __global__ void __launch_bounds__(kThreads, 1) gf2_tc_kernel(const __grid_consta
             }
             tc_fence_after();
             if (failed(&s_failed)) break;
-            const uint32_t mt = t % kMTiles, nt = t / kMTiles % n_tiles;
-            const uint32_t* to = dst ? dst + (size_t)(t / kMTiles / n_tiles) * n : nullptr;
+            const TcTile tile = tc_tile(maps, t);
+            const uint32_t mt = t % kMTiles, nt = tile.nt, n = maps.n[tile.j];
+            const uint32_t* to = dst ? dst + maps.at[tile.j] : nullptr;
             const uint32_t word = mt * (kBM / 32) + q;  // ring word of these 32 bits
             static_assert(kBN % 16 == 0, "columns are read 16 at a time");
             for (int c = 0; c < kBN; c += 32) {
@@ -497,12 +511,22 @@ cudaError_t gf2_tc_expand_matrix(const uint64_t* C, uint8_t* A, cudaStream_t s, 
 }
 
 cudaError_t gf2_tc_apply(int device, const uint8_t* const* A, int n_mats, const TcStates& in, uint32_t n, uint32_t* out,
-                         uint32_t out_stride, const uint32_t* dst, uint8_t* scratch, cudaStream_t s, bool dependent)
+                         uint32_t out_stride, const uint32_t* dst, uint8_t* scratch, cudaStream_t s, bool dependent,
+                         const uint32_t* counts)
 {
     if (n == 0 || n_mats == 0) return cudaSuccess;
     if (n_mats < 0 || n_mats > kGf2TcMaxMats) return cudaErrorInvalidValue;
     const uint32_t n_pad = gf2_tc_padded(n);
     TcMaps maps{};
+    uint32_t at = 0, tiles = 0;
+    for (int j = 0; j < n_mats; ++j) {
+        maps.n[j] = counts ? counts[j] : n;
+        maps.at[j] = at;
+        at += maps.n[j];
+        tiles += gf2_tc_padded(maps.n[j]) / kBN * (kGf2Bits / kBM);
+        maps.end[j] = tiles;
+    }
+    if (tiles == 0) return cudaSuccess;
     {
         std::lock_guard<std::mutex> lk(g_mu);
         if (!init_locked()) return cudaErrorNotSupported;
@@ -519,11 +543,9 @@ cudaError_t gf2_tc_apply(int device, const uint8_t* const* A, int n_mats, const 
     cudaError_t e = launch_dependent(dependent, dim3((unsigned)((words + 255) / 256)), dim3(256), s,
                                      expand_states_kernel, in, n, n_pad, scratch);
     if (e != cudaSuccess) return e;
-    const uint32_t n_tiles = n_pad / kBN;
-    const uint64_t tiles = (uint64_t)(kGf2Bits / kBM) * n_tiles * n_mats;
     int sms = 0;
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess || sms <= 0) sms = 1;
-    const unsigned grid = (unsigned)std::min<uint64_t>(tiles, (uint64_t)sms);
+    const unsigned grid = (unsigned)std::min<uint32_t>(tiles, (uint32_t)sms);
     const char* stall = std::getenv("XG_TC_TEST_STALL");
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3(grid);
@@ -535,7 +557,7 @@ cudaError_t gf2_tc_apply(int device, const uint8_t* const* A, int n_mats, const 
     attr.val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = &attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, gf2_tc_kernel, maps, (uint32_t)n_mats, n, n_tiles, dst, out, out_stride, g_status_dev,
+    return cudaLaunchKernelEx(&cfg, gf2_tc_kernel, maps, tiles, dst, out, out_stride, g_status_dev,
                               (stall && stall[0] == '1') ? 1u : 0u);
 }
 

@@ -50,6 +50,9 @@ struct TcStates {
 
 // out[dst[j n + i] out_stride ..] = C_j (state i) for i < n and j < n_mats (<=
 // kGf2TcMaxMats; dst null: one matrix, i), with A[j] from gf2_tc_expand_matrix.
+// counts (host, n_mats entries, each <= n, not increasing): matrix j applies to
+// the first counts[j] states, and the destinations of the matrices follow one
+// another in dst.
 // All states are read before the first is written: out may overlap the states
 // with one matrix, else if no destination is a source.  kNoState destinations
 // are skipped.  scratch: gf2_tc_scratch_bytes(n) bytes, 16-byte aligned, reused
@@ -57,7 +60,7 @@ struct TcStates {
 // launch_gf2_apply_pairs.
 cudaError_t gf2_tc_apply(int device, const uint8_t* const* A, int n_mats, const TcStates& in, uint32_t n, uint32_t* out,
                          uint32_t out_stride, const uint32_t* dst, uint8_t* scratch, cudaStream_t s,
-                         bool dependent = false);
+                         bool dependent = false, const uint32_t* counts = nullptr);
 
 // True (and cleared) if a tensor-core launch gave up a wait since the last
 // call: its results are not valid.  Read after synchronising.

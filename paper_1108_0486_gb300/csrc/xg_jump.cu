@@ -137,21 +137,23 @@ __global__ void __launch_bounds__(128) step_columns_kernel(uint32_t* __restrict_
 struct MatSet {
     const uint32_t* C[kMaxMats];
     const uint32_t* in[kMaxMats];   // the states that each one is applied to
+    uint32_t n[kMaxMats];           // how many of them
+    uint32_t at[kMaxMats];          // its destinations in the list
 };
 template <int kPairVecs>
 // The states and out may be the same array (sources are read, distinct
 // destinations are written), so neither is declared __restrict__.
 __global__ void __launch_bounds__(128) gf2_apply_pairs_kernel(MatSet mats, const uint32_t* __restrict__ src,
-                                                              const uint32_t* __restrict__ dst, uint32_t n,
-                                                              uint32_t* out, int cols, bool early)
+                                                              const uint32_t* __restrict__ dst, uint32_t* out, int cols, bool early)
 {
     __shared__ uint32_t vbits[kPairVecs * kR];   // this block's words of its states
     __shared__ uint32_t tbl[kPairVecs > 4 ? 16 : 1][kR];
     const uint32_t* __restrict__ C = mats.C[blockIdx.z];
     const uint32_t* rings = mats.in[blockIdx.z];
-    if (dst) dst += (size_t)blockIdx.z * n;
+    const uint32_t n = mats.n[blockIdx.z];
     const int t = threadIdx.x;
     const uint32_t base = blockIdx.x * kPairVecs;
+    if (base >= n) return;   // fewer states than the first matrix has
     const int nv = (int)umin((uint32_t)kPairVecs, n - base);
     const int nw = cols / 32, w0 = blockIdx.y * nw;
     uint32_t col[32];   // 32 columns of one input word
@@ -199,7 +201,7 @@ __global__ void __launch_bounds__(128) gf2_apply_pairs_kernel(MatSet mats, const
 #pragma unroll
     for (int v = 0; v < kPairVecs; ++v)
         if (v < nv && acc[v]) {
-            const uint32_t d = dst ? dst[base + v] : blockIdx.z * n + base + v;
+            const uint32_t at = mats.at[blockIdx.z] + base + v, d = dst ? dst[at] : at;
             if (d != kNoState) atomicXor(&out[(size_t)d * kR + t], acc[v]);
         }
 }
@@ -288,20 +290,25 @@ static cudaError_t launch_pairs(const MatSet& mats, int n_mats, uint32_t* out, u
     int chunks = 1;
     while (chunks < kBits / 32 && (uint64_t)groups * chunks * n_mats < (uint64_t)8 * sm_count) chunks *= 2;
     return launch_dependent(dependent, dim3(groups, chunks, n_mats), dim3(128), s, gf2_apply_pairs_kernel<NV>, mats,
-                            d_src, d_dst, n, out, kBits / chunks, early);
+                            d_src, d_dst, out, kBits / chunks, early);
 }
 
-// Matrix j applied to the states in[j] (null lists: state i to state j n + i).
+// Matrix j applied to the states in[j] (null lists: state i to state j n + i;
+// counts: to the first counts[j]).
 static cudaError_t apply_sets(const uint64_t* const* C, int n_mats, const uint32_t* const* in, uint32_t* out, uint32_t n,
                               const uint32_t* d_src, const uint32_t* d_dst, int sm_count, cudaStream_t s, bool dependent,
-                              bool early)
+                              bool early, const uint32_t* counts = nullptr)
 {
     if (n == 0 || n_mats == 0) return cudaSuccess;
     if (n_mats > kMaxMats) return cudaErrorInvalidValue;
     MatSet mats{};
+    uint32_t at = 0;
     for (int j = 0; j < n_mats; ++j) {
         mats.C[j] = reinterpret_cast<const uint32_t*>(C[j]);
         mats.in[j] = in[j];
+        mats.n[j] = counts ? counts[j] : n;
+        mats.at[j] = at;
+        at += mats.n[j];
     }
     if (n >= 4 * 48) return launch_pairs<48>(mats, n_mats, out, n, d_src, d_dst, sm_count, s, dependent, early);
     if (n > 4) return launch_pairs<16>(mats, n_mats, out, n, d_src, d_dst, sm_count, s, dependent, early);
@@ -310,11 +317,11 @@ static cudaError_t apply_sets(const uint64_t* const* C, int n_mats, const uint32
 
 cudaError_t launch_gf2_apply_multi(const uint64_t* const* C, int n_mats, const uint32_t* in, uint32_t* out, uint32_t n,
                                    const uint32_t* d_src, const uint32_t* d_dst, int sm_count, cudaStream_t s,
-                                   bool dependent, bool early)
+                                   bool dependent, bool early, const uint32_t* counts)
 {
     const uint32_t* all[kMaxMats];
     for (const uint32_t*& p : all) p = in;
-    return apply_sets(C, n_mats, all, out, n, d_src, d_dst, sm_count, s, dependent, early);
+    return apply_sets(C, n_mats, all, out, n, d_src, d_dst, sm_count, s, dependent, early, counts);
 }
 
 // C = M^J from the newest word's columns Y_b = M^J E_b (states, consecutive

@@ -35,10 +35,11 @@ cudaError_t launch_gf2_apply_pairs(const uint64_t* C, const uint32_t* in, uint32
 // skipped.  early: a dependent launch after it may become resident while it
 // runs.  Wrong for long kernels of many blocks, which would be spread over the
 // SMs by what this one has left free: 16 streams of 2^18 words in 128 pieces
-// 45 us early, 33 us not.
+// 45 us early, 33 us not.  counts as in gf2_tc_apply.
 cudaError_t launch_gf2_apply_multi(const uint64_t* const* C, int n_mats, const uint32_t* in, uint32_t* out, uint32_t n,
                                    const uint32_t* d_src, const uint32_t* d_dst, int sm_count, cudaStream_t s,
-                                   bool dependent = false, bool early = true);
+                                   bool dependent = false, bool early = true,
+                                   const uint32_t* counts = nullptr);
 
 // M^(j 2^k) for 1 <= j <= 7, built on first use like jump_matrix.
 const uint64_t* jump_matrix_multiple(int device, int param_set, int j, int k, cudaStream_t s, xg_status* st);

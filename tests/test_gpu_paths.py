@@ -434,3 +434,25 @@ def test_jump_by_the_number_of_set_bits(family, bits):
         with make(n) as st:
             st.jump(words)
             assert torch.equal(draw(st)[:3], ref)
+
+
+@pytest.mark.parametrize("tensor_cores", ["1", "0"])
+@pytest.mark.parametrize("calls", [(2,), (8, 9), (3, 64, 65, 1), (7, 512, 513, 20, 2, 100), tuple(range(1, 90)), (600,) * 40])
+def test_batch_prologue_steps(calls, tensor_cores, monkeypatch):
+    """Batches whose calls are cut into the given numbers of pieces (one to
+    three prologue steps, sources with one to seven results each) against
+    uncut batches, twice in a row."""
+    from paper_1108_0486_gb300 import Streams
+    monkeypatch.setenv("XG_JUMP_TENSOR_CORES", tensor_cores)
+    rows = []
+    for split in (64, 1):
+        with Streams(len(calls), param_set=len(calls) % 2, seeds=W.seeds(len(calls))) as st:
+            st.set_batch_split(split)
+            got = []
+            for call in range(2):
+                outs = [torch.zeros(64 * k - (5 if k % 3 else 0), dtype=torch.int32, device="cuda") for k in calls]
+                st.batch([(i, "u32", o.numel(), o) for i, o in enumerate(outs)])
+                got.append(torch.cat(outs))
+            got.append(st.u32(99).reshape(-1))
+            rows.append(torch.cat(got))
+    assert torch.equal(*rows)
