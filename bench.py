@@ -55,14 +55,14 @@ def _peaks():
         return 6800.0, "fallback"
 
 
-def _fp8_peak():
-    """Dense FP8 tensor peak: the measured bf16 GEMM rate times the nominal
-    FP8 / bf16 ratio of 2, else the nominal 4.5 PFLOP/s."""
+def _fp4_peak():
+    """Dense FP4 tensor peak: the measured bf16 GEMM rate times the nominal
+    FP4 / bf16 ratio of 6, else the nominal 13.5 PFLOP/s."""
     try:
         with open(os.path.join(ROOT, "MEASURED_PEAKS.json")) as f:
-            return 2.0 * float(json.load(f)["bf16_tflops"]), "measured bf16 x 2"
+            return 6.0 * float(json.load(f)["bf16_tflops"]), "measured bf16 x 6"
     except Exception:
-        return 4500.0, "nominal"
+        return 13500.0, "nominal"
 
 
 def _record(name):
@@ -95,7 +95,7 @@ def _traffic(kernel=None):
 
 def _issue_ceiling(sm_count, sm_mhz):
     """Normals per second at full instruction issue (4 warp instructions per
-    SM per clock) for the recorded instruction count of gen_kernel<normal>,
+    SM per clock) for the recorded instruction count of the normal kernel,
     or None when the record does not match the kernel sources."""
     rec = _record("gen_kernel_normal_issue.txt")
     if rec is None or not sm_mhz:
@@ -103,7 +103,7 @@ def _issue_ceiling(sm_count, sm_mhz):
     per_normal = float(rec["warp_instructions"]) / float(rec["normals"])
     return {"normals_per_s": sm_count * 4 * sm_mhz * 1e6 / per_normal,
             "instructions_per_normal": round(32 * per_normal, 2), "sm_mhz": sm_mhz,
-            "source": "profiles/gen_kernel_normal_issue.txt (ncu smsp__inst_executed.sum, 16384 x 4096 case)"}
+            "source": "profiles/gen_kernel_normal_issue.txt (ncu smsp__inst_executed.sum, 16384 x 8192 case)"}
 
 
 def _free_port() -> int:
@@ -577,28 +577,26 @@ def extra_rows(st, stream, torch, peak, sm_mhz=None):
     sp.close()
     rows["paper_parameter_set"] = paper
     del buf
-    # jump-ahead of every stream: J = 2^40 + 2^20 + 12345 words, 8 set bits,
-    # i.e. 8 applications of a 4096 x 4096 GF(2) matrix per stream
+    # jump-ahead of every stream: J = 2^40 + 2^20 + 12345 words, 8 set bits
     J = (1 << 40) + (1 << 20) + 12345
     ms = _time(lambda: st.jump(J), stream, torch)
     bits = bin(J).count("1")
-    # the powers are multiplied first ((bits - 1) applications to the 4096
-    # columns of a matrix), then the product is applied to the streams; each
-    # application of a 4096 x 4096 GF(2) matrix to one state is 2 * 4096^2
-    # FP8 tensor operations on the tensor-core path
-    apps = (bits - 1) * 4096 + STREAMS
+    # the powers are multiplied first (table kernel, 32 columns per power),
+    # then the product is applied to the streams: 2 * 4096^2 FP4 tensor
+    # operations per stream
+    apps = STREAMS
     tflops = 2 * 4096 ** 2 * apps / (ms / 1e3) / 1e12
-    fp8_peak = _fp8_peak()
+    fp4_peak = _fp4_peak()
     os.environ["XG_JUMP_TENSOR_CORES"] = "0"
     try:
         ms_table = _time(lambda: st.jump(J), stream, torch)
     finally:
         del os.environ["XG_JUMP_TENSOR_CORES"]
     rows["jump_16384_streams"] = {"words": J, "set_bits": bits, "ms": ms, "state_applications": apps,
-                                  "tensor_tflops": tflops, "fp8_peak_tflops": fp8_peak[0],
-                                  "fp8_peak_source": fp8_peak[1], "frac_of_fp8_peak": tflops / fp8_peak[0],
+                                  "tensor_tflops": tflops, "fp4_peak_tflops": fp4_peak[0],
+                                  "fp4_peak_source": fp4_peak[1], "frac_of_fp4_peak": tflops / fp4_peak[0],
                                   "ms_table_kernel": ms_table,
-                                  "note": "whole call: gather, FP8 expansion, tensor-core GEMMs, scatter"}
+                                  "note": "whole call: power product, FP4 expansion, one tensor-core GEMM in place"}
     # 16384 disjoint substreams of one sequence, 2^40 words apart (14 doubling
     # steps, one matrix application per stream); the streams are re-seeded
     # with their own seeds afterwards

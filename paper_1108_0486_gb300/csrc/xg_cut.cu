@@ -124,8 +124,8 @@ double word_ns(int kind, double w)
 }
 
 // Prologue time in us: the set-up launch, then per step a table-kernel launch
-// or an application on the tensor cores (a wave of output tiles is 240 states
-// by one matrix on 32 of the SMs).
+// or an application on the tensor cores (18 ns per operand row of a tile; the
+// last wave is rarely full).
 double prologue_us(uint32_t nstreams, uint64_t pieces, int sm_count)
 {
     const Steps p = plan_steps(nstreams, (uint32_t)pieces);
@@ -135,8 +135,10 @@ double prologue_us(uint32_t nstreams, uint64_t pieces, int sm_count)
         if (!p.step[k].tc) {
             t += 5.5 + 0.05 * (double)(n * p.step[k].mats);
         } else {
-            const uint64_t tiles = (n + 239) / 240 * 32 * p.step[k].mats;
-            t += 18.0 + 4.5 * (double)((tiles + sm_count - 1) / sm_count - 1);
+            uint32_t counts[kGf2TcMaxMats], waves = 1;
+            for (uint32_t& c : counts) c = (uint32_t)n;
+            const uint32_t bn = gf2_tc_tile(counts, (int)p.step[k].mats, sm_count, &waves);
+            t += 11.4 + 0.018 * (double)(128 + bn) * (1.0 + 0.7 * (double)(waves - 1));
         }
     }
     return t;

@@ -53,7 +53,7 @@ namespace xg {
 namespace {
 
 constexpr int kBM = 128;                  // output bits per tile (TMEM lanes)
-constexpr int kBN = 240;                  // states per tile (TMEM columns)
+constexpr int kBN = 240;                  // most states per tile (TMEM columns)
 constexpr int kRowBytes = kGf2Bits / 2;   // 4096 nibbles
 constexpr int kBK = 128;                  // bytes of K per stage: one 128-byte swizzle row
 constexpr int kKBlocks = kRowBytes / kBK; // 16
@@ -62,7 +62,7 @@ constexpr int kScaleA = 2 * kBN, kScaleB = 2 * kBN + 16;   // TMEM columns of th
 static_assert(kScaleB + 16 <= kTmemCols, "TMEM columns");
 constexpr int kStages = 4;
 constexpr int kABytes = kBM * kBK;        // 16 KiB
-constexpr int kBBytes = kBN * kBK;        // 32 KiB
+constexpr int kBBytes = kBN * kBK;        // 30 KiB
 constexpr int kStageBytes = kABytes + kBBytes;
 constexpr int kSmemBytes = kStages * kStageBytes + 1024 /* barriers */ + 1024 /* alignment */;
 constexpr int kEpilogueWarps = 4;
@@ -133,20 +133,23 @@ __device__ __forceinline__ uint64_t smem_desc(const void* p)
 }
 
 // Instruction descriptor, kind::mxf4: A and B E2M1, both K-major, UE8M0
-// scales (data id 0), K = 64, N = kBN, M = kBM.
-constexpr uint32_t kInstrDesc = (1u << 7) | (1u << 10)       // A, B: E2M1
-                                | (1u << 23)                 // scale type UE8M0
-                                | ((uint32_t)(kBN >> 3) << 17) | ((uint32_t)(kBM >> 7) << 27);
+// scales (data id 0), K = 64, N = bn (a multiple of 16), M = kBM.
+__device__ __forceinline__ uint32_t instr_desc(uint32_t bn)
+{
+    return (1u << 7) | (1u << 10)   // A, B: E2M1
+           | (1u << 23)             // scale type UE8M0
+           | ((bn >> 3) << 17) | ((uint32_t)(kBM >> 7) << 27);
+}
 
-__device__ __forceinline__ void mma_f4(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t sa_tmem,
-                                       uint32_t sb_tmem, uint32_t accumulate)
+__device__ __forceinline__ void mma_f4(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
+                                       uint32_t sa_tmem, uint32_t sb_tmem, uint32_t accumulate)
 {
     asm volatile(
         "{\n\t.reg .pred p;\n\t"
         "setp.ne.b32 p, %4, 0;\n\t"
         "tcgen05.mma.cta_group::1.kind::mxf4.block_scale.scale_vec::2X [%0], %1, %2, %3, [%5], [%6], p;\n\t}" ::"r"(
             d_tmem),
-        "l"(adesc), "l"(bdesc), "r"(kInstrDesc), "r"(accumulate), "r"(sa_tmem), "r"(sb_tmem)
+        "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate), "r"(sa_tmem), "r"(sb_tmem)
         : "memory");
 }
 
@@ -199,8 +202,10 @@ struct TcMaps {
 
 // out[dst[at_j + s]] = C_j x_s for the first n_j states of the B operand (rows
 // past them count for nothing).  Persistent: CTA b takes tiles b, b +
-// gridDim.x, ... of the matrices' (4096 / kBM) x (n_j / kBN) tiles, M fastest
-// (consecutive tiles share a B tile in L2).  A few hundred states fill a part
+// gridDim.x, ... of the matrices' (4096 / kBM) x (n_j / bn) tiles, M fastest
+// (consecutive tiles share a B tile in L2).  bn states per tile: 240 for many
+// states; fewer states take the width that gives the shortest waves (see
+// gf2_tc_tile), whose smaller B tiles are loaded and multiplied faster.  A few hundred states fill a part
 // of the SMs with one matrix, and a launch costs as much as its first tile
 // (14 us, each further wave 4), so several matrices share one: 500 states by 7
 // matrices 35 us, in three doubling launches 75 us.  192 threads: warp 0 = TMA producer, warp 1 = TMEM owner and
@@ -218,7 +223,7 @@ __device__ __forceinline__ TcTile tc_tile(const TcMaps& maps, uint32_t t)
     return TcTile{j, (t - from) / (uint32_t)(kGf2Bits / kBM)};
 }
 
-__global__ void __launch_bounds__(kThreads, 1) gf2_tc_kernel(const __grid_constant__ TcMaps maps, uint32_t total,
+__global__ void __launch_bounds__(kThreads, 1) gf2_tc_kernel(const __grid_constant__ TcMaps maps, uint32_t total, uint32_t bn,
                                                               const uint32_t* __restrict__ dst, uint32_t* out,
                                                               uint32_t out_stride, uint32_t* status, uint32_t stall)
 {
@@ -281,16 +286,17 @@ __global__ void __launch_bounds__(kThreads, 1) gf2_tc_kernel(const __grid_consta
                         s_failed = 1;
                         break;
                     }
-                    mbar_expect_tx(&full[s], kStageBytes);
+                    mbar_expect_tx(&full[s], kABytes + bn * kBK);
                     if (stall && blockIdx.x == 0 && issued == 0) continue;   // the failure-path test
                     tma_load_2d(sa + s * kABytes, ma, &full[s], kb * kBK, mt * kBM);
-                    tma_load_2d(sb + s * kBBytes, &maps.b, &full[s], kb * kBK, nt * kBN);
+                    tma_load_2d(sb + s * kBBytes, &maps.b, &full[s], kb * kBK, nt * (int)bn);
                 }
             }
         }
         __syncwarp();
     } else if (warp == 1) {
         if (lane == 0) {
+            const uint32_t idesc = instr_desc(bn);
             uint32_t it = 0, lt = 0;
             for (uint32_t t = blockIdx.x; t < total && !failed(&s_failed); t += gridDim.x, ++lt) {
                 const uint32_t acc = lt & 1, v = lt >> 1;
@@ -311,7 +317,7 @@ __global__ void __launch_bounds__(kThreads, 1) gf2_tc_kernel(const __grid_consta
                     const uint64_t bd = smem_desc(sb + s * kBBytes);
 #pragma unroll
                     for (int kk = 0; kk < kBK / 32; ++kk)  // K = 32 bytes per instruction: +2 in 16-byte units
-                        mma_f4(d, ad + 2 * kk, bd + 2 * kk, tmem + kScaleA, tmem + kScaleB, (kb | kk) != 0);
+                        mma_f4(d, ad + 2 * kk, bd + 2 * kk, idesc, tmem + kScaleA, tmem + kScaleB, (kb | kk) != 0);
                     mma_commit(&empty[s]);
                 }
                 mma_commit(&tfull[acc]);  // arrives once this tile's MMAs have completed
@@ -335,23 +341,23 @@ __global__ void __launch_bounds__(kThreads, 1) gf2_tc_kernel(const __grid_consta
             const uint32_t* to = dst ? dst + maps.at[tile.j] : nullptr;
             const uint32_t word = mt * (kBM / 32) + q;  // ring word of these 32 bits
             static_assert(kBN % 16 == 0, "columns are read 16 at a time");
-            for (int c = 0; c < kBN; c += 32) {
+            for (uint32_t c = 0; c < bn; c += 32) {
                 uint32_t vals[32];
-                const uint32_t col = tmem + ((q * 32) << 16) + acc * kBN + (uint32_t)c;
+                const uint32_t col = tmem + ((q * 32) << 16) + acc * kBN + c;
                 tmem_ld16(col, vals);
-                if (c + 16 < kBN) tmem_ld16(col + 16, vals + 16);
+                if (c + 16 < bn) tmem_ld16(col + 16, vals + 16);
                 tmem_ld_wait();
                 uint32_t mine = 0;
 #pragma unroll
                 for (int j = 0; j < 32; ++j) {
-                    if (j >= 16 && c + 16 >= kBN) break;
+                    if (j >= 16 && c + 16 >= bn) break;
                     // the count is an integer <= 4096: adding 2^23 puts its parity in the last bit
                     const uint32_t bit = __float_as_uint(__uint_as_float(vals[j]) + 8388608.0f) & 1u;
                     const uint32_t b = __ballot_sync(0xFFFFFFFFu, bit);
                     if (lane == j) mine = b;
                 }
-                const uint32_t st = nt * kBN + (uint32_t)c + (uint32_t)lane;
-                if (st < n && c + lane < kBN) {
+                const uint32_t st = nt * bn + c + (uint32_t)lane;
+                if (st < n && c + lane < bn) {
                     const uint32_t d = to ? to[st] : st;
                     if (d != kNoState) out[(size_t)d * out_stride + word] = mine;
                 }
@@ -409,23 +415,23 @@ __global__ void __launch_bounds__(256) expand_matrix_kernel(const uint32_t* __re
     *reinterpret_cast<uint4*>(A + (size_t)(32 * w + lane) * kRowBytes + 16 * kw) = spread32(row);
 }
 
-// B[s][k] = bit k of state s of `in` (s < n), 0 for n <= s < n_pad.  Thread =
-// one ring word = 16 bytes of B.
-__global__ void __launch_bounds__(256) expand_states_kernel(TcStates in, uint32_t n, uint32_t n_pad,
-                                                            uint8_t* __restrict__ B)
+// B[s][k] = bit k of state s of `in` (s < n; TMA fills rows past n with 0).  A warp
+// takes a state, a lane four of its words (16 bytes of B each), so that four
+// reads are under way: 16384 states 11.4 us with one word per thread, 7.1 us so.
+__global__ void __launch_bounds__(256) expand_states_kernel(TcStates in, uint32_t n, uint8_t* __restrict__ B)
 {
-    const uint64_t t = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const uint32_t s = blockIdx.x * 8 + threadIdx.x / 32, lane = threadIdx.x & 31u;
     cudaTriggerProgrammaticLaunchCompletion();
     if (!in.settled) cudaGridDependencySynchronize();
-    if (t < (uint64_t)n_pad * kGf2Words) {
-        const uint32_t s = (uint32_t)(t / kGf2Words), w = (uint32_t)(t % kGf2Words);
-        uint32_t x = 0;
-        if (s < n) {
-            const uint32_t* ring = in.base + (size_t)(in.list ? in.list[s] : s) * in.stride;
-            if (in.pend) ring -= in.pend[s] * in.word;
-            x = ring[w];
-        }
-        *reinterpret_cast<uint4*>(B + (size_t)s * kRowBytes + 16 * w) = spread32(x);
+    if (s < n) {
+        const uint32_t* ring = in.base + (size_t)(in.list ? in.list[s] : s) * in.stride;
+        if (in.pend) ring -= in.pend[s] * in.word;
+        uint32_t x[4];
+#pragma unroll
+        for (uint32_t i = 0; i < 4; ++i) x[i] = ring[32 * i + lane];
+#pragma unroll
+        for (uint32_t i = 0; i < 4; ++i)
+            *reinterpret_cast<uint4*>(B + (size_t)s * kRowBytes + 16 * (32 * i + lane)) = spread32(x[i]);
     }
     // the product waits for this kernel only: it ends after the one before it
     if (in.settled) cudaGridDependencySynchronize();
@@ -500,9 +506,34 @@ bool gf2_tc_available(int device)
     return major == 10 && minor == 3;
 }
 
-uint32_t gf2_tc_padded(uint32_t n) { return (n + kBN - 1) / kBN * kBN; }
+size_t gf2_tc_scratch_bytes(uint32_t n) { return (size_t)n * kRowBytes; }
 
-size_t gf2_tc_scratch_bytes(uint32_t n) { return (size_t)gf2_tc_padded(n) * kRowBytes; }
+// A tile's time grows with its bytes into shared memory, (kBM + bn) kRowBytes,
+// beside the latency of a stage and what the matrices take from HBM.  500
+// states by 7 matrices, 5 waves of 240 or of 176 states: 36.4 and 35.2 us; a
+// jump of 300 streams by one power, one wave of 240 or 80: 25.1 and 23.3 us; a
+// cut call of 400 x 131072 words 66.6 and 62.2 us.
+uint32_t gf2_tc_tile(const uint32_t* counts, int n_mats, int sms, uint32_t* waves)
+{
+    const bool equal = counts[0] == counts[n_mats - 1];   // they never increase
+    uint32_t best = kBN;
+    uint64_t best_cost = ~uint64_t(0);
+    for (uint32_t bn = kBN; bn >= 16; bn -= 16) {
+        uint32_t tiles = 0;
+        if (equal) tiles = (counts[0] + bn - 1) / bn * (uint32_t)n_mats;
+        else
+            for (int j = 0; j < n_mats; ++j) tiles += (counts[j] + bn - 1) / bn;
+        const uint32_t w = (tiles * (kGf2Bits / kBM) + sms - 1) / sms;
+        const uint64_t cost = (uint64_t)w * (kBM + bn);
+        if (cost < best_cost) {
+            best_cost = cost;
+            best = bn;
+            *waves = w;
+        }
+        if (w > 64) break;   // many states: the widest tile
+    }
+    return best;
+}
 
 cudaError_t gf2_tc_expand_matrix(const uint64_t* C, uint8_t* A, cudaStream_t s, bool dependent)
 {
@@ -516,14 +547,16 @@ cudaError_t gf2_tc_apply(int device, const uint8_t* const* A, int n_mats, const 
 {
     if (n == 0 || n_mats == 0) return cudaSuccess;
     if (n_mats < 0 || n_mats > kGf2TcMaxMats) return cudaErrorInvalidValue;
-    const uint32_t n_pad = gf2_tc_padded(n);
+    int sms = 0;
+    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess || sms <= 0) sms = 1;
     TcMaps maps{};
-    uint32_t at = 0, tiles = 0;
+    uint32_t at = 0, tiles = 0, waves = 0;
+    for (int j = 0; j < n_mats; ++j) maps.n[j] = counts ? counts[j] : n;
+    const uint32_t bn = gf2_tc_tile(maps.n, n_mats, sms, &waves);
     for (int j = 0; j < n_mats; ++j) {
-        maps.n[j] = counts ? counts[j] : n;
         maps.at[j] = at;
         at += maps.n[j];
-        tiles += gf2_tc_padded(maps.n[j]) / kBN * (kGf2Bits / kBM);
+        tiles += (maps.n[j] + bn - 1) / bn * (kGf2Bits / kBM);
         maps.end[j] = tiles;
     }
     if (tiles == 0) return cudaSuccess;
@@ -532,19 +565,15 @@ cudaError_t gf2_tc_apply(int device, const uint8_t* const* A, int n_mats, const 
         if (!init_locked()) return cudaErrorNotSupported;
         for (int j = 0; j < n_mats; ++j)
             if (!make_map(&maps.a[j], A[j], kGf2Bits, kBM)) return cudaErrorInvalidValue;
-        if (!make_map(&maps.b, scratch, n_pad, kBN)) return cudaErrorInvalidValue;
+        if (!make_map(&maps.b, scratch, n, bn)) return cudaErrorInvalidValue;
         if (device >= 0 && device < 64 && !g_attr_set[device]) {
             cudaError_t e = cudaFuncSetAttribute(gf2_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
             if (e != cudaSuccess) return e;
             g_attr_set[device] = true;
         }
     }
-    const uint64_t words = (uint64_t)n_pad * kGf2Words;
-    cudaError_t e = launch_dependent(dependent, dim3((unsigned)((words + 255) / 256)), dim3(256), s,
-                                     expand_states_kernel, in, n, n_pad, scratch);
+    cudaError_t e = launch_dependent(dependent, dim3((n + 7) / 8), dim3(256), s, expand_states_kernel, in, n, scratch);
     if (e != cudaSuccess) return e;
-    int sms = 0;
-    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess || sms <= 0) sms = 1;
     const unsigned grid = (unsigned)std::min<uint32_t>(tiles, (uint32_t)sms);
     const char* stall = std::getenv("XG_TC_TEST_STALL");
     cudaLaunchConfig_t cfg{};
@@ -557,7 +586,7 @@ cudaError_t gf2_tc_apply(int device, const uint8_t* const* A, int n_mats, const 
     attr.val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = &attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, gf2_tc_kernel, maps, tiles, dst, out, out_stride, g_status_dev,
+    return cudaLaunchKernelEx(&cfg, gf2_tc_kernel, maps, tiles, bn, dst, out, out_stride, g_status_dev,
                               (stall && stall[0] == '1') ? 1u : 0u);
 }
 

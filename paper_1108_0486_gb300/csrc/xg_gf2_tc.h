@@ -18,10 +18,13 @@ constexpr uint32_t kNoState = 0xFFFFFFFFu;
 // True on sm_103 with the driver's tensor-map encoder available.
 bool gf2_tc_available(int device);
 
-// States are padded to whole tiles of 240; the B operand scratch holds
-// gf2_tc_padded(n) * 2048 bytes.
-uint32_t gf2_tc_padded(uint32_t n);
+// Bytes of the B operand of n states.
 size_t gf2_tc_scratch_bytes(uint32_t n);
+
+// States per output tile (16 .. 240) that a launch of n_mats matrices on
+// counts[j] states each takes, and its waves of tiles over the SMs: the
+// smallest product of waves and bytes per tile (plain C++).
+uint32_t gf2_tc_tile(const uint32_t* counts, int n_mats, int sms, uint32_t* waves);
 
 // Bytes of a matrix as the A operand.
 constexpr size_t kGf2TcMatrixBytes = (size_t)kGf2Bits * kGf2Bits / 2;
