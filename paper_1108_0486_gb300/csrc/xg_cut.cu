@@ -42,7 +42,7 @@ struct Steps {
 
 // Up to 7 matrices per step, which makes the pieces eight times as many.  By
 // the table kernel as long as the states are few, where a step costs a launch
-// and the matrix read rather than the lookups (0.07 us per state and matrix);
+// and the matrix read rather than the lookups (0.05 us per state and matrix);
 // by the tensor cores from about 200 results on, where it costs the launches
 // and one tile's time and hardly more for seven matrices than for one.
 Steps plan_steps(uint32_t nstreams, uint32_t pieces)

@@ -506,16 +506,13 @@ const uint8_t* jump_matrix_tc(int device, int family, int j, int k, cudaStream_t
     return A;
 }
 
-bool gf2_use_tc(int device, uint32_t n)
+bool gf2_use_tc(int device, uint32_t n, uint32_t from)
 {
     // read on every call (a few hundred nanoseconds against a matrix application)
     const char* off = std::getenv("XG_JUMP_TENSOR_CORES");
     if (off && std::strcmp(off, "0") == 0) return false;
     const char* v = std::getenv("XG_GF2_TC_MIN_STATES");
-    // One application in a call, table kernel against tensor cores: 31 / 35 us
-    // for 64 states, 35 / 38 for 160, 39 / 36 for 192, 57 / 38 for 512,
-    // 68 / 42 for 1024 (the tensor cores take one tile's time up to 1140).
-    const uint32_t min_states = v ? (uint32_t)std::strtoul(v, nullptr, 10) : 192u;
+    const uint32_t min_states = v ? (uint32_t)std::strtoul(v, nullptr, 10) : from;
     return n >= std::max(1u, min_states) && gf2_tc_available(device);
 }
 
@@ -562,14 +559,18 @@ static size_t product_bytes(uint64_t words)
     return (size_t)__builtin_popcountll(words) * kMaxNewest * kR * 4 + kSeqBytes + (size_t)2 * kBits * kR * 4;
 }
 
+// The tensor cores beside the table kernel in jumps by one power: us per jump
+// of 8 / 64 / 160 / 256 streams 23.4 / 23.4 / 24.2 / 24.4 in place against 27.8
+// / 30.4 / 33.8 / 42.9 (gather, table kernel, scatter); by a product of 8 powers
+// 61 / 62 / 62 / 63 against 65 / 66 / 70 / 80.
+constexpr uint32_t kInPlaceStreams = 8;
+
 size_t gf2_jump_work_bytes(int device, uint32_t n, uint64_t words)
 {
     // the tensor-core operand, then the product's work area and its FP4 copy
-    size_t b = (gf2_apply_scratch(device, n) + 255) / 256 * 256;
-    if (jump_combines(words, n)) {
-        b += product_bytes(words);
-        if (gf2_use_tc(device, n)) b += kGf2TcMatrixBytes;
-    }
+    const bool in_place = gf2_jump_in_place(device, n, words);
+    size_t b = ((in_place ? gf2_tc_scratch_bytes(n) : gf2_apply_scratch(device, n)) + 255) / 256 * 256;
+    if (jump_combines(words, n)) b += product_bytes(words) + (in_place ? kGf2TcMatrixBytes : 0);
     return b;
 }
 
@@ -633,7 +634,7 @@ static cudaError_t power_product(int device, int family, uint64_t words, uint8_t
 
 bool gf2_jump_in_place(int device, uint32_t n, uint64_t words)
 {
-    return gf2_use_tc(device, n) && (__builtin_popcountll(words) == 1 || jump_combines(words, n));
+    return gf2_use_tc(device, n, kInPlaceStreams) && (__builtin_popcountll(words) == 1 || jump_combines(words, n));
 }
 
 cudaError_t gf2_jump_windows(int device, int family, uint64_t words, const JumpWindows& win, uint32_t n, uint8_t* work,
@@ -645,7 +646,7 @@ cudaError_t gf2_jump_windows(int device, int family, uint64_t words, const JumpW
         A = jump_matrix_tc(device, family, 1, __builtin_ctzll(words), s, st);
         if (!A) return cudaErrorMemoryAllocation;
     } else {
-        uint8_t* w = work + (gf2_apply_scratch(device, n) + 255) / 256 * 256;
+        uint8_t* w = work + (gf2_tc_scratch_bytes(n) + 255) / 256 * 256;
         uint8_t* abuf = w + product_bytes(words);
         const uint64_t* P = nullptr;
         cudaError_t e = power_product(device, family, words, w, sm_count, s, &P, st);
@@ -744,8 +745,9 @@ extern "C" xg_status xg_jump(xg_ctx* ctx, uint32_t first, uint32_t nstreams, uin
         if (((words >> k) & 1) && !jump_matrix(ctx->device, (int)ctx->param_set, k, s, &st)) return st;
     const uint32_t omega = ctx->weyl_on ? 0x9E3779B9u : 0u;
     const size_t wbytes = gf2_jump_work_bytes(ctx->device, nstreams, words);
+    const bool in_place = gf2_jump_in_place(ctx->device, nstreams, words);
     cudaError_t e;
-    if (gf2_jump_in_place(ctx->device, nstreams, words)) {
+    if (in_place) {
         if (xg_status g = ctx->ensure_jump_ws(wbytes)) return g;
         e = gf2_jump_windows(ctx->device, (int)ctx->param_set, words,
                              JumpWindows{ctx->st.win + (size_t)first * kWin, ctx->st.pend + first, 1}, nstreams,
@@ -779,10 +781,10 @@ extern "C" xg_status xg_jump(xg_ctx* ctx, uint32_t first, uint32_t nstreams, uin
         }
     }
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    const size_t sbytes = gf2_apply_scratch(ctx->device, nstreams);
+    const bool tc = in_place || gf2_apply_scratch(ctx->device, nstreams) != 0;
     if (st != XG_OK) return st;
     if (e != cudaSuccess) return cuda_fail(e, "xg_jump");
-    if (sbytes && gf2_tc_take_failure())
+    if (tc && gf2_tc_take_failure())
         return fail(XG_EDEVICE, "xg_jump: a tensor-core kernel gave up waiting; the streams are not valid");
     return XG_OK;
 }

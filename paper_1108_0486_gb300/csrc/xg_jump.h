@@ -47,10 +47,12 @@ const uint64_t* jump_matrix_multiple(int device, int param_set, int j, int k, cu
 // The same as the A operand of gf2_tc_apply.
 const uint8_t* jump_matrix_tc(int device, int family, int j, int k, cudaStream_t s, xg_status* st);
 
-// Whether an application to n states runs on the tensor cores (sm_103 and
-// n >= XG_GF2_TC_MIN_STATES, default 192; XG_JUMP_TENSOR_CORES=0 turns the
+// Whether an application with n results runs on the tensor cores (sm_103 and
+// n >= XG_GF2_TC_MIN_STATES, default `from`; XG_JUMP_TENSOR_CORES=0 turns the
 // tensor-core path off), and the device scratch it then needs (0 otherwise).
-bool gf2_use_tc(int device, uint32_t n);
+// A launch for 192 results costs 13 us on the tensor cores and 15 by the table
+// kernel (0.05 us per result), whose launches overlap better.
+bool gf2_use_tc(int device, uint32_t n, uint32_t from = 192);
 size_t gf2_apply_scratch(int device, uint32_t n);
 
 // rings[d_dst[i]] = C_k rings[d_src[i]] for n pairs, C_k the power 2^k of

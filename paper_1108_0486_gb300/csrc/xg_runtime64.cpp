@@ -386,9 +386,9 @@ xg_status xg_w64_jump(xg_w64_ctx* c, uint32_t first, uint32_t nstreams, uint64_t
         if (((words >> k) & 1) && !xg::jump_matrix(c->device, xg::kJumpSetW64, k, s, &st)) return st;
     const uint64_t omega = c->weyl_on ? xg64::kOmega : 0;
     const size_t wbytes = xg::gf2_jump_work_bytes(c->device, nstreams, words);
-    const size_t tc_bytes = xg::gf2_apply_scratch(c->device, nstreams);
+    const bool in_place = xg::gf2_jump_in_place(c->device, nstreams, words);
     cudaError_t e;
-    if (xg::gf2_jump_in_place(c->device, nstreams, words)) {
+    if (in_place) {
         if (xg_status g = ensure_jump_ws(c, wbytes)) return g;
         // the windows as 32-bit words, two per word (layout checked in generate_cut)
         e = xg::gf2_jump_windows(c->device, xg::kJumpSetW64, words,
@@ -422,7 +422,7 @@ xg_status xg_w64_jump(xg_w64_ctx* c, uint32_t first, uint32_t nstreams, uint64_t
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (st != XG_OK) return st;
     if (e != cudaSuccess) return cuda_fail(e, "xg_w64_jump");
-    if (tc_bytes && xg::gf2_tc_take_failure())
+    if ((in_place || xg::gf2_apply_scratch(c->device, nstreams)) && xg::gf2_tc_take_failure())
         return fail(XG_EDEVICE, "xg_w64_jump: a tensor-core kernel gave up waiting; the streams are not valid");
     return XG_OK;
 }

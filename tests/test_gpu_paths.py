@@ -456,3 +456,21 @@ def test_batch_prologue_steps(calls, tensor_cores, monkeypatch):
             got.append(st.u32(99).reshape(-1))
             rows.append(torch.cat(got))
     assert torch.equal(*rows)
+
+
+@pytest.mark.parametrize("family", [0, 64])
+@pytest.mark.parametrize("words", [1 << 21, (1 << 33) + (1 << 9) + 5, (1 << 30) + 12345])
+def test_jump_of_a_few_streams_in_the_windows(family, words, monkeypatch):
+    """The same on both sides of the least stream count that is jumped in place."""
+    from paper_1108_0486_gb300 import Streams, Streams64
+    for n, first, count in ((8, 0, 8), (20, 3, 7), (20, 3, 8), (20, 2, 17), (150, 50, 64), (150, 50, 65)):
+        got = []
+        for tc in ("1", "0"):
+            monkeypatch.setenv("XG_JUMP_TENSOR_CORES", tc)
+            seeds = W.seeds(n)
+            with (Streams64(n, seeds=seeds) if family == 64 else Streams(n, seeds=seeds)) as st:
+                draw = st.u64 if family == 64 else st.u32
+                draw(77)
+                st.jump(words, first=first, count=count)
+                got.append(torch.cat([draw(45), draw(200)], 1))
+        assert torch.equal(*got)
