@@ -56,8 +56,15 @@ typedef enum {
     XG_EDEVICE = 7,    /* device-side state read back by the host is corrupt (xg_get_state),
                           a server request's batch failed to launch and never ran, or a
                           jump-ahead kernel on the tensor cores gave up one of its bounded
-                          waits (xg_jump, xg_seed_substreams, a cut call: the streams being
-                          advanced are not valid; reseed or restore them) */
+                          waits (xg_jump, xg_seed_substreams, a cut call or batch: its
+                          outputs and the streams being advanced are not valid; reseed or
+                          restore them).  A call that returned before its kernels had ended
+                          reports it late: the first later call on the same context that
+                          finds it and reads or advances streams (generate, batch, jump,
+                          get and set_state(s), autotune, server start) or xg_destroy returns
+                          XG_EDEVICE, once; calls that generate or jump have then done
+                          nothing.  A server request of such a batch fails by itself.  Other
+                          contexts are not affected. */
     XG_ECANCELED = 8   /* the request was cancelled (xg_cancel) before it ran */
 } xg_status;
 
@@ -85,7 +92,9 @@ enum { XG_PARAMS_DEFAULT = 0, XG_PARAMS_PAPER = 1 };
 xg_status xg_create_streams(xg_ctx** out, uint32_t n_streams, uint32_t param_set,
                             uint32_t weyl_on, void* cuda_stream);
 
-/* Wait for the context's work, stop its server if running, free everything. */
+/* Wait for the context's work, stop its server if running, free everything.
+ * XG_EDEVICE (with everything freed) when a call's failure had not been
+ * reported yet. */
 xg_status xg_destroy(xg_ctx* ctx);
 
 /* Change the CUDA stream later calls enqueue on (cudaStream_t). */

@@ -52,9 +52,9 @@ class Streams:
             self.seed(seeds)
 
     def close(self):
-        if getattr(self, "ctx", None):
-            L.xg_destroy(self.ctx)
-            self.ctx = None
+        ctx, self.ctx = getattr(self, "ctx", None), None
+        if ctx:   # it is gone even where the call reports an earlier failure
+            L.xg_destroy(ctx)
 
     def __del__(self):
         try:
@@ -336,9 +336,9 @@ class Streams64:
         return L.xg_w64_params()
 
     def close(self):
-        if getattr(self, "ctx", None):
-            L.xg_w64_destroy(self.ctx)
-            self.ctx = None
+        ctx, self.ctx = getattr(self, "ctx", None), None
+        if ctx:   # it is gone even where the call reports an earlier failure
+            L.xg_w64_destroy(ctx)
 
     def __del__(self):
         try:

@@ -436,7 +436,7 @@ xg_status BatchLauncher::prologue(xg_ctx* c, cudaStream_t s)
         cudaError_t e;
         if (use_tc[k])
             e = gf2_tc_apply(c->device, tc_mats[k], n_mats, TcStates{rings, kGf2Words, src, nullptr, 0}, counts[k][0],
-                             rings, kGf2Words, dst, reinterpret_cast<uint8_t*>(db + off_tc), s, k > 0, counts[k]);
+                             rings, kGf2Words, dst, reinterpret_cast<uint8_t*>(db + off_tc), tc_, s, k > 0, counts[k]);
         else
             e = launch_gf2_apply_multi(mats[k], n_mats, rings, rings, counts[k][0], src, dst, c->sm_count, s, k > 0,
                                        k + 1 < nsteps, counts[k]);
@@ -452,10 +452,6 @@ xg_status BatchLauncher::launch(xg_ctx* c, const HostItem* items, uint32_t n, cu
         if (xg_status st = reserve(c, std::max<uint32_t>(n, 64))) return st;
     }
     if (launched_ && cudaEventSynchronize(done_) != cudaSuccess) return XG_ECUDA;
-    // a tensor-core jump-ahead that gave up waiting (in any earlier prologue)
-    // made its pieces' outputs invalid: report it here, the first point at
-    // which the host has synchronised with it
-    if (launched_ && gf2_tc_take_failure()) return XG_EDEVICE;
     // the jump prologue needs only the pieces: enqueue it before ordering the
     // heads, so that the GPU starts while the host finishes the plan
     plan_units(items, n, choose_piece_len(c, items, n, min_piece), c->n, plan_);
@@ -529,6 +525,7 @@ extern "C" xg_status xg_generate_batch(xg_ctx* ctx, const xg_item* items, uint32
         h[i] = HostItem{it.stream, it.type, it.count, it.out, nullptr};
     }
     std::lock_guard<std::mutex> lk(ctx->mu);
+    if (xg_status f = ctx->earlier_failure()) return f;
     BatchLauncher*& L = ctx->batch[ctx->batch_next];
     ctx->batch_next ^= 1;
     if (!L) L = new (std::nothrow) BatchLauncher();
@@ -594,6 +591,7 @@ extern "C" xg_status xg_autotune_batch(xg_ctx* ctx, const xg_item* items, uint32
         by_kind[it.type].push_back(HostItem{it.stream, it.type, it.count, it.out, nullptr});
     }
     std::lock_guard<std::mutex> lk(ctx->mu);
+    if (xg_status f = ctx->earlier_failure()) return f;
     BatchLauncher*& L = ctx->batch[0];
     if (!L) L = new (std::nothrow) BatchLauncher();
     if (!L) return fail(XG_ENOMEM, "host allocation failed");

@@ -8,6 +8,7 @@
 #include <cstdint>
 #include <vector>
 
+#include "xg_gf2_tc.h"
 #include "xg_launch.h"
 #include "xorgens_gb300.h"
 
@@ -78,6 +79,9 @@ public:
     size_t scratch_bytes() const { return bytes_; }
     cudaEvent_t done_event() const { return done_; }
     bool busy() const;
+    // Set when a jump prologue gave up waiting: the cut calls of its batch are
+    // not valid.
+    TcStatus& status() { return tc_; }
 
 private:
     xg_status build_graph(xg_ctx* c);
@@ -99,6 +103,7 @@ private:
     int max_grid_g_[2] = {0, 0};  // per variant (without, with group paths)
     BatchPlan plan_;
     // jump-ahead prologue buffers
+    TcStatus tc_;
     void* h_jstage_ = nullptr;
     void* d_jbuf_ = nullptr;
     size_t jbytes_ = 0;

@@ -206,22 +206,14 @@ xg_status CutWorkspace::ensure(size_t want)
 xg_status CutWorkspace::acquire(cudaStream_t s)
 {
     if (!used) return XG_OK;
-    // a tensor-core prologue that gave up waiting made its call's outputs
-    // invalid: reported by the first cut call after it has finished
-    if (tc_pending && cudaEventQuery(event) == cudaSuccess) {
-        tc_pending = false;
-        if (gf2_tc_take_failure())
-            return fail(XG_EDEVICE, "an earlier cut call's tensor-core kernel gave up waiting; its streams are not valid");
-    }
     if (stream != s && cudaStreamWaitEvent(s, event, 0) != cudaSuccess)
         return cuda_fail(cudaGetLastError(), "cut workspace");
     return XG_OK;
 }
 
-xg_status CutWorkspace::release(cudaStream_t s, bool tensor_cores)
+xg_status CutWorkspace::release(cudaStream_t s)
 {
     stream = s;
-    tc_pending = tc_pending || tensor_cores;
     if (cudaEventRecord(event, s) != cudaSuccess) return cuda_fail(cudaGetLastError(), "cut workspace");
     used = true;
     return XG_OK;
@@ -256,6 +248,7 @@ xg_status cut_prologue(CutWorkspace& ws, const CutStreams& streams, uint32_t fir
     const size_t tc_off = up(list_off + (size_t)steps.entries * 4);
     const size_t extra_off = up(tc_off + (most_tc ? gf2_tc_scratch_bytes(most_tc) : 0));
     if (ws.ensure(extra_off + extra_bytes) != XG_OK) return XG_OK;
+    if (most_tc && !streams.tc->device()) return XG_OK;
     char* base = static_cast<char*>(ws.mem);
     uint32_t* rings = reinterpret_cast<uint32_t*>(base);
     uint32_t* weyl0 = reinterpret_cast<uint32_t*>(base + weyl_off);
@@ -293,13 +286,13 @@ xg_status cut_prologue(CutWorkspace& ws, const CutStreams& streams, uint32_t fir
         const uint32_t* dst = src + m;
         if (use_tc[k])
             e = gf2_tc_apply(streams.device, tc_mats[k], n_mats, TcStates{rings, kGf2Words, src, nullptr, 0}, m, rings, kGf2Words,
-                             dst, tc, s, true);
+                             dst, tc, *streams.tc, s, true);
         else
             e = launch_gf2_apply_multi(mats[k], n_mats, rings, rings, m, src, dst, streams.sm_count, s, true,
                                        k + 1 < steps.n);
     }
     if (e != cudaSuccess) return cuda_fail(e, "cut prologue");
-    *out = CutRings{rings, weyl0, base + extra_off, most_tc != 0};
+    *out = CutRings{rings, weyl0, base + extra_off};
     return XG_OK;
 }
 
@@ -309,7 +302,7 @@ xg_status cut_generate(xg_ctx* c, int kind, uint32_t first, uint32_t nstreams, u
     const bool sum = kind == kNormalSum;
     const uint64_t words = kind == kNormal || sum ? n + (n & 1u) : n;
     const uint32_t pieces = (uint32_t)((words + (uint64_t(1) << q) - 1) >> q);
-    const CutStreams streams{c->device, c->sm_count, (int)c->param_set, c->st.win, c->st.pend, c->st.weyl, 1};
+    const CutStreams streams{c->device, c->sm_count, (int)c->param_set, c->st.win, c->st.pend, c->st.weyl, 1, &c->tc};
     CutRings r{};
     xg_status st = cut_prologue(c->cut, streams, first, nstreams, pieces, q, sum ? (size_t)pieces * nstreams * 4 : 0,
                                 c->stream, &r, ran);
@@ -332,7 +325,7 @@ xg_status cut_generate(xg_ctx* c, int kind, uint32_t first, uint32_t nstreams, u
         e = launch_dependent(true, dim3((nstreams + 1) / 2), dim3(64), c->stream, cut_sum_kernel,
                              reinterpret_cast<const float*>(r.extra), pieces, nstreams, static_cast<float*>(out));
     if (e != cudaSuccess) return cuda_fail(e, "cut generation");
-    return c->cut.release(c->stream, r.tensor_cores);
+    return c->cut.release(c->stream);
 }
 
 }  // namespace xg

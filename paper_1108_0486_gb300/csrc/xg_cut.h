@@ -6,6 +6,7 @@
 #include <cstdint>
 #include <cuda_runtime.h>
 
+#include "xg_gf2_tc.h"
 #include "xg_launch.h"
 #include "xorgens_gb300.h"
 
@@ -29,12 +30,11 @@ struct CutWorkspace {
     size_t bytes = 0;
     cudaEvent_t event = nullptr;
     cudaStream_t stream = nullptr;
-    bool used = false;         // the event has been recorded
-    bool tc_pending = false;   // a tensor-core prologue's status is unread
+    bool used = false;   // the event has been recorded
 
     xg_status ensure(size_t want);
-    xg_status acquire(cudaStream_t s);                      // before the first launch that uses it
-    xg_status release(cudaStream_t s, bool tensor_cores);   // after the last
+    xg_status acquire(cudaStream_t s);   // before the first launch that uses it
+    xg_status release(cudaStream_t s);   // after the last
     void destroy();
 };
 
@@ -48,6 +48,7 @@ struct CutStreams {
     const uint32_t* pend;
     const uint32_t* weyl;
     uint32_t word;
+    TcStatus* tc;           // the context's
 };
 
 // What the prologue leaves in the workspace: 128-word rings [nstreams][pieces],
@@ -56,7 +57,6 @@ struct CutRings {
     uint32_t* rings;
     uint32_t* weyl0;
     char* extra;
-    bool tensor_cores;
 };
 
 // Enqueue the prologue of a call on streams [first, first + nstreams) cut into

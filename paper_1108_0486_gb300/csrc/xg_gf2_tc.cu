@@ -34,7 +34,7 @@
 // were resident earlier would crowd onto the SMs that have no tile.
 //
 // Every wait is bounded (2 s of %globaltimer); a wait that gives up records
-// a failure in a host-visible status word, the CTA waits (bounded) for its
+// a failure in its owner's status word (TcStatus), the CTA waits (bounded) for its
 // own TMA copies still in flight, frees its TMEM and returns.  To test that
 // path, XG_TC_TEST_STALL=1 in the environment makes CTA 0 arm its first
 // stage's barrier without starting the stage's copies: the waits on that
@@ -45,6 +45,8 @@
 #include <cstdint>
 #include <cstdlib>
 #include <mutex>
+#include <utility>
+#include <vector>
 
 #include "xg_gf2_tc.h"
 #include "xg_runtime.h"
@@ -446,13 +448,12 @@ using EncodeTiled = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, 
 std::mutex g_mu;
 EncodeTiled g_encode = nullptr;
 bool g_probed = false;
-uint32_t* g_status_host = nullptr;  // mapped pinned word shared by every launch
-uint32_t* g_status_dev = nullptr;
 bool g_attr_set[64] = {};
+std::vector<std::pair<uint32_t*, uint32_t*>> g_status_free;   // status words without an owner (host, device)
 
 bool init_locked()
 {
-    if (g_probed) return g_encode != nullptr && g_status_dev != nullptr;
+    if (g_probed) return g_encode != nullptr;
     g_probed = true;
     void* fn = nullptr;
     cudaDriverEntryPointQueryResult q{};
@@ -462,21 +463,6 @@ bool init_locked()
         return false;
     }
     g_encode = reinterpret_cast<EncodeTiled>(fn);
-    void* h = nullptr;
-    if (cudaHostAlloc(&h, 64, cudaHostAllocMapped | cudaHostAllocPortable) != cudaSuccess) {
-        cudaGetLastError();
-        g_encode = nullptr;
-        return false;
-    }
-    g_status_host = static_cast<uint32_t*>(h);
-    *g_status_host = 0;
-    void* d = nullptr;
-    if (cudaHostGetDevicePointer(&d, h, 0) != cudaSuccess) {
-        cudaGetLastError();
-        g_encode = nullptr;
-        return false;
-    }
-    g_status_dev = static_cast<uint32_t*>(d);
     return true;
 }
 
@@ -542,11 +528,13 @@ cudaError_t gf2_tc_expand_matrix(const uint64_t* C, uint8_t* A, cudaStream_t s, 
 }
 
 cudaError_t gf2_tc_apply(int device, const uint8_t* const* A, int n_mats, const TcStates& in, uint32_t n, uint32_t* out,
-                         uint32_t out_stride, const uint32_t* dst, uint8_t* scratch, cudaStream_t s, bool dependent,
-                         const uint32_t* counts)
+                         uint32_t out_stride, const uint32_t* dst, uint8_t* scratch, TcStatus& status, cudaStream_t s,
+                         bool dependent, const uint32_t* counts)
 {
     if (n == 0 || n_mats == 0) return cudaSuccess;
     if (n_mats < 0 || n_mats > kGf2TcMaxMats) return cudaErrorInvalidValue;
+    uint32_t* const word = status.device();
+    if (!word) return cudaErrorMemoryAllocation;
     int sms = 0;
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess || sms <= 0) sms = 1;
     TcMaps maps{};
@@ -586,17 +574,46 @@ cudaError_t gf2_tc_apply(int device, const uint8_t* const* A, int n_mats, const 
     attr.val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = &attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, gf2_tc_kernel, maps, tiles, bn, dst, out, out_stride, g_status_dev,
+    return cudaLaunchKernelEx(&cfg, gf2_tc_kernel, maps, tiles, bn, dst, out, out_stride, word,
                               (stall && stall[0] == '1') ? 1u : 0u);
 }
 
-bool gf2_tc_take_failure()
+uint32_t* TcStatus::device()
 {
+    if (dev_) return dev_;
     std::lock_guard<std::mutex> lk(g_mu);
-    if (!g_status_host) return false;
-    const uint32_t v = *reinterpret_cast<volatile uint32_t*>(g_status_host);
-    if (v) *reinterpret_cast<volatile uint32_t*>(g_status_host) = 0;
-    return v != 0;
+    if (g_status_free.empty()) {
+        constexpr size_t kWords = 1024;   // one page
+        void *h = nullptr, *d = nullptr;
+        cudaError_t e = cudaHostAlloc(&h, kWords * 4, cudaHostAllocMapped | cudaHostAllocPortable);
+        if (e == cudaSuccess) e = cudaHostGetDevicePointer(&d, h, 0);
+        if (e != cudaSuccess) {
+            cudaGetLastError();
+            if (h) cudaFreeHost(h);
+            return nullptr;
+        }
+        for (size_t i = kWords; i-- > 0;)
+            g_status_free.emplace_back(static_cast<uint32_t*>(h) + i, static_cast<uint32_t*>(d) + i);
+    }
+    host_ = g_status_free.back().first;
+    dev_ = g_status_free.back().second;
+    g_status_free.pop_back();
+    *host_ = 0;
+    return dev_;
+}
+
+TcStatus::~TcStatus()
+{
+    if (!dev_) return;
+    std::lock_guard<std::mutex> lk(g_mu);
+    g_status_free.emplace_back(const_cast<uint32_t*>(host_), dev_);
+}
+
+bool TcStatus::take()
+{
+    if (!host_ || !*host_) return false;
+    *host_ = 0;
+    return true;
 }
 
 }  // namespace xg

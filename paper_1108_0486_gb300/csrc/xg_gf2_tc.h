@@ -37,6 +37,26 @@ cudaError_t gf2_tc_expand_matrix(const uint64_t* C, uint8_t* A, cudaStream_t s, 
 // Most matrices applied by one launch.
 constexpr int kGf2TcMaxMats = 7;
 
+// The word that a tensor-core launch sets when one of its waits gives up: its
+// results are then not valid.  One per owner of such launches (a context, a
+// batch launcher), so that a failure reaches its owner and no other.  The word
+// is mapped host memory from a process-wide list, taken at the owner's first
+// launch and given back with the owner, whose launches have finished by then.
+class TcStatus {
+public:
+    TcStatus() = default;
+    TcStatus(const TcStatus&) = delete;
+    TcStatus& operator=(const TcStatus&) = delete;
+    ~TcStatus();
+    uint32_t* device();                                    // null: no memory for the word
+    const volatile uint32_t* host() const { return host_; }   // null before the first launch
+    bool take();                                           // a wait gave up since the last call
+
+private:
+    volatile uint32_t* host_ = nullptr;
+    uint32_t* dev_ = nullptr;
+};
+
 // The states that are read: state i is the 128 words at base + list[i] stride
 // (list null: i), or, with pend, at base + i stride - pend[i] word (the ring in
 // a stream's window, base its position without pending words).  settled: no
@@ -62,11 +82,7 @@ struct TcStates {
 // once the launch has finished.  Asynchronous on s.  dependent: as in
 // launch_gf2_apply_pairs.
 cudaError_t gf2_tc_apply(int device, const uint8_t* const* A, int n_mats, const TcStates& in, uint32_t n, uint32_t* out,
-                         uint32_t out_stride, const uint32_t* dst, uint8_t* scratch, cudaStream_t s,
+                         uint32_t out_stride, const uint32_t* dst, uint8_t* scratch, TcStatus& status, cudaStream_t s,
                          bool dependent = false, const uint32_t* counts = nullptr);
-
-// True (and cleared) if a tensor-core launch gave up a wait since the last
-// call: its results are not valid.  Read after synchronising.
-bool gf2_tc_take_failure();
 
 }  // namespace xg

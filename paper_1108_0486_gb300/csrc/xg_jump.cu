@@ -522,7 +522,7 @@ size_t gf2_apply_scratch(int device, uint32_t n)
 }
 
 cudaError_t gf2_apply(int device, int family, int k, uint32_t* rings, uint32_t n, const uint32_t* d_src,
-                      const uint32_t* d_dst, uint8_t* scratch, int sm_count, cudaStream_t s, xg_status* st,
+                      const uint32_t* d_dst, uint8_t* scratch, TcStatus& tc, int sm_count, cudaStream_t s, xg_status* st,
                       bool dst_zeroed)
 {
     *st = XG_OK;
@@ -531,7 +531,7 @@ cudaError_t gf2_apply(int device, int family, int k, uint32_t* rings, uint32_t n
         const uint8_t* A = jump_matrix_tc(device, family, 1, k, s, st);
         if (!A) return cudaErrorMemoryAllocation;
         return gf2_tc_apply(device, &A, 1, TcStates{rings, kGf2Words, d_src, nullptr, 0}, n, rings, kGf2Words, d_dst, scratch,
-                            s);
+                            tc, s);
     }
     const uint64_t* C = jump_matrix(device, family, k, s, st);
     if (!C) return cudaErrorMemoryAllocation;
@@ -638,7 +638,7 @@ bool gf2_jump_in_place(int device, uint32_t n, uint64_t words)
 }
 
 cudaError_t gf2_jump_windows(int device, int family, uint64_t words, const JumpWindows& win, uint32_t n, uint8_t* work,
-                             int sm_count, cudaStream_t s, xg_status* st)
+                             TcStatus& tc, int sm_count, cudaStream_t s, xg_status* st)
 {
     *st = XG_OK;
     const uint8_t* A = nullptr;
@@ -657,11 +657,11 @@ cudaError_t gf2_jump_windows(int device, int family, uint64_t words, const JumpW
     // the windows were last written before the product's first launch
     uint32_t* ring = win.win + kRingBase;
     return gf2_tc_apply(device, &A, 1, TcStates{ring, kWin, nullptr, win.pend, win.word, true}, n, ring, kWin, nullptr,
-                        work, s, __builtin_popcountll(words) > 1);
+                        work, tc, s, __builtin_popcountll(words) > 1);
 }
 
 cudaError_t gf2_jump_states(int device, int family, uint64_t words, uint32_t* rings, uint32_t n,
-                            const uint32_t* d_idx, uint8_t* work, int sm_count, cudaStream_t s, xg_status* st,
+                            const uint32_t* d_idx, uint8_t* work, TcStatus& tc, int sm_count, cudaStream_t s, xg_status* st,
                             bool* result_hi)
 {
     *st = XG_OK;
@@ -674,7 +674,8 @@ cudaError_t gf2_jump_states(int device, int family, uint64_t words, uint32_t* ri
         bool in_lo = true;
         for (int k = 0; k < 64; ++k) {
             if (!((words >> k) & 1)) continue;
-            cudaError_t e = gf2_apply(device, family, k, rings, n, in_lo ? lo : hi, in_lo ? hi : lo, scratch, sm_count, s, st);
+            cudaError_t e = gf2_apply(device, family, k, rings, n, in_lo ? lo : hi, in_lo ? hi : lo, scratch, tc, sm_count, s,
+                                      st);
             if (e != cudaSuccess) return e;
             in_lo = !in_lo;
         }
@@ -737,6 +738,7 @@ extern "C" xg_status xg_jump(xg_ctx* ctx, uint32_t first, uint32_t nstreams, uin
     if (ctx->server) return fail(XG_EINVAL, "the request server owns this context; stop it first");
     if (nstreams == 0 || words == 0) return XG_OK;
     std::lock_guard<std::mutex> lk(ctx->mu);
+    if (xg_status f = ctx->earlier_failure()) return f;
     cudaStream_t s = ctx->stream;
     int top = 63;
     while (!((words >> top) & 1)) --top;
@@ -751,7 +753,7 @@ extern "C" xg_status xg_jump(xg_ctx* ctx, uint32_t first, uint32_t nstreams, uin
         if (xg_status g = ctx->ensure_jump_ws(wbytes)) return g;
         e = gf2_jump_windows(ctx->device, (int)ctx->param_set, words,
                              JumpWindows{ctx->st.win + (size_t)first * kWin, ctx->st.pend + first, 1}, nstreams,
-                             static_cast<uint8_t*>(ctx->jump_ws), ctx->sm_count, s, &st);
+                             static_cast<uint8_t*>(ctx->jump_ws), ctx->tc, ctx->sm_count, s, &st);
         if (e == cudaSuccess) {
             finish_jump_kernel<<<(nstreams + 255) / 256, 256, 0, s>>>(ctx->st, first, nstreams, words, omega);
             e = cudaGetLastError();
@@ -773,7 +775,7 @@ extern "C" xg_status xg_jump(xg_ctx* ctx, uint32_t first, uint32_t nstreams, uin
         bool hi = false;
         if (e == cudaSuccess)
             e = gf2_jump_states(ctx->device, (int)ctx->param_set, words, rings, nstreams, lo_idx,
-                                reinterpret_cast<uint8_t*>(ws + work_off), ctx->sm_count, s, &st, &hi);
+                                reinterpret_cast<uint8_t*>(ws + work_off), ctx->tc, ctx->sm_count, s, &st, &hi);
         if (e == cudaSuccess) {
             const uint32_t* res = hi ? rings + (size_t)nstreams * kR : rings;
             scatter_rings_kernel<<<nstreams, 128, 0, s>>>(ctx->st, first, nstreams, res, words, omega);
@@ -781,12 +783,9 @@ extern "C" xg_status xg_jump(xg_ctx* ctx, uint32_t first, uint32_t nstreams, uin
         }
     }
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    const bool tc = in_place || gf2_apply_scratch(ctx->device, nstreams) != 0;
     if (st != XG_OK) return st;
     if (e != cudaSuccess) return cuda_fail(e, "xg_jump");
-    if (tc && gf2_tc_take_failure())
-        return fail(XG_EDEVICE, "xg_jump: a tensor-core kernel gave up waiting; the streams are not valid");
-    return XG_OK;
+    return ctx->earlier_failure();
 }
 
 extern "C" xg_status xg_seed_substreams(xg_ctx* ctx, uint32_t first, uint32_t count, uint32_t seed,
@@ -838,7 +837,7 @@ extern "C" xg_status xg_seed_substreams(xg_ctx* ctx, uint32_t first, uint32_t co
     if (e == cudaSuccess && count > 1) e = cudaMemsetAsync(rings + kR, 0, (size_t)(count - 1) * kR * 4, s);
     for (int b = 0; b < steps && e == cudaSuccess; ++b) {
         const uint32_t lo = 1u << b, hi = (uint32_t)std::min<uint64_t>((uint64_t)lo << 1, count);
-        e = gf2_apply(ctx->device, (int)ctx->param_set, q + b, rings, hi - lo, iota, iota + lo, scratch,
+        e = gf2_apply(ctx->device, (int)ctx->param_set, q + b, rings, hi - lo, iota, iota + lo, scratch, ctx->tc,
                       ctx->sm_count, s, &st, true);
     }
     if (e == cudaSuccess) {
@@ -849,7 +848,5 @@ extern "C" xg_status xg_seed_substreams(xg_ctx* ctx, uint32_t first, uint32_t co
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (st != XG_OK) return st;
     if (e != cudaSuccess) return cuda_fail(e, "xg_seed_substreams");
-    if (sbytes && gf2_tc_take_failure())
-        return fail(XG_EDEVICE, "xg_seed_substreams: a tensor-core kernel gave up waiting; the streams are not valid");
-    return XG_OK;
+    return ctx->earlier_failure();
 }

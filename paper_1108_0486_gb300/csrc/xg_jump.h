@@ -9,6 +9,8 @@
 
 namespace xg {
 
+class TcStatus;
+
 constexpr int kMaxPow = 64;  // C_k = M^(2^k), k < 64
 // Matrix families: the 32-bit parameter sets 0 (default) and 1 (paper), and
 // the 64-bit-word generator.
@@ -60,11 +62,11 @@ size_t gf2_apply_scratch(int device, uint32_t n);
 // the tensor cores when gf2_use_tc(device, n) and scratch (gf2_apply_scratch
 // bytes) is given, else with the table kernel.  Asynchronous on s, except
 // that a power's first use builds it.  After synchronising, a caller that
-// may have used the tensor cores checks gf2_tc_take_failure().  The table
+// may have used the tensor cores checks the status.  The table
 // kernel XORs into the destinations, so it zeroes them first unless the
 // caller says they are zero already (dst_zeroed).
 cudaError_t gf2_apply(int device, int family, int k, uint32_t* rings, uint32_t n, const uint32_t* d_src,
-                      const uint32_t* d_dst, uint8_t* scratch, int sm_count, cudaStream_t s, xg_status* st,
+                      const uint32_t* d_dst, uint8_t* scratch, TcStatus& tc, int sm_count, cudaStream_t s, xg_status* st,
                       bool dst_zeroed = false);
 
 // Advance n states by `words` positions: M^words applied to rings[0, n),
@@ -76,7 +78,7 @@ cudaError_t gf2_apply(int device, int family, int k, uint32_t* rings, uint32_t n
 // the powers are multiplied first).  Not for jumps that gf2_jump_in_place takes.
 size_t gf2_jump_work_bytes(int device, uint32_t n, uint64_t words);
 cudaError_t gf2_jump_states(int device, int family, uint64_t words, uint32_t* rings, uint32_t n,
-                            const uint32_t* d_idx, uint8_t* work, int sm_count, cudaStream_t s, xg_status* st,
+                            const uint32_t* d_idx, uint8_t* work, TcStatus& tc, int sm_count, cudaStream_t s, xg_status* st,
                             bool* result_hi);
 
 // Whether a jump applies one matrix (a power, or the product of several) on
@@ -92,7 +94,7 @@ struct JumpWindows {
 };
 bool gf2_jump_in_place(int device, uint32_t n, uint64_t words);
 cudaError_t gf2_jump_windows(int device, int family, uint64_t words, const JumpWindows& win, uint32_t n, uint8_t* work,
-                             int sm_count, cudaStream_t s, xg_status* st);
+                             TcStatus& tc, int sm_count, cudaStream_t s, xg_status* st);
 
 // ids[i] = first + i for i < n, then ids[n + j] = j for j < 2n (3n entries).
 cudaError_t launch_jump_index(uint32_t* ids, uint32_t n, uint32_t first, cudaStream_t s);

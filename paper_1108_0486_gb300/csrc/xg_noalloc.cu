@@ -103,6 +103,7 @@ extern "C" xg_status xg_generate_batch_noalloc(xg_ctx* ctx, const xg_item* items
 
     std::lock_guard<std::mutex> lk(ctx->mu);
     if (ctx->server) return fail(XG_EINVAL, "the request server owns this context; use xg_submit");
+    if (xg_status f = ctx->earlier_failure()) return f;
     if (xg_status st = xg::noalloc_setup(ctx->device, ctx->sm_count)) return st;  // no-op after create
 
     std::lock_guard<std::mutex> lk_stage(g_stage_mu);

@@ -115,6 +115,15 @@ int xg_ctx::pick_block(int kind, int c) const
     return (cfg[t] == c && blk[t] > 0) ? blk[t] : block[c];
 }
 
+xg_status xg_ctx::earlier_failure()
+{
+    bool gave_up = tc.take();
+    for (xg::BatchLauncher* b : batch) gave_up = (b && b->status().take()) || gave_up;
+    return gave_up ? fail(XG_EDEVICE, "a tensor-core kernel of this context gave up waiting: the outputs of that call "
+                                      "and the streams it advanced are not valid")
+                   : XG_OK;
+}
+
 xg_status xg_ctx::ensure_jump_ws(size_t bytes)
 {
     if (jump_ws_bytes >= bytes) return XG_OK;
@@ -273,6 +282,7 @@ static xg_status generate_common(xg_ctx* ctx, int kind, uint32_t first, uint32_t
     if (reinterpret_cast<uintptr_t>(out) & 3u) return fail(XG_EINVAL, "output must be 4-byte aligned");
     if (c->server) return fail(XG_EINVAL, "the request server owns this context; use xg_submit");
     std::lock_guard<std::mutex> lk(c->mu);
+    if (xg_status f = c->earlier_failure()) return f;
     if (is_device_pointer(out)) {
         // few streams, long calls: a single stream is one serial chain (one
         // warp, ~1.5e9 words/s), so cut each call into pieces that run on
@@ -284,7 +294,8 @@ static xg_status generate_common(xg_ctx* ctx, int kind, uint32_t first, uint32_t
         }
         return enqueue_gen(c, kind, first, nstreams, n, out, ld, nullptr, c->stream);
     }
-    return generate_to_host(c, kind, first, nstreams, n, out, ld);
+    const xg_status st = generate_to_host(c, kind, first, nstreams, n, out, ld);
+    return st == XG_OK ? c->earlier_failure() : st;
 }
 
 extern "C" {
@@ -353,11 +364,15 @@ xg_status xg_destroy(xg_ctx* ctx)
     if (!ctx) return XG_OK;
     Ctx* c = ctx;
     c->shutdown_server();
+    if (c->stream || c->state_mem) cudaStreamSynchronize(c->stream);
+    c->cut.destroy();
+    for (xg::BatchLauncher* b : c->batch)
+        if (b && b->done_event()) cudaEventSynchronize(b->done_event());
+    const xg_status failed = c->earlier_failure();
     for (int b = 0; b < 2; ++b) {
         delete c->batch[b];
         c->batch[b] = nullptr;
     }
-    if (c->stream || c->state_mem) cudaStreamSynchronize(c->stream);
     for (int b = 0; b < xg_ctx::kStage; ++b) {
         if (c->copy_stream[b]) {
             cudaStreamSynchronize(c->copy_stream[b]);
@@ -370,10 +385,9 @@ xg_status xg_destroy(xg_ctx* ctx)
         if (c->staging[b]) cudaFree(c->staging[b]);
     }
     if (c->jump_ws) cudaFree(c->jump_ws);
-    c->cut.destroy();
     if (c->state_mem) cudaFree(c->state_mem);
     delete c;
-    return XG_OK;
+    return failed;
 }
 
 xg_status xg_set_stream(xg_ctx* ctx, void* cuda_stream)
@@ -426,6 +440,7 @@ xg_status xg_get_state(xg_ctx* ctx, uint32_t stream, uint32_t* ring, uint32_t* w
     XG_CUDA(cudaMemcpyAsync(&pend, c->st.pend + stream, 4, cudaMemcpyDeviceToHost, c->stream), "get_state");
     XG_CUDA(cudaMemcpyAsync(&w, c->st.weyl + stream, 4, cudaMemcpyDeviceToHost, c->stream), "get_state");
     XG_CUDA(cudaStreamSynchronize(c->stream), "get_state");
+    if (xg_status f = c->earlier_failure()) return f;
     if (pend >= (uint32_t)xg::kRingBase) return fail(XG_EDEVICE, "corrupt stream state (pend %u)", pend);
     std::memcpy(ring, win + xg::kRingBase - pend, 128 * 4);
     *weyl = w;
@@ -440,6 +455,7 @@ xg_status xg_set_state(xg_ctx* ctx, uint32_t stream, const uint32_t* ring, uint3
     if (!ring) return fail(XG_EINVAL, "null ring");
     if (c->server) return fail(XG_EINVAL, "the request server owns this context; stop it first");
     std::lock_guard<std::mutex> lk(c->mu);
+    if (xg_status f = c->earlier_failure()) return f;
     uint32_t win[xg::kWin] = {0};
     std::memcpy(win + xg::kRingBase, ring, 128 * 4);
     const uint32_t pend = 0, w = c->weyl_on ? weyl : 0u;
@@ -471,7 +487,7 @@ xg_status xg_get_states(xg_ctx* ctx, uint32_t first, uint32_t count, uint32_t* r
     if (e == cudaSuccess && pos) e = cudaMemcpyAsync(pos, d_pos, pb, cudaMemcpyDeviceToHost, c->stream);
     cudaFreeAsync(d, c->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
-    return e == cudaSuccess ? XG_OK : cuda_fail(e, "xg_get_states");
+    return e == cudaSuccess ? c->earlier_failure() : cuda_fail(e, "xg_get_states");
 }
 
 xg_status xg_set_states(xg_ctx* ctx, uint32_t first, uint32_t count, const uint32_t* rings, const uint32_t* weyl,
@@ -484,6 +500,7 @@ xg_status xg_set_states(xg_ctx* ctx, uint32_t first, uint32_t count, const uint3
     if (!rings || !weyl) return fail(XG_EINVAL, "null input");
     if (c->server) return fail(XG_EINVAL, "the request server owns this context; stop it first");
     std::lock_guard<std::mutex> lk(c->mu);
+    if (xg_status f = c->earlier_failure()) return f;
     const size_t rb = (size_t)count * 128 * 4, wb = (size_t)count * 4, pb = (size_t)count * 8;
     char* d = nullptr;
     XG_CUDA(cudaMallocAsync(reinterpret_cast<void**>(&d), rb + wb + pb + 16, c->stream), "cudaMallocAsync(states)");
@@ -526,6 +543,7 @@ xg_status xg_generate_normal_sum(xg_ctx* ctx, uint32_t first, uint32_t nstreams,
     if (!is_device_pointer(d_sums)) return fail(XG_EINVAL, "sums must be device memory");
     if (c->server) return fail(XG_EINVAL, "the request server owns this context; use xg_submit");
     std::lock_guard<std::mutex> lk(c->mu);
+    if (xg_status f = c->earlier_failure()) return f;
     if (const int q = cut_length(c, xg::kNormalSum, nstreams, n)) {
         bool ran = false;
         const xg_status st = xg::cut_generate(c, xg::kNormalSum, first, nstreams, n, d_sums, 0, q, &ran);
@@ -601,6 +619,7 @@ xg_status xg_autotune(xg_ctx* ctx, xg_type type, uint32_t nstreams, uint64_t n_p
     uint64_t nt = std::min<uint64_t>(n_per_stream, std::max<uint64_t>(256, (uint64_t(1) << 28) / nstreams));
     nt = align_up(nt, 64);
     std::lock_guard<std::mutex> lk(c->mu);
+    if (xg_status f = c->earlier_failure()) return f;
     const size_t state_bytes = (size_t)((char*)(c->st.pos + c->n) - (char*)c->state_mem);
     void* saved = nullptr;
     void* out = nullptr;

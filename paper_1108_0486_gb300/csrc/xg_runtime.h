@@ -55,7 +55,11 @@ struct xg_ctx {
     size_t jump_ws_bytes = 0;
 
     xg::CutWorkspace cut;
+    xg::TcStatus tc;   // of cut calls, jumps and substreams
 
+    // XG_EDEVICE, once, when a tensor-core kernel of an earlier call gave up
+    // waiting: looked at by every call that reads or advances streams.
+    xg_status earlier_failure();
     int pick_cfg(int kind, uint32_t nstreams, uint64_t n) const;
     xg::Store pick_store(int kind, int cfg, uint32_t nstreams, uint64_t n, const void* out, uint64_t ld) const;
     int pick_block(int kind, int cfg) const;

@@ -32,6 +32,7 @@ struct xg_w64_ctx {
     size_t staging_bytes = 0;
     uint64_t split_words = 0;   // cut calls: 0 automatic, 1 never, else the piece length
     xg::CutWorkspace cut;
+    xg::TcStatus tc;            // of cut calls, jumps and substreams
     // xg_w64_jump's workspace (grow-only, freed with the context): a call ends
     // synchronised, so that no use outlives it.  16384 streams, 404 us per jump
     // with an allocation per call, 148 us without
@@ -58,6 +59,15 @@ bool is_device_pointer(const void* p)
         return false;
     }
     return attr.type == cudaMemoryTypeDevice || attr.type == cudaMemoryTypeManaged;
+}
+
+// XG_EDEVICE, once, when a tensor-core kernel of an earlier call gave up
+// waiting: looked at by every call that reads or advances streams.
+xg_status earlier_failure(xg_w64_ctx* c)
+{
+    return c->tc.take() ? fail(XG_EDEVICE, "a tensor-core kernel of this context gave up waiting: the outputs of that "
+                                           "call and the streams it advanced are not valid")
+                        : XG_OK;
 }
 
 // Without a tuned choice, one warp per stream: the fastest shape for both
@@ -127,7 +137,7 @@ xg_status generate_cut(xg_w64_ctx* c, int kind, uint32_t first, uint32_t nstream
                   "window layout in 32-bit words");
     const uint32_t pieces = (uint32_t)((n + (uint64_t(1) << q) - 1) >> q);
     const xg::CutStreams streams{c->device, c->sm_count, xg::kJumpSetW64, reinterpret_cast<const uint32_t*>(c->st.win),
-                                 c->st.pend, reinterpret_cast<const uint32_t*>(c->st.weyl), 2};
+                                 c->st.pend, reinterpret_cast<const uint32_t*>(c->st.weyl), 2, &c->tc};
     xg::CutRings r{};
     xg_status st = xg::cut_prologue(c->cut, streams, first, nstreams, pieces, q, 0, c->stream, &r, ran);
     if (st != XG_OK || !*ran) return st;
@@ -145,7 +155,7 @@ xg_status generate_cut(xg_w64_ctx* c, int kind, uint32_t first, uint32_t nstream
     a.omega = c->weyl_on ? xg64::kOmega : 0;
     const cudaError_t e = xg64::launch_cut(kind, a, c->stream);
     if (e != cudaSuccess) return cuda_fail(e, "64-bit cut generation");
-    return c->cut.release(c->stream, r.tensor_cores);
+    return c->cut.release(c->stream);
 }
 
 // Host output: generate into one device buffer piece by piece and copy each
@@ -196,6 +206,7 @@ xg_status generate(xg_w64_ctx* c, int kind, uint32_t first, uint32_t nstreams, u
     if (ld > (UINT64_MAX / 16) / nstreams) return fail(XG_EINVAL, "output extent overflows");
     if (reinterpret_cast<uintptr_t>(out) & 7u) return fail(XG_EINVAL, "output must be 8-byte aligned");
     std::lock_guard<std::mutex> lk(c->mu);
+    if (xg_status f = earlier_failure(c)) return f;
     if (is_device_pointer(out)) {
         if (const int q = cut_length(c, kind, nstreams, n)) {
             bool ran = false;
@@ -204,7 +215,8 @@ xg_status generate(xg_w64_ctx* c, int kind, uint32_t first, uint32_t nstreams, u
         }
         return enqueue(c, kind, first, nstreams, n, out, ld);
     }
-    return to_host(c, kind, first, nstreams, n, out, ld);
+    const xg_status st = to_host(c, kind, first, nstreams, n, out, ld);
+    return st == XG_OK ? earlier_failure(c) : st;
 }
 
 }  // namespace
@@ -267,10 +279,11 @@ xg_status xg_w64_destroy(xg_w64_ctx* c)
     if (c->state_mem) cudaStreamSynchronize(c->stream);
     if (c->staging) cudaFree(c->staging);
     c->cut.destroy();
+    const xg_status failed = earlier_failure(c);
     if (c->jump_ws) cudaFree(c->jump_ws);
     if (c->state_mem) cudaFree(c->state_mem);
     delete c;
-    return XG_OK;
+    return failed;
 }
 
 xg_status xg_w64_set_stream(xg_w64_ctx* c, void* cuda_stream)
@@ -312,6 +325,7 @@ xg_status xg_w64_get_state(xg_w64_ctx* c, uint32_t stream, uint64_t* ring, uint6
     XG_CUDA(cudaMemcpyAsync(&pend, c->st.pend + stream, 4, cudaMemcpyDeviceToHost, c->stream), "get_state");
     XG_CUDA(cudaMemcpyAsync(&w, c->st.weyl + stream, 8, cudaMemcpyDeviceToHost, c->stream), "get_state");
     XG_CUDA(cudaStreamSynchronize(c->stream), "get_state");
+    if (xg_status f = earlier_failure(c)) return f;
     if (pend >= (uint32_t)xg64::kRingBase) return fail(XG_EDEVICE, "corrupt stream state (pend %u)", pend);
     std::memcpy(ring, win + xg64::kRingBase - pend, xg64::kR * 8);
     *weyl = w;
@@ -324,6 +338,7 @@ xg_status xg_w64_set_state(xg_w64_ctx* c, uint32_t stream, const uint64_t* ring,
     if (stream >= c->n) return fail(XG_EINVAL, "stream %u out of range", stream);
     if (!ring) return fail(XG_EINVAL, "null ring");
     std::lock_guard<std::mutex> lk(c->mu);
+    if (xg_status f = earlier_failure(c)) return f;
     uint64_t win[xg64::kWin] = {0};
     std::memcpy(win + xg64::kRingBase, ring, xg64::kR * 8);
     const uint32_t pend = 0;
@@ -378,6 +393,7 @@ xg_status xg_w64_jump(xg_w64_ctx* c, uint32_t first, uint32_t nstreams, uint64_t
     if ((uint64_t)first + nstreams > c->n) return fail(XG_EINVAL, "streams out of range");
     if (nstreams == 0 || words == 0) return XG_OK;
     std::lock_guard<std::mutex> lk(c->mu);
+    if (xg_status f = earlier_failure(c)) return f;
     cudaStream_t s = c->stream;
     int top = 63;
     while (!((words >> top) & 1)) --top;
@@ -394,7 +410,7 @@ xg_status xg_w64_jump(xg_w64_ctx* c, uint32_t first, uint32_t nstreams, uint64_t
         e = xg::gf2_jump_windows(c->device, xg::kJumpSetW64, words,
                                  xg::JumpWindows{reinterpret_cast<uint32_t*>(c->st.win + (size_t)first * xg64::kWin),
                                                  c->st.pend + first, 2},
-                                 nstreams, static_cast<uint8_t*>(c->jump_ws), c->sm_count, s, &st);
+                                 nstreams, static_cast<uint8_t*>(c->jump_ws), c->tc, c->sm_count, s, &st);
         if (e == cudaSuccess) e = xg64::launch_finish_jump(c->st, first, nstreams, words, omega, s);
     } else {
         // one allocation: rings[0, n) hold the states, rings[n, 2n) the second
@@ -414,7 +430,7 @@ xg_status xg_w64_jump(xg_w64_ctx* c, uint32_t first, uint32_t nstreams, uint64_t
         bool hi = false;
         if (e == cudaSuccess)
             e = xg::gf2_jump_states(c->device, xg::kJumpSetW64, words, rings32, nstreams, lo_idx,
-                                    reinterpret_cast<uint8_t*>(ws + work_off), c->sm_count, s, &st, &hi);
+                                    reinterpret_cast<uint8_t*>(ws + work_off), c->tc, c->sm_count, s, &st, &hi);
         if (e == cudaSuccess)
             e = xg64::launch_scatter_rings(c->st, first, nstreams, hi ? rings + (size_t)nstreams * xg64::kR : rings,
                                            words, omega, s);
@@ -422,9 +438,7 @@ xg_status xg_w64_jump(xg_w64_ctx* c, uint32_t first, uint32_t nstreams, uint64_t
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (st != XG_OK) return st;
     if (e != cudaSuccess) return cuda_fail(e, "xg_w64_jump");
-    if ((in_place || xg::gf2_apply_scratch(c->device, nstreams)) && xg::gf2_tc_take_failure())
-        return fail(XG_EDEVICE, "xg_w64_jump: a tensor-core kernel gave up waiting; the streams are not valid");
-    return XG_OK;
+    return earlier_failure(c);
 }
 
 xg_status xg_w64_seed_substreams(xg_w64_ctx* c, uint32_t first, uint32_t count, uint32_t seed,
@@ -478,7 +492,7 @@ xg_status xg_w64_seed_substreams(xg_w64_ctx* c, uint32_t first, uint32_t count, 
     for (int b = 0; b < steps && e == cudaSuccess; ++b) {
         const uint32_t lo = 1u << b, hi = (uint32_t)std::min<uint64_t>((uint64_t)lo << 1, count);
         e = xg::gf2_apply(c->device, xg::kJumpSetW64, q + b, rings32, hi - lo, iota, iota + lo, tc_scratch,
-                          c->sm_count, s, &st, true);
+                          c->tc, c->sm_count, s, &st, true);
     }
     if (e == cudaSuccess)
         e = xg64::launch_substream_scatter(c->st, first, count, rings, d_w0, q, c->weyl_on ? xg64::kOmega : 0, s);
@@ -486,9 +500,7 @@ xg_status xg_w64_seed_substreams(xg_w64_ctx* c, uint32_t first, uint32_t count, 
     cudaFreeAsync(ws, s);
     if (st != XG_OK) return st;
     if (e != cudaSuccess) return cuda_fail(e, "xg_w64_seed_substreams");
-    if (tc_bytes && xg::gf2_tc_take_failure())
-        return fail(XG_EDEVICE, "xg_w64_seed_substreams: a tensor-core kernel gave up waiting; the streams are not valid");
-    return XG_OK;
+    return earlier_failure(c);
 }
 
 xg_status xg_w64_transform_uniform_f64(xg_w64_ctx* c, const uint64_t* d_words, uint64_t n, double* d_out)
@@ -530,6 +542,7 @@ xg_status xg_w64_autotune(xg_w64_ctx* c, xg_w64_type type, uint32_t nstreams, ui
     uint64_t nt = std::min<uint64_t>(n_per_stream, std::max<uint64_t>(128, (uint64_t(1) << 26) / nstreams));
     nt = align_up(nt, 32);
     std::lock_guard<std::mutex> lk(c->mu);
+    if (xg_status f = earlier_failure(c)) return f;
     void* saved = nullptr;
     void* out = nullptr;
     cudaEvent_t e0 = nullptr, e1 = nullptr;

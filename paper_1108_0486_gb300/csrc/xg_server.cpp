@@ -220,6 +220,9 @@ struct Ticket {
     size_t bytes = 0;
     uint32_t slot = 0;
     uint32_t expected = 1;      // completion increments: 1, or the pieces it was cut into
+    // cut: the status word of its batch's jump prologue, which is set before the
+    // pieces start when their start rings are not valid (null: no tensor cores)
+    const volatile uint32_t* prologue = nullptr;
     std::atomic<int> state{0};  // kQueued, kRunning, kDone, kFailed, kCancelled
     // who owns a queued request: 0 = nobody yet, 1 = the scheduler took it
     // into a batch, 2 = xg_cancel took it (the one that swaps it from 0 wins)
@@ -503,8 +506,10 @@ public:
         if (t.state.load(std::memory_order_acquire) != kRunning) return false;
         volatile uint32_t* f = h_flags_ + t.slot;
         if (*f < t.expected) return false;
+        std::atomic_thread_fence(std::memory_order_acquire);   // the prologue's word after the flag
         int expect = kRunning;
-        if (t.state.compare_exchange_strong(expect, kDone)) t.t_done.store(now_ns());
+        const bool valid = !t.prologue || *t.prologue == 0;
+        if (t.state.compare_exchange_strong(expect, valid ? kDone : kFailed)) t.t_done.store(now_ns());
         return true;
     }
 
@@ -513,7 +518,7 @@ public:
         auto t = find(id);
         if (!t) return fail(XG_ENOTFOUND, "unknown ticket %llu", (unsigned long long)id);
         const bool d = check_flag(*t);
-        if (t->state.load() == kFailed) return fail(XG_EDEVICE, "ticket %llu failed: its batch did not run",
+        if (t->state.load() == kFailed) return fail(XG_EDEVICE, "ticket %llu failed: its batch did not run, or from wrong states",
                                                     (unsigned long long)id);
         if (t->state.load() == kCancelled)
             return fail(XG_ECANCELED, "ticket %llu was cancelled", (unsigned long long)id);
@@ -532,7 +537,7 @@ public:
                                                  (unsigned long long)id, timeout_ms);
             std::this_thread::yield();
         }
-        if (t->state.load() == kFailed) return fail(XG_EDEVICE, "ticket %llu failed: its batch did not run",
+        if (t->state.load() == kFailed) return fail(XG_EDEVICE, "ticket %llu failed: its batch did not run, or from wrong states",
                                                     (unsigned long long)id);
         if (t->state.load() == kCancelled)
             return fail(XG_ECANCELED, "ticket %llu was cancelled", (unsigned long long)id);
@@ -736,6 +741,7 @@ private:
                         trace_.push_back(TraceRec{(uint32_t)li, l.n_items, l.n_units, l.words, l.t_launch, l.t_host,
                                                   now_ns(), ms});
                     }
+                    l.launcher->status().take();   // the tickets have taken it over
                     l.busy = false;
                     l.inflight.clear();
                     l.words = 0;
@@ -800,6 +806,7 @@ private:
                 }
                 for (size_t j = 0; j < l.inflight.size(); ++j) {
                     l.inflight[j]->expected = lst == XG_OK ? units[j] : 1u;
+                    if (l.inflight[j]->expected > 1) l.inflight[j]->prologue = l.launcher->status().host();
                     l.inflight[j]->state.store(kRunning, std::memory_order_release);
                 }
                 if (lst != XG_OK) {
@@ -930,6 +937,7 @@ xg_status xg_server_start(xg_ctx* ctx, const xg_server_config* cfg)
     if (cfg) c = *cfg;
     std::lock_guard<std::mutex> lk(ctx->mu);
     cudaStreamSynchronize(ctx->stream);
+    if (xg_status st = ctx->earlier_failure()) return st;
     auto* s = new (std::nothrow) xg::Server(ctx);
     if (!s) return fail(XG_ENOMEM, "host allocation failed");
     if (xg_status st = s->start(c)) {

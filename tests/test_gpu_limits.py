@@ -1,0 +1,74 @@
+"""What calls do where something runs out -- a bounded wait, memory for the
+jump tables -- or goes on beside them: a capture, another CUDA stream.  Values
+against the CPU oracle or an undisturbed call, bit for bit."""
+import numpy as np
+import pytest
+
+import oracle as O
+from paper_1108_0486_gb300 import workloads as W
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("hear", ["whole call", "sum", "checkpoint", "jump", "batch", "close", "64-bit call", "64-bit close"])
+def test_wait_that_runs_out_in_a_cut_call_reaches_its_owner(hear, monkeypatch):
+    """One copy of a cut call's tensor-core prologue never starts (its waits
+    give up after 2 s): another context's jump and batch are right and hear
+    nothing of it, the next call on the failed context is refused, once, and
+    reseeded it is as good as new."""
+    from paper_1108_0486_gb300 import Streams, Streams64, XGError, _lib as L
+    wide = hear.startswith("64-bit")
+    n = 16 if wide else 64
+    seeds, n_other = W.seeds(n), 200
+    st = Streams64(n, seeds=seeds) if wide else Streams(n, seeds=seeds)
+    (st.set_split if wide else st.set_batch_split)(4096 if wide else 32768)
+    with Streams(n_other, seeds=W.seeds(n_other)) as other:
+        other.set_batch_split(4096)
+        torch.cuda.synchronize()
+        monkeypatch.setenv("XG_TC_TEST_STALL", "1")
+        st.u64(1 << 18) if wide else st.u32(1 << 18)
+        monkeypatch.delenv("XG_TC_TEST_STALL")
+        torch.cuda.synchronize()
+        other.jump(3)
+        outs = [torch.empty(32768, dtype=torch.int32, device="cuda") for _ in range(n_other)]
+        other.batch([(i, "u32", 32768, o) for i, o in enumerate(outs)])
+        got = other.u32(5)
+        for s in (0, n_other - 1):
+            w = O.streams(W.seeds(1, 1 + s), 3 + 32768 + 5)[0]
+            assert np.array_equal(outs[s].cpu().numpy().view(np.uint32), w[3:-5])
+            assert np.array_equal(got[s].cpu().numpy().view(np.uint32), w[-5:])
+    calls = {"whole call": lambda: st.u32(10), "sum": lambda: st.normal_sum(10), "checkpoint": lambda: st.checkpoint(),
+             "jump": lambda: st.jump(1), "batch": lambda: st.batch([(0, "u32", 32768, outs[0])]), "close": st.close,
+             "64-bit call": lambda: st.u64(10), "64-bit close": st.close}
+    with pytest.raises(XGError) as err:
+        calls[hear]()
+    assert err.value.status == L.XG_EDEVICE and "gave up waiting" in str(err.value)
+    if hear.endswith("close"):
+        assert st.ctx is None
+        return
+    st.seed(seeds)
+    got = (st.u64(70) if wide else st.u32(70)).cpu().numpy()
+    assert np.array_equal(got.view(np.uint64), O.streams64(seeds, 70)) if wide else \
+        np.array_equal(got.view(np.uint32), O.streams(seeds, 70))
+    st.close()
+
+
+def test_wait_that_runs_out_fails_the_servers_cut_requests(monkeypatch):
+    """The same in a server's batch: the request that was cut fails, the
+    uncut one of the batch and a later one are right."""
+    from paper_1108_0486_gb300 import Streams, XGError, _lib as L
+    seeds = W.seeds(3)
+    with Streams(3, seeds=seeds) as st:
+        monkeypatch.setenv("XG_TC_TEST_STALL", "1")
+        with st.serve(mem_cap_bytes=1 << 28, lanes=1) as srv:
+            cut, small = srv.submit_many([(0, "u32", 1 << 23), (1, "u32", 1000)])
+            with pytest.raises(XGError) as err:
+                srv.wait(cut, 60000)
+            assert err.value.status == L.XG_EDEVICE
+            monkeypatch.delenv("XG_TC_TEST_STALL")
+            got = srv.result(small, "u32", 1000).cpu().numpy().view(np.uint32)
+            assert np.array_equal(got, O.streams(seeds[1:2], 1000)[0])
+            late = srv.submit(2, "u32", 1 << 23)
+            got = srv.result(late, "u32", 1 << 23).cpu().numpy().view(np.uint32)
+            assert np.array_equal(got, O.streams(seeds[2:], 1 << 23)[0])
