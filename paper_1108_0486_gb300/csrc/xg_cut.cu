@@ -206,15 +206,18 @@ xg_status CutWorkspace::ensure(size_t want)
 xg_status CutWorkspace::acquire(cudaStream_t s)
 {
     if (!used) return XG_OK;
-    if (stream != s && cudaStreamWaitEvent(s, event, 0) != cudaSuccess)
-        return cuda_fail(cudaGetLastError(), "cut workspace");
+    unsigned long long id = 0;
+    cudaError_t e = cudaStreamGetId(s, &id);
+    if (e == cudaSuccess && id != stream_id) e = cudaStreamWaitEvent(s, event, 0);
+    if (e != cudaSuccess) return cuda_fail(e, "cut workspace");
     return XG_OK;
 }
 
 xg_status CutWorkspace::release(cudaStream_t s)
 {
-    stream = s;
-    if (cudaEventRecord(event, s) != cudaSuccess) return cuda_fail(cudaGetLastError(), "cut workspace");
+    cudaError_t e = cudaStreamGetId(s, &stream_id);
+    if (e == cudaSuccess) e = cudaEventRecord(event, s);
+    if (e != cudaSuccess) return cuda_fail(e, "cut workspace");
     used = true;
     return XG_OK;
 }
@@ -291,7 +294,10 @@ xg_status cut_prologue(CutWorkspace& ws, const CutStreams& streams, uint32_t fir
             e = launch_gf2_apply_multi(mats[k], n_mats, rings, rings, m, src, dst, streams.sm_count, s, true,
                                        k + 1 < steps.n);
     }
-    if (e != cudaSuccess) return cuda_fail(e, "cut prologue");
+    if (e != cudaSuccess) {
+        ws.release(s);
+        return cuda_fail(e, "cut prologue");
+    }
     *out = CutRings{rings, weyl0, base + extra_off};
     return XG_OK;
 }
@@ -324,8 +330,8 @@ xg_status cut_generate(xg_ctx* c, int kind, uint32_t first, uint32_t nstreams, u
     if (sum && e == cudaSuccess)
         e = launch_dependent(true, dim3((nstreams + 1) / 2), dim3(64), c->stream, cut_sum_kernel,
                              reinterpret_cast<const float*>(r.extra), pieces, nstreams, static_cast<float*>(out));
-    if (e != cudaSuccess) return cuda_fail(e, "cut generation");
-    return c->cut.release(c->stream);
+    st = c->cut.release(c->stream);
+    return e == cudaSuccess ? st : cuda_fail(e, "cut generation");
 }
 
 }  // namespace xg

@@ -24,17 +24,19 @@ int cut_choose(int kind, uint32_t nstreams, uint64_t n, int sm_count, uint64_t f
 
 // A context's workspace for cut calls (grow-only, freed with the context).
 // Used on the context's stream of the moment: the event follows the last use,
-// and a use on another stream waits for it.
+// and a use on another stream waits for it.  Streams are told apart by their
+// ids: a handle may name another stream later (one made after it was
+// destroyed, or another thread's per-thread default stream).
 struct CutWorkspace {
     void* mem = nullptr;
     size_t bytes = 0;
     cudaEvent_t event = nullptr;
-    cudaStream_t stream = nullptr;
-    bool used = false;   // the event has been recorded
+    unsigned long long stream_id = 0;   // of the last use
+    bool used = false;                  // the event has been recorded
 
     xg_status ensure(size_t want);
     xg_status acquire(cudaStream_t s);   // before the first launch that uses it
-    xg_status release(cudaStream_t s);   // after the last
+    xg_status release(cudaStream_t s);   // after the last one that was enqueued
     void destroy();
 };
 

@@ -154,8 +154,8 @@ xg_status generate_cut(xg_w64_ctx* c, int kind, uint32_t first, uint32_t nstream
     a.weyl0 = reinterpret_cast<const uint64_t*>(r.weyl0);
     a.omega = c->weyl_on ? xg64::kOmega : 0;
     const cudaError_t e = xg64::launch_cut(kind, a, c->stream);
-    if (e != cudaSuccess) return cuda_fail(e, "64-bit cut generation");
-    return c->cut.release(c->stream);
+    st = c->cut.release(c->stream);
+    return e == cudaSuccess ? st : cuda_fail(e, "64-bit cut generation");
 }
 
 // Host output: generate into one device buffer piece by piece and copy each

@@ -72,3 +72,24 @@ def test_wait_that_runs_out_fails_the_servers_cut_requests(monkeypatch):
             late = srv.submit(2, "u32", 1 << 23)
             got = srv.result(late, "u32", 1 << 23).cpu().numpy().view(np.uint32)
             assert np.array_equal(got, O.streams(seeds[2:], 1 << 23)[0])
+
+
+def test_cut_calls_on_two_streams_of_one_handle():
+    """Cut calls of one context from two threads in turn on their per-thread
+    default streams: two streams with the same handle, which nothing else
+    orders (the calls are on disjoint streams of the context)."""
+    from concurrent.futures import ThreadPoolExecutor
+    from paper_1108_0486_gb300 import Streams, _lib as L
+    per_thread = 2   # cudaStreamPerThread
+    n, calls = 1 << 20, 12
+    outs = [torch.empty((1, n), dtype=torch.int32, device="cuda") for _ in range(calls)]
+    with Streams(2, seeds=W.seeds(2)) as st, ThreadPoolExecutor(1) as a, ThreadPoolExecutor(1) as b:
+        torch.cuda.synchronize()
+        L.xg_set_stream(st.ctx, per_thread)
+        for k, out in enumerate(outs):
+            (a, b)[k % 2].submit(st.u32, n, first=k % 2, count=1, out=out).result()
+        torch.cuda.synchronize()
+        L.xg_set_stream(st.ctx, torch.cuda.current_stream().cuda_stream)
+        for s in range(2):
+            got = torch.cat(outs[s::2], 1).cpu().numpy().view(np.uint32)[0]
+            assert np.array_equal(got, O.streams(W.seeds(1, 1 + s), n * calls // 2)[0])
