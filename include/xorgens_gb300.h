@@ -328,8 +328,11 @@ typedef struct {
  * batches, and long requests are cut into fewer, longer pieces (jump-ahead
  * work only pays while the GPU would otherwise idle).  Each result is identical
  * to the same request run alone.  Start-up allocates the pool, each lane's
- * buffers and the jump-ahead powers (about 70 MiB) so that serving itself
- * does not allocate.  A request whose batch fails to launch is
+ * buffers (for max_batch calls or pieces, at most 2048 pieces) and the
+ * jump-ahead matrices that requests within the cap need (about 0.7 GiB with
+ * the default cap, kept until the process exits; see xg_jump) so that serving
+ * itself does not allocate; a batch of more pieces grows its lane's buffers.
+ * A request whose batch fails to launch is
  * reported as XG_EDEVICE by xg_poll / xg_wait and leaves its stream where it
  * was; the server keeps serving.  (For testing that path without a GPU
  * fault, the environment variable XG_INJECT_LAUNCH_FAILURES=N, read at

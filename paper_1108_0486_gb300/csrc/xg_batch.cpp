@@ -313,8 +313,9 @@ xg_status BatchLauncher::grow_jump(size_t want)
 
 xg_status BatchLauncher::reserve_jump(uint32_t pieces, uint32_t pairs)
 {
-    // the layout of prologue(): rings, weyls, streams, skips, pair lists,
-    // then the tensor-core operand of one doubling step (at most all pieces)
+    (void)tc_.device();
+    // the layout of prologue(): rings, weyls, streams, skips, step lists,
+    // then the tensor-core operand of one step (at most all pieces)
     return grow_jump((size_t)pieces * (512 + 4 + 4 + 8 + 64) + (size_t)pairs * 8 + 4096 + gf2_tc_scratch_bytes(pieces));
 }
 

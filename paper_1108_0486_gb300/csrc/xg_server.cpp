@@ -333,12 +333,7 @@ public:
             // room for requests cut into pieces, so the first ones do not allocate
             if (xg_status s = l.launcher->reserve_jump(2048, 4096)) return fail(s, "server: jump buffers");
         }
-        // the jump powers a cut request can need (pieces of 2^15..2^22 words,
-        // calls up to 2^32 words), built now rather than on the first request
-        for (int k = 0; k <= 32; ++k) {
-            xg_status st = XG_OK;
-            if (!jump_matrix(c_->device, (int)c_->param_set, k, lanes_[0].stream, &st)) return st;
-        }
+        if (xg_status s = build_matrices()) return s;
         // host-side fault injection for tests: the first N batch launches
         // report failure without reaching the GPU
         if (const char* f = std::getenv("XG_INJECT_LAUNCH_FAILURES")) inject_failures_ = std::atoi(f);
@@ -657,6 +652,32 @@ private:
         uint64_t words, t_launch_ns, host_ns, t_seen_done_ns;
         float gpu_ms;
     };
+
+    // The matrices that cut requests can need, built now rather than by the
+    // first request of each length: the powers up to 2^32 and, for the steps of
+    // the prologue (pieces of 2^q words, q >= 15 or as set), the multiples
+    // M^(j 2^e), j = 1 .. 7, with their FP4 copies, as far as a request of the
+    // whole cap goes.  Without the memory for these, requests are served with
+    // what there is.
+    xg_status build_matrices()
+    {
+        const int family = (int)c_->param_set;
+        xg_status st = XG_OK;
+        for (int k = 0; k <= 32; ++k)
+            if (!jump_matrix(c_->device, family, k, lanes_[0].stream, &st)) return st;
+        if (c_->split_words == 1) return XG_OK;
+        const uint64_t words = cfg_.mem_cap_bytes / 4;
+        int q = 0;
+        while ((uint64_t(1) << q) < (c_->split_words ? c_->split_words : BatchLauncher::kMinPiece)) ++q;
+        // the automatic length varies, so every exponent; a set one, every step's
+        const int step = c_->split_words ? 3 : 1;
+        for (int e = q; e < 60 && (uint64_t(1) << e) < words; e += step)
+            for (int j = 1; j <= 7 && (uint64_t)j << e < words; ++j)
+                if (!(gf2_use_tc(c_->device, ~0u) ? (const void*)jump_matrix_tc(c_->device, family, j, e, lanes_[0].stream, &st)
+                                                  : jump_matrix_multiple(c_->device, family, j, e, lanes_[0].stream, &st)))
+                    return st == XG_ENOMEM ? XG_OK : st;
+        return XG_OK;
+    }
 
     // Shortest piece a new batch may cut its calls into, from the words the
     // GPU already has in flight: cutting shortens one call's critical path

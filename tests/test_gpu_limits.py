@@ -93,3 +93,34 @@ def test_cut_calls_on_two_streams_of_one_handle():
         for s in range(2):
             got = torch.cat(outs[s::2], 1).cpu().numpy().view(np.uint32)[0]
             assert np.array_equal(got, O.streams(W.seeds(1, 1 + s), n * calls // 2)[0])
+
+
+FIRST_BURSTS = """
+import sys
+import torch
+from paper_1108_0486_gb300 import Streams, workloads as W
+with Streams(12, seeds=W.seeds(12)) as st:
+    st.u32(10)
+    with st.serve(mem_cap_bytes=5 << 28, max_batch=2048, lanes=8) as srv:
+        torch.cuda.synchronize()
+        free = torch.cuda.mem_get_info()[0]
+        # pieces of 2^15 words, and of 2^16 beside enough words in flight; at most 2048 at once
+        for sizes in ([1 << 24], [3 << 24, 1 << 24], [1 << 24, 1 << 22, 1 << 18], [1 << 20] * 10):
+            tickets = [srv.submit(i, "u32", n) for i, n in enumerate(sizes)]
+            for t in tickets:
+                srv.wait(t, 60000)
+                srv.release(t)
+        print(free - torch.cuda.mem_get_info()[0])
+"""
+
+
+def test_first_cut_requests_allocate_nothing():
+    """In a process of its own, where no matrix exists before the server:
+    free device memory stays as it is from the server's start through the
+    first requests of several lengths, cut into few and many pieces."""
+    import subprocess
+    import sys
+    out = subprocess.run([sys.executable, "-c", FIRST_BURSTS], capture_output=True, text=True,
+                         cwd=W.__file__.rsplit("/", 2)[0])
+    assert out.returncode == 0, out.stderr
+    assert out.stdout.strip() == "0"
