@@ -272,7 +272,12 @@ xg_status xg_set_batch_split(xg_ctx* ctx, uint64_t piece_words);
  * the jump is a product of precomputed powers M^(2^k) of its transition
  * matrix, one per set bit of `words`; the Weyl word advances by
  * words * omega).  The first use of each power builds it on the GPU (2 MiB
- * each, kept until exit).  Synchronous.  Useful for provably disjoint
+ * each, kept until exit); jumps of 8 and more streams by one power on the
+ * tensor cores, and the calls and batches that are cut, also build matrices
+ * derived from the powers (2 and 8 MiB each), which are kept too, in at most
+ * 3 GiB per device.  The environment variable XG_JUMP_TABLE_MIB=<n> replaces
+ * that limit; past it, or where device memory has run out, calls do without
+ * new ones, by slower paths with the same results.  Synchronous.  Useful for provably disjoint
  * substreams: stream i jumped by i * 2^64 would never overlap, here by any
  * 64-bit distance. */
 xg_status xg_jump(xg_ctx* ctx, uint32_t first, uint32_t nstreams, uint64_t words);

@@ -326,26 +326,29 @@ xg_status BatchLauncher::reserve_jump(uint32_t pieces, uint32_t pairs)
 // all seven: the sources are listed by how many results they have, most
 // first, so that matrix j applies to a prefix of them.  256 requests of a
 // server burst took 6 doubling launches of 15 to 25 us each, a batch of 4096
-// calls five of 25 to 37 us.
-xg_status BatchLauncher::prologue(xg_ctx* c, cudaStream_t s)
+// calls five of 25 to 37 us.  Radix 2 (log2_radix = 1) needs the powers alone,
+// one per step.  XG_ENOMEM, with nothing enqueued, where a matrix is not to be
+// had; a step whose FP4 copies are missing runs on the table kernel.
+xg_status BatchLauncher::prologue(xg_ctx* c, cudaStream_t s, int log2_radix)
 {
     const uint32_t P = (uint32_t)plan_.pieces.size();
     if (P == 0) return XG_OK;
-    constexpr int kSteps = 11;   // 8^11 > 2^32 pieces
+    const uint64_t radix = uint64_t(1) << log2_radix;
+    constexpr int kSteps = 33;   // 2^32 pieces and more
     constexpr uint32_t kMats = 7;
     static_assert(kMats <= (uint32_t)kMaxMats && kMats <= (uint32_t)kGf2TcMaxMats, "matrices per launch");
     uint32_t with[kSteps][kMats + 1] = {};   // sources with exactly d results
     int nsteps = 0;
-    // f(step, piece, results, 8^step) for every source
+    // f(step, piece, results, radix^step) for every source
     auto for_sources = [&](auto&& f) {
         for (uint32_t k0 = 0, k1; k0 < P; k0 = k1) {
             k1 = k0 + 1;
             while (k1 < P && plan_.piece_index[k1] != 0) ++k1;
             const uint64_t K = k1 - k0;
             int step = 0;
-            for (uint64_t have = 1; have < K; have *= 8, ++step)
+            for (uint64_t have = 1; have < K; have *= radix, ++step)
                 for (uint64_t m = 0; m < have && m + have < K; ++m)
-                    f(step, k0 + (uint32_t)m, (uint32_t)std::min<uint64_t>(kMats, (K - 1 - m) / have), (uint32_t)have);
+                    f(step, k0 + (uint32_t)m, (uint32_t)std::min<uint64_t>(radix - 1, (K - 1 - m) / have), (uint32_t)have);
             nsteps = std::max(nsteps, step);
         }
     };
@@ -363,7 +366,7 @@ xg_status BatchLauncher::prologue(xg_ctx* c, cudaStream_t s)
             counts[k][j] = with[k][j + 1] + (j + 1 < kMats ? counts[k][j + 1] : 0u);
             results += counts[k][j];
         }
-        use_tc[k] = gf2_use_tc(c->device, results);
+        use_tc[k] = gf2_use_tc(c->device, results) && tc_.device();
         if (use_tc[k]) most = std::max(most, counts[k][0]);
     }
     // device buffer: rings | weyls | gather streams | gather skips | lists
@@ -380,7 +383,7 @@ xg_status BatchLauncher::prologue(xg_ctx* c, cudaStream_t s)
     char* hb = static_cast<char*>(h_jstage_);
     char* db = static_cast<char*>(d_jbuf_);
     // every piece's Weyl word comes from the gather (its own skip); its ring
-    // from the gather (m = 0) or a doubling step
+    // from the gather (m = 0) or a step
     std::memcpy(hb + off_streams, plan_.piece_stream.data(), (size_t)P * 4);
     std::memcpy(hb + off_skip, plan_.piece_skip.data(), (size_t)P * 8);
     // per step: its sources, then each matrix's destinations
@@ -409,19 +412,24 @@ xg_status BatchLauncher::prologue(xg_ctx* c, cudaStream_t s)
     // matrices first (the first use builds them and synchronises)
     const uint64_t* mats[kSteps][kMats] = {};
     const uint8_t* tc_mats[kSteps][kMats] = {};
-    for (int k = 0; k < nsteps; ++k)
-        for (uint32_t j = 0; j < kMats && counts[k][j]; ++j) {
-            xg_status st = XG_OK;
-            const int e = plan_.split_log2 + 3 * k;
-            if (use_tc[k]) tc_mats[k][j] = jump_matrix_tc(c->device, (int)c->param_set, (int)j + 1, e, s, &st);
-            else mats[k][j] = jump_matrix_multiple(c->device, (int)c->param_set, (int)j + 1, e, s, &st);
-            if (!tc_mats[k][j] && !mats[k][j]) return st;
+    for (int k = 0; k < nsteps; ++k) {
+        xg_status st = XG_OK;
+        const int family = (int)c->param_set, e = plan_.split_log2 + log2_radix * k;
+        for (uint32_t j = 0; use_tc[k] && j < kMats && counts[k][j]; ++j) {
+            tc_mats[k][j] = jump_matrix_tc(c->device, family, (int)j + 1, e, s, &st);
+            if (!tc_mats[k][j] && st != XG_ENOMEM) return st;
+            if (!tc_mats[k][j]) use_tc[k] = false;
         }
+        for (uint32_t j = 0; !use_tc[k] && j < kMats && counts[k][j]; ++j) {
+            mats[k][j] = jump_matrix_multiple(c->device, family, (int)j + 1, e, s, &st);
+            if (!mats[k][j]) return st;
+        }
+    }
     if (cudaMemcpyAsync(db + off_streams, hb + off_streams, off_lists + o * 4 - off_streams, cudaMemcpyHostToDevice,
                         s) != cudaSuccess)
         return XG_ECUDA;
     // piece 0 of each call gets its stream's ring, the others (nonzero skip)
-    // a zero ring, into which their doubling step XORs
+    // a zero ring, into which their step XORs
     if (launch_gather_rings(c->st, reinterpret_cast<const uint32_t*>(db + off_streams), P,
                             reinterpret_cast<uint32_t*>(db + off_rings),
                             reinterpret_cast<const uint64_t*>(db + off_skip),
@@ -456,9 +464,16 @@ xg_status BatchLauncher::launch(xg_ctx* c, const HostItem* items, uint32_t n, cu
     // the jump prologue needs only the pieces: enqueue it before ordering the
     // heads, so that the GPU starts while the host finishes the plan
     plan_units(items, n, choose_piece_len(c, items, n, min_piece), c->n, plan_);
-    const uint32_t nu = (uint32_t)plan_.units.size();
+    uint32_t nu = (uint32_t)plan_.units.size();
     if (xg_status st = reserve(c, nu)) return st;
-    if (xg_status st = prologue(c, s)) return st;
+    xg_status jump = prologue(c, s, 3);
+    if (jump == XG_ENOMEM) jump = prologue(c, s, 1);
+    if (jump == XG_ENOMEM) {   // the uncut batch needs no matrices
+        plan_units(items, n, 0, c->n, plan_);
+        nu = (uint32_t)plan_.units.size();
+        jump = XG_OK;
+    }
+    if (jump) return jump;
     plan_order(plan_);
     // group only units of at most 1/8 of a resident warp's share of the
     // batch (XG_BATCH_GROUP_MAX_WORDS=<n> sets the limit instead)

@@ -85,7 +85,7 @@ public:
 
 private:
     xg_status build_graph(xg_ctx* c);
-    xg_status prologue(xg_ctx* c, cudaStream_t s);
+    xg_status prologue(xg_ctx* c, cudaStream_t s, int log2_radix);
     xg_status grow_jump(size_t want);
     uint64_t choose_piece_len(const xg_ctx* c, const HostItem* items, uint32_t n, uint64_t min_piece) const;
     uint32_t capacity_ = 0;

@@ -25,6 +25,7 @@
 // Products of matrices are therefore applications to 32 (64) states and one
 // pass that writes the columns, instead of applications to 4096 states.
 #include <algorithm>
+#include <atomic>
 #include <cstdlib>
 #include <cstring>
 #include <mutex>
@@ -366,6 +367,31 @@ struct Tables {
 };
 std::mutex g_tab_mu;
 Tables g_tabs[64][3];  // per device, per matrix family
+
+// Device memory of the odd multiples and the FP4 copies, which 64 exponents of
+// three families would take 7 GiB of; the limit is what the powers' FP8 copies
+// of an earlier form could take.
+std::atomic<size_t> g_derived[64];
+
+size_t derived_limit()
+{
+    const char* v = std::getenv("XG_JUMP_TABLE_MIB");
+    return v ? (size_t)std::strtoull(v, nullptr, 10) << 20 : size_t(3) << 30;
+}
+
+cudaError_t derived_alloc(int device, void** p, size_t bytes)
+{
+    cudaError_t e = cudaErrorMemoryAllocation;
+    if (g_derived[device].fetch_add(bytes) + bytes <= derived_limit()) e = cudaMalloc(p, bytes);
+    if (e != cudaSuccess) g_derived[device].fetch_sub(bytes);
+    return e;
+}
+
+void derived_free(int device, void* p, size_t bytes)
+{
+    cudaFree(p);
+    g_derived[device].fetch_sub(bytes);
+}
 }  // namespace
 
 // out = A B (powers of one matrix): A applied to B's newest columns.
@@ -454,16 +480,17 @@ const uint64_t* jump_matrix_multiple(int device, int param_set, int j, int k, cu
     uint64_t*& C = T.odd[(j - 3) / 2][k];
     if (C) return C;
     void* p = nullptr;
-    cudaError_t e = cudaMalloc(&p, (size_t)kBits * kWords64 * 8);
+    const size_t bytes = (size_t)kBits * kWords64 * 8;
+    cudaError_t e = derived_alloc(device, &p, bytes);
     if (e != cudaSuccess) {
         cudaGetLastError();
-        *st = fail(XG_ENOMEM, "jump tables: cudaMalloc(2 MiB) failed for %d times power %d", j, k);
+        *st = fail(XG_ENOMEM, "jump tables: no 2 MiB for %d times power %d", j, k);
         return nullptr;
     }
     e = multiply_matrices(device, param_set, T, a, b, static_cast<uint64_t*>(p), s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);  // other CUDA streams may use it next
     if (e != cudaSuccess) {
-        cudaFree(p);
+        derived_free(device, p, bytes);
         *st = cuda_fail(e, "jump table build");
         return nullptr;
     }
@@ -489,16 +516,16 @@ const uint8_t* jump_matrix_tc(int device, int family, int j, int k, cudaStream_t
     uint8_t*& A = g_tc_mats[device][family][j / 2][k];
     if (A) return A;
     void* p = nullptr;
-    cudaError_t e = cudaMalloc(&p, kGf2TcMatrixBytes);
+    cudaError_t e = derived_alloc(device, &p, kGf2TcMatrixBytes);
     if (e != cudaSuccess) {
         cudaGetLastError();
-        *st = fail(XG_ENOMEM, "jump tables: cudaMalloc(8 MiB) failed for the FP4 power %d", k);
+        *st = fail(XG_ENOMEM, "jump tables: no 8 MiB for the FP4 copy of %d times power %d", j, k);
         return nullptr;
     }
     e = gf2_tc_expand_matrix(C, static_cast<uint8_t*>(p), s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);  // other CUDA streams may use it next
     if (e != cudaSuccess) {
-        cudaFree(p);
+        derived_free(device, p, kGf2TcMatrixBytes);
         *st = cuda_fail(e, "jump tables: FP4 expansion");
         return nullptr;
     }
@@ -527,13 +554,13 @@ cudaError_t gf2_apply(int device, int family, int k, uint32_t* rings, uint32_t n
 {
     *st = XG_OK;
     if (n == 0) return cudaSuccess;
-    if (scratch && gf2_use_tc(device, n)) {
+    if (scratch && gf2_use_tc(device, n) && tc.device()) {
         const uint8_t* A = jump_matrix_tc(device, family, 1, k, s, st);
-        if (!A) return cudaErrorMemoryAllocation;
-        return gf2_tc_apply(device, &A, 1, TcStates{rings, kGf2Words, d_src, nullptr, 0}, n, rings, kGf2Words, d_dst, scratch,
+        if (!A && *st != XG_ENOMEM) return cudaErrorUnknown;   // with *st
+        if (A) return gf2_tc_apply(device, &A, 1, TcStates{rings, kGf2Words, d_src, nullptr, 0}, n, rings, kGf2Words, d_dst, scratch,
                             tc, s);
     }
-    const uint64_t* C = jump_matrix(device, family, k, s, st);
+    const uint64_t* C = jump_matrix(device, family, k, s, st);   // *st is XG_OK again
     if (!C) return cudaErrorMemoryAllocation;
     cudaError_t e = dst_zeroed ? cudaSuccess : zero_rings(rings, d_dst, n, s);
     if (e == cudaSuccess) e = launch_gf2_apply_pairs(C, rings, rings, n, d_src, d_dst, sm_count, s);
@@ -565,13 +592,12 @@ static size_t product_bytes(uint64_t words)
 // 61 / 62 / 62 / 63 against 65 / 66 / 70 / 80.
 constexpr uint32_t kInPlaceStreams = 8;
 
-size_t gf2_jump_work_bytes(int device, uint32_t n, uint64_t words)
+size_t gf2_jump_work_bytes(int device, uint32_t n, uint64_t words, bool in_place)
 {
+    const size_t product = jump_combines(words, n) ? product_bytes(words) : 0;
+    if (!in_place) return product ? product : gf2_apply_scratch(device, n);
     // the tensor-core operand, then the product's work area and its FP4 copy
-    const bool in_place = gf2_jump_in_place(device, n, words);
-    size_t b = ((in_place ? gf2_tc_scratch_bytes(n) : gf2_apply_scratch(device, n)) + 255) / 256 * 256;
-    if (jump_combines(words, n)) b += product_bytes(words) + (in_place ? kGf2TcMatrixBytes : 0);
-    return b;
+    return (gf2_tc_scratch_bytes(n) + 255) / 256 * 256 + (product ? product + kGf2TcMatrixBytes : 0);
 }
 
 // The product of the powers in `words` in column form (in w, product_bytes):
@@ -632,9 +658,12 @@ static cudaError_t power_product(int device, int family, uint64_t words, uint8_t
     return e;
 }
 
-bool gf2_jump_in_place(int device, uint32_t n, uint64_t words)
+bool gf2_jump_in_place(int device, int family, uint32_t n, uint64_t words, TcStatus& tc, cudaStream_t s)
 {
-    return gf2_use_tc(device, n, kInPlaceStreams) && (__builtin_popcountll(words) == 1 || jump_combines(words, n));
+    if (!gf2_use_tc(device, n, kInPlaceStreams) || !tc.device()) return false;
+    xg_status st = XG_OK;
+    if (__builtin_popcountll(words) == 1) return jump_matrix_tc(device, family, 1, __builtin_ctzll(words), s, &st) != nullptr;
+    return jump_combines(words, n);
 }
 
 cudaError_t gf2_jump_windows(int device, int family, uint64_t words, const JumpWindows& win, uint32_t n, uint8_t* work,
@@ -668,9 +697,8 @@ cudaError_t gf2_jump_states(int device, int family, uint64_t words, uint32_t* ri
     *result_hi = false;
     const uint32_t* lo = d_idx;       // 0 .. n-1
     const uint32_t* hi = d_idx + n;   // n .. 2n-1
-    const size_t sbytes = gf2_apply_scratch(device, n);
     if (!jump_combines(words, n)) {
-        uint8_t* scratch = sbytes ? work : nullptr;
+        uint8_t* scratch = gf2_apply_scratch(device, n) ? work : nullptr;
         bool in_lo = true;
         for (int k = 0; k < 64; ++k) {
             if (!((words >> k) & 1)) continue;
@@ -683,7 +711,7 @@ cudaError_t gf2_jump_states(int device, int family, uint64_t words, uint32_t* ri
         return cudaSuccess;
     }
     const uint64_t* P = nullptr;
-    cudaError_t e = power_product(device, family, words, work + (sbytes + 255) / 256 * 256, sm_count, s, &P, st);
+    cudaError_t e = power_product(device, family, words, work, sm_count, s, &P, st);
     if (e == cudaSuccess) e = zero_rings(rings, hi, n, s);
     if (e == cudaSuccess) e = launch_gf2_apply_pairs(P, rings, rings, n, lo, hi, sm_count, s);
     *result_hi = true;
@@ -746,11 +774,10 @@ extern "C" xg_status xg_jump(xg_ctx* ctx, uint32_t first, uint32_t nstreams, uin
     for (int k = 0; k <= top; ++k)
         if (((words >> k) & 1) && !jump_matrix(ctx->device, (int)ctx->param_set, k, s, &st)) return st;
     const uint32_t omega = ctx->weyl_on ? 0x9E3779B9u : 0u;
-    const size_t wbytes = gf2_jump_work_bytes(ctx->device, nstreams, words);
-    const bool in_place = gf2_jump_in_place(ctx->device, nstreams, words);
+    const bool in_place = gf2_jump_in_place(ctx->device, (int)ctx->param_set, nstreams, words, ctx->tc, s) &&
+                          ctx->ensure_jump_ws(gf2_jump_work_bytes(ctx->device, nstreams, words, true)) == XG_OK;
     cudaError_t e;
     if (in_place) {
-        if (xg_status g = ctx->ensure_jump_ws(wbytes)) return g;
         e = gf2_jump_windows(ctx->device, (int)ctx->param_set, words,
                              JumpWindows{ctx->st.win + (size_t)first * kWin, ctx->st.pend + first, 1}, nstreams,
                              static_cast<uint8_t*>(ctx->jump_ws), ctx->tc, ctx->sm_count, s, &st);
@@ -765,6 +792,7 @@ extern "C" xg_status xg_jump(xg_ctx* ctx, uint32_t first, uint32_t nstreams, uin
         const size_t rings_bytes = (size_t)2 * nstreams * kR * 4;
         const size_t ids_off = rings_bytes;
         const size_t work_off = (ids_off + (size_t)3 * nstreams * 4 + 255) / 256 * 256;
+        const size_t wbytes = gf2_jump_work_bytes(ctx->device, nstreams, words, false);
         if (xg_status g = ctx->ensure_jump_ws(work_off + wbytes)) return g;
         char* ws = static_cast<char*>(ctx->jump_ws);
         uint32_t* rings = reinterpret_cast<uint32_t*>(ws);

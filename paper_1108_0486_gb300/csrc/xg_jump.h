@@ -43,7 +43,11 @@ cudaError_t launch_gf2_apply_multi(const uint64_t* const* C, int n_mats, const u
                                    bool dependent = false, bool early = true,
                                    const uint32_t* counts = nullptr);
 
-// M^(j 2^k) for 1 <= j <= 7, built on first use like jump_matrix.
+// M^(j 2^k) for 1 <= j <= 7, built on first use like jump_matrix.  The odd
+// multiples and the FP4 copies of a device take at most 3 GiB in all
+// (XG_JUMP_TABLE_MIB sets another limit); past it, and where the device has no
+// memory left, a new one is XG_ENOMEM, and the callers do without: jumps and
+// batches with the powers and the table kernel, cut calls as whole calls.
 const uint64_t* jump_matrix_multiple(int device, int param_set, int j, int k, cudaStream_t s, xg_status* st);
 
 // The same as the A operand of gf2_tc_apply.
@@ -59,8 +63,9 @@ size_t gf2_apply_scratch(int device, uint32_t n);
 
 // rings[d_dst[i]] = C_k rings[d_src[i]] for n pairs, C_k the power 2^k of
 // the matrix family (destinations distinct and not among the sources).  On
-// the tensor cores when gf2_use_tc(device, n) and scratch (gf2_apply_scratch
-// bytes) is given, else with the table kernel.  Asynchronous on s, except
+// the tensor cores when gf2_use_tc(device, n), scratch (gf2_apply_scratch
+// bytes) is given and the FP4 copy is to be had, else with the table kernel.
+// Asynchronous on s, except
 // that a power's first use builds it.  After synchronising, a caller that
 // may have used the tensor cores checks the status.  The table
 // kernel XORs into the destinations, so it zeroes them first unless the
@@ -71,18 +76,18 @@ cudaError_t gf2_apply(int device, int family, int k, uint32_t* rings, uint32_t n
 
 // Advance n states by `words` positions: M^words applied to rings[0, n),
 // with rings[n, 2n) as the second buffer (*result_hi: the result ended there)
-// and d_idx the identity list 0 .. 2n - 1.  With several set bits and more
-// than 64 states the powers are multiplied first and the product applied once.
-// work: gf2_jump_work_bytes(device, n, words) bytes of device memory,
-// 256-byte aligned (the tensor-core operand, and the product's work area when
-// the powers are multiplied first).  Not for jumps that gf2_jump_in_place takes.
-size_t gf2_jump_work_bytes(int device, uint32_t n, uint64_t words);
+// and d_idx the identity list 0 .. 2n - 1.  With several set bits (2, 4 or 7 by
+// the number of states) the powers are multiplied first and the product applied
+// once.  work: gf2_jump_work_bytes bytes of device memory, 256-byte aligned
+// (the tensor-core operand or the product's work area).
+size_t gf2_jump_work_bytes(int device, uint32_t n, uint64_t words, bool in_place);
 cudaError_t gf2_jump_states(int device, int family, uint64_t words, uint32_t* rings, uint32_t n,
                             const uint32_t* d_idx, uint8_t* work, TcStatus& tc, int sm_count, cudaStream_t s, xg_status* st,
                             bool* result_hi);
 
 // Whether a jump applies one matrix (a power, or the product of several) on
-// the tensor cores; then gf2_jump_windows reads the rings of n consecutive
+// the tensor cores (false too where there is no memory for a power's FP4 copy,
+// which is built here); then gf2_jump_windows reads the rings of n consecutive
 // streams in their windows and writes them back there, without pending words:
 // for 16384 streams it saves the copies of all rings out of the windows and
 // back (25 of 229 us).  The caller resets pend and advances the Weyl words.
@@ -92,7 +97,7 @@ struct JumpWindows {
     uint32_t* pend;   // of the first stream
     uint32_t word;    // 32-bit words per generator word
 };
-bool gf2_jump_in_place(int device, uint32_t n, uint64_t words);
+bool gf2_jump_in_place(int device, int family, uint32_t n, uint64_t words, TcStatus& tc, cudaStream_t s);
 cudaError_t gf2_jump_windows(int device, int family, uint64_t words, const JumpWindows& win, uint32_t n, uint8_t* work,
                              TcStatus& tc, int sm_count, cudaStream_t s, xg_status* st);
 

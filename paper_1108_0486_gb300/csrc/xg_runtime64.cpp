@@ -401,11 +401,10 @@ xg_status xg_w64_jump(xg_w64_ctx* c, uint32_t first, uint32_t nstreams, uint64_t
     for (int k = 0; k <= top; ++k)
         if (((words >> k) & 1) && !xg::jump_matrix(c->device, xg::kJumpSetW64, k, s, &st)) return st;
     const uint64_t omega = c->weyl_on ? xg64::kOmega : 0;
-    const size_t wbytes = xg::gf2_jump_work_bytes(c->device, nstreams, words);
-    const bool in_place = xg::gf2_jump_in_place(c->device, nstreams, words);
+    const bool in_place = xg::gf2_jump_in_place(c->device, xg::kJumpSetW64, nstreams, words, c->tc, s) &&
+                          ensure_jump_ws(c, xg::gf2_jump_work_bytes(c->device, nstreams, words, true)) == XG_OK;
     cudaError_t e;
     if (in_place) {
-        if (xg_status g = ensure_jump_ws(c, wbytes)) return g;
         // the windows as 32-bit words, two per word (layout checked in generate_cut)
         e = xg::gf2_jump_windows(c->device, xg::kJumpSetW64, words,
                                  xg::JumpWindows{reinterpret_cast<uint32_t*>(c->st.win + (size_t)first * xg64::kWin),
@@ -419,6 +418,7 @@ xg_status xg_w64_jump(xg_w64_ctx* c, uint32_t first, uint32_t nstreams, uint64_t
         // the jump's work area
         const size_t rings_bytes = (size_t)2 * nstreams * xg64::kR * 8;
         const size_t work_off = (rings_bytes + (size_t)3 * nstreams * 4 + 255) / 256 * 256;
+        const size_t wbytes = xg::gf2_jump_work_bytes(c->device, nstreams, words, false);
         if (xg_status g = ensure_jump_ws(c, work_off + wbytes)) return g;
         char* ws = static_cast<char*>(c->jump_ws);
         uint64_t* rings = reinterpret_cast<uint64_t*>(ws);

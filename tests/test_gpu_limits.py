@@ -124,3 +124,67 @@ def test_first_cut_requests_allocate_nothing():
                          cwd=W.__file__.rsplit("/", 2)[0])
     assert out.returncode == 0, out.stderr
     assert out.stdout.strip() == "0"
+
+
+WITHOUT_TABLES = """
+import sys
+import numpy as np
+import torch
+from paper_1108_0486_gb300 import Streams, Streams64, workloads as W
+torch.zeros(1, device="cuda")
+start = None
+rows = []
+for kind in (Streams, Streams64):
+    for n in (9, 300):
+        with kind(n, seeds=W.seeds(n)) as st:
+            draw = st.u64 if kind is Streams64 else st.u32
+            draw(77)
+            if start is None:
+                torch.cuda.synchronize()
+                start = torch.cuda.mem_get_info()[0]
+            st.jump(1 << 20)
+            rows.append(draw(70))
+            st.seed_substreams(5, 12)
+            rows.append(draw(70))
+    with kind(3, seeds=W.seeds(3)) as st:
+        (st.set_split if kind is Streams64 else st.set_batch_split)(4096)
+        rows += [(st.u64 if kind is Streams64 else st.u32)(1 << 18) for _ in range(2)]
+calls = (1, 9, 65, 600) + (13,) * 30
+with Streams(len(calls), seeds=W.seeds(len(calls))) as st:
+    st.set_batch_split(64)
+    for _ in range(2):
+        outs = [torch.zeros(64 * k + 5, dtype=torch.int32, device="cuda") for k in calls]
+        st.batch([(i, "u32", o.numel(), o) for i, o in enumerate(outs)])
+        rows += [torch.cat(outs), st.u32(9)]
+with Streams(2, seeds=W.seeds(2)) as st:
+    with st.serve(mem_cap_bytes=1 << 28, lanes=2) as srv:
+        tickets = [srv.submit(i % 2, "u32", 5 << 20) for i in range(4)]
+        rows += [srv.result(t, "u32", 5 << 20) for t in tickets]
+        rows = [r.cpu().numpy().reshape(-1) for r in rows]
+torch.cuda.synchronize()
+torch.cuda.empty_cache()
+print(start - torch.cuda.mem_get_info()[0])
+np.savez(sys.argv[1], *rows)
+"""
+
+
+def test_calls_without_memory_for_derived_tables(tmp_path):
+    """Jumps, substreams, cut calls, batches and requests where no odd multiple
+    and no FP4 copy of a power may be built, in a process where none exists: the
+    results of a process without the limit, and no more memory kept than the
+    powers (2 MiB, 33 in the 32-bit family, 24 in the other) and their scratch."""
+    import os
+    import subprocess
+    import sys
+    got = []
+    for limit in ("0", "3072"):
+        path = str(tmp_path / f"{limit}.npz")
+        out = subprocess.run([sys.executable, "-c", WITHOUT_TABLES, path], capture_output=True, text=True,
+                             cwd=W.__file__.rsplit("/", 2)[0], env=dict(os.environ, XG_JUMP_TABLE_MIB=limit))
+        assert out.returncode == 0, out.stderr
+        if limit == "0":
+            assert int(out.stdout) <= (57 * 2 + 6) << 20
+        got.append(np.load(path))
+    assert len(got[0].files) == 20
+    for name in got[0].files:
+        assert np.array_equal(got[0][name], got[1][name]), name
