@@ -149,7 +149,10 @@ xg_status xg_set_states(xg_ctx* ctx, uint32_t first, uint32_t count, const uint3
  * pieces generated at once where that is predicted to be the faster (see
  * xg_set_batch_split; 1 turns this off; a set or tuned launch shape keeps it
  * to at most 64 streams of at least 2^18 outputs), but not while the CUDA
- * stream is being captured; the outputs are the same. */
+ * stream is being captured; the outputs are the same.  The first call cut to
+ * a piece length builds what it needs (a workspace of the context, the
+ * matrices of xg_jump) and waits for it, some milliseconds; a capture of
+ * another CUDA stream goes on beside that. */
 xg_status xg_generate_u32(xg_ctx* ctx, uint32_t first, uint32_t nstreams,
                           uint64_t n_per_stream, uint32_t* out, uint64_t ld);
 xg_status xg_generate_uniform(xg_ctx* ctx, uint32_t first, uint32_t nstreams,

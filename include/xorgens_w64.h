@@ -103,7 +103,9 @@ xg_status xg_w64_autotune(xg_w64_ctx* ctx, xg_w64_type type, uint32_t nstreams, 
  * cut is predicted to be the faster; a set or tuned launch shape keeps it to
  * at most 16 streams of at least 2^18 words), 1 = never cut, else a power of
  * two >= 64, for at most 16 streams of at least 2^18 words.  Not while the
- * CUDA stream is being captured.  XG_EINVAL for other values. */
+ * CUDA stream is being captured.  The first call cut to a piece length builds
+ * a workspace and matrices and waits for them, as xg_generate_u32 says.
+ * XG_EINVAL for other values. */
 xg_status xg_w64_set_split(xg_w64_ctx* ctx, uint64_t piece_words);
 
 /* Jump-ahead: advance streams [first, first+nstreams) by `words` positions

@@ -144,6 +144,20 @@ double prologue_us(uint32_t nstreams, uint64_t pieces, int sm_count)
     return t;
 }
 
+// While it lives, what this thread allocates and waits for is no part of a
+// capture that another CUDA stream is in: in the default (global) capture mode
+// that capture would be refused and invalidated.
+class OutsideCaptures {
+public:
+    OutsideCaptures() { cudaThreadExchangeStreamCaptureMode(&mode_); }
+    ~OutsideCaptures() { cudaThreadExchangeStreamCaptureMode(&mode_); }
+    OutsideCaptures(const OutsideCaptures&) = delete;
+    OutsideCaptures& operator=(const OutsideCaptures&) = delete;
+
+private:
+    cudaStreamCaptureMode mode_ = cudaStreamCaptureModeRelaxed;
+};
+
 }  // namespace
 
 int cut_choose(int kind, uint32_t nstreams, uint64_t n, int sm_count, uint64_t forced)
@@ -236,6 +250,7 @@ xg_status cut_prologue(CutWorkspace& ws, const CutStreams& streams, uint32_t fir
                        int q, size_t extra_bytes, cudaStream_t s, CutRings* out, bool* ran)
 {
     *ran = false;
+    OutsideCaptures outside;   // the workspace, the matrices
     const uint32_t total = pieces * nstreams;
     const Steps steps = plan_steps(nstreams, pieces);
     uint32_t most_tc = 0;   // states of the largest tensor-core step

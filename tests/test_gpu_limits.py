@@ -188,3 +188,30 @@ def test_calls_without_memory_for_derived_tables(tmp_path):
     assert len(got[0].files) == 20
     for name in got[0].files:
         assert np.array_equal(got[0][name], got[1][name]), name
+
+
+@pytest.mark.parametrize("wide", [False, True])
+def test_first_cut_call_beside_a_capture(wide):
+    """A context's first cut call, which allocates and may build matrices,
+    while another CUDA stream is captured in the default mode, by this thread
+    or another: the call's words and the captured graph are both good."""
+    from concurrent.futures import ThreadPoolExecutor
+    from paper_1108_0486_gb300 import Streams, Streams64
+    n, dtype = 1 << 20, torch.int64 if wide else torch.int32
+    cs, own = torch.cuda.Stream(), torch.cuda.Stream()
+    x = torch.zeros(1000, device="cuda")
+    for other_thread in (False, True):
+        with (Streams64 if wide else Streams)(2, seeds=W.seeds(2), stream=own) as st, ThreadPoolExecutor(1) as pool:
+            draw = st.u64 if wide else st.u32
+            out = torch.empty((2, n), dtype=dtype, device="cuda")
+            torch.cuda.synchronize()
+            g = torch.cuda.CUDAGraph()
+            with torch.cuda.graph(g, stream=cs, capture_error_mode="global"):
+                x += 1
+                pool.submit(draw, n, out=out).result() if other_thread else draw(n, out=out)
+                x += 1
+            g.replay()
+            torch.cuda.synchronize()
+            ref = O.streams64(W.seeds(2), n) if wide else O.streams(W.seeds(2), n)
+            assert np.array_equal(out.cpu().numpy().view(ref.dtype), ref)
+    assert float(x.sum()) == 4000.0
