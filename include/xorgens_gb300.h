@@ -167,7 +167,10 @@ xg_status xg_generate_normal(xg_ctx* ctx, uint32_t first, uint32_t nstreams,
  * its own values in sequence order, then the lanes of a stream are combined
  * by a butterfly over lane offsets TPG/2, ..., 1.  A long call on few streams
  * without a set or tuned launch shape may be summed in pieces that way (see
- * xg_set_batch_split), the pieces' sums added in FP64 and rounded once. */
+ * xg_set_batch_split), with 32 lanes and two words each: 32 partial sums in
+ * FP64, of every 32nd piece in order, then the same butterfly and one rounding.
+ * The order depends on the numbers of streams and outputs, the split set and
+ * the GPU's number of SMs, not on whether the call was captured. */
 xg_status xg_generate_normal_sum(xg_ctx* ctx, uint32_t first, uint32_t nstreams,
                                  uint64_t n_per_stream, float* d_sums);
 

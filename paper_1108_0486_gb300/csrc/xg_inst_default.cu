@@ -20,6 +20,11 @@ cudaError_t launch_cut_default(int out_kind, bool vec, const CutArgs& a, cudaStr
     return launch_cut_impl<ParamsDefault>(out_kind, vec, a, s);
 }
 
+cudaError_t launch_sum_in_pieces_default(const GenArgs& a, uint32_t log2_len, cudaStream_t s)
+{
+    return launch_sum_in_pieces_impl<ParamsDefault>(a, log2_len, s);
+}
+
 const void* batch_kernel_ptr_default(bool groups) { return batch_kernel_ptr<ParamsDefault>(groups); }
 
 }  // namespace xg

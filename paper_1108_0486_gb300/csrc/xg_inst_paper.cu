@@ -20,6 +20,11 @@ cudaError_t launch_cut_paper(int out_kind, bool vec, const CutArgs& a, cudaStrea
     return launch_cut_impl<ParamsPaper>(out_kind, vec, a, s);
 }
 
+cudaError_t launch_sum_in_pieces_paper(const GenArgs& a, uint32_t log2_len, cudaStream_t s)
+{
+    return launch_sum_in_pieces_impl<ParamsPaper>(a, log2_len, s);
+}
+
 const void* batch_kernel_ptr_paper(bool groups) { return batch_kernel_ptr<ParamsPaper>(groups); }
 
 }  // namespace xg

@@ -612,6 +612,69 @@ __global__ void __launch_bounds__(256, 1) cut_kernel(CutArgs a)
     }
 }
 
+// The sums of a call that would be cut where it cannot be (its CUDA stream is
+// being captured, or there is no memory for the prologue): a warp generates the
+// whole stream and adds in the cut call's order, so that the sum's bits do not
+// depend on how it came about.  A piece's sum goes to the lane that adds it in
+// cut_sum_kernel.  The voted loop runs piece by piece: one stream of 2^20
+// 1084 us (995 as one chain, 39 cut), 500 streams of 500000 507 (499, 363).
+template <class P>
+__global__ void __launch_bounds__(256, 1) sum_in_pieces_kernel(GenArgs a, uint32_t log2_len)
+{
+    using E = Engine<P, 32, 2>;
+    using Em = Emit<E, kNormalSum, true>;
+    static_assert(E::NROWS == 2 && E::RW <= 64, "pieces are whole rounds");
+    const uint32_t g = (blockIdx.x * blockDim.x + threadIdx.x) / 32;
+    if (g >= a.nstreams) return;
+    const uint32_t s = a.first + g;
+    const int lane = (int)(threadIdx.x & 31u);
+    constexpr unsigned kFull = 0xFFFFFFFFu;
+    E eng;
+    eng.lane = lane;
+    eng.mask = kFull;
+    uint32_t* win_s = a.st.win + (uint64_t)s * kWin;
+    load_ring(eng, win_s, a.st.pend[s]);
+    const uint32_t wp = a.st.weyl[s];
+    Em em;
+    em.omega = a.omega;
+    em.lane_off = 2 * (uint64_t)lane;
+    em.wl = wp + (uint32_t)(2 * lane + 1) * a.omega;
+    em.dst = nullptr;
+    const uint64_t nwords = a.n + (a.n & 1u), len = uint64_t(1) << log2_len;
+    uint32_t retired[2], pend = 0;
+    double acc = 0.0;
+    uint32_t m = 0;
+    for (uint64_t at = 0; at < nwords; at += len, ++m) {
+        const uint64_t words = nwords - at < len ? nwords - at : len;
+        em.limit = a.n - at < len ? a.n - at : len;
+        em.acc = 0.0f;
+        const uint64_t nr = (words + E::RW - 1) / E::RW;
+        if (drive<E, Em, true, kVotedBlocks>(eng, nr, em, retired)) {   // an odd number of rounds: oldest row first again
+#pragma unroll
+            for (int i = 0; i < 2; ++i) {
+                const uint32_t t = eng.ring[0][i];
+                eng.ring[0][i] = eng.ring[1][i];
+                eng.ring[1][i] = t;
+            }
+        }
+        pend = (uint32_t)(nr * E::RW - words);
+        float sum = em.acc;
+#pragma unroll
+        for (int off = 16; off >= 1; off /= 2) sum = __fadd_rn(sum, __shfl_xor_sync(kFull, sum, off));
+        if (lane == (int)(m % 32)) acc += (double)sum;
+    }
+#pragma unroll
+    for (int off = 16; off >= 1; off /= 2) acc += __shfl_xor_sync(kFull, acc, off);
+    __syncwarp();
+    store_window(eng, win_s, 0, retired);
+    if (lane == 0) {
+        a.sums[g] = (float)acc;
+        a.st.weyl[s] = wp + (uint32_t)nwords * a.omega;
+        a.st.pend[s] = pend;
+        a.st.pos[s] += nwords;
+    }
+}
+
 // Persistent batch kernel.  Each warp repeatedly takes the next task
 // (atomic counter; tasks are ordered costliest first by the host).  A chain
 // task runs every item of one chain -- the calls on one stream, in order --
@@ -814,6 +877,13 @@ cudaError_t launch_cut_impl(int out_kind, bool vec, const CutArgs& a, cudaStream
     case kNormalSum: return launch_cut_one<P, kNormalSum, kAligned>(a, s);
     default: return cudaErrorInvalidValue;
     }
+}
+
+template <class P>
+cudaError_t launch_sum_in_pieces_impl(const GenArgs& a, uint32_t log2_len, cudaStream_t s)
+{
+    sum_in_pieces_kernel<P><<<(a.nstreams + 1) / 2, 64, 0, s>>>(a, log2_len);
+    return cudaGetLastError();
 }
 
 template <class P>

@@ -189,6 +189,8 @@ cudaError_t launch_export_states(const State& st, uint32_t first, uint32_t n, ui
 cudaError_t launch_import_states(const State& st, uint32_t first, uint32_t n, const uint32_t* rings,
                                  const uint32_t* weyl, const uint64_t* pos, uint32_t weyl_on, cudaStream_t s);
 cudaError_t launch_cut(int param_set, int out_kind, bool vec, const CutArgs& a, cudaStream_t s);
+// Fused sums (a.sums) of whole streams, added as if cut into pieces of 2^log2_len.
+cudaError_t launch_sum_in_pieces(int param_set, const GenArgs& a, uint32_t log2_len, cudaStream_t s);
 // The persistent batch kernel of a parameter set; groups: the variant with
 // the group-task paths.
 const void* batch_kernel_ptr(int param_set, bool groups);
@@ -200,6 +202,8 @@ cudaError_t launch_gen_default(int cfg, int out_kind, Store store, int block, co
 cudaError_t launch_gen_paper(int cfg, int out_kind, Store store, int block, const GenArgs&, cudaStream_t);
 cudaError_t launch_cut_default(int out_kind, bool vec, const CutArgs&, cudaStream_t);
 cudaError_t launch_cut_paper(int out_kind, bool vec, const CutArgs&, cudaStream_t);
+cudaError_t launch_sum_in_pieces_default(const GenArgs&, uint32_t log2_len, cudaStream_t);
+cudaError_t launch_sum_in_pieces_paper(const GenArgs&, uint32_t log2_len, cudaStream_t);
 const void* batch_kernel_ptr_default(bool groups);
 const void* batch_kernel_ptr_paper(bool groups);
 

@@ -150,6 +150,11 @@ cudaError_t launch_cut(int param_set, int out_kind, bool vec, const CutArgs& a, 
     return param_set == 1 ? launch_cut_paper(out_kind, vec, a, s) : launch_cut_default(out_kind, vec, a, s);
 }
 
+cudaError_t launch_sum_in_pieces(int param_set, const GenArgs& a, uint32_t log2_len, cudaStream_t s)
+{
+    return param_set == 1 ? launch_sum_in_pieces_paper(a, log2_len, s) : launch_sum_in_pieces_default(a, log2_len, s);
+}
+
 const void* batch_kernel_ptr(int param_set, bool groups)
 {
     return param_set == 1 ? batch_kernel_ptr_paper(groups) : batch_kernel_ptr_default(groups);

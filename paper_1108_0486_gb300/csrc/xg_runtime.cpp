@@ -187,9 +187,8 @@ static xg_status enqueue_gen(Ctx* c, int kind, uint32_t first, uint32_t nstreams
 // call.  A piece length set by the caller applies to at most 64 streams of at
 // least 2^18 outputs; by itself the library cuts where its prediction says
 // so, unless a launch shape was set or tuned for more streams or shorter
-// calls than those.  Not while the stream is being captured: a first use builds matrices
-// and the workspace.
-static int cut_length(Ctx* c, int kind, uint32_t nstreams, uint64_t n)
+// calls than those.
+static int cut_length(const Ctx* c, int kind, uint32_t nstreams, uint64_t n)
 {
     if (c->split_words == 1 || n < (uint64_t(1) << 13)) return 0;
     // fused sums: a launch shape that was set fixes the order of the additions
@@ -197,14 +196,19 @@ static int cut_length(Ctx* c, int kind, uint32_t nstreams, uint64_t n)
     if (kind == xg::kNormalSum && shaped) return 0;
     const bool always = nstreams <= 64 && n >= (uint64_t(1) << 18);   // whatever the launch shape set
     if (!always && (c->split_words > 1 || shaped)) return 0;
-    const int q = xg::cut_choose(kind, nstreams, n, c->sm_count, c->split_words);
-    if (!q) return 0;
+    return xg::cut_choose(kind, nstreams, n, c->sm_count, c->split_words);
+}
+
+// Whether a call may be cut now: not while its CUDA stream is being captured,
+// since a first use builds matrices and the workspace.
+static bool may_cut(const Ctx* c)
+{
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     if (cudaStreamIsCapturing(c->stream, &cap) != cudaSuccess) {
         cudaGetLastError();
-        return 0;
+        return false;
     }
-    return cap == cudaStreamCaptureStatusNone ? q : 0;
+    return cap == cudaStreamCaptureStatusNone;
 }
 
 static bool is_device_pointer(const void* p)
@@ -287,7 +291,7 @@ static xg_status generate_common(xg_ctx* ctx, int kind, uint32_t first, uint32_t
         // few streams, long calls: a single stream is one serial chain (one
         // warp, ~1.5e9 words/s), so cut each call into pieces that run on
         // many warps at once (jump-ahead; the output is the same)
-        if (const int q = cut_length(c, kind, nstreams, n)) {
+        if (const int q = cut_length(c, kind, nstreams, n); q && may_cut(c)) {
             bool ran = false;
             const xg_status st = xg::cut_generate(c, kind, first, nstreams, n, out, ld, q, &ran);
             if (ran || st != XG_OK) return st;
@@ -545,9 +549,20 @@ xg_status xg_generate_normal_sum(xg_ctx* ctx, uint32_t first, uint32_t nstreams,
     std::lock_guard<std::mutex> lk(c->mu);
     if (xg_status f = c->earlier_failure()) return f;
     if (const int q = cut_length(c, xg::kNormalSum, nstreams, n)) {
-        bool ran = false;
-        const xg_status st = xg::cut_generate(c, xg::kNormalSum, first, nstreams, n, d_sums, 0, q, &ran);
-        if (ran || st != XG_OK) return st;
+        if (may_cut(c)) {
+            bool ran = false;
+            const xg_status st = xg::cut_generate(c, xg::kNormalSum, first, nstreams, n, d_sums, 0, q, &ran);
+            if (ran || st != XG_OK) return st;
+        }
+        xg::GenArgs a{};
+        a.st = c->st;
+        a.first = first;
+        a.nstreams = nstreams;
+        a.n = n;
+        a.sums = d_sums;
+        a.omega = c->weyl_on ? kOmegaHost : 0u;
+        const cudaError_t e = xg::launch_sum_in_pieces((int)c->param_set, a, (uint32_t)q, c->stream);
+        return e == cudaSuccess ? XG_OK : cuda_fail(e, "sum kernel launch");
     }
     return enqueue_gen(c, xg::kNormalSum, first, nstreams, n, nullptr, 0, d_sums, c->stream);
 }

@@ -215,3 +215,55 @@ def test_first_cut_call_beside_a_capture(wide):
             ref = O.streams64(W.seeds(2), n) if wide else O.streams(W.seeds(2), n)
             assert np.array_equal(out.cpu().numpy().view(ref.dtype), ref)
     assert float(x.sum()) == 4000.0
+
+
+def sum_in_pieces(z, q):
+    """One row's normals added in the documented order of a call cut into
+    pieces of 2^q: per piece, each lane's values in sequence and a butterfly in
+    FP32; lane l of 32 adds the pieces l, l + 32, ... in FP64, a butterfly."""
+    def butterfly(v):
+        for off in (16, 8, 4, 2, 1):
+            v = v + v[..., np.arange(32) ^ off]
+        return v[..., 0]
+    pieces = -(-(z.size + (z.size & 1)) >> q)
+    v = np.zeros((pieces << q,), dtype=np.float32)
+    v[:z.size] = z
+    v = v.reshape(pieces, -1, 32, 2).transpose(0, 2, 1, 3).reshape(pieces, 32, -1)
+    sums = butterfly(np.add.accumulate(v, axis=2, dtype=np.float32)[..., -1]).astype(np.float64)
+    lanes = np.zeros((-(-pieces // 32) * 32,))
+    lanes[:pieces] = sums
+    return np.float32(butterfly(np.add.accumulate(lanes.reshape(-1, 32), axis=0)[-1]))
+
+
+@pytest.mark.parametrize("streams,n,piece", [(1, 32769, 0), (1, (1 << 18) + 3, 4096), (3, 262145, 64), (2, 1 << 20, 0),
+                                              (7, 300001, 0), (64, 1 << 18, 65536), (100, 70001, 0), (500, 200001, 0)])
+def test_sums_of_cut_calls_bit_for_bit(streams, n, piece):
+    """Sums of calls cut into pieces of a set or a chosen length (none is left
+    out or taken twice: the exact bits), called, then captured and replayed
+    twice; the streams end where whole calls end."""
+    import ctypes
+    from paper_1108_0486_gb300 import Streams, _lib as L
+    choose = L.lib()._ZN2xg10cut_chooseEijmim   # xg::cut_choose, kind 3: fused sums
+    choose.argtypes = [ctypes.c_int, ctypes.c_uint32, ctypes.c_uint64, ctypes.c_int, ctypes.c_uint64]
+    q = choose(3, streams, n, torch.cuda.get_device_properties(0).multi_processor_count, piece)
+    assert q >= 6 and (not piece or 1 << q == piece)
+    ps, cs = streams % 2, torch.cuda.Stream()
+    with Streams(streams, param_set=ps, seeds=W.seeds(streams), stream=cs) as a, \
+            Streams(streams, param_set=ps, seeds=W.seeds(streams), stream=cs) as b, torch.cuda.stream(cs):
+        a.set_batch_split(piece)
+        b.set_batch_split(1)
+        got = [a.normal_sum(n)]
+        out = torch.empty(streams, device="cuda")
+        torch.cuda.synchronize()
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g, stream=cs):
+            a.normal_sum(n, out=out)
+        for _ in range(2):
+            g.replay()
+            got.append(out.clone())
+        for sums in got:
+            z = b.normal(n).cpu().numpy()
+            for s in {0, streams // 2, streams - 1}:
+                assert float(sums[s]) == float(sum_in_pieces(z[s], q)), s
+        assert torch.equal(a.u32(77), b.u32(77))
+        assert np.array_equal(a.checkpoint()["pos"], b.checkpoint()["pos"])
