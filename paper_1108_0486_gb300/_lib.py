@@ -151,7 +151,9 @@ def check(status: int) -> None:
 
 def call(name: str, *args) -> None:
     """Call an entry point.  Pointer arguments may be plain integers or None:
-    the argument types bound at load convert them."""
+    the argument types bound at load convert them (and would take text and bytes
+    for the address of their characters, so an output that is no integer goes
+    through vp, which refuses those)."""
     fn = _entry.get(name)
     if fn is None:
         fn = getattr(lib(), name)
@@ -209,19 +211,19 @@ def xg_set_states(ctx, first, count, rings_ptr, weyl_ptr, pos_ptr=0) -> None:
 
 
 def xg_generate_u32(ctx, first, nstreams, n_per_stream, out_ptr, ld) -> None:
-    call("xg_generate_u32", ctx, first, nstreams, n_per_stream, out_ptr, ld)
+    call("xg_generate_u32", ctx, first, nstreams, n_per_stream, out_ptr if type(out_ptr) is int else vp(out_ptr), ld)
 
 
 def xg_generate_uniform(ctx, first, nstreams, n_per_stream, out_ptr, ld) -> None:
-    call("xg_generate_uniform", ctx, first, nstreams, n_per_stream, out_ptr, ld)
+    call("xg_generate_uniform", ctx, first, nstreams, n_per_stream, out_ptr if type(out_ptr) is int else vp(out_ptr), ld)
 
 
 def xg_generate_normal(ctx, first, nstreams, n_per_stream, out_ptr, ld) -> None:
-    call("xg_generate_normal", ctx, first, nstreams, n_per_stream, out_ptr, ld)
+    call("xg_generate_normal", ctx, first, nstreams, n_per_stream, out_ptr if type(out_ptr) is int else vp(out_ptr), ld)
 
 
 def xg_generate_normal_sum(ctx, first, nstreams, n_per_stream, sums_ptr) -> None:
-    call("xg_generate_normal_sum", ctx, first, nstreams, n_per_stream, sums_ptr)
+    call("xg_generate_normal_sum", ctx, first, nstreams, n_per_stream, sums_ptr if type(sums_ptr) is int else vp(sums_ptr))
 
 
 def xg_transform_uniform(ctx, words_ptr, n, out_ptr) -> None:
@@ -232,7 +234,8 @@ def xg_transform_normal(ctx, words_ptr, n, out_ptr) -> None:
     call("xg_transform_normal", ctypes.c_void_p(ctx), ctypes.c_void_p(words_ptr), n, ctypes.c_void_p(out_ptr))
 
 
-_ROW = [("stream", "<u4"), ("type", "<u4"), ("count", "<u8"), ("out", "<u8")]   # xg_item and xg_request
+_ROW = [("stream", "<u4"), ("type", "<u4"), ("count", "<u8"), ("out", "<u8")]   # xg_item
+_REQUEST = _ROW[:3] + [("d_out", "<u8")]                                         # xg_request
 
 
 def pack_columns(streams, types, counts, pointers):
@@ -252,11 +255,14 @@ def pack_columns(streams, types, counts, pointers):
 
 def pack_rows(rows):
     """Rows (stream, type, count, pointer) as pack_columns gives them; a record
-    array that it made is returned as it is."""
+    array with the fields of xg_item or xg_request is taken as it is, one with
+    other fields is refused."""
     import numpy as np
     if isinstance(rows, np.ndarray):
         if rows.dtype.names:
-            return rows
+            if rows.dtype not in (np.dtype(_ROW), np.dtype(_REQUEST)):
+                raise TypeError(f"rows of {rows.dtype}, not of (stream, type, count, out)")
+            return np.ascontiguousarray(rows.reshape(-1))
         rows = rows.astype(np.uint64, copy=False).reshape(-1, 4)
         return pack_columns(*(rows[:, k].tolist() for k in range(4)))
     rows = rows if isinstance(rows, (list, tuple)) else list(rows)
@@ -343,7 +349,7 @@ def xg_submit(ctx, stream, out_type, count, d_out=0) -> int:
 def make_requests(reqs):
     """A numpy record array laid out as xg_request[] from (stream, type,
     count, d_out) tuples (build it once, submit slices of it)."""
-    rec = pack_rows(reqs).view([(n if n != "out" else "d_out", t) for n, t in _ROW])
+    rec = pack_rows(reqs).view(_REQUEST)
     assert rec.itemsize == ctypes.sizeof(XgRequest)
     return rec
 
@@ -476,11 +482,13 @@ def xg_w64_set_state(ctx: int, stream: int, host_ring_ptr: int, weyl: int) -> No
 
 
 def xg_w64_generate_u64(ctx, first, nstreams, n_per_stream, out_ptr, ld) -> None:
-    call("xg_w64_generate_u64", ctx, first, nstreams, n_per_stream, out_ptr, ld)
+    call("xg_w64_generate_u64", ctx, first, nstreams, n_per_stream,
+         out_ptr if type(out_ptr) is int else vp(out_ptr), ld)
 
 
 def xg_w64_generate_uniform_f64(ctx, first, nstreams, n_per_stream, out_ptr, ld) -> None:
-    call("xg_w64_generate_uniform_f64", ctx, first, nstreams, n_per_stream, out_ptr, ld)
+    call("xg_w64_generate_uniform_f64", ctx, first, nstreams, n_per_stream,
+         out_ptr if type(out_ptr) is int else vp(out_ptr), ld)
 
 
 def xg_w64_transform_uniform_f64(ctx, words_ptr, n, out_ptr) -> None:
