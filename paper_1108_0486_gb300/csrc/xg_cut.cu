@@ -41,18 +41,18 @@ struct Steps {
 };
 
 // Up to 7 matrices per step, which makes the pieces eight times as many.  By
-// the table kernel as long as the states are few, where a step costs a launch
-// and the matrix read rather than the lookups (0.05 us per state and matrix);
-// by the tensor cores from about 200 results on, where it costs the launches
-// and one tile's time and hardly more for seven matrices than for one.
+// the table kernel as long as the results are few, where a step costs a launch
+// and the matrix read rather than the lookups (0.05 us per result); by the
+// tensor cores from kTcMinResults on, where it costs the launches and one
+// tile's time and hardly more for seven matrices than for one.  The price of a
+// step (cut_prologue_us) and its launch go by the same limit.
 Steps plan_steps(uint32_t nstreams, uint32_t pieces)
 {
     Steps p{};
     for (uint64_t have = 1; have < pieces && p.n < kMaxSteps; ++p.n) {
         const uint64_t sources = have * nstreams;
         const uint64_t left = std::min<uint64_t>(7, (pieces + have - 1) / have - 1);
-        const bool table = sources <= 16 || (sources <= 48 && left <= 3) || (sources < 192 && left == 1);
-        p.step[p.n] = Step{(uint32_t)have, (uint32_t)left, table ? 0u : 1u, p.entries};
+        p.step[p.n] = Step{(uint32_t)have, (uint32_t)left, sources * left >= kTcMinResults ? 1u : 0u, p.entries};
         p.entries += sources * (1 + left);
         have *= 1 + left;
     }
@@ -123,10 +123,26 @@ double word_ns(int kind, double w)
     }
 }
 
-// Prologue time in us: the set-up launch, then per step a table-kernel launch
+// While it lives, what this thread allocates and waits for is no part of a
+// capture that another CUDA stream is in: in the default (global) capture mode
+// that capture would be refused and invalidated.
+class OutsideCaptures {
+public:
+    OutsideCaptures() { cudaThreadExchangeStreamCaptureMode(&mode_); }
+    ~OutsideCaptures() { cudaThreadExchangeStreamCaptureMode(&mode_); }
+    OutsideCaptures(const OutsideCaptures&) = delete;
+    OutsideCaptures& operator=(const OutsideCaptures&) = delete;
+
+private:
+    cudaStreamCaptureMode mode_ = cudaStreamCaptureModeRelaxed;
+};
+
+}  // namespace
+
+// The set-up launch, then per step a table-kernel launch
 // or an application on the tensor cores (18 ns per operand row of a tile; the
 // last wave is rarely full).
-double prologue_us(uint32_t nstreams, uint64_t pieces, int sm_count)
+double cut_prologue_us(uint32_t nstreams, uint64_t pieces, int sm_count)
 {
     const Steps p = plan_steps(nstreams, (uint32_t)pieces);
     double t = 5.0;
@@ -143,22 +159,6 @@ double prologue_us(uint32_t nstreams, uint64_t pieces, int sm_count)
     }
     return t;
 }
-
-// While it lives, what this thread allocates and waits for is no part of a
-// capture that another CUDA stream is in: in the default (global) capture mode
-// that capture would be refused and invalidated.
-class OutsideCaptures {
-public:
-    OutsideCaptures() { cudaThreadExchangeStreamCaptureMode(&mode_); }
-    ~OutsideCaptures() { cudaThreadExchangeStreamCaptureMode(&mode_); }
-    OutsideCaptures(const OutsideCaptures&) = delete;
-    OutsideCaptures& operator=(const OutsideCaptures&) = delete;
-
-private:
-    cudaStreamCaptureMode mode_ = cudaStreamCaptureModeRelaxed;
-};
-
-}  // namespace
 
 int cut_choose(int kind, uint32_t nstreams, uint64_t n, int sm_count, uint64_t forced)
 {
@@ -185,7 +185,7 @@ int cut_choose(int kind, uint32_t nstreams, uint64_t n, int sm_count, uint64_t f
         if (pieces * nstreams > kMaxPieces) continue;
         const double run = 6.0 + 1e-3 * (double)len * word_ns(kind, warps(nstreams * ((pieces + 1) / 2)));
         if (run >= best) continue;
-        const double t = prologue_us(nstreams, pieces, sm_count) + run + (kind == kNormalSum ? 2.0 : 0.0);
+        const double t = cut_prologue_us(nstreams, pieces, sm_count) + run + (kind == kNormalSum ? 2.0 : 0.0);
         if (t < best) {
             best = t;
             best_q = q;

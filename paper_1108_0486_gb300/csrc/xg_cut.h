@@ -22,6 +22,9 @@ constexpr int kCutUniform64 = 5;
 // of two >= 64), or 0.
 int cut_choose(int kind, uint32_t nstreams, uint64_t n, int sm_count, uint64_t forced);
 
+// Predicted time of the prologue in us (the same).
+double cut_prologue_us(uint32_t nstreams, uint64_t pieces, int sm_count);
+
 // A context's workspace for cut calls (grow-only, freed with the context).
 // Used on the context's stream of the moment: the event follows the last use,
 // and a use on another stream waits for it.  Streams are told apart by their

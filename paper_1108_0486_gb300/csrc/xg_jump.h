@@ -58,7 +58,8 @@ const uint8_t* jump_matrix_tc(int device, int family, int j, int k, cudaStream_t
 // tensor-core path off), and the device scratch it then needs (0 otherwise).
 // A launch for 192 results costs 13 us on the tensor cores and 15 by the table
 // kernel (0.05 us per result), whose launches overlap better.
-bool gf2_use_tc(int device, uint32_t n, uint32_t from = 192);
+constexpr uint32_t kTcMinResults = 192;
+bool gf2_use_tc(int device, uint32_t n, uint32_t from = kTcMinResults);
 size_t gf2_apply_scratch(int device, uint32_t n);
 
 // rings[d_dst[i]] = C_k rings[d_src[i]] for n pairs, C_k the power 2^k of
