@@ -267,3 +267,52 @@ def test_sums_of_cut_calls_bit_for_bit(streams, n, piece):
                 assert float(sums[s]) == float(sum_in_pieces(z[s], q)), s
         assert torch.equal(a.u32(77), b.u32(77))
         assert np.array_equal(a.checkpoint()["pos"], b.checkpoint()["pos"])
+
+
+def test_tensor_core_jump_at_the_edges_of_its_tiles():
+    """One power applied to as many states as fill the last tile, leave one
+    place free in it or start another, for tiles of every width between 16 and
+    240 that the library takes: the table kernel's states."""
+    import ctypes
+    import os
+    from paper_1108_0486_gb300 import Streams, _lib as L
+    fn, waves = L.lib()._ZN2xg11gf2_tc_tileEPKjiiPj, ctypes.c_uint32()   # xg::gf2_tc_tile
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    tile = lambda n: fn(ctypes.byref(ctypes.c_uint32(n)), 1, sms, ctypes.byref(waves))
+    sizes = {}
+    for n in range(8, 20000):
+        w = tile(n)
+        if n % w in (0, 1, w - 1):
+            sizes.setdefault((w, n % w), n)
+    assert {w for w, _ in sizes} >= {16, 240} and len(sizes) >= 20
+    for n in sorted(set(sizes.values())):
+        rows = []
+        for tc in ("1", "0"):
+            os.environ["XG_JUMP_TENSOR_CORES"] = tc
+            try:
+                with Streams(n, seeds=W.seeds(n)) as st:
+                    st.jump(1 << 37)
+                    rows.append(st.u32(128))
+            finally:
+                del os.environ["XG_JUMP_TENSOR_CORES"]
+        assert torch.equal(*rows), n
+
+
+@pytest.mark.parametrize("family", [0, 1, 64])
+@pytest.mark.parametrize("words", [(1 << 33) + 12, (1 << 30) + (1 << 20) + 9, (1 << 41) + 0x3F])
+def test_table_kernel_jumps_at_the_limits_of_products(family, words, monkeypatch):
+    """Without the tensor cores: streams on both sides of the counts from which
+    3, 4 or 7 powers are multiplied first (65, 5, 1) and of the table kernel's
+    forms (4, 192 states), against jumps by one power after another."""
+    from paper_1108_0486_gb300 import Streams, Streams64
+    monkeypatch.setenv("XG_JUMP_TENSOR_CORES", "0")
+    rows = []
+    for n in (1, 4, 5, 64, 65, 191, 192):
+        for jumps in ([words], [1 << k for k in range(64) if words >> k & 1]):
+            seeds = W.seeds(n)
+            with (Streams64(n, seeds=seeds) if family == 64 else Streams(n, param_set=family, seeds=seeds)) as st:
+                for j in jumps:
+                    st.jump(j)
+                rows.append((st.u64 if family == 64 else st.u32)(140))
+        assert torch.equal(rows[-1], rows[-2]), n
+        assert torch.equal(rows[-1][0], rows[0][0])
