@@ -9,6 +9,7 @@ from __future__ import annotations
 
 import array
 import ctypes
+import functools
 import os
 import threading
 
@@ -234,8 +235,13 @@ def xg_transform_normal(ctx, words_ptr, n, out_ptr) -> None:
     call("xg_transform_normal", ctypes.c_void_p(ctx), ctypes.c_void_p(words_ptr), n, ctypes.c_void_p(out_ptr))
 
 
-_ROW = [("stream", "<u4"), ("type", "<u4"), ("count", "<u8"), ("out", "<u8")]   # xg_item
-_REQUEST = _ROW[:3] + [("d_out", "<u8")]                                         # xg_request
+@functools.lru_cache(maxsize=None)
+def _row_dtypes():
+    """Record layouts of xg_item and xg_request (a structured dtype takes some
+    microseconds to make)."""
+    import numpy as np
+    head = [("stream", "<u4"), ("type", "<u4"), ("count", "<u8")]
+    return np.dtype(head + [("out", "<u8")]), np.dtype(head + [("d_out", "<u8")])
 
 
 def pack_columns(streams, types, counts, pointers):
@@ -243,8 +249,9 @@ def pack_columns(streams, types, counts, pointers):
     integers go through machine-integer arrays, a quarter of the time that one
     nested list of rows takes to convert."""
     import numpy as np
-    rec = np.zeros(len(streams), dtype=_ROW)
-    for (name, _), c in zip(_ROW, (streams, types, counts, pointers)):
+    row, _ = _row_dtypes()
+    rec = np.zeros(len(streams), dtype=row)
+    for name, c in zip(row.names, (streams, types, counts, pointers)):
         try:
             c = array.array("Q", c)
         except TypeError:                  # not integers as they stand
@@ -260,7 +267,7 @@ def pack_rows(rows):
     import numpy as np
     if isinstance(rows, np.ndarray):
         if rows.dtype.names:
-            if rows.dtype not in (np.dtype(_ROW), np.dtype(_REQUEST)):
+            if rows.dtype not in _row_dtypes():
                 raise TypeError(f"rows of {rows.dtype}, not of (stream, type, count, out)")
             return np.ascontiguousarray(rows.reshape(-1))
         rows = rows.astype(np.uint64, copy=False).reshape(-1, 4)
@@ -349,7 +356,7 @@ def xg_submit(ctx, stream, out_type, count, d_out=0) -> int:
 def make_requests(reqs):
     """A numpy record array laid out as xg_request[] from (stream, type,
     count, d_out) tuples (build it once, submit slices of it)."""
-    rec = pack_rows(reqs).view(_REQUEST)
+    rec = pack_rows(reqs).view(_row_dtypes()[1])
     assert rec.itemsize == ctypes.sizeof(XgRequest)
     return rec
 

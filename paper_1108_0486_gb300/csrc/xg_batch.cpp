@@ -326,29 +326,29 @@ xg_status BatchLauncher::reserve_jump(uint32_t pieces, uint32_t pairs)
 // all seven: the sources are listed by how many results they have, most
 // first, so that matrix j applies to a prefix of them.  256 requests of a
 // server burst took 6 doubling launches of 15 to 25 us each, a batch of 4096
-// calls five of 25 to 37 us.  Radix 2 (log2_radix = 1) needs the powers alone,
-// one per step.  XG_ENOMEM, with nothing enqueued, where a matrix is not to be
+// calls five of 25 to 37 us.  Radix 2 needs the powers alone, one per step.  XG_ENOMEM, with nothing enqueued, where a matrix is not to be
 // had; a step whose FP4 copies are missing runs on the table kernel.
-xg_status BatchLauncher::prologue(xg_ctx* c, cudaStream_t s, int log2_radix)
+template <int LOG2_RADIX>
+xg_status BatchLauncher::prologue(xg_ctx* c, cudaStream_t s)
 {
     const uint32_t P = (uint32_t)plan_.pieces.size();
     if (P == 0) return XG_OK;
-    const uint64_t radix = uint64_t(1) << log2_radix;
-    constexpr int kSteps = 33;   // 2^32 pieces and more
-    constexpr uint32_t kMats = 7;
+    constexpr uint64_t kRadix = uint64_t(1) << LOG2_RADIX;
+    constexpr int kSteps = 32 / LOG2_RADIX + 1;   // 2^32 pieces and more
+    constexpr uint32_t kMats = kRadix - 1;
     static_assert(kMats <= (uint32_t)kMaxMats && kMats <= (uint32_t)kGf2TcMaxMats, "matrices per launch");
     uint32_t with[kSteps][kMats + 1] = {};   // sources with exactly d results
     int nsteps = 0;
-    // f(step, piece, results, radix^step) for every source
+    // f(step, piece, results, kRadix^step) for every source
     auto for_sources = [&](auto&& f) {
         for (uint32_t k0 = 0, k1; k0 < P; k0 = k1) {
             k1 = k0 + 1;
             while (k1 < P && plan_.piece_index[k1] != 0) ++k1;
             const uint64_t K = k1 - k0;
             int step = 0;
-            for (uint64_t have = 1; have < K; have *= radix, ++step)
+            for (uint64_t have = 1; have < K; have *= kRadix, ++step)
                 for (uint64_t m = 0; m < have && m + have < K; ++m)
-                    f(step, k0 + (uint32_t)m, (uint32_t)std::min<uint64_t>(radix - 1, (K - 1 - m) / have), (uint32_t)have);
+                    f(step, k0 + (uint32_t)m, (uint32_t)std::min<uint64_t>(kMats, (K - 1 - m) / have), (uint32_t)have);
             nsteps = std::max(nsteps, step);
         }
     };
@@ -414,7 +414,7 @@ xg_status BatchLauncher::prologue(xg_ctx* c, cudaStream_t s, int log2_radix)
     const uint8_t* tc_mats[kSteps][kMats] = {};
     for (int k = 0; k < nsteps; ++k) {
         xg_status st = XG_OK;
-        const int family = (int)c->param_set, e = plan_.split_log2 + log2_radix * k;
+        const int family = (int)c->param_set, e = plan_.split_log2 + LOG2_RADIX * k;
         for (uint32_t j = 0; use_tc[k] && j < kMats && counts[k][j]; ++j) {
             tc_mats[k][j] = jump_matrix_tc(c->device, family, (int)j + 1, e, s, &st);
             if (!tc_mats[k][j] && st != XG_ENOMEM) return st;
@@ -454,6 +454,15 @@ xg_status BatchLauncher::prologue(xg_ctx* c, cudaStream_t s, int log2_radix)
     return XG_OK;
 }
 
+// With the powers alone, or, where not even these are to be had, no cut.
+[[gnu::cold, gnu::noinline]] xg_status BatchLauncher::prologue_without_tables(xg_ctx* c, const HostItem* items, uint32_t n,
+                                                                              cudaStream_t s)
+{
+    const xg_status st = prologue<1>(c, s);
+    if (st == XG_ENOMEM) plan_units(items, n, 0, c->n, plan_);
+    return st == XG_ENOMEM ? XG_OK : st;
+}
+
 xg_status BatchLauncher::launch(xg_ctx* c, const HostItem* items, uint32_t n, cudaStream_t s,
                                 uint32_t* units_per_item, uint64_t min_piece)
 {
@@ -464,16 +473,12 @@ xg_status BatchLauncher::launch(xg_ctx* c, const HostItem* items, uint32_t n, cu
     // the jump prologue needs only the pieces: enqueue it before ordering the
     // heads, so that the GPU starts while the host finishes the plan
     plan_units(items, n, choose_piece_len(c, items, n, min_piece), c->n, plan_);
-    uint32_t nu = (uint32_t)plan_.units.size();
-    if (xg_status st = reserve(c, nu)) return st;
-    xg_status jump = prologue(c, s, 3);
-    if (jump == XG_ENOMEM) jump = prologue(c, s, 1);
-    if (jump == XG_ENOMEM) {   // the uncut batch needs no matrices
-        plan_units(items, n, 0, c->n, plan_);
-        nu = (uint32_t)plan_.units.size();
-        jump = XG_OK;
+    if (xg_status st = reserve(c, (uint32_t)plan_.units.size())) return st;
+    if (xg_status st = prologue<3>(c, s)) {
+        if (st == XG_ENOMEM) st = prologue_without_tables(c, items, n, s);
+        if (st) return st;
     }
-    if (jump) return jump;
+    const uint32_t nu = (uint32_t)plan_.units.size();
     plan_order(plan_);
     // group only units of at most 1/8 of a resident warp's share of the
     // batch (XG_BATCH_GROUP_MAX_WORDS=<n> sets the limit instead)

@@ -85,7 +85,9 @@ public:
 
 private:
     xg_status build_graph(xg_ctx* c);
-    xg_status prologue(xg_ctx* c, cudaStream_t s, int log2_radix);
+    template <int LOG2_RADIX>
+    xg_status prologue(xg_ctx* c, cudaStream_t s);
+    xg_status prologue_without_tables(xg_ctx* c, const HostItem* items, uint32_t n, cudaStream_t s);
     xg_status grow_jump(size_t want);
     uint64_t choose_piece_len(const xg_ctx* c, const HostItem* items, uint32_t n, uint64_t min_piece) const;
     uint32_t capacity_ = 0;

@@ -499,9 +499,8 @@ public:
         const int st = t.state.load(std::memory_order_acquire);
         if (st == kDone || st == kFailed || st == kCancelled) return true;
         if (t.state.load(std::memory_order_acquire) != kRunning) return false;
-        volatile uint32_t* f = h_flags_ + t.slot;
-        if (*f < t.expected) return false;
-        std::atomic_thread_fence(std::memory_order_acquire);   // the prologue's word after the flag
+        // acquire: the prologue's word is read after the flag
+        if (__atomic_load_n(h_flags_ + t.slot, __ATOMIC_ACQUIRE) < t.expected) return false;
         int expect = kRunning;
         const bool valid = !t.prologue || *t.prologue == 0;
         if (t.state.compare_exchange_strong(expect, valid ? kDone : kFailed)) t.t_done.store(now_ns());
