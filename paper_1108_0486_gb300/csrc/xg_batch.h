@@ -67,11 +67,12 @@ public:
     // receives how many completion increments each item will produce.
     // min_piece: the shortest piece the automatic choice may cut (a caller
     // that knows the GPU is already busy raises it: cutting buys latency at
-    // the price of jump-ahead work, about 2.2e4 words' worth per piece).
+    // the price of jump-ahead work, about 4.6e3 words' worth per piece).
     xg_status launch(xg_ctx* c, const HostItem* items, uint32_t n, cudaStream_t s,
                      uint32_t* units_per_item = nullptr, uint64_t min_piece = kMinPiece);
-    // 2^15: on an idle GPU the serving p99 is lowest there (2^14 and 2^13 add
-    // more jump-ahead than they save; 2^16 leaves longer chains)
+    // 2^15: on an idle GPU the serving p99 was lowest there (2^14 and 2^13 added
+    // more jump-ahead than they saved, at five times its present price; 2^16
+    // leaves longer chains)
     static constexpr uint64_t kMinPiece = uint64_t(1) << 15;
     // Preallocate the jump prologue's buffers for up to `pieces` pieces (so
     // that a later launch does not allocate).

@@ -11,20 +11,20 @@
 // (M = 4096 output bits, N = states, K = 4096 input bits, both operands
 // K-major), followed by a parity epilogue that packs bits back into 32-bit
 // ring words.  FP4 halves the bytes per operand of the same kernel in FP8
-// (kind::f8f6f4): one application to 16384 states 149 -> 98.6 us.  Bound by
-// the bytes into shared memory, 47 KB per 128 x 240 x 256 block or about
-// 114 B/ns per SM (17 TB/s over the GPU); the tensor pipe is 61% active.
+// (kind::f8f6f4): one application to 16384 states 150 -> 86 us.  Bound by
+// shared memory: 47 KB per 128 x 240 x 256 block are written and read once,
+// about 130 B per clock and SM; the tensor pipe is 66% active.
 //
 // Order of K: both operands hold the 32 bits of an input word as 32 nibbles
 // in the order that three shifts and masks give (spread32); a dot product
 // does not depend on it.
 //
-// Kernel: persistent, one CTA per SM, 128 x 240 output tiles (two FP32
-// accumulators of 240 columns and 32 columns of scales fill the 512 TMEM
-// columns).  Warp 0 (one lane) streams 128-byte-wide K blocks (256 bits) of A
+// Kernel: persistent, one CTA per SM, output tiles of 128 bits by bn states, bn
+// up to 240 (gf2_tc_tile; two FP32 accumulators of 240 columns and 32 columns
+// of scales fill the 512 TMEM columns).  Warp 0 (one lane) streams 128-byte-wide K blocks (256 bits) of A
 // and B into a 4-stage shared-memory ring with TMA (128B swizzle, mbarrier
 // transaction counts); warp 1 (one lane) issues tcgen05.mma (kind::mxf4,
-// E2M1 x E2M1 -> F32, 128 x 240 x 64 each) into one of two TMEM accumulators
+// E2M1 x E2M1 -> F32, 128 x bn x 64 each) into one of two TMEM accumulators
 // and frees each stage with tcgen05.commit; four epilogue warps read the
 // other accumulator with tcgen05.ld (32 TMEM lanes = 32 output bits each),
 // take each count's parity and pack the 32 lanes' bits with a warp ballot:
@@ -202,6 +202,17 @@ struct TcMaps {
     uint32_t end[kGf2TcMaxMats];  // tiles of the matrices up to j
 };
 
+// Matrix and state tile of tile t.
+struct TcTile {
+    uint32_t j, nt;
+};
+__device__ __forceinline__ TcTile tc_tile(const TcMaps& maps, uint32_t t)
+{
+    uint32_t j = 0, from = 0;
+    while (t >= maps.end[j]) from = maps.end[j++];
+    return TcTile{j, (t - from) / (uint32_t)(kGf2Bits / kBM)};
+}
+
 // out[dst[at_j + s]] = C_j x_s for the first n_j states of the B operand (rows
 // past them count for nothing).  Persistent: CTA b takes tiles b, b +
 // gridDim.x, ... of the matrices' (4096 / kBM) x (n_j / bn) tiles, M fastest
@@ -214,17 +225,6 @@ struct TcMaps {
 // MMA issuer, warps 2-5 = epilogue (warp w reads TMEM lanes 32 (w mod 4) ..).
 // Two accumulators of kBN columns alternate, so that the epilogue of one
 // tile overlaps the MMAs of the next.
-// Matrix and state tile of tile t.
-struct TcTile {
-    uint32_t j, nt;
-};
-__device__ __forceinline__ TcTile tc_tile(const TcMaps& maps, uint32_t t)
-{
-    uint32_t j = 0, from = 0;
-    while (t >= maps.end[j]) from = maps.end[j++];
-    return TcTile{j, (t - from) / (uint32_t)(kGf2Bits / kBM)};
-}
-
 __global__ void __launch_bounds__(kThreads, 1) gf2_tc_kernel(const __grid_constant__ TcMaps maps, uint32_t total, uint32_t bn,
                                                               const uint32_t* __restrict__ dst, uint32_t* out,
                                                               uint32_t out_stride, uint32_t* status, uint32_t stall)

@@ -141,9 +141,9 @@ struct MatSet {
     uint32_t n[kMaxMats];           // how many of them
     uint32_t at[kMaxMats];          // its destinations in the list
 };
-template <int kPairVecs>
 // The states and out may be the same array (sources are read, distinct
 // destinations are written), so neither is declared __restrict__.
+template <int kPairVecs>
 __global__ void __launch_bounds__(128) gf2_apply_pairs_kernel(MatSet mats, const uint32_t* __restrict__ src,
                                                               const uint32_t* __restrict__ dst, uint32_t* out, int cols, bool early)
 {
@@ -368,9 +368,10 @@ struct Tables {
 std::mutex g_tab_mu;
 Tables g_tabs[64][3];  // per device, per matrix family
 
-// Device memory of the odd multiples and the FP4 copies, which 64 exponents of
-// three families would take 7 GiB of; the limit is what the powers' FP8 copies
-// of an earlier form could take.
+// Device memory of the odd multiples and the FP4 copies.  64 exponents of three
+// families would take 7 GiB; a server of the default size needs 0.6 GiB of one
+// family, so the limit leaves each of them as many exponents as calls of up to
+// 2^37 words have.
 std::atomic<size_t> g_derived[64];
 
 size_t derived_limit()

@@ -680,11 +680,13 @@ private:
 
     // Shortest piece a new batch may cut its calls into, from the words the
     // GPU already has in flight: cutting shortens one call's critical path
-    // but costs jump-ahead work (about 2.2e4 words' worth per piece), which
-    // only pays while the GPU would otherwise idle.  B is about 1.5 ms of
-    // work: 2^18 words for each of 32 warps per SM.  2^15 only while the GPU
-    // is nearly idle (below B/32): at about a third of the GPU's rate the
-    // extra jump-ahead of 2^15-word pieces tripled the p99 against 2^16.
+    // but costs jump-ahead work, which only pays while the GPU would otherwise
+    // idle: 5 ns of the whole GPU per piece in large steps, 4.6e3 words' worth.
+    // The limits were measured when it was 25 ns and have not been since.  B is
+    // about 1.5 ms of work: 2^18 words for each of 32 warps per SM.  2^15 only
+    // while the GPU is nearly idle (below B/32): at about a third of the GPU's
+    // rate the extra jump-ahead of 2^15-word pieces then tripled the p99 against
+    // 2^16.
     uint64_t min_piece_for_backlog() const
     {
         const uint64_t B = (uint64_t)c_->sm_count * 32 * (uint64_t(1) << 18);
