@@ -55,6 +55,7 @@ xg_status xg_w64_params(uint32_t* host_rsabcd6, uint64_t* omega);
  * all zero until seeded.  weyl_on: 1 for Eq. (1), 0 for the bare recurrence.
  * cuda_stream: the CUDA stream for all work (NULL: legacy default stream). */
 xg_status xg_w64_create(xg_w64_ctx** out, uint32_t n_streams, uint32_t weyl_on, void* cuda_stream);
+/* As xg_destroy (a failure not reported yet is XG_EDEVICE; all is freed). */
 xg_status xg_w64_destroy(xg_w64_ctx* ctx);
 xg_status xg_w64_set_stream(xg_w64_ctx* ctx, void* cuda_stream);
 
